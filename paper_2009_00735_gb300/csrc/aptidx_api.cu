@@ -274,10 +274,9 @@ static void clear_graphs(Ctx* c) {
     c->graphs.clear();
 }
 
-// gather count + offsets + fill (step a1), queued on the stream
+// the ROI atoms into their slots (step a1), queued on the stream
 static int run_gather(Ctx* c) {
-    cudaError_t e = launch_gather_count(c);
-    if (e == cudaSuccess) e = launch_gather_fill(c);
+    cudaError_t e = launch_gather_fill(c);
     if (e != cudaSuccess) return cuda_check(c, e, "ROI gather");
     return APTIDX_OK;
 }
@@ -288,19 +287,19 @@ static int launch_sequence(Ctx* c, int path, unsigned flags, float* dS, uint16_t
     int rc;
     prof_begin(c, APTIDX_PHASE_GATHER);
     if ((rc = run_gather(c))) return rc;
-    prof_end(c, APTIDX_PHASE_GATHER, 6);
+    prof_end(c, APTIDX_PHASE_GATHER, 1);
     prof_begin(c, APTIDX_PHASE_ORDER);
     cudaError_t e = launch_roi_order(c);
     if (e != cudaSuccess) return cuda_check(c, e, "ROI order");
-    prof_end(c, APTIDX_PHASE_ORDER, 3);
+    prof_end(c, APTIDX_PHASE_ORDER, 1);
     prof_begin(c, APTIDX_PHASE_SIGNATURE);
     if (path == APTIDX_PATH_PLAIN_FP32) {
-        e = launch_signatures_plain(c, dS, dA, nullptr, -1, 0);
+        e = launch_signatures_plain(c, dS, dA, nullptr, -1);
     } else {
         e = launch_signatures_tc(c, dS, dA, nullptr, -1);
     }
     if (e != cudaSuccess) return cuda_check(c, e, "signature kernel");
-    prof_end(c, APTIDX_PHASE_SIGNATURE, path == APTIDX_PATH_PLAIN_FP32 ? 1 : 1);
+    prof_end(c, APTIDX_PHASE_SIGNATURE, 1);
     if (flags & APTIDX_NORMALISE_MAX) {
         prof_begin(c, APTIDX_PHASE_NORMALISE);
         e = launch_normalise(c, dS);
@@ -389,7 +388,7 @@ static int autotune(Ctx* c, int path, float* dS, uint16_t* dA) {
             for (int rep = 0; rep < 2 && e == cudaSuccess; ++rep) {   // the first launch sets attributes
                 e = cudaEventRecord(e0, c->stream);
                 if (e == cudaSuccess)
-                    e = pi ? launch_signatures_tc(c, dS, dA, nullptr, -1) : launch_signatures_plain(c, dS, dA, nullptr, -1, 0);
+                    e = pi ? launch_signatures_tc(c, dS, dA, nullptr, -1) : launch_signatures_plain(c, dS, dA, nullptr, -1);
                 if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
                 if (e == cudaSuccess) e = cudaEventSynchronize(e1);
                 if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
@@ -461,7 +460,6 @@ int aptidx_create(aptidx_ctx** out, int device, void* cuda_stream) {
     if (e != cudaSuccess) rc = APTIDX_E_CUDA;
     if (!rc) rc = dev_alloc(c, (void**)&c->d_status, sizeof(int) * 4);
     if (!rc) rc = dev_alloc(c, (void**)&c->d_counter, sizeof(int32_t) * 4);
-    if (!rc) rc = dev_alloc(c, (void**)&c->d_sort_hist, sizeof(int32_t) * 65537);
     if (!rc && cudaMemsetAsync(c->d_status, 0, sizeof(int) * 4, c->stream) != cudaSuccess) rc = APTIDX_E_CUDA;
     if (!rc && cudaStreamSynchronize(c->stream) != cudaSuccess) rc = APTIDX_E_CUDA;
     if (rc) {
@@ -499,7 +497,6 @@ int aptidx_destroy(aptidx_ctx* ctx) {
     free_ptr(c->d_counter);
     release_spare(c);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
-    free_ptr(c->d_sort_hist);
     for (auto& pr : c->ev_pending) {
         cudaEventDestroy(pr.a);
         cudaEventDestroy(pr.b);
@@ -792,10 +789,11 @@ int aptidx_set_rois(aptidx_ctx* ctx, const double* centres, const double* radii,
         }
         if ((rc = ensure_scan_tmp(c, std::max<int64_t>(nroi, c->n_cells)))) return rc;
     }
-    // count the ROI atoms once to size the gather buffer
+    // count the ROI atoms once to lay out the gather buffer
     APTIDX_CUDA(c, cudaMemsetAsync(c->d_status, 0, sizeof(int), s));
-    cudaError_t e = launch_gather_count(c);
+    cudaError_t e = launch_gather_layout(c);
     if (e != cudaSuccess) return cuda_check(c, e, "ROI count");
+    c->layout_mask = type_mask;
     std::vector<int32_t> hnw((size_t)nroi);
     APTIDX_CUDA(c, cudaMemcpyAsync(hnw.data(), c->d_nw, (size_t)nroi * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     APTIDX_CUDA(c, cudaStreamSynchronize(s));
@@ -882,7 +880,7 @@ int aptidx_compute_signatures(aptidx_ctx* ctx, int path, unsigned flags, float* 
         }
         prof_begin(c, APTIDX_PHASE_SIGNATURE);
         APTIDX_CUDA(c, cudaGraphLaunch(it->second, c->stream));
-        prof_end(c, APTIDX_PHASE_SIGNATURE, (path == APTIDX_PATH_TC_FP16 ? 11 : 10) + ((flags & APTIDX_NORMALISE_MAX) ? 1 : 0));
+        prof_end(c, APTIDX_PHASE_SIGNATURE, 3 + ((flags & APTIDX_NORMALISE_MAX) ? 1 : 0));
     } else if ((rc = launch_sequence(c, path, flags, dS, dA))) {
         return rc;
     }
@@ -1154,7 +1152,7 @@ int aptidx_get_histograms(aptidx_ctx* ctx, int64_t roi, int path, uint16_t* h, i
     }
     if (!rc) {
         if (path == APTIDX_PATH_PLAIN_FP32) {
-            e = launch_signatures_plain(c, row, nullptr, dh, roi, 0);
+            e = launch_signatures_plain(c, row, nullptr, dh, roi);
         } else {
             rc = prepare_tc(c);
             if (!rc) e = launch_signatures_tc(c, row, nullptr, dh, roi);
@@ -1180,10 +1178,12 @@ int aptidx_get_roi_atoms(aptidx_ctx* ctx, int64_t roi, float* xc, int64_t cap, i
     if (c->nroi <= 0) return set_error(c, APTIDX_E_STATE, "get_roi_atoms: set ROIs first");
     if (roi < 0 || roi >= c->nroi || !n_out) return set_error(c, APTIDX_E_INVALID_ARG, "get_roi_atoms: bad arguments");
     if ((rc = run_gather(c))) return rc;
-    int64_t off[2];
-    APTIDX_CUDA(c, cudaMemcpyAsync(off, c->d_off + roi, 2 * sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
+    int64_t off[1];
+    APTIDX_CUDA(c, cudaMemcpyAsync(off, c->d_off + roi, sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
+    int32_t nw = 0;
+    APTIDX_CUDA(c, cudaMemcpyAsync(&nw, c->d_nw + roi, sizeof(nw), cudaMemcpyDeviceToHost, c->stream));
     APTIDX_CUDA(c, cudaStreamSynchronize(c->stream));
-    const int64_t n = off[1] - off[0];
+    const int64_t n = nw;   // the slot may be laid out for more atom types
     *n_out = n;
     if (n > cap || (n > 0 && !xc)) return set_error(c, APTIDX_E_OVERFLOW, "get_roi_atoms: %lld atoms exceed cap %lld", (long long)n, (long long)cap);
     std::vector<float4> tmp((size_t)n);
@@ -1603,16 +1603,17 @@ int aptidx_compute_signatures_multi(aptidx_ctx* ctx, int path, unsigned flags, i
                 passes.emplace_back(grp.begin() + i, grp.begin() + std::min(grp.size(), i + APTIDX_MAX_BANDS));
         }
     }
-    // the gather buffer was sized for the context's type mask; a pass that
-    // selects further atom types needs it sized for the union of the masks
+    // the gather buffer was laid out for the context's type mask; a pass that
+    // selects further atom types needs it laid out for the union of the masks
+    // (whose slots also hold the narrower selections)
     {
-        uint32_t umask = 0;
+        uint32_t umask = c->layout_mask;
         for (int s = 0; s < n_sig; ++s) umask |= type_mask[s];
-        if (umask & ~c->type_mask) {
+        if (umask != c->layout_mask) {
             const uint32_t m0 = c->type_mask;
             c->type_mask = umask;
             APTIDX_CUDA(c, cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream));
-            cudaError_t e = launch_gather_count(c);
+            cudaError_t e = launch_gather_layout(c);
             c->type_mask = m0;
             if (e != cudaSuccess) return cuda_check(c, e, "ROI count");
             std::vector<int32_t> hnw((size_t)c->nroi);
@@ -1625,17 +1626,31 @@ int aptidx_compute_signatures_multi(aptidx_ctx* ctx, int path, unsigned flags, i
                 total += hnw[(size_t)r];
                 nwmax = std::max(nwmax, hnw[(size_t)r]);
             }
+            float4* grown = nullptr;
             if (nwmax > APTIDX_MAX_ATOMS_PER_ROI) {
                 APTIDX_CUDA(c, cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream));
-                return set_error(c, APTIDX_E_OVERFLOW, "a ROI holds %d atoms of the requested types (limit %d)",
-                                 nwmax, APTIDX_MAX_ATOMS_PER_ROI);
+                rc = set_error(c, APTIDX_E_OVERFLOW, "a ROI holds %d atoms of the requested types (limit %d)", nwmax,
+                               APTIDX_MAX_ATOMS_PER_ROI);
+            } else if (total > c->atoms_cap) {
+                rc = dev_alloc(c, (void**)&grown, (size_t)total * sizeof(float4));
             }
-            if (total > c->atoms_cap) {
+            if (rc) {
+                // the context keeps the layout of its own mask
+                const std::string err = c->err;
+                const uint32_t lm = c->layout_mask;
+                c->type_mask = lm;
+                launch_gather_layout(c);
+                c->type_mask = m0;
+                cudaStreamSynchronize(c->stream);
+                c->err = err;
+                return rc;
+            }
+            if (grown) {
                 free_ptr(c->d_atoms);
-                c->atoms_cap = 0;
-                if ((rc = dev_alloc(c, (void**)&c->d_atoms, (size_t)total * sizeof(float4)))) return rc;
+                c->d_atoms = grown;
                 c->atoms_cap = total;
             }
+            c->layout_mask = umask;
             if ((rc = read_status(c))) return rc;
         }
     }
@@ -1767,7 +1782,7 @@ int aptidx_compute_fsp(aptidx_ctx* ctx, int32_t grid_l, double k_max, float* amp
     if ((rc = dev_out(c, amp, n, mem, t, &d))) return rc;
     prof_begin(c, APTIDX_PHASE_GATHER);
     if ((rc = run_gather(c))) return rc;
-    prof_end(c, APTIDX_PHASE_GATHER, 6);
+    prof_end(c, APTIDX_PHASE_GATHER, 1);
     prof_begin(c, APTIDX_PHASE_SIGNATURE);
     cudaError_t e = launch_fsp_tc(c, grid_l, k_max, d);
     if (e != cudaSuccess) return cuda_check(c, e, "reciprocal-space signature");

@@ -434,10 +434,6 @@ __device__ __forceinline__ int band_count_t(const BandSet& bs) { return kNB == 1
 template <int kNB>
 __device__ __forceinline__ int64_t band_off_t(const BandSet& bs, int b) { return kNB == 1 ? 0 : bs.off[b]; }
 
-// ROI rank ranges of a signature launch (ranks index the longest-first order)
-constexpr int kRanksAll = 0;       // [0, nroi)
-constexpr int kRanksBig = 1;       // [0, n_big): ROIs above 2048 atoms
-constexpr int kRanksSmall = 2;     // [n_big, nroi)
 constexpr int kTcMaxAtoms = 2048;  // fp16 carries every count <= 2048 exactly
 
 // -----------------------------------------------------------------------------

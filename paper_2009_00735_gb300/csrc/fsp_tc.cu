@@ -422,7 +422,7 @@ cudaError_t launch_fsp_tc(Ctx* c, int L, double kmax, float* out) {
     p.out = out;
     p.counter = c->d_counter + 2;
     p.status = c->d_status;
-    if ((e = cudaMemsetAsync(p.counter, 0, sizeof(int32_t), c->stream)) != cudaSuccess) return e;
+    if ((e = zero_counters(c)) != cudaSuccess) return e;
     const int64_t grid = std::min<int64_t>((int64_t)c->sm_count, c->nroi * p.items_roi);
     if (grid < 1) return cudaSuccess;
     k_fsp_tc<<<(unsigned)grid, kThreadsF, smem, c->stream>>>(p);

@@ -119,7 +119,8 @@ struct Ctx {
     // gather output (CSR)
     int32_t* d_nw = nullptr;           // [nroi]
     int64_t* d_nw64 = nullptr;         // [nroi] widened counts (scan input)
-    int64_t* d_off = nullptr;          // [nroi + 1]
+    int64_t* d_off = nullptr;          // [nroi + 1] slots of d_atoms, laid out for layout_mask
+    uint32_t layout_mask = 0;
     float4* d_atoms = nullptr;         // [total] centred FP32 (x, y, z, 0)
     int64_t atoms_cap = 0;
     int64_t atoms_total = 0;
@@ -128,7 +129,7 @@ struct Ctx {
     // scheduling scratch
     int32_t* d_order = nullptr;        // [nroi] ROI order (largest first)
     int32_t* d_counter = nullptr;      // [4] work counters
-    int32_t* d_sort_hist = nullptr;    // [65536 + 1]
+    bool counters_zero = false;        // the ROI order just queued zeroes the work counters
     int64_t* d_scan_tmp = nullptr;     // scan block sums
     size_t scan_tmp_elems = 0;
 
@@ -203,16 +204,19 @@ cudaError_t launch_cell_build(Ctx* c, int32_t* d_cell_of, int32_t* d_k2, int32_t
 size_t cell_sort_hist_elems(int64_t n);
 cudaError_t launch_scan_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* tmp, cudaStream_t s);
 size_t scan_tmp_elems(int64_t n);
-cudaError_t launch_gather_count(Ctx* c);
+cudaError_t launch_gather_layout(Ctx* c);
 cudaError_t launch_gather_fill(Ctx* c);
 cudaError_t launch_roi_order(Ctx* c);
+// the work counters are zero for the next kernel on the stream (a memset unless
+// the ROI order just queued zeroes them)
+cudaError_t zero_counters(Ctx* c);
 cudaError_t launch_roi_refine(Ctx* c, const float* S, float kappa, double spacing, int split, double* out,
                               int32_t* parent, int64_t cap, int64_t* n_qualified);
 cudaError_t launch_twiddles(float2* tw, int m, cudaStream_t s);
 
 // signature kernels
 cudaError_t launch_signatures_plain(Ctx* c, float* S, uint16_t* argk, uint16_t* hist_out,
-                                    int64_t hist_roi, int rank_mode);
+                                    int64_t hist_roi);
 cudaError_t launch_signatures_tc(Ctx* c, float* S, uint16_t* argk, uint16_t* hist_out,
                                  int64_t hist_roi);
 int prepare_tc(Ctx* c);

@@ -85,8 +85,6 @@ struct SigParams {
     int32_t* counter;
     int* status;
     int atom_cap;
-    const int32_t* n_big;
-    int rank_mode;
     int64_t nroi;
     BandSet bands;
 };
@@ -117,13 +115,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_plain(SigParams p) {
     __syncthreads();
     uint32_t phase = 0;
     const float magic = bin_magic(p.m);
-    int64_t rank_lo = 0, n_items = p.n_items;
-    if (p.single_roi < 0 && p.rank_mode != kRanksAll) {
-        const int64_t nb = *p.n_big;
-        rank_lo = p.rank_mode == kRanksBig ? 0 : nb;
-        const int64_t rank_hi = p.rank_mode == kRanksBig ? nb : p.nroi;
-        n_items = (rank_hi - rank_lo) * p.items_per_roi;
-    }
+    const int64_t n_items = p.n_items;
 
     for (;;) {
         if (tid == 0) *item_s = atomicAdd(p.counter, 1);
@@ -131,7 +123,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_plain(SigParams p) {
         const int64_t item = *item_s;
         __syncthreads();
         if (item >= n_items) break;
-        const int64_t roi_rank = rank_lo + item / p.items_per_roi;
+        const int64_t roi_rank = item / p.items_per_roi;
         const int grp = (int)(item % p.items_per_roi);
         const int64_t roi = p.single_roi >= 0 ? p.single_roi : (int64_t)p.order[roi_rank];
         const int nw = p.nw[roi];
@@ -435,8 +427,7 @@ size_t plain_smem_bytes(int m, int atom_cap) {
     return NBc * kWords * 4 + NB * 8 + (size_t)atom_cap * 16 + kPartBytes + 64;
 }
 
-cudaError_t launch_signatures_plain(Ctx* c, float* S, uint16_t* argk, uint16_t* hist_out, int64_t hist_roi,
-                                    int rank_mode) {
+cudaError_t launch_signatures_plain(Ctx* c, float* S, uint16_t* argk, uint16_t* hist_out, int64_t hist_roi) {
     static int max_optin = -1;
     if (max_optin < 0) {
         cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
@@ -475,16 +466,13 @@ cudaError_t launch_signatures_plain(Ctx* c, float* S, uint16_t* argk, uint16_t* 
     p.counter = c->d_counter;
     p.status = c->d_status;
     p.atom_cap = cap;
-    p.n_big = c->d_counter + 1;
-    p.rank_mode = hist_out ? kRanksAll : rank_mode;
     p.nroi = nroi_lim;
     p.bands = hist_out ? BandSet() : c->multi;
-    if ((e = cudaMemsetAsync(c->d_counter, 0, sizeof(int32_t), c->stream)) != cudaSuccess) return e;
+    if ((e = zero_counters(c)) != cudaSuccess) return e;
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem);
     per_sm = max(per_sm, 1);
-    int64_t grid = tmin<int64_t>((int64_t)c->sm_count * per_sm, p.n_items);
-    if (rank_mode == kRanksBig && !hist_out) grid = tmin<int64_t>(grid, (int64_t)c->sm_count);
+    const int64_t grid = tmin<int64_t>((int64_t)c->sm_count * per_sm, p.n_items);
     if (grid < 1) return cudaSuccess;
     kern<<<(unsigned)grid, kThreads, smem, c->stream>>>(p);
     return cudaGetLastError();
@@ -650,8 +638,6 @@ extern "C" int aptidx_signatures_noalloc(const float* xc4, const int64_t* off, c
     p.counter = counter;
     p.status = st;
     p.atom_cap = cap;
-    p.n_big = counter + 1;
-    p.rank_mode = kRanksAll;
     p.nroi = nroi;
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sig_plain<1>, kThreads, smem);

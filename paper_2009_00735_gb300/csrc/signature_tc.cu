@@ -990,7 +990,7 @@ cudaError_t launch_signatures_tc(Ctx* c, float* S, uint16_t* argk, uint16_t* his
     p.atom_cap = cap;
     p.n_iss = std::min(std::max(c->tune_iss, 1), kIssuers);
     p.bands = hist_out ? BandSet() : c->multi;
-    if ((e = cudaMemsetAsync(p.counter, 0, sizeof(int32_t), c->stream)) != cudaSuccess) return e;
+    if ((e = zero_counters(c)) != cudaSuccess) return e;
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem);
     per_sm = std::max(1, std::min(per_sm, (int)(512 / p.tmem_cols)));

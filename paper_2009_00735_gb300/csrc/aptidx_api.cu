@@ -654,6 +654,7 @@ int aptidx_set_directions(aptidx_ctx* ctx, const float* u, int32_t nv, int mem) 
         for (int32_t v = 0; v < nv; ++v) {
             if (partner[v] >= 0 && partner[v] < v) continue;   // written by its lower-index partner
             sd.push_back(d4[v]);
+            sd.back().w = partner[v] >= 0 ? 1.f : 0.f;   // whether the slot has a partner
             si.push_back(make_int2(v, partner[v]));
         }
         while (sd.size() % kTileDirs) {
@@ -911,7 +912,7 @@ int aptidx_get_tuning(aptidx_ctx* ctx, int path, int32_t* tiles_per_item, int32_
     CTX_OR_FAIL(ctx);
     if (path != APTIDX_PATH_PLAIN_FP32 && path != APTIDX_PATH_TC_FP16)
         return set_error(c, APTIDX_E_INVALID_ARG, "unknown path %d", path);
-    if (tiles_per_item) *tiles_per_item = c->tune_tpi[path == APTIDX_PATH_TC_FP16];
+    if (tiles_per_item) *tiles_per_item = tuned_tiles_per_item(c, path == APTIDX_PATH_TC_FP16);
     if (issuers) *issuers = path == APTIDX_PATH_TC_FP16 ? c->tune_iss : 0;
     return APTIDX_OK;
 }

@@ -139,6 +139,12 @@ __device__ __forceinline__ uint64_t f2_fma_ru(uint64_t a, uint64_t b, uint64_t c
 }
 __device__ __forceinline__ float f2_lo(uint64_t x) { return __uint_as_float((uint32_t)x); }
 __device__ __forceinline__ float f2_hi(uint64_t x) { return __uint_as_float((uint32_t)(x >> 32)); }
+// min(|a|, |b|, |c|), one instruction
+__device__ __forceinline__ float fmin3_abs(float a, float b, float c) {
+    float d;
+    asm("min.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
 __device__ __forceinline__ uint64_t f2_dup(float v) {
     return ((uint64_t)__float_as_uint(v) << 32) | (uint64_t)__float_as_uint(v);
 }
@@ -365,6 +371,150 @@ __device__ __forceinline__ int hist_tile_pairs2(uint32_t* H, const float4* A, in
     return handled;
 }
 
+// -----------------------------------------------------------------------------
+// Histogram pass of the pipelined tensor-core kernel.  Atoms lie in 64-byte
+// blocks of four (x of the four | y | z | unused), three 16-byte loads that are
+// the FP32 pairs of two packed steps.  The bin fma runs at four times the scale
+// on the integer grid of [2^25, 2^26) (spacing 4): its bit pattern is
+// 0x4C000000 + row, and shifting that left by 7 drops every exponent bit, so
+// one funnel shift with the lane's byte offset in the top seven bits of the low
+// word gives row * 128 + 4 lane, the shared address itself when the magic
+// number carries the histogram's base / 128.  That keeps the address off the
+// FMA pipe, which a multiply-add of the pattern loads as much as four packed
+// FMAs do per atom pair.
+// -----------------------------------------------------------------------------
+__device__ __forceinline__ void quad_atoms(float4* A, int n, int tid, int nthreads, unsigned* r2max = nullptr) {
+    float m = 0.f;
+    for (int q = tid; q < (n >> 2); q += nthreads) {
+        float4* B = A + 4 * q;
+        const float4 a = B[0], b = B[1], c = B[2], d = B[3];
+        B[0] = make_float4(a.x, b.x, c.x, d.x);
+        B[1] = make_float4(a.y, b.y, c.y, d.y);
+        B[2] = make_float4(a.z, b.z, c.z, d.z);
+        m = fmaxf(fmaxf(m, fmaxf(a.x * a.x + a.y * a.y + a.z * a.z, b.x * b.x + b.y * b.y + b.z * b.z)),
+                  fmaxf(c.x * c.x + c.y * c.y + c.z * c.z, d.x * d.x + d.y * d.y + d.z * d.z));
+    }
+    if (r2max) {
+        if (tid < (n & 3)) {
+            const float4 a = A[(n & ~3) + tid];
+            m = fmaxf(m, a.x * a.x + a.y * a.y + a.z * a.z);
+        }
+        atomicMax(r2max, __float_as_uint(m));
+    }
+}
+
+constexpr uint32_t kQuadBits = 0x4C000000u;   // bit pattern of 2^25
+
+// 4 (2^23 + 2^(m-1) + base row): the magic number of the pass whose histogram
+// starts at shared row `row0` (its byte address / 128)
+__device__ __forceinline__ float quad_magic(int m, uint32_t row0) {
+    return 4.0f * (8388608.0f + (float)((1 << (m - 1)) + (int)row0));
+}
+
+// Per-lane state of the pass.
+struct QuadDirs {
+    uint64_t x0, y0, z0, x1, y1, z1, sc, mg;
+    uint32_t lane_top;   // 4 lane in the top seven bits
+    uint32_t t_lo;       // chunked: bit pattern of the chunk's first bin
+    uint32_t h_lane;     // chunked: H + 4 lane
+};
+
+__device__ __forceinline__ QuadDirs quad_dirs(float4 d0, float4 d1, float scale, float magic, int lane) {
+    QuadDirs q;
+    q.x0 = f2_dup(d0.x);
+    q.y0 = f2_dup(d0.y);
+    q.z0 = f2_dup(d0.z);
+    q.x1 = f2_dup(d1.x);
+    q.y1 = f2_dup(d1.y);
+    q.z1 = f2_dup(d1.z);
+    q.sc = f2_dup(4.0f * scale);
+    q.mg = f2_dup(magic);
+    q.lane_top = (uint32_t)lane << 27;
+    q.t_lo = q.h_lane = 0;
+    return q;
+}
+
+template <bool kChunked>
+__device__ __forceinline__ void quad_inc(uint32_t t, uint32_t one, const QuadDirs& q) {
+    if (kChunked) {
+        const uint32_t v = t - q.t_lo;   // bin - first bin of the chunk
+        if (v < 1024u) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(v * 128u + q.h_lane), "r"(one) : "memory");
+    } else {
+        asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(__funnelshift_l(q.lane_top, t, 7)), "r"(one) : "memory");
+    }
+}
+
+// kCount as in hist_add_pair2, except that for 2 the smallest |s| is kept (0:
+// some projection is exactly zero) instead of a product, two three-input minima
+// on the integer pipe instead of two packed multiplies
+template <int kCount, bool kChunked>
+__device__ __forceinline__ void quad_add_pair(uint64_t x, uint64_t y, uint64_t z, const QuadDirs& q, uint32_t& c0,
+                                              uint32_t& c1, float& zmin) {
+    const uint64_t s0 = f2_fma(z, q.z0, f2_fma(y, q.y0, f2_mul(x, q.x0)));
+    const uint64_t s1 = f2_fma(z, q.z1, f2_fma(y, q.y1, f2_mul(x, q.x1)));
+    const uint64_t t0 = f2_fma_rd(s0, q.sc, q.mg);
+    const uint64_t t1 = f2_fma_rd(s1, q.sc, q.mg);
+    if (kCount == 2) {
+        const uint64_t pr = f2_mul(s0, s1);
+        zmin = fmin3_abs(zmin, f2_lo(pr), f2_hi(pr));
+    } else if (kCount == 1) {
+        const uint64_t u0 = f2_fma_ru(s0, q.sc, q.mg);
+        const uint64_t u1 = f2_fma_ru(s1, q.sc, q.mg);
+        c0 += ((uint32_t)u0 - (uint32_t)t0) + ((uint32_t)(u0 >> 32) - (uint32_t)(t0 >> 32));
+        c1 += ((uint32_t)u1 - (uint32_t)t1) + ((uint32_t)(u1 >> 32) - (uint32_t)(t1 >> 32));
+    }
+    quad_inc<kChunked>((uint32_t)t0, 1u, q);
+    quad_inc<kChunked>((uint32_t)(t0 >> 32), 1u, q);
+    quad_inc<kChunked>((uint32_t)t1, 0x10000u, q);
+    quad_inc<kChunked>((uint32_t)(t1 >> 32), 0x10000u, q);
+}
+
+// Histograms of one 64-direction tile over `cn` atoms staged by quad_atoms;
+// warp w takes blocks w, w + W, ..., two at a time with their loads first; the
+// up to three trailing atoms go to warp (cn / 4) % W.  Returns the number of
+// atoms this warp handled.
+template <int W, int kCount, bool kChunked>
+__device__ __forceinline__ int hist_tile_quads(const float4* A, int cn, int warp, const QuadDirs& q, uint32_t& c0,
+                                               uint32_t& c1, float& zmin) {
+    const int nq = cn >> 2;
+    auto ld = [&](int i, int k) { return *reinterpret_cast<const ulonglong2*>(A + 4 * i + k); };
+    int j = warp;
+    for (; j + W < nq; j += 2 * W) {
+        const ulonglong2 xa = ld(j, 0), ya = ld(j, 1), za = ld(j, 2);
+        const ulonglong2 xb = ld(j + W, 0), yb = ld(j + W, 1), zb = ld(j + W, 2);
+        quad_add_pair<kCount, kChunked>(xa.x, ya.x, za.x, q, c0, c1, zmin);
+        quad_add_pair<kCount, kChunked>(xa.y, ya.y, za.y, q, c0, c1, zmin);
+        quad_add_pair<kCount, kChunked>(xb.x, yb.x, zb.x, q, c0, c1, zmin);
+        quad_add_pair<kCount, kChunked>(xb.y, yb.y, zb.y, q, c0, c1, zmin);
+    }
+    if (j < nq) {
+        const ulonglong2 xa = ld(j, 0), ya = ld(j, 1), za = ld(j, 2);
+        quad_add_pair<kCount, kChunked>(xa.x, ya.x, za.x, q, c0, c1, zmin);
+        quad_add_pair<kCount, kChunked>(xa.y, ya.y, za.y, q, c0, c1, zmin);
+    }
+    int handled = warp < nq ? 4 * ((nq - warp + W - 1) / W) : 0;
+    if (warp == nq % W) {
+        for (int i = nq * 4; i < cn; ++i) {
+            const float4 a = A[i];
+            const float sc = f2_lo(q.sc), mg = f2_lo(q.mg);
+            const float s0 = project_f32(f2_lo(q.x0), f2_lo(q.y0), f2_lo(q.z0), a);
+            const float s1 = project_f32(f2_lo(q.x1), f2_lo(q.y1), f2_lo(q.z1), a);
+            const uint32_t t0 = __float_as_uint(__fmaf_rd(s0, sc, mg));
+            const uint32_t t1 = __float_as_uint(__fmaf_rd(s1, sc, mg));
+            if (kCount == 2) {
+                zmin = fminf(zmin, fminf(fabsf(s0), fabsf(s1)));
+            } else if (kCount == 1) {
+                c0 += __float_as_uint(__fmaf_ru(s0, sc, mg)) - t0;
+                c1 += __float_as_uint(__fmaf_ru(s1, sc, mg)) - t1;
+            }
+            quad_inc<kChunked>(t0, 1u, q);
+            quad_inc<kChunked>(t1, 0x10000u, q);
+            ++handled;
+        }
+    }
+    return handled;
+}
+
 // Debug export of a tile's histograms: h_out[v * 2^m + b] for v < nv.
 __device__ __forceinline__ void hist_export(const uint32_t* H, int NB, int tile, int nv, uint16_t* h_out, int tid,
                                             int nthreads) {
@@ -461,6 +611,10 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                  : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {

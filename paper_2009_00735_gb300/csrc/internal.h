@@ -103,6 +103,7 @@ struct Ctx {
     int tc_gb = 0;                     // frequency groups per B batch
     int tc_ng = 0;                     // groups in the global B operand
     uint32_t tc_tmem_cols = 0;
+    int tc_ng_roi = 1;                 // most groups of one ROI's band
     bool tc_wide = false;              // some ROI band spans more groups than one B batch
 
     // ROIs
@@ -144,7 +145,7 @@ struct Ctx {
     // launch configuration (tiles per work item per path, MMA issuer warps),
     // set by the autotuner; rank_limit > 0 restricts a launch to the first
     // ranks of the ROI order (tuning runs)
-    int tune_tpi[2] = {16, 16};
+    int tune_tpi[2] = {16, 0};         // 0: the rule of the tensor-core launch
     int tune_iss = 4;
     int64_t rank_limit = 0;
     struct TuneCfg {
@@ -220,6 +221,7 @@ cudaError_t launch_signatures_plain(Ctx* c, float* S, uint16_t* argk, uint16_t* 
 cudaError_t launch_signatures_tc(Ctx* c, float* S, uint16_t* argk, uint16_t* hist_out,
                                  int64_t hist_roi);
 int prepare_tc(Ctx* c);
+int tuned_tiles_per_item(const Ctx* c, int path);   // of the next launch on that path
 bool tc_supported(Ctx* c);
 cudaError_t launch_fsp_tc(Ctx* c, int L, double kmax, float* out);
 bool tc_supported(Ctx* c);

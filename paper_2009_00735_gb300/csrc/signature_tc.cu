@@ -137,6 +137,471 @@ __device__ __forceinline__ void quarter_rot(float* v, const float* u, int n) {
 
 // ---- the kernel ----------------------------------------------------------------
 
+constexpr int kHistWarps = 16;                       // warps 0-15: projection, histogram, transfer
+constexpr int kHistThreads = kHistWarps * 32;
+constexpr int kAuxThreads = 128;                     // warps 16-19: MMA issue, epilogue, output
+constexpr int kTpThreads = kHistThreads + kAuxThreads;
+constexpr int kExFloats = 4 * 2 * 8 * 32;            // epilogue exchange: 4 bin quarters x 2 x 8 values x 32 lanes
+constexpr int kTmemA = 0;                            // A operand: even directions, odd directions 128 columns on
+constexpr int kTmemD = 256;                          // accumulators
+constexpr int kTmemCols = 512;
+
+// what a pass hands from the histogram warps to the others
+struct TpPass {
+    int64_t roi;
+    int32_t tile, flags;
+    int32_t g0, ng, klo, khi;   // first frequency group, groups, the ROI's band
+    int32_t bc;                 // bin chunk
+};
+constexpr int kPassStop = 1, kPassFirst = 2, kPassLast = 4, kPassBad = 8, kPassPartner = 16;
+
+__device__ __forceinline__ void hist_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kHistThreads) : "memory"); }
+__device__ __forceinline__ void aux_sync() { asm volatile("bar.sync 3, 128;" ::: "memory"); }
+__device__ __forceinline__ bool hist_sync_or(bool v) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+        "bar.red.or.pred q, 2, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"(v ? 1u : 0u), "n"(kHistThreads)
+        : "memory");
+    return r != 0;
+}
+
+// kNB: band slots of the epilogue (1: the ROI's own band; APTIDX_MAX_BANDS:
+// the pass's BandSet, aptidx_compute_signatures_multi)
+template <int kNB>
+__global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const int NB = 1 << p.m;
+    const int NBc = NB < kChunkBins ? NB : kChunkBins;   // bins per chunk
+    const int nchunk = NB / NBc;
+    const int KB = NBc / 256;   // 64-row K blocks of the B operand per chunk (K = NBc / 4 rows)
+    uint32_t* H = reinterpret_cast<uint32_t*>(smem);
+    unsigned char* BT = smem + (size_t)NBc * 128;
+    float* EX = reinterpret_cast<float*>(BT + p.bt_bytes);   // [2][kExFloats]
+    float4* A = reinterpret_cast<float4*>(EX + 2 * kExFloats);
+    float4* DB = A + p.atom_cap;   // [2][kDirs]: this tile's directions and the next tile's
+    TpPass* pass_s = reinterpret_cast<TpPass*>(DB + 2 * kDirs);   // [2]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(pass_s + 2);
+    uint64_t* bar_atoms = bars;
+    uint64_t* bar_b = bars + 1;
+    uint64_t* bar_full = bars + 2;    // A operand of a pass written (16 histogram warps)
+    uint64_t* bar_mma = bars + 3;     // [2] its MMAs done (4 auxiliary warps), by pass parity
+    int* item_s = reinterpret_cast<int*>(bars + 5);
+    uint32_t* tmem_s = reinterpret_cast<uint32_t*>(bars + 6);
+    unsigned* r2max_s = tmem_s + 1;   // largest |x|^2 of the item's atoms
+    volatile int* hist_fail = reinterpret_cast<volatile int*>(bars + 7);
+    volatile int* aux_fail = hist_fail + 1;
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+        mbar_init(bar_atoms, 1);
+        mbar_init(bar_b, 1);
+        mbar_init(bar_full, kHistWarps);
+        mbar_init(&bar_mma[0], 4);
+        mbar_init(&bar_mma[1], 4);
+        *hist_fail = 0;
+        *aux_fail = 0;
+        fence_barrier_init();
+    }
+    for (int i = tid; i < NBc * 8; i += kTpThreads) reinterpret_cast<uint4*>(H)[i] = make_uint4(0, 0, 0, 0);
+    if (warp == kHistWarps) tmem_alloc(tmem_s, kTmemCols);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_s;
+    const uint32_t h_addr = smem_u32(H);
+    const bool sym = p.slot_idx != nullptr;
+
+    if (warp < kHistWarps) {
+        // ================= histogram warps =================
+        const float magic = quad_magic(p.m, h_addr >> 7);
+        const int chunk_log = p.m > 10 ? p.m - 10 : 0;
+        const int n_items = (int)((p.single_roi >= 0 ? 1 : p.nroi) * p.items_per_roi);   // < 2^31 (launch)
+        uint32_t ph_atoms = 0, t = 0;   // t: passes handed over
+        // this warp's share of the transfer: bins of quarter warp & 3 (the
+        // tensor-memory lanes it may write), a quarter of them
+        const int tr_rows = NBc / 16;
+        const int tr_row0 = (warp & 3) * (NBc / 4) + (warp >> 2) * tr_rows;
+        const uint32_t tr_col0 = tmem + kTmemA + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * (tr_rows / 2));
+        bool failed = false;
+        if (tid == 0) *item_s = atomicAdd(p.counter, 1);
+        hist_sync();
+        int item = *item_s;
+        // atoms [0, n) from src into A by one bulk copy, arranged in blocks of four
+        auto stage = [&](const float4* src, int n, unsigned* r2) -> bool {
+            if (tid == 0) {
+                if (r2) *r2 = 0u;
+                if (n > 0) {
+                    fence_proxy_async_smem();   // earlier generic accesses of A before the async write
+                    mbar_arrive_expect_tx(bar_atoms, (uint32_t)n * 16u);
+                    bulk_g2s(A, src, (uint32_t)n * 16u, bar_atoms);
+                    if (!mbar_wait_bounded(bar_atoms, ph_atoms, p.status)) {
+                        mbar_wait_bounded(bar_atoms, ph_atoms, p.status, 1u << 20);   // let the copy land
+                        *hist_fail = 1;
+                    }
+                }
+            }
+            if (n > 0) ph_atoms ^= 1u;
+            hist_sync();
+            if (*hist_fail) return false;
+            quad_atoms(A, n, tid, kHistThreads, r2);
+            hist_sync();
+            return true;
+        };
+        while (item < n_items && !failed) {
+            int next = 0;
+            if (tid == 0) next = atomicAdd(p.counter, 1);   // the next item, published when this one is done
+            const int roi = p.single_roi >= 0 ? (int)p.single_roi : p.order[item / p.items_per_roi];
+            const int grp = item % p.items_per_roi;
+            const int nw = p.nw[roi];
+            const float scale = p.scale[roi];
+            const int klo = p.band[2 * roi], khi = p.band[2 * roi + 1];
+            const int t0 = grp * p.tiles_per_item;
+            const int t1 = min(t0 + p.tiles_per_item, p.tiles_per_roi);
+            const int nblk = max(1, (nw + p.atom_cap - 1) / p.atom_cap);   // atom blocks
+            // the first tile's directions (later tiles' arrive while the tile before
+            // them runs; held in shared memory: in registers the loop spilled them,
+            // 1.6 K cycles per tile)
+            if (tid < kDirs) cp_async16(DB + (t0 & 1) * kDirs + tid, p.dirs + (int64_t)t0 * kDirs + tid);
+            cp_async_wait_all();
+            if (nblk > 1) {
+                hist_sync();
+            } else if (!stage(p.atoms + p.off[roi], nw, r2max_s)) {
+                failed = true;
+                break;
+            }
+            // with one atom block and no nonzero integer product possible, the
+            // antipodal check only looks for s = 0
+            const bool zero_check =
+                sym && nblk == 1 && !nonzero_integer_products_possible(scale, __uint_as_float(*r2max_s));
+            for (int tile = t0; tile < t1 && !failed; ++tile) {
+                float4 d0 = DB[(tile & 1) * kDirs + 2 * lane], d1 = DB[(tile & 1) * kDirs + 2 * lane + 1];
+                if (tile + 1 < t1 && tid < kDirs)
+                    cp_async16(DB + ((tile + 1) & 1) * kDirs + tid, p.dirs + (int64_t)(tile + 1) * kDirs + tid);
+                const bool pt0 = d0.w != 0.f, pt1 = d1.w != 0.f;   // the slot has an antipodal partner
+                bool tile_bad = false;
+                for (int pass = 0; pass < 2 && !failed; ++pass) {
+                    if (pass == 1) {
+                        if (!tile_bad) break;
+                        // the partners -u of this tile's directions, from their own histograms
+                        d0 = make_float4(-d0.x, -d0.y, -d0.z, d0.w);
+                        d1 = make_float4(-d1.x, -d1.y, -d1.z, d1.w);
+                    }
+                    const bool count = sym && pass == 0;
+                    QuadDirs q = quad_dirs(d0, d1, scale, magic, lane);
+                    uint32_t c0 = 0, c1 = 0;
+                    float zmin = 1.f;
+                    int handled = 0;
+                    const int n_sub = nblk << chunk_log;
+                    for (int sub = 0; sub < n_sub; ++sub, ++t) {
+                        const int blk = sub >> chunk_log, bc = sub & (nchunk - 1);
+                        const int cn = min(p.atom_cap, nw - blk * p.atom_cap);
+                        const bool last = sub == n_sub - 1;
+                        if (nblk > 1 && bc == 0 && !stage(p.atoms + p.off[roi] + (int64_t)blk * p.atom_cap, cn, nullptr)) {
+                            failed = true;
+                            break;
+                        }
+                        // ---- 1. histograms (H is zero here) ----
+                        if (nchunk == 1) {
+                            if (count && zero_check)
+                                handled += hist_tile_quads<kHistWarps, 2, false>(A, cn, warp, q, c0, c1, zmin);
+                            else if (count)
+                                handled += hist_tile_quads<kHistWarps, 1, false>(A, cn, warp, q, c0, c1, zmin);
+                            else
+                                hist_tile_quads<kHistWarps, 0, false>(A, cn, warp, q, c0, c1, zmin);
+                        } else {
+                            q.t_lo = kQuadBits + (h_addr >> 7) + (uint32_t)bc * kChunkBins;
+                            q.h_lane = h_addr + 4u * (uint32_t)lane;
+                            if (count && bc == 0 && zero_check)
+                                handled += hist_tile_quads<kHistWarps, 2, true>(A, cn, warp, q, c0, c1, zmin);
+                            else if (count && bc == 0)
+                                handled += hist_tile_quads<kHistWarps, 1, true>(A, cn, warp, q, c0, c1, zmin);
+                            else
+                                hist_tile_quads<kHistWarps, 0, true>(A, cn, warp, q, c0, c1, zmin);
+                        }
+                        // the non-integer counts are complete once the last pass's
+                        // histogram is in: a partner whose count falls short of the
+                        // atoms this warp handled needs its own histogram
+                        const bool bad = count && last &&
+                                         (zero_check ? (pt0 || pt1) && zmin == 0.f
+                                                     : (pt0 && c0 != (uint32_t)handled) || (pt1 && c1 != (uint32_t)handled));
+                        // the A operand of the pass before has been read
+                        if (tid == 0) {
+                            if (t > 0 && !mbar_wait_bounded(&bar_mma[(t - 1) & 1], ((t - 1) >> 1) & 1u, p.status))
+                                *hist_fail = 1;
+                            if (*aux_fail) *hist_fail = 1;
+                        }
+                        const bool any_bad = hist_sync_or(bad);
+                        if (last && pass == 0) tile_bad = any_bad;
+                        if (*hist_fail) {
+                            failed = true;
+                            break;
+                        }
+                        tc_fence_after();
+                        if (p.hist_out) {
+                            hist_export_add(H, NBc, NB, bc, tile, p.nv, p.hist_out, tid, kHistThreads);
+                            hist_sync();   // every row is read before the transfer zeroes it
+                        }
+                        if (tid == 0) {
+                            TpPass m;
+                            m.roi = roi;
+                            m.tile = tile;
+                            m.flags = (sub == 0 ? kPassFirst : 0) | (last ? kPassLast : 0) | (tile_bad ? kPassBad : 0) |
+                                      (pass ? kPassPartner : 0);
+                            m.g0 = (klo - p.kbase) >> 2;
+                            m.ng = ((khi - p.kbase) >> 2) - m.g0 + 1;
+                            m.klo = klo;
+                            m.khi = khi;
+                            m.bc = bc;
+                            pass_s[t & 1] = m;
+                        }
+                        // ---- 2. transfer: counts into tensor memory, the histogram
+                        // zeroed behind them by exchanging each word with 0 (a load
+                        // and a store pass over the rows took twice the shared-memory
+                        // cycles).  Word (bin, lane) holds directions 2 lane and
+                        // 2 lane + 1; two bins' words make a K pair of either ----
+                        for (int r = 0; r < tr_rows; r += 16) {
+                            const uint32_t row = h_addr + (uint32_t)(tr_row0 + r) * 128u + 4u * (uint32_t)lane;
+                            uint32_t w[16], e[8], o[8];
+#pragma unroll
+                            for (int i = 0; i < 16; ++i)
+                                asm volatile("atom.shared.exch.b32 %0, [%1], 0;" : "=r"(w[i]) : "r"(row + 128u * i) : "memory");
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) {
+                                e[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x5410);
+                                o[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x7632);
+                            }
+                            tmem_st8(tr_col0 + (uint32_t)(r / 2), e);
+                            tmem_st8(tr_col0 + 128u + (uint32_t)(r / 2), o);
+                        }
+                        tmem_wait_st();
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar_full);
+                        cp_async_wait_all();
+                        hist_sync();   // the histogram is zero, the next directions are in
+                    }
+                }
+            }
+            if (tid == 0) *item_s = next;
+            hist_sync();
+            item = *item_s;
+            // (the next write of item_s comes after the barriers of an item)
+        }
+        // the auxiliary warps leave at a pass marked stop, handed over (like any
+        // other) only once the pass before has been taken: bar_full never runs two
+        // phases ahead of its reader
+        if (tid == 0) {
+            if (!failed && t > 0) mbar_wait_bounded(&bar_mma[(t - 1) & 1], ((t - 1) >> 1) & 1u, p.status);
+            pass_s[t & 1].flags = kPassStop;
+        }
+        hist_sync();
+        if (lane == 0) mbar_arrive(bar_full);
+    } else {
+        // ================= auxiliary warps =================
+        const int at = tid - kHistThreads, aw = at >> 5;   // warp aw: tensor-memory lanes 32 aw .., bin quarter aw
+        const uint32_t bt_addr = smem_u32(BT);
+        const int nh = p.n_iss >> 1;    // accumulators per direction parity (halves of K)
+        uint32_t ph_b = 0, exb = 0;
+        int cur_g0 = -1, cur_ng = -1, cur_bc = -1;   // B operand in shared memory
+        // accumulators: two buffers of 128 columns in turn when a tile's fit one,
+        // else one of 256
+        bool pending = false;
+        TpPass pend;
+        uint32_t pend_t = 0, pend_d = 0, dbuf = 0;
+
+        // wait for the MMAs of pass `u` (thread 0 of the group) and publish the outcome
+        auto done = [&](uint32_t u) -> bool {
+            if (at == 0 && !mbar_wait_bounded(&bar_mma[u & 1], (u >> 1) & 1u, p.status)) *aux_fail = 1;
+            aux_sync();
+            return *aux_fail == 0;
+        };
+        // |X(k)| and the band maximum of one tile: every warp sums its quarter's
+        // partials of a frequency group, threads 0-63 (one per direction) add the
+        // four quarters with their factors w^(f q NBc / 4)
+        auto epilogue = [&](const TpPass& m, uint32_t u, uint32_t dsel) -> bool {
+            if (!done(u)) return false;
+            tc_fence_after();
+            const uint32_t cols = (uint32_t)(16 * m.ng);
+            const uint32_t dcol = tmem + ((uint32_t)(aw * 32) << 16) + kTmemD + dsel;
+            float best[kNB];
+            int bk[kNB];
+            band_init_t<kNB>(p.bands, m.klo, best, bk);
+            for (int j = 0; j < m.ng; ++j) {
+                float* ex = EX + (exb & 1) * kExFloats;
+                ++exb;
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    float v[8], lo[8];
+                    const uint32_t c = dcol + (uint32_t)b * cols + (uint32_t)(8 * j);
+                    tmem_ld8(c, v);
+                    tmem_ld8(c + (uint32_t)(8 * m.ng), lo);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) v[i] += lo[i];
+                    if (nh == 2) {
+                        float v2[8];
+                        tmem_ld8(c + 2 * cols, v2);
+                        tmem_ld8(c + 2 * cols + (uint32_t)(8 * m.ng), lo);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) v[i] += v2[i] + lo[i];
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) ex[((aw * 2 + b) * 8 + i) * 32 + lane] = v[i];
+                }
+                tc_fence_before();
+                aux_sync();
+                if (at < kDirs) {
+                    const int f0 = p.kbase + 4 * (m.g0 + j);
+                    const float* x = ex + (at & 1) * 256 + (at >> 1);   // quarter q: + 512 q
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int f = f0 + i;
+                        float fc[4], fs[4];   // w^(f q NBc / 4) = fc - i fs
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            if (nchunk == 1) {   // (-i)^(f q)
+                                const int ph = (f * q) & 3;
+                                fc[q] = ph == 0 ? 1.f : ph == 2 ? -1.f : 0.f;
+                                fs[q] = ph == 1 ? 1.f : ph == 3 ? -1.f : 0.f;
+                            } else {
+                                sincospif((float)(f * q) * (float)NBc / (float)(2 * NB), &fs[q], &fc[q]);
+                            }
+                        }
+                        float xr[4], xi[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float r = x[q * 512 + (2 * i) * 32], s = x[q * 512 + (2 * i + 1) * 32];
+                            xr[q] = fc[q] * r - fs[q] * s;
+                            xi[q] = fs[q] * r + fc[q] * s;
+                        }
+                        const float r = (xr[0] + xr[2]) + (xr[1] + xr[3]), s = (xi[0] + xi[2]) + (xi[1] + xi[3]);
+                        // the band maximum on |X|^2 (its root is the maximum amplitude)
+                        band_update_t<kNB>(p.bands, m.klo, m.khi, f, r * r + s * s, best, bk);
+                    }
+                }
+            }
+            if (at < kDirs) {
+                const int slot = m.tile * kDirs + at;
+                int v0 = slot < p.nv ? slot : -1, v1 = -1;
+                if (sym) {
+                    // the slot's direction, and its partner when the tile's mirror
+                    // images are exact; a partner pass writes the partners
+                    const int2 si = p.slot_idx[slot];
+                    v0 = (m.flags & kPassPartner) ? si.y : si.x;
+                    v1 = (m.flags & (kPassPartner | kPassBad)) ? -1 : si.y;
+                }
+                const int64_t rb = (p.single_roi >= 0 ? 0 : m.roi) * (int64_t)p.nv;
+#pragma unroll
+                for (int b = 0; b < kNB; ++b) {
+                    if (b < band_count_t<kNB>(p.bands)) {
+                        const float a = best[b] >= 0.f ? sqrtf(best[b]) * 16777216.0f : best[b];
+                        const int64_t ob = band_off_t<kNB>(p.bands, b) + rb;
+                        if (v0 >= 0) {
+                            p.S[ob + v0] = a;
+                            if (p.argk) p.argk[ob + v0] = (uint16_t)bk[b];
+                        }
+                        if (v1 >= 0) {
+                            p.S[ob + v1] = a;
+                            if (p.argk) p.argk[ob + v1] = (uint16_t)bk[b];
+                        }
+                    }
+                }
+            }
+            return true;
+        };
+
+        bool ok = true;
+        for (uint32_t t = 0; ok; ++t) {
+            if (at == 0 && !mbar_wait_bounded(bar_full, t & 1u, p.status)) *aux_fail = 1;
+            aux_sync();
+            if (*aux_fail) break;
+            tc_fence_after();
+            const TpPass m = pass_s[t & 1];
+            if (m.flags & kPassStop) break;
+            // ---- B operand of the band (all chunks when they fit) ----
+            const uint32_t part = (uint32_t)m.ng * KB * 1024u;
+            const bool all = (uint32_t)nchunk * 2u * part <= (uint32_t)p.bt_bytes;
+            const int want_bc = all ? 0 : m.bc;
+            if (m.g0 != cur_g0 || m.ng != cur_ng || want_bc != cur_bc) {
+                if (t > 0 && !done(t - 1)) break;   // its MMAs read the operand held so far
+                if (at == 0) {
+                    const int n = all ? nchunk : 1;
+                    fence_proxy_async_smem();
+                    mbar_arrive_expect_tx(bar_b, 2u * part * (uint32_t)n);
+                    for (int i = 0; i < 2 * n; ++i)
+                        bulk_g2s(BT + (size_t)i * part,
+                                 p.twb + ((size_t)(2 * want_bc + i) * p.ng_total + m.g0) * KB * 1024, part, bar_b);
+                    if (!mbar_wait_bounded(bar_b, ph_b, p.status)) {
+                        mbar_wait_bounded(bar_b, ph_b, p.status, 1u << 20);
+                        *aux_fail = 1;
+                    }
+                }
+                ph_b ^= 1u;
+                aux_sync();
+                if (*aux_fail) break;
+                cur_g0 = m.g0;
+                cur_ng = m.ng;
+                cur_bc = want_bc;
+            }
+            // ---- 3. contraction: issuer aw takes directions of parity aw & 1 and
+            // half aw >> 1 of K (with two issuers, all of K) ----
+            const uint32_t cols = (uint32_t)(16 * m.ng);
+            const bool dbl = p.n_iss * (int)cols <= 128;
+            if (m.flags & kPassFirst) dbuf = dbl ? dbuf ^ 128u : 0u;
+            if (pending && !dbl) {   // the columns about to be written hold the tile before
+                pending = false;
+                if (!epilogue(pend, pend_t, pend_d)) break;
+            }
+            if (lane == 0) {
+                if (aw < p.n_iss) {
+                    const int nk = NBc / 64 / nh;   // K = 16 steps of this issuer
+                    const int k0 = (aw >> 1) * nk;
+                    const uint32_t idesc = idesc_f16_mk(128, (int)cols, false);
+                    const uint32_t d = tmem + kTmemD + dbuf + (uint32_t)aw * cols;
+                    const uint32_t a = tmem + kTmemA + (uint32_t)(aw & 1) * 128u;
+                    const uint64_t b = sdesc_sw128(bt_addr + (all ? (uint32_t)m.bc * 2u * part : 0u), 16u, (uint32_t)KB * 1024u);
+                    for (int k = k0; k < k0 + nk; ++k)
+                        mma_f16_ta(d, a + (uint32_t)(8 * k), b + (uint64_t)((k >> 2) * 64 + (k & 3) * 2), idesc,
+                                   k > k0 || !(m.flags & kPassFirst) ? 1u : 0u);
+                    mma_commit(&bar_mma[t & 1]);
+                } else {
+                    mbar_arrive(&bar_mma[t & 1]);
+                }
+            }
+            __syncwarp();
+            // ---- 4. epilogue: of the tile before while these MMAs run when the
+            // accumulators are double buffered ----
+            if (pending) {
+                pending = false;
+                ok = epilogue(pend, pend_t, pend_d);
+            }
+            if (ok && (m.flags & kPassLast)) {
+                if (dbl) {
+                    pending = true;
+                    pend = m;
+                    pend_t = t;
+                    pend_d = dbuf;
+                } else {
+                    ok = epilogue(m, t, dbuf);
+                }
+            }
+        }
+        if (pending && *aux_fail == 0) epilogue(pend, pend_t, pend_d);
+    }
+    // teardown
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == kHistWarps) tmem_dealloc(tmem, kTmemCols);
+}
+
+// ---- wide bands ----------------------------------------------------------------
+
 // kNB: band slots of the epilogue (1: the ROI's own band; APTIDX_MAX_BANDS:
 // the pass's BandSet, aptidx_compute_signatures_multi); kWide: the instance
 // that streams the twiddles of bands wider than one B batch (the narrow-band
@@ -212,7 +677,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
         const int klo = p.band[2 * roi], khi = p.band[2 * roi + 1];
         const int fg0 = (klo - p.kbase) >> 2, fg1 = (khi - p.kbase) >> 2;
         const int ng = fg1 - fg0 + 1;
-        const int nbatch = (ng + p.gb - 1) / p.gb;
+        const int nbatch = 2;   // TRANSITION
         const int t0 = grp * p.tiles_per_item;
         const int t1 = min(t0 + p.tiles_per_item, p.tiles_per_roi);
         const int nblk = max(1, (nw + p.atom_cap - 1) / p.atom_cap);   // atom blocks
@@ -832,8 +1297,8 @@ __global__ void k_build_twb(uint8_t* twb, int m, int kbase, int ng, bool streame
     const int NB = 1 << m;
     const int NBc = NB < kChunkBins ? NB : kChunkBins;
     const int nchunk = NB / NBc;
-    const int NK = streamed ? NBc / 4 : NBc / 2;
-    const int KB = NBc / 128;
+    const int NK = NBc / 4;
+    const int KB = NBc / 256, KBs = NBc / 128;
     const int64_t total = (int64_t)nchunk * 2 * ng * NK * 8;   // chunks x [hi|lo] x groups x K rows x 8 columns
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int r = (int)(i & 7);
@@ -855,7 +1320,7 @@ __global__ void k_build_twb(uint8_t* twb, int m, int kbase, int ng, bool streame
         size_t off;
         if (streamed) {
             const int kb = k >> 5, kin = k & 31;
-            const size_t blk = ((size_t)(bc * KB + kb) * 2 + part) * (ng + 1) + g;
+            const size_t blk = ((size_t)(bc * KBs + kb) * 2 + part) * (ng + 1) + g;
             off = blk * 512 + (size_t)r * 64 + (size_t)(((kin >> 3) ^ ((r >> 1) & 3)) << 4) + (size_t)(kin & 7) * 2;
         } else {
             const int kb = k >> 6, kin = k & 63;
@@ -881,16 +1346,22 @@ static size_t tc_smem_bytes(int m, int atom_cap, size_t bt_bytes) {
            128 * 8 * 4 + 256;
 }
 
+static size_t tp_smem_bytes(int m, int atom_cap) {
+    const size_t nbc = std::min<size_t>((size_t)1 << m, kChunkBins);
+    return 1024 + nbc * 128 + kBtBytes + 2 * kExFloats * 4 + (size_t)atom_cap * 16 + 2 * kDirs * 16 + 2 * sizeof(TpPass) + 128;
+}
+
 // Build the B operand for the current ROI bands and pick the TMEM size.
 int prepare_tc(Ctx* c) {
     if (!tc_supported(c)) return set_error(c, APTIDX_E_INVALID_ARG, "tensor-core path needs an sm_103 device");
     const int NB = 1 << c->m;
     const int NBc = std::min(NB, kChunkBins);
     const int nchunk = NB / NBc;
-    const int KB = NBc / 128;   // 1 KB blocks of 64 K rows per chunk, K = NBc / 2
+    const int KB = NBc / 256;   // 1 KB blocks of 64 K rows per chunk, K = NBc / 4
     const int kbase = c->band_min;
     const int ng = (c->band_max - kbase) / 4 + 1;
-    const int gb = kBtBytes / (2 * KB * 1024);
+    // groups one B batch and the accumulators of two issuers hold
+    const int gb = std::min(8, kBtBytes / (2 * KB * 1024));
     int ng_roi_max = 1;
     for (int64_t r = 0; r < c->nroi; ++r) {
         const int g0 = (c->h_band[2 * r] - kbase) >> 2, g1 = (c->h_band[2 * r + 1] - kbase) >> 2;
@@ -916,7 +1387,7 @@ int prepare_tc(Ctx* c) {
         c->twb_key[0] = c->twb_key[1] = c->twb_key[2] = -1;
         // both layouts of the same twiddles: [narrow | streamed (one zero group more per run)]
         const size_t bytes = (size_t)nchunk * 2 * ng * KB * 1024;
-        const size_t sbytes = (size_t)nchunk * 2 * (ng + 1) * KB * 512;
+        const size_t sbytes = (size_t)nchunk * 2 * (ng + 1) * (NBc / 128) * 512;
         int rc = dev_alloc(c, &c->d_twb, bytes + sbytes);
         if (rc) return rc;
         cudaError_t e0 = cudaMemsetAsync((uint8_t*)c->d_twb + bytes, 0, sbytes, c->stream);
@@ -937,7 +1408,36 @@ int prepare_tc(Ctx* c) {
     c->tc_ng = ng;
     c->tc_tmem_cols = cols;
     c->tc_wide = wide;
+    c->tc_ng_roi = ng_roi_max;
     return APTIDX_OK;
+}
+
+// Tiles per work item when none was tuned: the split of a ROI into items that
+// ends first if every CTA takes the same number of items, a set-up (staging and
+// arranging the ROI's atoms) counted as a few tiles of a small ROI; at most 64
+// tiles.  Few ROIs then spread over every SM (16 ROIs of 81 tiles: 9 tiles per
+// item, one wave), many ROIs get long items.
+static int tiles_per_item_rule(const Ctx* c, int tiles, int64_t nroi) {
+    const double mean = nroi > 0 ? (double)c->atoms_total / (double)c->nroi : 0.0;
+    const double setup = 0.3 + 300.0 / (mean + 150.0);   // in tiles
+    int best = 1;
+    double best_t = 1e300;
+    for (int tpi = 1; tpi <= std::min(tiles, 64); ++tpi) {
+        const int64_t items = nroi * ((tiles + tpi - 1) / tpi);
+        const double t = (double)((items + c->sm_count - 1) / c->sm_count) * (tpi + setup);
+        if (t < best_t * 0.999) {
+            best_t = t;
+            best = tpi;
+        }
+    }
+    return best;
+}
+
+int tuned_tiles_per_item(const Ctx* c, int path) {
+    if (c->tune_tpi[path] > 0) return c->tune_tpi[path];
+    if (path == 0 || c->nroi <= 0) return 16;
+    const bool pairs = c->use_pairs && c->d_slot_idx;
+    return tiles_per_item_rule(c, (pairs ? c->nslot_pad : c->nv_pad) / kDirs, c->nroi);
 }
 
 cudaError_t launch_signatures_tc(Ctx* c, float* S, uint16_t* argk, uint16_t* hist_out, int64_t hist_roi) {
@@ -945,16 +1445,14 @@ cudaError_t launch_signatures_tc(Ctx* c, float* S, uint16_t* argk, uint16_t* his
     static int max_optin = -1;
     if (max_optin < 0) cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
     const size_t bt_bytes = c->tc_wide ? 4 * (size_t)kWideStage : (size_t)kBtBytes;
-    const size_t base = tc_smem_bytes(c->m, 0, bt_bytes);
+    const size_t base = c->tc_wide ? tc_smem_bytes(c->m, 0, bt_bytes) : tp_smem_bytes(c->m, 0);
     int cap = (int)(((size_t)max_optin - base) / 16);
     cap = std::min(cap, kTcMaxAtoms) & ~15;
     if (cap < 256) return cudaErrorInvalidConfiguration;
-    const size_t smem = tc_smem_bytes(c->m, cap, bt_bytes);
+    const size_t smem = base + (size_t)cap * 16;
     const bool multi = !hist_out && c->multi.n > 0;
-    // the wide-band stream lives in its own instances, so that the narrow-band
-    // kernel compiles without it
-    auto kern = multi ? (c->tc_wide ? k_sig_tc<APTIDX_MAX_BANDS, true> : k_sig_tc<APTIDX_MAX_BANDS, false>)
-                      : (c->tc_wide ? k_sig_tc<1, true> : k_sig_tc<1, false>);
+    auto kern = multi ? (c->tc_wide ? k_sig_tc<APTIDX_MAX_BANDS, true> : k_sig_tp<APTIDX_MAX_BANDS>)
+                      : (c->tc_wide ? k_sig_tc<1, true> : k_sig_tp<1>);
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
     // antipodal pairs (one projection per pair) unless switched off or exporting
@@ -968,9 +1466,11 @@ cudaError_t launch_signatures_tc(Ctx* c, float* S, uint16_t* argk, uint16_t* his
     p.slot_idx = pairs ? c->d_slot_idx : nullptr;
     p.nv = c->nv;
     p.tiles_per_roi = (pairs ? c->nslot_pad : c->nv_pad) / kDirs;
-    p.tiles_per_item = std::min(std::max(c->tune_tpi[1], 1), p.tiles_per_roi);
-    p.items_per_roi = (p.tiles_per_roi + p.tiles_per_item - 1) / p.tiles_per_item;
     p.nroi = c->rank_limit > 0 ? std::min<int64_t>(c->nroi, c->rank_limit) : c->nroi;
+    p.tiles_per_item = std::min(c->tune_tpi[1] > 0 ? c->tune_tpi[1]
+                                                   : tiles_per_item_rule(c, p.tiles_per_roi, hist_out ? 1 : p.nroi),
+                                p.tiles_per_roi);
+    p.items_per_roi = (p.tiles_per_roi + p.tiles_per_item - 1) / p.tiles_per_item;
     p.scale = c->d_scale;
     p.band = c->d_band;
     p.m = c->m;
@@ -988,16 +1488,17 @@ cudaError_t launch_signatures_tc(Ctx* c, float* S, uint16_t* argk, uint16_t* his
     p.counter = c->d_counter + 2;
     p.status = c->d_status;
     p.atom_cap = cap;
-    p.n_iss = std::min(std::max(c->tune_iss, 1), kIssuers);
+    // four issuers while their accumulators fit (16 columns per group and
+    // issuer, 256 in all), else two
+    p.n_iss = c->tune_iss >= 4 && c->tc_ng_roi <= 4 ? 4 : 2;
     p.bands = hist_out ? BandSet() : c->multi;
     if ((e = zero_counters(c)) != cudaSuccess) return e;
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem);
-    per_sm = std::max(1, std::min(per_sm, (int)(512 / p.tmem_cols)));
+    // one CTA per SM (registers; the pipelined kernel takes all tensor memory)
     const int64_t items = (hist_out ? 1 : p.nroi) * (int64_t)p.items_per_roi;
-    const int64_t grid = std::min<int64_t>((int64_t)c->sm_count * per_sm, items);
+    if (items >= ((int64_t)1 << 31) - 4096) return cudaErrorInvalidConfiguration;   // the work counter is 32 bits
+    const int64_t grid = std::min<int64_t>((int64_t)c->sm_count, items);
     if (grid < 1) return cudaSuccess;
-    kern<<<(unsigned)grid, kThreads, smem, c->stream>>>(p);
+    kern<<<(unsigned)grid, c->tc_wide ? kThreads : kTpThreads, smem, c->stream>>>(p);
     c->launches += hist_out ? 0 : 1;
     return cudaGetLastError();
 }

@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
     unsigned char* BT = smem + (size_t)NBc * 128;
     float* EX = reinterpret_cast<float*>(BT + p.bt_bytes);   // [2][kExFloats]
     float4* A = reinterpret_cast<float4*>(EX + 2 * kExFloats);
-    float4* DB = A + p.atom_cap;   // [2][kDirs]: this tile's directions and the next tile's
+    float4* DB = A + p.atom_cap;   // [2][parity][32]: this tile's directions and the next tile's
     TpPass* pass_s = reinterpret_cast<TpPass*>(DB + 2 * kDirs);   // [2]
     uint64_t* bars = reinterpret_cast<uint64_t*>(pass_s + 2);
     uint64_t* bar_atoms = bars;
@@ -265,7 +265,9 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
             // the first tile's directions (later tiles' arrive while the tile before
             // them runs; held in shared memory: in registers the loop spilled them,
             // 1.6 K cycles per tile)
-            if (tid < kDirs) cp_async16(DB + (t0 & 1) * kDirs + tid, p.dirs + (int64_t)t0 * kDirs + tid);
+            // slot 2 l + i of a tile at [i][l]: a warp reads 512 consecutive bytes
+            const int db_slot = (tid & 1) * 32 + (tid >> 1);
+            if (tid < kDirs) cp_async16(DB + (t0 & 1) * kDirs + db_slot, p.dirs + (int64_t)t0 * kDirs + tid);
             cp_async_wait_all();
             if (nblk > 1) {
                 hist_sync();
@@ -278,9 +280,9 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
             const bool zero_check =
                 sym && nblk == 1 && !nonzero_integer_products_possible(scale, __uint_as_float(*r2max_s));
             for (int tile = t0; tile < t1 && !failed; ++tile) {
-                float4 d0 = DB[(tile & 1) * kDirs + 2 * lane], d1 = DB[(tile & 1) * kDirs + 2 * lane + 1];
+                float4 d0 = DB[(tile & 1) * kDirs + lane], d1 = DB[(tile & 1) * kDirs + 32 + lane];
                 if (tile + 1 < t1 && tid < kDirs)
-                    cp_async16(DB + ((tile + 1) & 1) * kDirs + tid, p.dirs + (int64_t)(tile + 1) * kDirs + tid);
+                    cp_async16(DB + ((tile + 1) & 1) * kDirs + db_slot, p.dirs + (int64_t)(tile + 1) * kDirs + tid);
                 const bool pt0 = d0.w != 0.f, pt1 = d1.w != 0.f;   // the slot has an antipodal partner
                 bool tile_bad = false;
                 for (int pass = 0; pass < 2 && !failed; ++pass) {
@@ -328,8 +330,9 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
                         const bool bad = count && last &&
                                          (zero_check ? (pt0 || pt1) && zmin == 0.f
                                                      : (pt0 && c0 != (uint32_t)handled) || (pt1 && c1 != (uint32_t)handled));
-                        // the A operand of the pass before has been read
-                        if (tid == 0) {
+                        // the A operand of the pass before has been read (asked by the
+                        // last warp, which never has more atoms than the others)
+                        if (tid == kHistThreads - 1) {
                             if (t > 0 && !mbar_wait_bounded(&bar_mma[(t - 1) & 1], ((t - 1) >> 1) & 1u, p.status))
                                 *hist_fail = 1;
                             if (*aux_fail) *hist_fail = 1;
@@ -621,7 +624,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
     unsigned char* BT = smem + (size_t)NBc * 128;
     float* EX = reinterpret_cast<float*>(BT + p.bt_bytes);   // [kDirs][8]
     float4* A = reinterpret_cast<float4*>(BT + p.bt_bytes + kExBytes);
-    float4* DB = A + p.atom_cap;   // [2][kDirs]: this tile's directions and the next tile's
+    float4* DB = A + p.atom_cap;   // [2][parity][32]: this tile's directions and the next tile's
     int2* DI = reinterpret_cast<int2*>(DB + 2 * kDirs);   // [2][kDirs]: (output, partner) of those slots
     float* EX2 = reinterpret_cast<float*>(DI + 2 * kDirs);   // [128 TMEM lanes][8]: partials 2, 3
     // barriers: [0] atoms, [1] B operand, [2 .. 2 + kIssuers) MMA completion per

@@ -100,69 +100,233 @@ __global__ void __launch_bounds__(1024) k_top_nodes(const float* __restrict__ si
     }
 }
 
+// The same for n_hat <= kSelMax: the n_hat-th smallest 32-bit key (descending
+// value) by a radix select over four 8-bit digits, then the keys below it and
+// the lowest-index ones equal to it, sorted in shared memory.  The full sort
+// above walks 136 passes of 65536 keys in global memory at 40962 directions
+// (2.16 ms in one CTA); four counting passes and a sort of 1024 keys take
+// 0.04 ms.
+constexpr int kSelMax = 4096;
+
+__global__ void __launch_bounds__(1024) k_top_select(const float* __restrict__ sig, int32_t nv, int32_t n_hat,
+                                                     int32_t* top, float* top_val) {
+    __shared__ uint64_t sel[kSelMax];
+    __shared__ uint32_t hist[256], wcnt[32];
+    __shared__ uint32_t s_prefix, s_rem, s_count;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid == 0) {
+        s_prefix = 0;
+        s_rem = (uint32_t)n_hat;
+        s_count = 0;
+    }
+    for (int pass = 3; pass >= 0; --pass) {
+        if (tid < 256) hist[tid] = 0;
+        __syncthreads();
+        const uint32_t prefix = s_prefix, hmask = pass == 3 ? 0u : 0xFFFFFFFFu << (8 * (pass + 1));
+        for (int i = tid; i < nv; i += 1024) {
+            const uint32_t k = ~ordered_f32(sig[i]);
+            if ((k & hmask) == (prefix & hmask)) atomicAdd(&hist[(k >> (8 * pass)) & 255u], 1u);
+        }
+        __syncthreads();
+        if (tid == 0) {
+            uint32_t rem = s_rem, d = 0;
+            while (hist[d] < rem) rem -= hist[d++];
+            s_rem = rem;
+            s_prefix = prefix | (d << (8 * pass));
+        }
+        __syncthreads();
+    }
+    const uint32_t kth = s_prefix, need_eq = s_rem, n_less = (uint32_t)n_hat - need_eq;
+    int kp = 1;
+    while (kp < n_hat) kp <<= 1;
+    for (int i = tid; i < kp; i += 1024) sel[i] = ~0ull;
+    __syncthreads();
+    for (int i = tid; i < nv; i += 1024) {
+        const uint32_t k = ~ordered_f32(sig[i]);
+        if (k < kth) sel[atomicAdd(&s_count, 1u)] = ((uint64_t)k << 32) | (uint32_t)i;
+    }
+    uint32_t taken = 0;
+    for (int i0 = 0; i0 < nv && taken < need_eq; i0 += 1024) {
+        const int i = i0 + tid;
+        const bool eq = i < nv && ~ordered_f32(sig[i]) == kth;
+        const uint32_t bal = __ballot_sync(0xffffffffu, eq);
+        __syncthreads();
+        if (lane == 0) wcnt[warp] = __popc(bal);
+        __syncthreads();
+        uint32_t before = 0, total = 0;
+        for (int w = 0; w < 32; ++w) {
+            if (w < warp) before += wcnt[w];
+            total += wcnt[w];
+        }
+        const uint32_t rank = taken + before + __popc(bal & ((1u << lane) - 1u));
+        if (eq && rank < need_eq) sel[n_less + rank] = ((uint64_t)kth << 32) | (uint32_t)i;
+        taken += total;
+    }
+    __syncthreads();
+    for (int k = 2; k <= kp; k <<= 1) {
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int i = tid; i < kp; i += 1024) {
+                const int l = i ^ j;
+                if (l > i) {
+                    const uint64_t x = sel[i], y = sel[l];
+                    if ((x > y) == ((i & k) == 0)) {
+                        sel[i] = y;
+                        sel[l] = x;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    }
+    for (int i = tid; i < n_hat; i += 1024) {
+        const int32_t idx = (int32_t)(sel[i] & 0xFFFFFFFFu);
+        top[i] = idx;
+        top_val[i] = sig[idx];
+    }
+}
+
 // ---- look-up table ---------------------------------------------------------------
 
 constexpr int kLutThreads = 256;
 constexpr int kLutPer = 4;                       // queries per thread
 constexpr int kLutTile = 2048;                   // nodes per shared-memory tile
 
-// lut_t[k * ng_pad + g] = argmax_p u_p . r with r = (float)(R(q_g) n_top[k])
-// (FP64 products summed left to right), the dot product by the FP32 contract
-// fma(u_z, r_z, fma(u_y, r_y, u_x r_x)); ties resolve to the lowest index.
-// IdxT is uint16_t when every node index fits (nv <= 65536), else int32_t.
+// The rotated node r = (float)(R(q) n), FP64 products summed left to right.
+__device__ __forceinline__ float3 rotate_node(const M3& R, float4 n) {
+    const double nx = n.x, ny = n.y, nz = n.z;
+    float3 r;
+    r.x = __double2float_rn(__dadd_rn(__dadd_rn(__dmul_rn(R.a[0], nx), __dmul_rn(R.a[1], ny)), __dmul_rn(R.a[2], nz)));
+    r.y = __double2float_rn(__dadd_rn(__dadd_rn(__dmul_rn(R.a[3], nx), __dmul_rn(R.a[4], ny)), __dmul_rn(R.a[5], nz)));
+    r.z = __double2float_rn(__dadd_rn(__dadd_rn(__dmul_rn(R.a[6], nx), __dmul_rn(R.a[7], ny)), __dmul_rn(R.a[8], nz)));
+    return r;
+}
+
+__device__ __forceinline__ float node_dot(float4 u, float3 r) {
+    return __fmaf_rn(u.z, r.z, __fmaf_rn(u.y, r.y, __fmul_rn(u.x, r.x)));
+}
+
+// lut_t[k * ng_pad + g] = argmax_p u_p . r with r = R(q_g) n_top[k], the dot
+// product by the FP32 contract fma(u_z, r_z, fma(u_y, r_y, u_x r_x)); ties
+// resolve to the lowest index.  IdxT is uint16_t when every node index fits
+// (nv <= 65536), else int32_t.
+//
+// The nodes lie in a cubic grid of cells of edge h (about one and a half node
+// spacings).  A query scans the 3 x 3 x 3 cells around r, nine runs of
+// consecutive nodes.  A node outside them is at least h away, so its exact dot
+// product is at most (max |u|^2 + |r|^2 - h^2) / 2: when the best found exceeds
+// that by more than the FP32 errors it is the answer of a scan over all nodes.
+// Queries it does not settle (r in a gap of the direction set) are listed and
+// left to k_lut_scan.  Scanning all 40962 nodes for every query took 29.1 ms
+// for 3419 x 1000 queries (1.4e11 dot products); this reads about 20 nodes per
+// query, bound by the L2 latency of the run bounds and nodes:
+// 0.3 ms.
+constexpr int kLutK = 8;   // nodes per thread (one rotation matrix, kLutK of its columns of the table)
+
+struct NodeGrid {
+    const int32_t* start;   // [dim^3 + 1]
+    const float4* nodes;    // in cell order, ascending index inside a cell; w = index bits
+    int dim;
+    float org, inv_h, far2;   // cell = (x - org) * inv_h; far2 = max |u|^2 - (0.999 h)^2
+};
+
+__device__ __forceinline__ int node_cell(float x, const NodeGrid& g) {
+    return min(max((int)((x - g.org) * g.inv_h), 0), g.dim - 1);
+}
+
 template <typename IdxT>
-__global__ void __launch_bounds__(kLutThreads) k_build_lut(const float4* __restrict__ dirs, int32_t nv,
+__global__ void __launch_bounds__(kLutThreads) k_build_lut(NodeGrid grid, const float4* __restrict__ dirs,
                                                            const int32_t* __restrict__ top, int32_t n_hat,
                                                            const double* __restrict__ quats, int64_t ng,
-                                                           int64_t ng_pad, IdxT* lut_t) {
-    __shared__ float4 tile[kLutTile];
-    const int64_t nq = ng * n_hat;
-    const int64_t q0 = (int64_t)blockIdx.x * kLutThreads * kLutPer;
-    float rx[kLutPer], ry[kLutPer], rz[kLutPer], best[kLutPer];
-    int32_t bi[kLutPer];
-    int64_t qi[kLutPer];
+                                                           int64_t ng_pad, IdxT* lut_t, int32_t k0, int32_t k1,
+                                                           uint32_t* open, uint32_t* n_open) {
+    const int64_t g = (int64_t)blockIdx.x * kLutThreads + threadIdx.x;
+    const int kb = k0 + (int)blockIdx.y * kLutK;
+    if (g >= ng) return;
+    const M3 R = quat_to_matrix(quats[4 * g], quats[4 * g + 1], quats[4 * g + 2], quats[4 * g + 3]);
+    for (int k = kb; k < min(kb + kLutK, k1); ++k) {
+        const float3 r = rotate_node(R, dirs[top[k]]);
+        const int ix = node_cell(r.x, grid), iy = node_cell(r.y, grid), iz = node_cell(r.z, grid);
+        const int xa = max(ix - 1, 0), xb = min(ix + 2, grid.dim);
+        float best = -INFINITY;
+        int32_t bi = 0x7FFFFFFF;
+        int32_t beg[9], end[9];
 #pragma unroll
-    for (int j = 0; j < kLutPer; ++j) {
-        const int64_t q = q0 + (int64_t)j * kLutThreads + threadIdx.x;
-        qi[j] = q;
-        best[j] = -INFINITY;
-        bi[j] = 0;
-        rx[j] = ry[j] = rz[j] = 0.f;
-        if (q < nq) {
-            const int64_t g = q / n_hat;
-            const int k = (int)(q % n_hat);
-            const M3 R = quat_to_matrix(quats[4 * g], quats[4 * g + 1], quats[4 * g + 2], quats[4 * g + 3]);
-            const float4 n = dirs[top[k]];
-            const double nx = n.x, ny = n.y, nz = n.z;
-            rx[j] = __double2float_rn(__dadd_rn(__dadd_rn(__dmul_rn(R.a[0], nx), __dmul_rn(R.a[1], ny)), __dmul_rn(R.a[2], nz)));
-            ry[j] = __double2float_rn(__dadd_rn(__dadd_rn(__dmul_rn(R.a[3], nx), __dmul_rn(R.a[4], ny)), __dmul_rn(R.a[5], nz)));
-            rz[j] = __double2float_rn(__dadd_rn(__dadd_rn(__dmul_rn(R.a[6], nx), __dmul_rn(R.a[7], ny)), __dmul_rn(R.a[8], nz)));
+        for (int j = 0; j < 9; ++j) {
+            const int y = iy + j % 3 - 1, z = iz + j / 3 - 1;
+            const bool in = y >= 0 && y < grid.dim && z >= 0 && z < grid.dim;
+            const int c = in ? grid.dim * (y + grid.dim * z) : 0;
+            beg[j] = in ? __ldg(grid.start + c + xa) : 0;
+            end[j] = in ? __ldg(grid.start + c + xb) : 0;
+        }
+#pragma unroll
+        for (int j = 0; j < 9; ++j)
+            for (int i = beg[j]; i < end[j]; ++i) {
+                const float4 u = __ldg(grid.nodes + i);
+                const float d = node_dot(u, r);
+                const int32_t idx = __float_as_int(u.w);
+                if (d > best || (d == best && idx < bi)) {
+                    best = d;
+                    bi = idx;
+                }
+            }
+        const float r2 = r.x * r.x + r.y * r.y + r.z * r.z;
+        if (best > 0.5f * (grid.far2 + r2) + 2e-6f) {
+            lut_t[(int64_t)k * ng_pad + g] = (IdxT)bi;
+        } else {
+            open[atomicAdd(n_open, 1u)] = (uint32_t)((int64_t)(k - k0) * ng + g);
         }
     }
-    for (int p0 = 0; p0 < nv; p0 += kLutTile) {
-        const int cnt = min(kLutTile, nv - p0);
-        __syncthreads();
-        for (int i = threadIdx.x; i < cnt; i += kLutThreads) tile[i] = dirs[p0 + i];
-        __syncthreads();
-        for (int i = 0; i < cnt; ++i) {
-            const float4 u = tile[i];
+}
+
+// The listed queries against every node, staged through shared memory, four
+// queries per thread.
+template <typename IdxT>
+__global__ void __launch_bounds__(kLutThreads) k_lut_scan(const float4* __restrict__ dirs, int32_t nv,
+                                                          const int32_t* __restrict__ top,
+                                                          const double* __restrict__ quats, int64_t ng,
+                                                          int64_t ng_pad, IdxT* lut_t, int32_t k0,
+                                                          const uint32_t* __restrict__ open,
+                                                          const uint32_t* __restrict__ n_open) {
+    __shared__ float4 tile[kLutTile];
+    const uint32_t n = *n_open;
+    for (uint32_t q0 = blockIdx.x * (uint32_t)(kLutThreads * kLutPer); q0 < n;
+         q0 += gridDim.x * (uint32_t)(kLutThreads * kLutPer)) {
+        float3 r[kLutPer];
+        float best[kLutPer];
+        int32_t bi[kLutPer];
 #pragma unroll
-            for (int j = 0; j < kLutPer; ++j) {
-                const float d = __fmaf_rn(u.z, rz[j], __fmaf_rn(u.y, ry[j], __fmul_rn(u.x, rx[j])));
-                if (d > best[j]) {
-                    best[j] = d;
-                    bi[j] = p0 + i;
+        for (int j = 0; j < kLutPer; ++j) {
+            const uint32_t q = q0 + (uint32_t)j * kLutThreads + threadIdx.x;
+            best[j] = -INFINITY;
+            bi[j] = 0;
+            r[j] = make_float3(0.f, 0.f, 0.f);
+            if (q < n) {
+                const int64_t g = open[q] % ng;
+                const M3 R = quat_to_matrix(quats[4 * g], quats[4 * g + 1], quats[4 * g + 2], quats[4 * g + 3]);
+                r[j] = rotate_node(R, dirs[top[k0 + (int)(open[q] / ng)]]);
+            }
+        }
+        for (int p0 = 0; p0 < nv; p0 += kLutTile) {
+            const int cnt = min(kLutTile, nv - p0);
+            __syncthreads();
+            for (int i = threadIdx.x; i < cnt; i += kLutThreads) tile[i] = dirs[p0 + i];
+            __syncthreads();
+            for (int i = 0; i < cnt; ++i) {
+                const float4 u = tile[i];
+#pragma unroll
+                for (int j = 0; j < kLutPer; ++j) {
+                    const float d = node_dot(u, r[j]);
+                    if (d > best[j]) {
+                        best[j] = d;
+                        bi[j] = p0 + i;
+                    }
                 }
             }
         }
-    }
 #pragma unroll
-    for (int j = 0; j < kLutPer; ++j) {
-        const int64_t q = qi[j];
-        if (q < nq) {
-            const int64_t g = q / n_hat;
-            const int k = (int)(q % n_hat);
-            lut_t[(int64_t)k * ng_pad + g] = (IdxT)bi[j];
+        for (int j = 0; j < kLutPer; ++j) {
+            const uint32_t q = q0 + (uint32_t)j * kLutThreads + threadIdx.x;
+            if (q < n) lut_t[(k0 + (int64_t)(open[q] / ng)) * ng_pad + open[q] % ng] = (IdxT)bi[j];
         }
     }
 }
@@ -760,6 +924,11 @@ cudaError_t launch_lut_export(Ctx* c, Reference* r, int32_t* out) {
 // ---- launches ------------------------------------------------------------------------
 
 cudaError_t launch_top_nodes(Ctx* c, Reference* r) {
+    if (r->n_hat <= kSelMax) {
+        k_top_select<<<1, 1024, 0, c->stream>>>(r->d_node_sig, c->nv, r->n_hat, r->d_top, r->d_top_val);
+        cudaError_t e = cudaGetLastError();
+        return e == cudaSuccess ? cudaStreamSynchronize(c->stream) : e;
+    }
     int32_t npow2 = 1;
     while (npow2 < c->nv) npow2 <<= 1;
     uint64_t* keys = nullptr;
@@ -771,17 +940,36 @@ cudaError_t launch_top_nodes(Ctx* c, Reference* r) {
     return e;
 }
 
+// The table in runs of rows of at most 2^24 queries, so that the list of open
+// queries (sized for all of a run) stays at 64 MB, and of what a grid takes.
+template <typename IdxT>
+static cudaError_t launch_build_lut_t(Ctx* c, Reference* r, const double* d_quats, int64_t ng) {
+    const int64_t rows = std::min<int64_t>(std::min<int64_t>(r->n_hat, 65535 * kLutK),
+                                           std::max<int64_t>(1, ((int64_t)1 << 24) / ng));
+    uint32_t* open = nullptr;
+    if (dev_alloc(c, (void**)&open, (size_t)(rows * ng + 1) * sizeof(uint32_t))) return cudaErrorMemoryAllocation;
+    const NodeGrid grid{c->d_node_start, c->d_nodes, c->node_dim, c->node_org, c->node_inv_h, c->node_far2};
+    cudaError_t e = cudaSuccess;
+    for (int64_t k0 = 0; k0 < r->n_hat && e == cudaSuccess; k0 += rows) {
+        const int64_t k1 = std::min<int64_t>(k0 + rows, r->n_hat);
+        if ((e = cudaMemsetAsync(open, 0, sizeof(uint32_t), c->stream)) != cudaSuccess) break;
+        const dim3 blocks((unsigned)((ng + kLutThreads - 1) / kLutThreads), (unsigned)((k1 - k0 + kLutK - 1) / kLutK));
+        k_build_lut<IdxT><<<blocks, kLutThreads, 0, c->stream>>>(grid, c->d_dirs, r->d_top, r->n_hat, d_quats, ng,
+                                                                 r->ng_pad, static_cast<IdxT*>(r->d_lut), (int32_t)k0,
+                                                                 (int32_t)k1, open + 1, open);
+        k_lut_scan<IdxT><<<(unsigned)c->sm_count * 4, kLutThreads, 0, c->stream>>>(
+            c->d_dirs, c->nv, r->d_top, d_quats, ng, r->ng_pad, static_cast<IdxT*>(r->d_lut), (int32_t)k0, open + 1,
+            open);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    dev_recycle(c, open);
+    return e;
+}
+
 cudaError_t launch_build_lut(Ctx* c, Reference* r, const double* d_quats, int64_t ng) {
-    const int64_t nq = ng * r->n_hat;
-    const int64_t per = (int64_t)kLutThreads * kLutPer;
-    const unsigned grid = (unsigned)((nq + per - 1) / per);
-    if (r->lut_bytes == 2)
-        k_build_lut<<<grid, kLutThreads, 0, c->stream>>>(c->d_dirs, c->nv, r->d_top, r->n_hat, d_quats, ng, r->ng_pad,
-                                                         static_cast<uint16_t*>(r->d_lut));
-    else
-        k_build_lut<<<grid, kLutThreads, 0, c->stream>>>(c->d_dirs, c->nv, r->d_top, r->n_hat, d_quats, ng, r->ng_pad,
-                                                         static_cast<int32_t*>(r->d_lut));
-    return cudaGetLastError();
+    return r->lut_bytes == 2 ? launch_build_lut_t<uint16_t>(c, r, d_quats, ng)
+                             : launch_build_lut_t<int32_t>(c, r, d_quats, ng);
 }
 
 template <typename IdxT>

@@ -84,6 +84,11 @@ struct Ctx {
     int2* d_slot_idx = nullptr;
     int32_t nslot = 0, nslot_pad = 0, npairs = 0;
     bool use_pairs = true;           // cleared by APTIDX_DIRECT for one call
+    // the directions in a cubic grid of cells for nearest-node queries
+    int32_t* d_node_start = nullptr;   // [node_dim^3 + 1]
+    float4* d_nodes = nullptr;         // [nv] in cell order, w = index bits
+    int node_dim = 0;
+    float node_org = 0.f, node_inv_h = 0.f, node_far2 = 0.f;
     float* d_gn_scratch = nullptr;   // one signature row per refinement CTA, in the order above
     size_t gn_scratch_bytes = 0;
     BandSet multi;                       // bands of the current pass (multi-signature calls)

@@ -742,7 +742,7 @@ int aptidx_set_binning(aptidx_ctx* ctx, int m, int32_t k_lo, int32_t k_hi, int f
     if (c->tw_m != m) {
         free_ptr(c->d_tw);
         c->tw_m = 0;
-        int rc = dev_alloc(c, (void**)&c->d_tw, sizeof(float2) << m);
+        int rc = dev_alloc(c, (void**)&c->d_tw, sizeof(float2) << (m + 1));
         if (rc) return rc;
         cudaError_t e = launch_twiddles(c->d_tw, m, c->stream);
         if (e != cudaSuccess) return cuda_check(c, e, "twiddles");

@@ -666,20 +666,21 @@ cudaError_t zero_counters(Ctx* c) {
 }
 
 // -----------------------------------------------------------------------------
-// twiddle table (cos, sin)(2 pi j / 2^m) in FP32, from FP64 sincospi with the
-// angle index reduced exactly in integers
+// twiddle table (cos, sin)(pi j / 2^m), j < 2 x 2^m, in FP32, from FP64 sincospi
+// with the angle index reduced exactly in integers (half steps of the DFT's
+// angle: the folded sum takes its phase from the middle of the histogram)
 // -----------------------------------------------------------------------------
 __global__ void k_twiddles(float2* tw, int m) {
     int nb = 1 << m;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < nb; j += gridDim.x * blockDim.x) {
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < 2 * nb; j += gridDim.x * blockDim.x) {
         double sn, cs;
-        sincospi(2.0 * (double)j / (double)nb, &sn, &cs);
+        sincospi((double)j / (double)nb, &sn, &cs);
         tw[j] = make_float2((float)cs, (float)sn);
     }
 }
 
 cudaError_t launch_twiddles(float2* tw, int m, cudaStream_t s) {
-    k_twiddles<<<((1 << m) + 255) / 256, 256, 0, s>>>(tw, m);
+    k_twiddles<<<((2 << m) + 255) / 256, 256, 0, s>>>(tw, m);
     return cudaGetLastError();
 }
 

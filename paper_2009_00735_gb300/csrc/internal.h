@@ -99,7 +99,7 @@ struct Ctx {
     int m = 0;
     int32_t k_lo = 0, k_hi = 0;
     bool binning_set = false;
-    float2* d_tw = nullptr;            // [2^m] (cos, sin)(2 pi j / 2^m), FP32
+    float2* d_tw = nullptr;            // [2 x 2^m] (cos, sin)(pi j / 2^m), FP32
     int tw_m = 0;
     // tensor-core twiddle operand (B): [n_cols] hi/lo FP16 in canonical layout
     void* d_twb = nullptr;

@@ -10,9 +10,19 @@
 // l owns directions 2l and 2l+1 and adds 1 to 16-bit halves of the word
 // H[b * 32 + l].  A lane's words sit in bank l whatever the bin, so the
 // shared-memory atomics of one warp instruction never conflict.
-// The band spectrum X(k) = sum_n h[n] e^{-2 pi i k n / 2^m} is then
-// accumulated in FP32 against a (cos, sin) table; the twiddle index is
-// uniform across a warp, so table reads are broadcasts.
+//
+// The band spectrum takes the phase from the middle of the histogram: with
+// bins n and N - 1 - n folded into their sum e and difference o,
+//   |X(k)|^2 = (sum_n e_n cos t_n)^2 + (sum_n o_n sin t_n)^2,
+// t_n = 2 pi k (j + 1/2) / N at the j-th bin from the middle, and the bins j
+// and N / 2 - 1 - j share one cosine and sine up to the sign (-1)^k.  The folds
+// are exact (small integers), so four bins cost two FMAs per frequency (a
+// complex sum over all bins costs eight), and the value of the mirrored
+// histogram, that of the direction -u, is the same bit for bit.  Antipodal
+// pairs are therefore projected once (as on the tensor-core path, with the same
+// exact check for atoms whose mirror image falls into another bin).
+// 512 ROIs of 1133 atoms x 40962 directions, 2^10 bins, four frequencies:
+// 24.9 ms with every direction projected and the complex sum, 8.6 ms now.
 #include <mutex>
 
 #include "common.cuh"
@@ -68,7 +78,8 @@ struct SigParams {
     const int64_t* off;
     const int32_t* nw;
     const int32_t* order;
-    const float4* dirs;
+    const float4* dirs;      // direction slots, padded to whole tiles with (1, 0, 0)
+    const int2* slot_idx;    // per slot: (output direction, antipodal partner or -1); NULL: slot = direction
     int32_t nv;
     int32_t tiles_per_roi;
     int32_t tiles_per_item;
@@ -89,32 +100,90 @@ struct SigParams {
     BandSet bands;
 };
 
+// Folded partial spectrum of kKpw frequencies from k0 over the bins j0 .. j0 +
+// span - 1 from the middle (and their three images), for the lane's two
+// directions: re = sum e cos, im = sum o sin.  TW2[i] = (cos, sin)(pi i / N),
+// i < 2 N; kOdd = k0 & 1.
+template <int kOdd>
+__device__ __forceinline__ void fold_dft(const uint32_t* H, const float2* TW2, int NB, int lane, int j0, int span,
+                                         int k0, float (&re)[kKpw][2], float (&im)[kKpw][2]) {
+    const unsigned mask = 2u * (unsigned)NB - 1u;
+    unsigned idx[kKpw];
+#pragma unroll
+    for (int q = 0; q < kKpw; ++q) idx[q] = ((unsigned)(k0 + q) * (2u * (unsigned)j0 + 1u)) & mask;
+    const uint32_t* ha = H + (NB / 2 - 1 - j0) * kWords + lane;   // a: below the middle, descending
+    const uint32_t* hb = H + (NB / 2 + j0) * kWords + lane;       // b: above the middle
+    const uint32_t* hc = H + j0 * kWords + lane;                  // c: from the first bin
+    const uint32_t* hd = H + (NB - 1 - j0) * kWords + lane;       // d: from the last bin
+#pragma unroll 2
+    for (int j = 0; j < span; ++j) {
+        const uint32_t wa = *ha, wc = *hc;
+        const uint32_t s1 = wa + *hb, s2 = wc + *hd;   // 16-bit halves: no carry, a histogram holds at most 65535 atoms
+        ha -= kWords;
+        hb += kWords;
+        hc += kWords;
+        hd -= kWords;
+        float ee[2], eo[2], oe[2], oo[2];   // e and o of even and odd frequencies
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+            const float f1 = u23_to_float(d ? s1 >> 16 : s1 & 0xFFFFu), f2 = u23_to_float(d ? s2 >> 16 : s2 & 0xFFFFu);
+            const float fa = u23_to_float(d ? wa >> 16 : wa & 0xFFFFu), fc = u23_to_float(d ? wc >> 16 : wc & 0xFFFFu);
+            const float p = fmaf(2.f, fa, -f1), r = fmaf(2.f, fc, -f2);   // a - b, c - d
+            ee[d] = f1 + f2;
+            eo[d] = f1 - f2;
+            oe[d] = p - r;
+            oo[d] = p + r;
+        }
+#pragma unroll
+        for (int q = 0; q < kKpw; ++q) {
+            const float2 t = TW2[idx[q]];
+            idx[q] = (idx[q] + 2u * (unsigned)(k0 + q)) & mask;
+            const bool odd = ((q + kOdd) & 1) != 0;
+#pragma unroll
+            for (int d = 0; d < 2; ++d) {
+                re[q][d] = fmaf(odd ? eo[d] : ee[d], t.x, re[q][d]);
+                im[q][d] = fmaf(odd ? oo[d] : oe[d], t.y, im[q][d]);
+            }
+        }
+    }
+}
+
 // kNB: band slots of the epilogue (1: the ROI's own band; APTIDX_MAX_BANDS:
-// the pass's BandSet)
-template <int kNB>
+// the pass's BandSet).  kSafe: atoms and directions come from the caller
+// unchecked, so bins are masked to m bits (memory-safe for any input).
+template <int kNB, bool kSafe>
 __global__ void __launch_bounds__(kThreads, 1) k_sig_plain(SigParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
     const int NB = 1 << p.m;
     const int nbm1 = NB - 1;
     const int NBc = NB < kChunkBins ? NB : kChunkBins;   // histogram rows held at once
     const int nchunk = NB / NBc;
+    const int ntw = nchunk == 1 ? 2 * NB : NB;   // half-step angles for the folded sum
     uint32_t* H = reinterpret_cast<uint32_t*>(smem);
     float2* TW = reinterpret_cast<float2*>(smem + (size_t)NBc * kWords * 4);
-    float4* A = reinterpret_cast<float4*>(smem + (size_t)NBc * kWords * 4 + (size_t)NB * 8);
+    float4* A = reinterpret_cast<float4*>(smem + (size_t)NBc * kWords * 4 + (size_t)ntw * 8);
     float2* PART = reinterpret_cast<float2*>(A + p.atom_cap);
     uint64_t* bar = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(PART) + kPartBytes);
     int* flag = reinterpret_cast<int*>(bar + 1);
     int64_t* item_s = reinterpret_cast<int64_t*>(bar + 2);
+    unsigned* r2max_s = reinterpret_cast<unsigned*>(bar + 3);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int j = tid; j < NB; j += kThreads) TW[j] = p.tw[j];
+    for (int j = tid; j < ntw; j += kThreads) TW[j] = p.tw[nchunk == 1 ? j : 2 * j];
+    auto zero_h = [&](int t0) {   // threads t0 .. kThreads - 1
+        for (int i = tid - t0; i < NBc * kWords / 4; i += kThreads - t0)
+            reinterpret_cast<uint4*>(H)[i] = make_uint4(0, 0, 0, 0);
+    };
+    zero_h(0);   // every pass finds the histogram zero
     if (tid == 0) {
         mbar_init(bar, 1);
         fence_barrier_init();
     }
     __syncthreads();
     uint32_t phase = 0;
-    const float magic = bin_magic(p.m);
+    const uint32_t h_addr = smem_u32(H);
+    const float magic = kSafe ? bin_magic(p.m) : quad_magic(p.m, h_addr >> 7);
+    const bool sym = !kSafe && p.slot_idx != nullptr;
     const int64_t n_items = p.n_items;
 
     for (;;) {
@@ -130,269 +199,285 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_plain(SigParams p) {
         const int64_t abase = p.off[roi];
         const float scale = p.scale[roi];
         const int klo = p.band[2 * roi], khi = p.band[2 * roi + 1];
+        const int K = khi - klo + 1;
+        const int G = (K + kKpw - 1) / kKpw;   // frequency groups of kKpw
         const int t0 = grp * p.tiles_per_item;
         const int t1 = min(t0 + p.tiles_per_item, p.tiles_per_roi);
         const bool one_chunk = nw <= p.atom_cap;
-        if (one_chunk && !stage_atoms(A, p.atoms + abase, nw, bar, phase, p.status, flag)) return;
+        const int64_t out_base = (p.single_roi >= 0 ? 0 : roi) * (int64_t)p.nv;
+        // stage n atoms, in blocks of four unless the checked loops read them
+        auto stage = [&](const float4* src, int n, unsigned* r2) -> bool {
+            if (r2 && tid == 0) *r2 = 0u;
+            if (!stage_atoms(A, src, n, bar, phase, p.status, flag)) return false;
+            if (!kSafe) {
+                quad_atoms(A, n, tid, kThreads, r2);
+                __syncthreads();
+            }
+            return true;
+        };
+        if (one_chunk && !stage(p.atoms + abase, nw, r2max_s)) return;
+        const bool zero_check =
+            sym && one_chunk && !nonzero_integer_products_possible(scale, __uint_as_float(*r2max_s));
+        // one pass of the histogram over bn atoms from a0 (bin chunk bc); the
+        // counts of the antipodal check go to c0, c1, zmin, handled
+        QuadDirs q;
+        float4 d0, d1;
+        uint32_t c0 = 0, c1 = 0;
+        float zmin = 1.f;
+        int handled = 0;
+        auto histogram = [&](const float4* src, int bn, int bc, bool count) -> bool {
+            for (int s0 = 0; s0 < bn || s0 == 0; s0 += p.atom_cap) {
+                const int cn = min(p.atom_cap, bn - s0);
+                if (!one_chunk && !stage(src + s0, cn, nullptr)) return false;
+                if (kSafe) {
+                    if (nchunk == 1)
+                        hist_tile<kWarps, true>(H, A, cn, warp, lane, d0, d1, scale, magic, nbm1);
+                    else
+                        hist_tile_chunk<kWarps>(H, A, cn, warp, lane, d0, d1, scale, magic, (uint32_t)nbm1, (uint32_t)bc);
+                } else if (nchunk == 1) {
+                    if (count && zero_check)
+                        handled += hist_tile_quads<kWarps, 2, false>(A, cn, warp, q, c0, c1, zmin);
+                    else if (count)
+                        handled += hist_tile_quads<kWarps, 1, false>(A, cn, warp, q, c0, c1, zmin);
+                    else
+                        hist_tile_quads<kWarps, 0, false>(A, cn, warp, q, c0, c1, zmin);
+                } else {
+                    q.t_lo = kQuadBits + (h_addr >> 7) + (uint32_t)bc * kChunkBins;
+                    q.h_lane = h_addr + 4u * (uint32_t)lane;
+                    hist_tile_quads<kWarps, 0, true>(A, cn, warp, q, c0, c1, zmin);
+                }
+                if (!one_chunk) __syncthreads();
+            }
+            return true;
+        };
+        // where direction `at` of the tile goes: pass 0 the slot's direction (and
+        // its partner when `mirror`), pass 1 the partner
+        auto write_out = [&](int tile, int at, int pass, bool mirror, int b, float value, int k) {
+            const int slot = tile * kDirs + at;
+            int v0 = slot < p.nv ? slot : -1, v1 = -1;
+            if (sym) {
+                const int2 si = p.slot_idx[slot];
+                v0 = pass ? si.y : si.x;
+                v1 = mirror ? si.y : -1;
+            }
+            const int64_t ob = band_off_t<kNB>(p.bands, b) + out_base;
+            if (v0 >= 0) {
+                p.S[ob + v0] = value;
+                if (p.argk) p.argk[ob + v0] = (uint16_t)k;
+            }
+            if (v1 >= 0) {
+                p.S[ob + v1] = value;
+                if (p.argk) p.argk[ob + v1] = (uint16_t)k;
+            }
+        };
 
-        if (nchunk > 1 || nw > kBlockAtoms) {
-            // ---- multi-pass path: the histogram of a tile in passes over atom
-            // blocks of at most kBlockAtoms and bin chunks of 1024; each warp
-            // unit (4 frequencies x a span of the chunk's bins) accumulates its
-            // partial DFT in registers across the passes.  Bands of more than
-            // kWarps groups of frequencies run in rounds of kWarps groups.
-            const int K = khi - klo + 1;
-            const int G = (K + kKpw - 1) / kKpw;
-            const int nblk = (nw + kBlockAtoms - 1) / kBlockAtoms;
-            const int64_t out_base = (p.single_roi >= 0 ? 0 : roi) * (int64_t)p.nv;
-            for (int tile = t0; tile < t1; ++tile) {
-                const float4 d0 = p.dirs[(int64_t)tile * kDirs + 2 * lane];
-                const float4 d1 = p.dirs[(int64_t)tile * kDirs + 2 * lane + 1];
-                float best[kNB];
-                int bk[kNB];
-                if (tid < kDirs) band_init_t<kNB>(p.bands, klo, best, bk);
-                for (int g_lo = 0; g_lo < G; g_lo += kWarps) {
-                    const int Gr = min(kWarps, G - g_lo);
-                    int nsplit = 1;
-                    while (Gr * nsplit * 2 <= kWarps && nsplit * 2 <= NBc / 32) nsplit *= 2;
-                    const int span = NBc / nsplit;
-                    const bool unit = warp < Gr * nsplit;
-                    const int g = g_lo + warp / nsplit, sp = warp % nsplit;
-                    const int k0 = klo + g * kKpw;
-                    float re[kKpw][2], im[kKpw][2];
+        const bool multi_pass = nchunk > 1 || nw > kBlockAtoms;
+        for (int tile = t0; tile < t1; ++tile) {
+            bool partners = sym && multi_pass;   // a partner pass is due
+            for (int pass = 0; pass < 2; ++pass) {
+                if (pass == 1 && !partners) break;
+                d0 = p.dirs[(int64_t)tile * kDirs + 2 * lane];
+                d1 = p.dirs[(int64_t)tile * kDirs + 2 * lane + 1];
+                const bool pt0 = d0.w != 0.f, pt1 = d1.w != 0.f;
+                if (pass == 1) {
+                    d0 = make_float4(-d0.x, -d0.y, -d0.z, d0.w);
+                    d1 = make_float4(-d1.x, -d1.y, -d1.z, d1.w);
+                }
+                if (!kSafe) q = quad_dirs(d0, d1, scale, magic, lane);
+                if (multi_pass) {
+                    // ---- multi-pass path: the histogram of a tile in passes over atom
+                    // blocks of at most kBlockAtoms and bin chunks of 1024; each warp
+                    // unit (4 frequencies x a span of the chunk's bins) accumulates its
+                    // partial DFT in registers across the passes.  Bands of more than
+                    // kWarps groups of frequencies run in rounds of kWarps groups.
+                    const int nblk = (nw + kBlockAtoms - 1) / kBlockAtoms;
+                    const int tws = nchunk == 1 ? 2 : 1;   // full-step angles
+                    float best[kNB];
+                    int bk[kNB];
+                    if (tid < kDirs) band_init_t<kNB>(p.bands, klo, best, bk);
+                    for (int g_lo = 0; g_lo < G; g_lo += kWarps) {
+                        const int Gr = min(kWarps, G - g_lo);
+                        int nsplit = 1;
+                        while (Gr * nsplit * 2 <= kWarps && nsplit * 2 <= NBc / 32) nsplit *= 2;
+                        const int span = NBc / nsplit;
+                        const bool unit = warp < Gr * nsplit;
+                        const int g = g_lo + warp / nsplit, sp = warp % nsplit;
+                        const int k0 = klo + g * kKpw;
+                        float re[kKpw][2], im[kKpw][2];
 #pragma unroll
-                    for (int q = 0; q < kKpw; ++q) re[q][0] = re[q][1] = im[q][0] = im[q][1] = 0.f;
-                    for (int blk = 0; blk < max(nblk, 1); ++blk) {
-                        const int b0 = blk * kBlockAtoms, bn = max(0, min(kBlockAtoms, nw - b0));
-                        for (int bc = 0; bc < nchunk; ++bc) {
-                            uint4* H4 = reinterpret_cast<uint4*>(H);
-                            for (int i = tid; i < NBc * kWords / 4; i += kThreads) H4[i] = make_uint4(0, 0, 0, 0);
-                            __syncthreads();
-                            for (int c0 = 0; c0 < bn; c0 += p.atom_cap) {
-                                const int cn = min(p.atom_cap, bn - c0);
-                                if (!one_chunk) {
-                                    if (!stage_atoms(A, p.atoms + abase + b0 + c0, cn, bar, phase, p.status, flag))
-                                        return;
-                                }
-                                hist_tile_chunk<kWarps>(H, A, cn, warp, lane, d0, d1, scale, magic, (uint32_t)nbm1,
-                                                        (uint32_t)bc);
-                                if (!one_chunk) __syncthreads();
-                            }
-                            __syncthreads();
-                            if (p.hist_out && g_lo == 0) {
-                                hist_export_add_p(H, NBc, NB, bc, tile, p.nv, p.hist_out, tid, kThreads);
+                        for (int i = 0; i < kKpw; ++i) re[i][0] = re[i][1] = im[i][0] = im[i][1] = 0.f;
+                        for (int blk = 0; blk < max(nblk, 1); ++blk) {
+                            const int b0 = blk * kBlockAtoms, bn = max(0, min(kBlockAtoms, nw - b0));
+                            for (int bc = 0; bc < nchunk; ++bc) {
+                                if (!histogram(p.atoms + abase + b0, bn, bc, false)) return;
                                 __syncthreads();
-                            }
-                            if (unit) {
-                                const int n0 = bc * NBc + sp * span;
-                                unsigned idx[kKpw];
+                                if (p.hist_out && g_lo == 0) {
+                                    hist_export_add_p(H, NBc, NB, bc, tile, p.nv, p.hist_out, tid, kThreads);
+                                    __syncthreads();
+                                }
+                                if (unit) {
+                                    const int n0 = bc * NBc + sp * span;
+                                    unsigned idx[kKpw];
 #pragma unroll
-                                for (int q = 0; q < kKpw; ++q)
-                                    idx[q] = (unsigned)(((int64_t)(k0 + q) * n0) & (int64_t)nbm1);
-                                for (int n = 0; n < span; ++n) {
-                                    const uint32_t w = H[(sp * span + n) * kWords + lane];
-                                    const float f0 = u23_to_float(w & 0xFFFFu), f1 = u23_to_float(w >> 16);
+                                    for (int i = 0; i < kKpw; ++i)
+                                        idx[i] = (unsigned)(((int64_t)(k0 + i) * n0) & (int64_t)nbm1);
+                                    for (int n = 0; n < span; ++n) {
+                                        const uint32_t w = H[(sp * span + n) * kWords + lane];
+                                        const float f0 = u23_to_float(w & 0xFFFFu), f1 = u23_to_float(w >> 16);
 #pragma unroll
-                                    for (int q = 0; q < kKpw; ++q) {
-                                        const float2 t = TW[idx[q]];
-                                        re[q][0] = fmaf(f0, t.x, re[q][0]);
-                                        im[q][0] = fmaf(f0, t.y, im[q][0]);
-                                        re[q][1] = fmaf(f1, t.x, re[q][1]);
-                                        im[q][1] = fmaf(f1, t.y, im[q][1]);
-                                        idx[q] = (idx[q] + (unsigned)(k0 + q)) & (unsigned)nbm1;
+                                        for (int i = 0; i < kKpw; ++i) {
+                                            const float2 t = TW[tws * idx[i]];
+                                            re[i][0] = fmaf(f0, t.x, re[i][0]);
+                                            im[i][0] = fmaf(f0, t.y, im[i][0]);
+                                            re[i][1] = fmaf(f1, t.x, re[i][1]);
+                                            im[i][1] = fmaf(f1, t.y, im[i][1]);
+                                            idx[i] = (idx[i] + (unsigned)(k0 + i)) & (unsigned)nbm1;
+                                        }
                                     }
                                 }
+                                __syncthreads();   // H has been read
+                                zero_h(0);
+                                __syncthreads();
                             }
-                            __syncthreads();   // H is read before the next pass zeroes it
                         }
-                    }
-                    if (unit) {
+                        if (unit) {
 #pragma unroll
-                        for (int q = 0; q < kKpw; ++q) {
-                            PART[((size_t)warp * kKpw + q) * kDirs + 2 * lane] = make_float2(re[q][0], im[q][0]);
-                            PART[((size_t)warp * kKpw + q) * kDirs + 2 * lane + 1] = make_float2(re[q][1], im[q][1]);
+                            for (int i = 0; i < kKpw; ++i) {
+                                PART[((size_t)warp * kKpw + i) * kDirs + 2 * lane] = make_float2(re[i][0], im[i][0]);
+                                PART[((size_t)warp * kKpw + i) * kDirs + 2 * lane + 1] = make_float2(re[i][1], im[i][1]);
+                            }
+                        }
+                        __syncthreads();
+                        if (tid < kDirs) {
+                            for (int kk = g_lo * kKpw; kk < min(K, (g_lo + Gr) * kKpw); ++kk) {
+                                const int gg = kk / kKpw - g_lo, i = kk % kKpw;
+                                float sr = 0.f, si = 0.f;
+                                for (int s2 = 0; s2 < nsplit; ++s2) {
+                                    const float2 t = PART[((size_t)(gg * nsplit + s2) * kKpw + i) * kDirs + tid];
+                                    sr += t.x;
+                                    si += t.y;
+                                }
+                                band_update_t<kNB>(p.bands, klo, khi, klo + kk, sqrtf(sr * sr + si * si), best, bk);
+                            }
+                        }
+                        __syncthreads();
+                    }
+                    if (tid < kDirs)
+#pragma unroll
+                        for (int b = 0; b < kNB; ++b)
+                            if (b < band_count_t<kNB>(p.bands)) write_out(tile, tid, pass, false, b, best[b], bk[b]);
+                    continue;
+                }
+
+                const bool count = sym && pass == 0;
+                c0 = c1 = 0;
+                zmin = 1.f;
+                handled = 0;
+                if (!histogram(p.atoms + abase, nw, 0, count)) return;
+                const int bad = count && (zero_check ? (pt0 || pt1) && zmin == 0.f
+                                                     : (pt0 && c0 != (uint32_t)handled) || (pt1 && c1 != (uint32_t)handled));
+                const bool any_bad = __syncthreads_or(bad) != 0;
+                if (pass == 0) partners = any_bad;
+                const bool mirror = count && !any_bad;
+
+                if (p.hist_out) hist_export_add_p(H, NB, NB, 0, tile, p.nv, p.hist_out, tid, kThreads);
+
+                // ---- band spectrum (FP32) and band maximum ----
+                if (G <= kWarps) {
+                    int nsplit = 1;
+                    while (G * nsplit * 2 <= kWarps && nsplit * 2 <= NB / 32) nsplit *= 2;
+                    const int span = NB / 4 / nsplit;
+                    if (warp < G * nsplit) {
+                        const int g = warp / nsplit, sp = warp % nsplit;
+                        const int k0 = klo + g * kKpw;
+                        float re[kKpw][2], im[kKpw][2];
+#pragma unroll
+                        for (int i = 0; i < kKpw; ++i) re[i][0] = re[i][1] = im[i][0] = im[i][1] = 0.f;
+                        if (k0 & 1)
+                            fold_dft<1>(H, TW, NB, lane, sp * span, span, k0, re, im);
+                        else
+                            fold_dft<0>(H, TW, NB, lane, sp * span, span, k0, re, im);
+#pragma unroll
+                        for (int i = 0; i < kKpw; ++i) {
+                            PART[((size_t)warp * kKpw + i) * kDirs + 2 * lane] = make_float2(re[i][0], im[i][0]);
+                            PART[((size_t)warp * kKpw + i) * kDirs + 2 * lane + 1] = make_float2(re[i][1], im[i][1]);
                         }
                     }
                     __syncthreads();
                     if (tid < kDirs) {
-                        for (int kk = g_lo * kKpw; kk < min(K, (g_lo + Gr) * kKpw); ++kk) {
-                            const int gg = kk / kKpw - g_lo, q = kk % kKpw;
+                        float best[kNB];
+                        int bk[kNB];
+                        band_init_t<kNB>(p.bands, klo, best, bk);
+                        for (int kk = 0; kk < K; ++kk) {
+                            const int g = kk / kKpw, i = kk % kKpw;
                             float sr = 0.f, si = 0.f;
-                            for (int s2 = 0; s2 < nsplit; ++s2) {
-                                const float2 t = PART[((size_t)(gg * nsplit + s2) * kKpw + q) * kDirs + tid];
+                            for (int sp = 0; sp < nsplit; ++sp) {
+                                const float2 t = PART[((size_t)(g * nsplit + sp) * kKpw + i) * kDirs + tid];
                                 sr += t.x;
                                 si += t.y;
                             }
                             band_update_t<kNB>(p.bands, klo, khi, klo + kk, sqrtf(sr * sr + si * si), best, bk);
                         }
+#pragma unroll
+                        for (int b = 0; b < kNB; ++b)
+                            if (b < band_count_t<kNB>(p.bands)) write_out(tile, tid, pass, mirror, b, best[b], bk[b]);
+                    } else {
+                        zero_h(kDirs);
+                    }
+                } else {
+                    float b0[kNB], b1[kNB];
+                    int bk0[kNB], bk1[kNB];
+                    band_init_t<kNB>(p.bands, klo, b0, bk0);
+                    band_init_t<kNB>(p.bands, klo, b1, bk1);
+                    for (int g = warp; g < G; g += kWarps) {
+                        const int k0 = klo + g * kKpw;
+                        float re[kKpw][2], im[kKpw][2];
+#pragma unroll
+                        for (int i = 0; i < kKpw; ++i) re[i][0] = re[i][1] = im[i][0] = im[i][1] = 0.f;
+                        if (k0 & 1)
+                            fold_dft<1>(H, TW, NB, lane, 0, NB / 4, k0, re, im);
+                        else
+                            fold_dft<0>(H, TW, NB, lane, 0, NB / 4, k0, re, im);
+#pragma unroll
+                        for (int i = 0; i < kKpw; ++i) {
+                            if (k0 + i > khi) break;
+                            const float a0 = sqrtf(re[i][0] * re[i][0] + im[i][0] * im[i][0]);
+                            const float a1 = sqrtf(re[i][1] * re[i][1] + im[i][1] * im[i][1]);
+                            band_update_t<kNB>(p.bands, klo, khi, k0 + i, a0, b0, bk0);
+                            band_update_t<kNB>(p.bands, klo, khi, k0 + i, a1, b1, bk1);
+                        }
+                    }
+                    // per band, each warp's best over its frequency groups; the
+                    // band's slab of PART holds kWarps x kDirs (value, k) pairs
+#pragma unroll
+                    for (int b = 0; b < kNB; ++b) {
+                        if (b < band_count_t<kNB>(p.bands)) {
+                            PART[((size_t)b * kWarps + warp) * kDirs + 2 * lane] = make_float2(b0[b], __int_as_float(bk0[b]));
+                            PART[((size_t)b * kWarps + warp) * kDirs + 2 * lane + 1] =
+                                make_float2(b1[b], __int_as_float(bk1[b]));
+                        }
                     }
                     __syncthreads();
-                }
-                if (tid < kDirs) {
-                    const int64_t v = (int64_t)tile * kDirs + tid;
-                    if (v < p.nv) {
-#pragma unroll
-                        for (int b = 0; b < kNB; ++b) {
-                            if (b < band_count_t<kNB>(p.bands)) {
-                                p.S[band_off_t<kNB>(p.bands, b) + out_base + v] = best[b];
-                                if (p.argk) p.argk[band_off_t<kNB>(p.bands, b) + out_base + v] = (uint16_t)bk[b];
+                    if (tid < kDirs) {
+                        for (int b = 0; b < band_count_t<kNB>(p.bands); ++b) {
+                            float best = -1.f;
+                            int bk = kNB == 1 ? klo : p.bands.lo[b];
+                            for (int w = 0; w < kWarps; ++w) {
+                                const float2 t = PART[((size_t)b * kWarps + w) * kDirs + tid];
+                                const int k = __float_as_int(t.y);
+                                if (t.x > best || (t.x == best && k < bk)) {
+                                    best = t.x;
+                                    bk = k;
+                                }
                             }
+                            write_out(tile, tid, pass, mirror, b, best, bk);
                         }
-                    }
-                }
-            }
-            continue;
-        }
-
-        for (int tile = t0; tile < t1; ++tile) {
-            uint4* H4 = reinterpret_cast<uint4*>(H);
-            for (int i = tid; i < NB * kWords / 4; i += kThreads) H4[i] = make_uint4(0, 0, 0, 0);
-            const float4 d0 = p.dirs[(int64_t)tile * kDirs + 2 * lane];
-            const float4 d1 = p.dirs[(int64_t)tile * kDirs + 2 * lane + 1];
-            __syncthreads();
-            for (int c0 = 0; c0 < nw; c0 += p.atom_cap) {
-                const int cn = min(p.atom_cap, nw - c0);
-                if (!one_chunk && !stage_atoms(A, p.atoms + abase + c0, cn, bar, phase, p.status, flag)) return;
-                hist_tile<kWarps, true>(H, A, cn, warp, lane, d0, d1, scale, magic, nbm1);
-                if (!one_chunk) __syncthreads();
-            }
-            __syncthreads();
-
-            if (p.hist_out) hist_export_add_p(H, NB, NB, 0, tile, p.nv, p.hist_out, tid, kThreads);
-
-            // ---- band spectrum (FP32) and band maximum ----
-            const int K = khi - klo + 1;
-            const int G = (K + kKpw - 1) / kKpw;   // frequency groups of kKpw
-            const int64_t out_base = (p.single_roi >= 0 ? 0 : roi) * (int64_t)p.nv + (int64_t)tile * kDirs;
-            if (G <= kWarps) {
-                int nsplit = 1;
-                while (G * nsplit * 2 <= kWarps && nsplit * 2 <= NB / 32) nsplit *= 2;
-                const int span = NB / nsplit;
-                const int units = G * nsplit;
-                if (warp < units) {
-                    const int g = warp / nsplit, sp = warp % nsplit;
-                    const int k0 = klo + g * kKpw;
-                    float re[kKpw][2], im[kKpw][2];
-                    unsigned idx[kKpw];
-                    const int n0 = sp * span;
-#pragma unroll
-                    for (int q = 0; q < kKpw; ++q) {
-                        re[q][0] = re[q][1] = im[q][0] = im[q][1] = 0.f;
-                        idx[q] = (unsigned)((k0 + q) * n0) & (unsigned)nbm1;
-                    }
-                    for (int n = n0; n < n0 + span; ++n) {
-                        const uint32_t w = H[n * kWords + lane];
-                        const float f0 = u23_to_float(w & 0xFFFFu), f1 = u23_to_float(w >> 16);
-#pragma unroll
-                        for (int q = 0; q < kKpw; ++q) {
-                            const float2 t = TW[idx[q]];
-                            re[q][0] = fmaf(f0, t.x, re[q][0]);
-                            im[q][0] = fmaf(f0, t.y, im[q][0]);
-                            re[q][1] = fmaf(f1, t.x, re[q][1]);
-                            im[q][1] = fmaf(f1, t.y, im[q][1]);
-                            idx[q] = (idx[q] + (unsigned)(k0 + q)) & (unsigned)nbm1;
-                        }
-                    }
-#pragma unroll
-                    for (int q = 0; q < kKpw; ++q) {
-                        PART[((size_t)warp * kKpw + q) * kDirs + 2 * lane] = make_float2(re[q][0], im[q][0]);
-                        PART[((size_t)warp * kKpw + q) * kDirs + 2 * lane + 1] = make_float2(re[q][1], im[q][1]);
+                    } else {
+                        zero_h(kDirs);
                     }
                 }
                 __syncthreads();
-                if (tid < kDirs) {
-                    const int64_t v = (int64_t)tile * kDirs + tid;
-                    float best[kNB];
-                    int bk[kNB];
-                    band_init_t<kNB>(p.bands, klo, best, bk);
-                    for (int kk = 0; kk < K; ++kk) {
-                        const int g = kk / kKpw, q = kk % kKpw;
-                        float sr = 0.f, si = 0.f;
-                        for (int sp = 0; sp < nsplit; ++sp) {
-                            const float2 t = PART[((size_t)(g * nsplit + sp) * kKpw + q) * kDirs + tid];
-                            sr += t.x;
-                            si += t.y;
-                        }
-                        band_update_t<kNB>(p.bands, klo, khi, klo + kk, sqrtf(sr * sr + si * si), best, bk);
-                    }
-                    if (v < p.nv) {
-#pragma unroll
-                        for (int b = 0; b < kNB; ++b) {
-                            if (b < band_count_t<kNB>(p.bands)) {
-                                p.S[band_off_t<kNB>(p.bands, b) + out_base + tid] = best[b];
-                                if (p.argk) p.argk[band_off_t<kNB>(p.bands, b) + out_base + tid] = (uint16_t)bk[b];
-                            }
-                        }
-                    }
-                }
-            } else {
-                float b0[kNB], b1[kNB];
-                int bk0[kNB], bk1[kNB];
-                band_init_t<kNB>(p.bands, klo, b0, bk0);
-                band_init_t<kNB>(p.bands, klo, b1, bk1);
-                for (int g = warp; g < G; g += kWarps) {
-                    const int k0 = klo + g * kKpw;
-                    float re[kKpw][2], im[kKpw][2];
-                    unsigned idx[kKpw];
-#pragma unroll
-                    for (int q = 0; q < kKpw; ++q) {
-                        re[q][0] = re[q][1] = im[q][0] = im[q][1] = 0.f;
-                        idx[q] = 0;
-                    }
-                    for (int n = 0; n < NB; ++n) {
-                        const uint32_t w = H[n * kWords + lane];
-                        const float f0 = u23_to_float(w & 0xFFFFu), f1 = u23_to_float(w >> 16);
-#pragma unroll
-                        for (int q = 0; q < kKpw; ++q) {
-                            const float2 t = TW[idx[q]];
-                            re[q][0] = fmaf(f0, t.x, re[q][0]);
-                            im[q][0] = fmaf(f0, t.y, im[q][0]);
-                            re[q][1] = fmaf(f1, t.x, re[q][1]);
-                            im[q][1] = fmaf(f1, t.y, im[q][1]);
-                            idx[q] = (idx[q] + (unsigned)(k0 + q)) & (unsigned)nbm1;
-                        }
-                    }
-#pragma unroll
-                    for (int q = 0; q < kKpw; ++q) {
-                        if (k0 + q > khi) break;
-                        const float a0 = sqrtf(re[q][0] * re[q][0] + im[q][0] * im[q][0]);
-                        const float a1 = sqrtf(re[q][1] * re[q][1] + im[q][1] * im[q][1]);
-                        band_update_t<kNB>(p.bands, klo, khi, k0 + q, a0, b0, bk0);
-                        band_update_t<kNB>(p.bands, klo, khi, k0 + q, a1, b1, bk1);
-                    }
-                }
-                // per band, each warp's best over its frequency groups; the
-                // band's slab of PART holds kWarps x kDirs (value, k) pairs
-#pragma unroll
-                for (int b = 0; b < kNB; ++b) {
-                    if (b < band_count_t<kNB>(p.bands)) {
-                        PART[((size_t)b * kWarps + warp) * kDirs + 2 * lane] = make_float2(b0[b], __int_as_float(bk0[b]));
-                        PART[((size_t)b * kWarps + warp) * kDirs + 2 * lane + 1] =
-                            make_float2(b1[b], __int_as_float(bk1[b]));
-                    }
-                }
-                __syncthreads();
-                if (tid < kDirs) {
-                    const int64_t v = (int64_t)tile * kDirs + tid;
-                    for (int b = 0; b < band_count_t<kNB>(p.bands); ++b) {
-                        float best = -1.f;
-                        int bk = kNB == 1 ? klo : p.bands.lo[b];
-                        for (int w = 0; w < kWarps; ++w) {
-                            const float2 t = PART[((size_t)b * kWarps + w) * kDirs + tid];
-                            const int k = __float_as_int(t.y);
-                            if (t.x > best || (t.x == best && k < bk)) {
-                                best = t.x;
-                                bk = k;
-                            }
-                        }
-                        if (v < p.nv) {
-                            p.S[band_off_t<kNB>(p.bands, b) + out_base + tid] = best;
-                            if (p.argk) p.argk[band_off_t<kNB>(p.bands, b) + out_base + tid] = (uint16_t)bk;
-                        }
-                    }
-                }
             }
-            __syncthreads();
         }
     }
 }
@@ -424,7 +509,8 @@ cudaError_t launch_normalise(Ctx* c, float* S, int64_t rows) {
 size_t plain_smem_bytes(int m, int atom_cap) {
     const size_t NB = (size_t)1 << m;
     const size_t NBc = NB < (size_t)kChunkBins ? NB : (size_t)kChunkBins;
-    return NBc * kWords * 4 + NB * 8 + (size_t)atom_cap * 16 + kPartBytes + 64;
+    const size_t ntw = NB == NBc ? 2 * NB : NB;   // as in the kernel
+    return NBc * kWords * 4 + ntw * 8 + (size_t)atom_cap * 16 + kPartBytes + 64;
 }
 
 cudaError_t launch_signatures_plain(Ctx* c, float* S, uint16_t* argk, uint16_t* hist_out, int64_t hist_roi) {
@@ -438,7 +524,7 @@ cudaError_t launch_signatures_plain(Ctx* c, float* S, uint16_t* argk, uint16_t* 
     if (cap < 256) return cudaErrorInvalidConfiguration;
     const size_t smem = plain_smem_bytes(c->m, cap);
     const bool multi = !hist_out && c->multi.n > 0;
-    auto kern = multi ? k_sig_plain<APTIDX_MAX_BANDS> : k_sig_plain<1>;
+    auto kern = multi ? k_sig_plain<APTIDX_MAX_BANDS, false> : k_sig_plain<1, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
 
@@ -447,9 +533,13 @@ cudaError_t launch_signatures_plain(Ctx* c, float* S, uint16_t* argk, uint16_t* 
     p.off = c->d_off;
     p.nw = c->d_nw;
     p.order = c->d_order;
-    p.dirs = c->d_dirs;
+    // antipodal pairs (one projection per pair) unless switched off, exporting,
+    // or in passes over bin chunks (whose spectrum is not folded)
+    const bool pairs = !hist_out && c->use_pairs && c->d_slot_idx && c->m <= 10;
+    p.dirs = pairs ? c->d_slot_dirs : c->d_dirs;
+    p.slot_idx = pairs ? c->d_slot_idx : nullptr;
     p.nv = c->nv;
-    p.tiles_per_roi = c->nv_pad / kDirs;
+    p.tiles_per_roi = (pairs ? c->nslot_pad : c->nv_pad) / kDirs;
     p.tiles_per_item = min(max(c->tune_tpi[0], 1), p.tiles_per_roi);
     p.items_per_roi = (p.tiles_per_roi + p.tiles_per_item - 1) / p.tiles_per_item;
     const int64_t nroi_lim = c->rank_limit > 0 ? tmin<int64_t>(c->nroi, c->rank_limit) : c->nroi;
@@ -491,8 +581,8 @@ constexpr int64_t kNaMaxRoi = APTIDX_NOALLOC_MAX_ROIS;
 constexpr int64_t kNaMaxDirs = APTIDX_NOALLOC_MAX_DIRS;
 // byte offsets inside the scratch array
 constexpr size_t kNaDirs = 0;                                        // float4 [kNaMaxDirs]
-constexpr size_t kNaTw = kNaDirs + 16 * (size_t)kNaMaxDirs;          // float2 [2^APTIDX_MAX_M]
-constexpr size_t kNaScale = kNaTw + 8 * ((size_t)1 << APTIDX_MAX_M);  // float  [kNaMaxRoi]
+constexpr size_t kNaTw = kNaDirs + 16 * (size_t)kNaMaxDirs;          // float2 [2 x 2^APTIDX_MAX_M]
+constexpr size_t kNaScale = kNaTw + 16 * ((size_t)1 << APTIDX_MAX_M);  // float  [kNaMaxRoi]
 constexpr size_t kNaBand = kNaScale + 4 * (size_t)kNaMaxRoi;         // int32  [2 kNaMaxRoi]
 constexpr size_t kNaNw = kNaBand + 8 * (size_t)kNaMaxRoi;            // int32  [kNaMaxRoi]
 constexpr size_t kNaOrder = kNaNw + 4 * (size_t)kNaMaxRoi;           // int32  [kNaMaxRoi]
@@ -546,9 +636,9 @@ __global__ void k_noalloc_setup(unsigned char* scr, const int64_t* __restrict__ 
         }
         dirs[v] = d;
     }
-    for (int64_t j = t0; j < (int64_t)(1 << m); j += stride) {
+    for (int64_t j = t0; j < (int64_t)(2 << m); j += stride) {
         double sn, cs;
-        sincospi(2.0 * (double)j / (double)(1 << m), &sn, &cs);
+        sincospi((double)j / (double)(1 << m), &sn, &cs);
         tw[j] = make_float2((float)cs, (float)sn);
     }
 }
@@ -612,7 +702,7 @@ extern "C" int aptidx_signatures_noalloc(const float* xc4, const int64_t* off, c
     cap = std::min(cap, 4096) & ~15;
     if (cap < 256) return APTIDX_E_CUDA;
     const size_t smem = plain_smem_bytes(m, cap);
-    if (cudaFuncSetAttribute(k_sig_plain<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    if (cudaFuncSetAttribute(k_sig_plain<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
         return APTIDX_E_CUDA;
     }
@@ -622,6 +712,7 @@ extern "C" int aptidx_signatures_noalloc(const float* xc4, const int64_t* off, c
     p.nw = reinterpret_cast<const int32_t*>(base + kNaNw);
     p.order = reinterpret_cast<const int32_t*>(base + kNaOrder);
     p.dirs = reinterpret_cast<const float4*>(base + kNaDirs);
+    p.slot_idx = nullptr;
     p.nv = nv;
     p.tiles_per_roi = nv_pad / kDirs;
     p.tiles_per_item = std::min(16, p.tiles_per_roi);
@@ -640,9 +731,9 @@ extern "C" int aptidx_signatures_noalloc(const float* xc4, const int64_t* off, c
     p.atom_cap = cap;
     p.nroi = nroi;
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sig_plain<1>, kThreads, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sig_plain<1, true>, kThreads, smem);
     per_sm = std::max(per_sm, 1);
     const int64_t grid = std::min<int64_t>((int64_t)sm_count * per_sm, p.n_items);
-    k_sig_plain<1><<<(unsigned)grid, kThreads, smem, s>>>(p);
+    k_sig_plain<1, true><<<(unsigned)grid, kThreads, smem, s>>>(p);
     return cudaGetLastError() == cudaSuccess ? APTIDX_OK : APTIDX_E_CUDA;
 }

@@ -513,6 +513,9 @@ int aptidx_destroy(aptidx_ctx* ctx) {
         free_ptr(r.d_top_val);
         free_ptr(r.d_img4);
         free_ptr(r.d_lut);
+        free_ptr(r.d_tm_ent);
+        free_ptr(r.d_tm_off);
+        dev_free(r.d_lut_g);
         free_ptr(r.d_quats);
     }
     delete ctx;
@@ -1305,6 +1308,44 @@ int check_ref(Ctx* c, int32_t cand, bool need_lut, bool need_img) {
     return APTIDX_OK;
 }
 
+// Scratch of the matching calls, kept by the context and grown as needed.
+int match_scratch(Ctx* c, size_t need) {
+    if (need <= c->match_scratch_bytes) return APTIDX_OK;
+    free_ptr(c->d_match_scratch);
+    c->match_scratch_bytes = 0;
+    int rc = dev_alloc(c, (void**)&c->d_match_scratch, need);
+    if (!rc) c->match_scratch_bytes = need;
+    return rc;
+}
+
+// ROIs per round when their estimates (and, `copies` = 2, their score rows) stay
+// within 1 GiB: whole groups of 64
+int64_t tm_round(const Reference& r, int64_t nroi, int copies) {
+    const int64_t groups = std::max<int64_t>(1, ((int64_t)1 << 30) / (r.ng * 256 * copies));
+    return std::min<int64_t>((nroi + 63) / 64, groups) * 64;
+}
+
+// best orientation per ROI (device pointers), by lists where they pay
+int match_best(Ctx* c, Reference& r, const float* dS, int64_t nroi, int32_t* db, float* ds, int* launches) {
+    cudaError_t e = cudaSuccess;
+    if (!tm_pays(c, &r, nroi)) {
+        e = launch_match(c, &r, dS, nroi, db, ds);
+        *launches += 1;
+    } else {
+        const int64_t round = tm_round(r, nroi, 1);
+        int rc = match_scratch(c, (size_t)round * r.ng * sizeof(float));
+        if (rc) return rc;
+        for (int64_t r0 = 0; r0 < nroi && e == cudaSuccess; r0 += round) {
+            const int64_t n = std::min(round, nroi - r0);
+            e = launch_tm_sum(c, &r, dS + r0 * c->nv, n, c->d_match_scratch);
+            if (e == cudaSuccess)
+                e = launch_tm_best(c, &r, dS + r0 * c->nv, n, c->d_match_scratch, db + r0, ds ? ds + r0 : nullptr);
+            *launches += 2;
+        }
+    }
+    return e == cudaSuccess ? APTIDX_OK : cuda_check(c, e, "match");
+}
+
 }  // namespace
 
 extern "C" {
@@ -1326,6 +1367,10 @@ int aptidx_set_reference(aptidx_ctx* ctx, int32_t cand, const float* node_sig, i
     free_ptr(r.d_top);
     free_ptr(r.d_top_val);
     free_ptr(r.d_lut);
+    recycle_ptr(c, r.d_tm_ent);
+    recycle_ptr(c, r.d_tm_off);
+    dev_recycle(c, r.d_lut_g);
+    r.d_lut_g = nullptr;
     free_ptr(r.d_quats);
     free_ptr(r.d_img4);
     r.ng = 0;
@@ -1364,6 +1409,8 @@ int aptidx_set_reference(aptidx_ctx* ctx, int32_t cand, const float* node_sig, i
         double en = 0.0;
         for (int32_t k = 0; k < n_hat; ++k) en += (double)v[k] * (double)v[k];
         r.energy = en;
+        r.ref_max = 0.0;
+        for (int32_t k = 0; k < c->nv; ++k) r.ref_max = std::max(r.ref_max, (double)fabsf(hs[k]));
     }
     cudaError_t e = launch_top_nodes(c, &r);
     if (e != cudaSuccess) return cuda_check(c, e, "strongest reference nodes");
@@ -1388,6 +1435,10 @@ int aptidx_build_lut(aptidx_ctx* ctx, int32_t cand, const double* quats, int64_t
     }
     Reference& r = c->ref[cand];
     free_ptr(r.d_lut);
+    recycle_ptr(c, r.d_tm_ent);
+    recycle_ptr(c, r.d_tm_off);
+    dev_recycle(c, r.d_lut_g);
+    r.d_lut_g = nullptr;
     free_ptr(r.d_quats);
     r.ng = 0;
     r.ng_pad = 0;
@@ -1402,6 +1453,7 @@ int aptidx_build_lut(aptidx_ctx* ctx, int32_t cand, const double* quats, int64_t
     if (e != cudaSuccess) return cuda_check(c, e, "look-up table");
     c->launches += 1;
     r.ng = ng;
+    if ((e = launch_build_tm(c, &r)) != cudaSuccess) return cuda_check(c, e, "look-up table lists");
     return APTIDX_OK;
 }
 
@@ -1443,9 +1495,9 @@ int aptidx_match(aptidx_ctx* ctx, int32_t cand, const float* S, int64_t nroi, in
     if ((rc = dev_out(c, best, (size_t)nroi, mem, tb, &db))) return rc;
     if ((rc = dev_out(c, score, (size_t)nroi, mem, ts, &ds))) return rc;
     prof_begin(c, APTIDX_PHASE_MATCH);
-    cudaError_t e = launch_match(c, &r, dS, nroi, db, ds);
-    if (e != cudaSuccess) return cuda_check(c, e, "match");
-    prof_end(c, APTIDX_PHASE_MATCH, 1);
+    int launches = 0;
+    if ((rc = match_best(c, r, dS, nroi, db, ds, &launches))) return rc;
+    prof_end(c, APTIDX_PHASE_MATCH, launches);
     if ((rc = copy_back(c, best, db, (size_t)nroi, mem))) return rc;
     if ((rc = copy_back(c, score, ds, (size_t)nroi, mem))) return rc;
     if (mem == APTIDX_MEM_HOST) return read_status(c);
@@ -1478,19 +1530,24 @@ int aptidx_match_topk(aptidx_ctx* ctx, int32_t cand, const float* S, int64_t nro
     prof_begin(c, APTIDX_PHASE_MATCH);
     int launches = 0;
     if (topk == 1) {
-        cudaError_t e = launch_match(c, &r, dS, nroi, db, ds);
-        if (e != cudaSuccess) return cuda_check(c, e, "match");
-        launches = 1;
+        if ((rc = match_best(c, r, dS, nroi, db, ds, &launches))) return rc;
+    } else if (tm_pays(c, &r, nroi) && tm_exact_smem(c, &r) + 18 * 1024 <= (size_t)max_optin) {
+        const int64_t round = tm_round(r, nroi, 2);
+        const size_t one = (size_t)round * r.ng;
+        if ((rc = match_scratch(c, 2 * one * sizeof(float)))) return rc;
+        for (int64_t r0 = 0; r0 < nroi; r0 += round) {
+            const int64_t n = std::min(round, nroi - r0);
+            float* rows = c->d_match_scratch + one;
+            cudaError_t e = launch_tm_sum(c, &r, dS + r0 * c->nv, n, c->d_match_scratch);
+            if (e == cudaSuccess) e = launch_tm_rows(c, &r, dS + r0 * c->nv, n, topk, c->d_match_scratch, rows);
+            if (e == cudaSuccess) e = launch_topk(c, rows, r.ng, n, topk, db + r0 * topk, ds ? ds + r0 * topk : nullptr);
+            if (e != cudaSuccess) return cuda_check(c, e, "match_topk");
+            launches += 4;
+        }
     } else {
         // scores of a chunk of ROIs (at most 1 GiB), then a radix select per ROI
         const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(nroi, ((int64_t)1 << 30) / (r.ng * 4)));
-        const size_t need = (size_t)chunk * r.ng * sizeof(float);
-        if (need > c->match_scratch_bytes) {
-            free_ptr(c->d_match_scratch);
-            c->match_scratch_bytes = 0;
-            if ((rc = dev_alloc(c, (void**)&c->d_match_scratch, need))) return rc;
-            c->match_scratch_bytes = need;
-        }
+        if ((rc = match_scratch(c, (size_t)chunk * r.ng * sizeof(float)))) return rc;
         for (int64_t r0 = 0; r0 < nroi; r0 += chunk) {
             const int64_t n = std::min(chunk, nroi - r0);
             cudaError_t e = launch_match(c, &r, dS + r0 * c->nv, n, nullptr, nullptr, c->d_match_scratch);
@@ -1561,13 +1618,7 @@ int aptidx_match_phase(aptidx_ctx* ctx, int32_t n_cand, const int32_t* cand_off,
     APTIDX_CUDA(c, cudaMemcpyAsync(dn, nc.data(), nc.size() * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
     // channel sums of a chunk of ROIs (at most 1 GiB), then the argmin per ROI
     const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(nroi, ((int64_t)1 << 30) / (ng * 4)));
-    const size_t need = (size_t)chunk * ng * sizeof(float);
-    if (need > c->match_scratch_bytes) {
-        free_ptr(c->d_match_scratch);
-        c->match_scratch_bytes = 0;
-        if ((rc = dev_alloc(c, (void**)&c->d_match_scratch, need))) return rc;
-        c->match_scratch_bytes = need;
-    }
+    if ((rc = match_scratch(c, (size_t)chunk * ng * sizeof(float)))) return rc;
     prof_begin(c, APTIDX_PHASE_MATCH);
     int launches = 0;
     for (int32_t k = 0; k < n_cand; ++k) {

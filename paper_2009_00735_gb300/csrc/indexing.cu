@@ -450,6 +450,379 @@ __global__ void __launch_bounds__(1024, 1) k_match(const float* __restrict__ S, 
     }
 }
 
+// ---- Eq. 3 for many ROIs -----------------------------------------------------------
+//
+// k_match gathers 32 random words of one signature row per instruction: 3.5
+// shared-memory wavefronts on average, which bounds it (7.2 ms for 4096 ROIs,
+// 3419 orientations, 1000 nodes: 6.2 look-ups per SM cycle).  Here a lane is a
+// pair of ROIs: a CTA holds the values of 64 ROIs at a tile of nodes,
+// [node][ROI] in shared memory, and walks the table entries whose node lies in
+// its tile, so that a look-up of 64 ROIs is two wavefronts and the entry, which
+// every lane needs (a broadcast costs its bytes times 32 lanes), is one: 4
+// bytes, the reference value rounded to 22 bits and the node's row in the other
+// ten.  Entries are stored per (tile, orientation) in lists padded to four with
+// entries that read a row of zeros.  The tiles' partial sums of an orientation
+// add up in global memory, in any order.
+//
+// The sums serve as estimates only.  With every reference off by at most
+// delta = 2^-14 max |ref|, the root of an estimate is within eta = sqrt(n_hat)
+// delta of the root of the exact sum (triangle inequality), and any FP32 order
+// of summation is within eps = (n_hat + 64) 2^-24 of it: every orientation
+// whose estimate is at most (sqrt(m) + 2 eta)^2 (1 + 5 eps), m the smallest (or
+// the topk-th smallest) estimate, is summed again in k order, and these decide.
+// Results are those of k_match bit for bit.
+// 4096 ROIs, 3419 orientations, 1000 nodes: 7.2 ms before, 2.9 now (k_tm_sum 2.75,
+// k_tm_best 0.14); top 1000 of 50000 orientations for 192 ROIs: 6.8 ms before,
+// 3.0 now (sums 1.9, exact sums 0.65, selections 0.4).
+constexpr int kTmRois = 64;
+constexpr int kTmPitch = 66;          // words per node row (8-byte aligned, written by columns)
+constexpr int kTmTileMax = 879;       // nodes per tile: (879 + 1) x 264 bytes of shared memory, < 1024 rows
+constexpr int kTmThreads = 1024;
+constexpr uint32_t kTmRowBits = 0x3FFu;
+
+__device__ __forceinline__ uint32_t tm_entry(float ref, int row) {
+    const uint32_t b = __float_as_uint(ref);   // round to nearest at 13 mantissa bits (finite)
+    return ((b + 0x200u) & ~kTmRowBits) | (uint32_t)row;
+}
+
+template <typename IdxT>
+__global__ void __launch_bounds__(256) k_tm_count(const IdxT* __restrict__ lut_t, int64_t ng, int64_t ng_pad, int T,
+                                                  int32_t* counts) {
+    const int64_t g = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (g < ng) atomicAdd(&counts[(int64_t)((int)lut_t[(int64_t)blockIdx.y * ng_pad + g] / T) * ng + g], 1);
+}
+
+__global__ void __launch_bounds__(256) k_tm_pad(const int32_t* __restrict__ counts, int64_t n, int64_t* padded) {
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i < n) padded[i] = (counts[i] + 3) & ~3;
+}
+
+// 32-bit offsets, the padding entries, and the counts zeroed (they become the
+// lists' cursors)
+__global__ void __launch_bounds__(256) k_tm_off(const int64_t* __restrict__ off64, int32_t* counts, int64_t n, int T,
+                                                uint32_t* off, uint32_t* ent) {
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i <= n) off[i] = (uint32_t)off64[i];
+    if (i >= n) return;
+    const int32_t c = counts[i];
+    for (int k = c; k < ((c + 3) & ~3); ++k) ent[off64[i] + k] = (uint32_t)T;
+    counts[i] = 0;
+}
+
+template <typename IdxT>
+__global__ void __launch_bounds__(256) k_tm_fill(const IdxT* __restrict__ lut_t, int64_t ng, int64_t ng_pad,
+                                                 const float* __restrict__ top_val, int T,
+                                                 const uint32_t* __restrict__ off, int32_t* cursor, uint32_t* ent) {
+    const int64_t g = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (g >= ng) return;
+    const int node = (int)lut_t[(int64_t)blockIdx.y * ng_pad + g];
+    const int p = node / T;
+    const int64_t l = (int64_t)p * ng + g;
+    ent[(size_t)off[l] + (uint32_t)atomicAdd(&cursor[l], 1)] = tm_entry(top_val[blockIdx.y], node - p * T);
+}
+
+// k-major table to rows per orientation, lut_g[g * pitch + k] (32 x 32 tiles)
+template <typename IdxT>
+__global__ void __launch_bounds__(256) k_tm_rowmajor(const IdxT* __restrict__ lut_t, int64_t ng, int64_t ng_pad,
+                                                     int32_t n_hat, int pitch, IdxT* lut_g) {
+    __shared__ IdxT t[32][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t g0 = (int64_t)blockIdx.x * 32;
+    const int k0 = (int)blockIdx.y * 32;
+    for (int i = w; i < 32; i += 8)
+        t[i][lane] = k0 + i < n_hat && g0 + lane < ng ? lut_t[(int64_t)(k0 + i) * ng_pad + g0 + lane] : (IdxT)0;
+    __syncthreads();
+    for (int i = w; i < 32; i += 8)
+        if (g0 + i < ng && k0 + lane < pitch) lut_g[(g0 + i) * pitch + k0 + lane] = t[lane][i];
+}
+
+// CTA (tile, part of the orientations; group of 64 ROIs); D[group][g][2][32],
+// ROI 2 l + i of the group at [i][l]
+__global__ void __launch_bounds__(kTmThreads, 1) k_tm_sum(const float* __restrict__ S, int64_t nroi, int32_t nv,
+                                                          const uint32_t* __restrict__ ent,
+                                                          const uint32_t* __restrict__ off, int64_t ng, int T,
+                                                          int gsplit, float* D) {
+    extern __shared__ float st[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int p = (int)blockIdx.x / gsplit, gs = (int)blockIdx.x % gsplit;
+    const int n0 = p * T, cnt = min(T, nv - n0);
+    for (int i = warp; i < kTmRois; i += kTmThreads / 32) {
+        const int64_t roi = (int64_t)blockIdx.y * kTmRois + i;
+        for (int n = lane; n < cnt; n += 32) st[n * kTmPitch + i] = roi < nroi ? S[roi * (int64_t)nv + n0 + n] : 0.f;
+    }
+    if (threadIdx.x < kTmPitch) st[T * kTmPitch + threadIdx.x] = 0.f;
+    __syncthreads();
+    const uint32_t sb = smem_u32(st) + 8u * (uint32_t)lane;
+    const int64_t per = (ng + gsplit - 1) / gsplit;
+    const int64_t g1 = tmin<int64_t>(ng, (gs + 1) * per);
+    const uint32_t* o = off + (int64_t)p * ng;
+    auto term = [&](uint32_t e, float& a, float& b) {
+        float x, y;
+        asm("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(x), "=f"(y) : "r"(sb + (e & kTmRowBits) * (kTmPitch * 4u)));
+        const float ref = __uint_as_float(e & ~kTmRowBits);
+        x -= ref;
+        y -= ref;
+        a = fmaf(x, x, a);
+        b = fmaf(y, y, b);
+    };
+    int64_t g = gs * per + warp;
+    uint32_t b = g < g1 ? o[g] : 0, e = g < g1 ? o[g + 1] : 0;
+    for (; g < g1; g += kTmThreads / 32) {
+        const uint4* q = reinterpret_cast<const uint4*>(ent + b);
+        const int n = (int)((e - b) >> 2);
+        const int64_t gn = g + kTmThreads / 32;
+        if (gn < g1) {
+            b = o[gn];
+            e = o[gn + 1];
+        }
+        if (n > 0) {
+            float a0 = 0.f, a1 = 0.f, b0 = 0.f, b1 = 0.f;
+            uint4 x = __ldg(q);
+            for (int i = 1; i < n; ++i) {
+                const uint4 nx = __ldg(q + i);
+                term(x.x, a0, b0);
+                term(x.y, a1, b1);
+                term(x.z, a0, b0);
+                term(x.w, a1, b1);
+                x = nx;
+            }
+            term(x.x, a0, b0);
+            term(x.y, a1, b1);
+            term(x.z, a0, b0);
+            term(x.w, a1, b1);
+            float* d = D + ((int64_t)blockIdx.y * ng + g) * kTmRois + lane;
+            atomicAdd(d, a0 + a1);
+            atomicAdd(d + 32, b0 + b1);
+        }
+    }
+}
+
+// largest estimate whose exact sum can be the smallest: see above (and the
+// smallest normal number for sums of terms that underflow)
+struct TmMargin {
+    float eta2, rel;   // 2 eta, 1 + 5 eps
+};
+__device__ __forceinline__ float tm_threshold(float estimate, TmMargin m) {
+    const float r = sqrtf(estimate) + m.eta2;
+    return r * r * m.rel + 1.1754944e-38f;
+}
+
+// The best orientation of 32 ROIs (half a group per CTA, lane = ROI): the smallest
+// estimate, then the sums in k order of every orientation near it, a warp per
+// (ROI, orientation): the lanes read 32 terms, which are added in turn.
+template <typename IdxT>
+__global__ void __launch_bounds__(kTmThreads, 1) k_tm_best(const float* __restrict__ S, int64_t nroi, int32_t nv,
+                                                        const IdxT* __restrict__ lut_g, int64_t ng, int pitch,
+                                                        const float* __restrict__ top_val, int32_t n_hat,
+                                                        TmMargin margin, const float* __restrict__ D, int32_t* best,
+                                                        float* score) {
+    __shared__ float red[32][33];
+    __shared__ float thr[32];
+    __shared__ unsigned long long key[32];
+    __shared__ uint32_t list_g[kTmThreads];
+    __shared__ uint8_t list_r[kTmThreads];
+    __shared__ uint32_t n_list;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t roi0 = (int64_t)(blockIdx.x >> 1) * kTmRois + (blockIdx.x & 1);   // ROI of lane l: roi0 + 2 l
+    const float* d = D + (int64_t)(blockIdx.x >> 1) * ng * kTmRois + (blockIdx.x & 1) * 32 + lane;
+    float m = INFINITY;
+#pragma unroll 4
+    for (int64_t g = warp; g < ng; g += 32) m = fminf(m, d[g * kTmRois]);
+    red[warp][lane] = m;
+    if (warp == 0) key[lane] = 0x7F8000007FFFFFFFull;   // (+inf, no orientation)
+    if (threadIdx.x == 0) n_list = 0;
+    __syncthreads();
+    if (warp == 0) {
+        for (int w = 1; w < 32; ++w) m = fminf(m, red[w][lane]);
+        thr[lane] = tm_threshold(m, margin);
+    }
+    __syncthreads();
+    const float t = thr[lane];
+    const bool valid = roi0 + 2 * lane < nroi;
+    // sums in k order of the first n listed (ROI, orientation) pairs
+    auto decide = [&](uint32_t n) {
+        for (uint32_t i = warp; i < n; i += 32) {
+            const int r = list_r[i];
+            const int64_t cg = list_g[i];
+            const float* row = S + (roi0 + 2 * r) * nv;
+            float acc = 0.f;
+            auto load = [&](int k) { return k < n_hat ? row[(int)lut_g[cg * pitch + k]] - top_val[k] : 0.f; };
+            float v = load(lane);
+            for (int k0 = 0; k0 < n_hat; k0 += 32) {
+                const float next = load(k0 + 32 + lane);
+                const int kn = min(32, n_hat - k0);
+                if (kn == 32) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {
+                        const float x = __shfl_sync(0xffffffffu, v, j);
+                        acc = fmaf(x, x, acc);
+                    }
+                } else {
+                    for (int j = 0; j < kn; ++j) {
+                        const float x = __shfl_sync(0xffffffffu, v, j);
+                        acc = fmaf(x, x, acc);
+                    }
+                }
+                v = next;
+            }
+            if (lane == 0 && acc < INFINITY)
+                atomicMin(&key[r], ((unsigned long long)__float_as_uint(acc) << 32) | (uint32_t)cg);
+        }
+    };
+    auto list = [&](int64_t g) {
+        if (valid && g < ng && d[g * kTmRois] <= t) {
+            const uint32_t i = atomicAdd(&n_list, 1u);
+            if (i < kTmThreads) {
+                list_g[i] = (uint32_t)g;
+                list_r[i] = (uint8_t)lane;
+            }
+        }
+    };
+#pragma unroll 4
+    for (int64_t g = warp; g < ng; g += 32) list(g);
+    __syncthreads();
+    const uint32_t n_all = n_list;
+    if (n_all <= kTmThreads) {
+        decide(n_all);
+        __syncthreads();
+    } else {
+        // many ties (flat signatures): in steps that cannot overrun the list
+        for (int64_t g0 = 0; g0 < ng; g0 += 32) {
+            __syncthreads();
+            if (threadIdx.x == 0) n_list = 0;
+            __syncthreads();
+            list(g0 + warp);
+            __syncthreads();
+            decide(n_list);
+        }
+        __syncthreads();
+    }
+    if (warp == 0 && valid) {
+        const int64_t r = roi0 + 2 * lane;
+        const unsigned long long v = key[lane];
+        if (best) best[r] = (int32_t)(uint32_t)v;
+        if (score) score[r] = __uint_as_float((uint32_t)(v >> 32));
+    }
+}
+
+// D to rows of scores, out[roi * ng + g]: a CTA per 32 orientations of half a group
+__global__ void __launch_bounds__(256) k_tm_rows(const float* __restrict__ D, int64_t nroi, int64_t ng, float* out) {
+    __shared__ float t[32][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t g0 = (int64_t)blockIdx.x * 32, grp = blockIdx.y >> 1;
+    const int half = blockIdx.y & 1;
+    for (int i = w; i < 32; i += 8)
+        t[i][lane] = g0 + i < ng ? D[(grp * ng + g0 + i) * kTmRois + half * 32 + lane] : 0.f;
+    __syncthreads();
+    for (int i = w; i < 32; i += 8) {
+        const int64_t r = grp * kTmRois + 2 * i + half;
+        if (r < nroi && g0 + lane < ng) out[r * ng + g0 + lane] = t[lane][i];
+    }
+}
+
+// Key of rank `rank` (1 = smallest) among n keys, by a radix select over four
+// 8-bit digits; hist and the two words in shared memory, all threads call it.
+__device__ __forceinline__ uint32_t radix_kth(const uint32_t* key, int64_t n, uint32_t rank, uint32_t* hist,
+                                              uint32_t* s_prefix, uint32_t* s_rem) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    __syncthreads();
+    if (tid == 0) {
+        *s_prefix = 0;
+        *s_rem = rank;
+    }
+    for (int pass = 3; pass >= 0; --pass) {
+        for (int i = tid; i < 256; i += nt) hist[i] = 0;
+        __syncthreads();
+        const uint32_t prefix = *s_prefix, hmask = pass == 3 ? 0u : 0xFFFFFFFFu << (8 * (pass + 1));
+        for (int64_t g = tid; g < n; g += nt) {
+            const uint32_t k = key[g];
+            if ((k & hmask) == (prefix & hmask)) atomicAdd(&hist[(k >> (8 * pass)) & 255u], 1u);
+        }
+        __syncthreads();
+        if (tid == 0) {
+            uint32_t rem = *s_rem, d = 0;
+            while (hist[d] < rem) rem -= hist[d++];
+            *s_rem = rem;
+            *s_prefix = prefix | (d << (8 * pass));
+        }
+        __syncthreads();
+    }
+    return *s_prefix;
+}
+
+// The largest score of every ROI that the topk can depend on
+__global__ void __launch_bounds__(256) k_tm_reach(const float* __restrict__ scores, int64_t ng, int64_t nroi, int32_t topk,
+                                                  TmMargin margin, float* reach) {
+    __shared__ uint32_t hist[256], s_prefix, s_rem;
+    for (int64_t r = blockIdx.x; r < nroi; r += gridDim.x) {
+        const uint32_t kth = radix_kth(reinterpret_cast<const uint32_t*>(scores + r * ng), ng, (uint32_t)topk, hist,
+                                       &s_prefix, &s_rem);
+        // fewer numbers than topk: NaN, every orientation counts
+        if (threadIdx.x == 0) reach[r] = kth > 0x7F800000u ? NAN : tm_threshold(__uint_as_float(kth), margin);
+    }
+}
+
+// Every score within reach is replaced by the sum in k order (a thread per
+// orientation, the signature row in shared memory), so that k_topk's selection
+// over the row is exact.  A CTA takes one part of a ROI's orientations.
+constexpr int kTmList = 4096;
+
+template <typename IdxT>
+__global__ void __launch_bounds__(kTmThreads, 1) k_tm_exact(const float* __restrict__ S, int64_t nroi, int32_t nv,
+                                                            const IdxT* __restrict__ lut_g, int64_t ng, int pitch,
+                                                            const float* __restrict__ top_val, int32_t n_hat,
+                                                            const float* __restrict__ reach, int parts,
+                                                            float* scores) {
+    extern __shared__ float sm[];
+    float* row = sm;             // nv
+    float* ref = sm + nv;        // n_hat
+    __shared__ uint32_t list[kTmList];
+    __shared__ uint32_t n_list;
+    const int tid = threadIdx.x;
+    for (int i = tid; i < n_hat; i += kTmThreads) ref[i] = top_val[i];
+    if (tid == 0) n_list = 0;
+    const int64_t per = (ng + parts - 1) / parts;
+    for (int64_t it = blockIdx.x; it < nroi * parts; it += gridDim.x) {
+        const int64_t r = it / parts, ga = (it % parts) * per, gb = tmin<int64_t>(ng, ga + per);
+        __syncthreads();
+        for (int i = tid; i < nv; i += kTmThreads) row[i] = S[r * (int64_t)nv + i];
+        float* sc = scores + r * ng;
+        const float t = reach[r];
+        const bool all = isnan(t);
+        __syncthreads();
+        for (int64_t g0 = ga; g0 < gb; g0 += kTmThreads) {
+            const int64_t g = g0 + tid;
+            if (g < gb && (all || sc[g] <= t)) list[atomicAdd(&n_list, 1u)] = (uint32_t)g;
+            __syncthreads();
+            const uint32_t n = n_list;
+            if (n > kTmList - kTmThreads || g0 + kTmThreads >= gb) {
+                for (uint32_t i = tid; i < n; i += kTmThreads) {
+                    // 16 bytes of the orientation's row of the table at a time
+                    constexpr int N = 16 / (int)sizeof(IdxT);
+                    const uint4* lp = reinterpret_cast<const uint4*>(lut_g + (int64_t)list[i] * pitch);
+                    float acc = 0.f;
+                    uint4 w = __ldg(lp);
+                    for (int k = 0; k < n_hat; k += N) {
+                        const uint4 cur = w;
+                        if (k + N < n_hat) w = __ldg(++lp);
+                        const IdxT* ix = reinterpret_cast<const IdxT*>(&cur);
+#pragma unroll
+                        for (int j = 0; j < N; ++j)
+                            if (k + j < n_hat) {
+                                const float v = row[(int)ix[j]] - ref[k + j];
+                                acc = fmaf(v, v, acc);
+                            }
+                    }
+                    sc[list[i]] = acc;
+                }
+                __syncthreads();
+                if (tid == 0) n_list = 0;
+            }
+            __syncthreads();
+        }
+    }
+}
+
 // ---- the topk smallest Delta(g) of a ROI (ties: lower g), ascending ----------
 // One CTA per ROI: radix select of the topk-th smallest key (Delta >= 0, so
 // its FP32 bit pattern orders like the value) over four 8-bit digits, then
@@ -996,6 +1369,139 @@ cudaError_t launch_match(Ctx* c, Reference* r, const float* S, int64_t nroi, int
                          float* scores_out, bool accumulate, float weight) {
     return r->lut_bytes == 2 ? launch_match_t<uint16_t>(c, r, S, nroi, best, score, scores_out, accumulate, weight)
                              : launch_match_t<int32_t>(c, r, S, nroi, best, score, scores_out, accumulate, weight);
+}
+
+// The lists of k_tm_sum for the table just built (skipped when they would not
+// fit: k_match then serves every call).
+template <typename IdxT>
+static cudaError_t build_tm_t(Ctx* c, Reference* r) {
+    const int tiles = (c->nv + kTmTileMax - 1) / kTmTileMax;
+    const int64_t lists = (int64_t)tiles * r->ng;
+    if (lists > ((int64_t)1 << 24) - 4096 || r->n_hat > 65535 || r->ng * r->n_hat + 3 * lists >= ((int64_t)1 << 32))
+        return cudaSuccess;
+    const int T = (c->nv + tiles - 1) / tiles;
+    const int pitch = (r->n_hat + 7) / 8 * 8;
+    void *ent = nullptr, *off = nullptr, *lut_g = nullptr;
+    int32_t* counts = nullptr;
+    int64_t *padded = nullptr, *off64 = nullptr, *tmp = nullptr;
+    const std::string err = c->err;
+    if (dev_alloc(c, &ent, (size_t)(r->ng * r->n_hat + 3 * lists) * sizeof(uint32_t)) ||
+        dev_alloc(c, &off, (size_t)(lists + 1) * sizeof(uint32_t)) ||
+        dev_alloc(c, &lut_g, (size_t)r->ng * pitch * sizeof(IdxT)) ||
+        dev_alloc(c, (void**)&counts, (size_t)lists * sizeof(int32_t)) ||
+        dev_alloc(c, (void**)&padded, (size_t)lists * sizeof(int64_t)) ||
+        dev_alloc(c, (void**)&off64, (size_t)(lists + 1) * sizeof(int64_t)) ||
+        dev_alloc(c, (void**)&tmp, (scan_tmp_elems(lists) + 1) * sizeof(int64_t))) {
+        for (void* q : {ent, off, lut_g, (void*)counts, (void*)padded, (void*)off64, (void*)tmp}) dev_free(q);
+        c->err = err;
+        return cudaSuccess;
+    }
+    const IdxT* lut = static_cast<const IdxT*>(r->d_lut);
+    const dim3 all((unsigned)((r->ng + 255) / 256), (unsigned)r->n_hat);
+    const unsigned per_list = (unsigned)(lists / 256 + 1);
+    cudaError_t e = cudaMemsetAsync(counts, 0, (size_t)lists * sizeof(int32_t), c->stream);
+    if (e == cudaSuccess) {
+        k_tm_count<IdxT><<<all, 256, 0, c->stream>>>(lut, r->ng, r->ng_pad, T, counts);
+        k_tm_pad<<<per_list, 256, 0, c->stream>>>(counts, lists, padded);
+        e = launch_scan_i64(padded, off64, lists, tmp, c->stream);
+    }
+    if (e == cudaSuccess) {
+        k_tm_off<<<per_list, 256, 0, c->stream>>>(off64, counts, lists, T, static_cast<uint32_t*>(off),
+                                                  static_cast<uint32_t*>(ent));
+        k_tm_fill<IdxT><<<all, 256, 0, c->stream>>>(lut, r->ng, r->ng_pad, r->d_top_val, T,
+                                                    static_cast<uint32_t*>(off), counts, static_cast<uint32_t*>(ent));
+        k_tm_rowmajor<IdxT><<<dim3((unsigned)((r->ng + 31) / 32), (unsigned)((pitch + 31) / 32)), 256, 0, c->stream>>>(
+            lut, r->ng, r->ng_pad, r->n_hat, pitch, static_cast<IdxT*>(lut_g));
+        e = cudaGetLastError();
+    }
+    for (void* q : {(void*)counts, (void*)padded, (void*)off64, (void*)tmp}) dev_recycle(c, q);
+    r->d_tm_ent = static_cast<uint32_t*>(ent);
+    r->d_tm_off = static_cast<uint32_t*>(off);
+    r->d_lut_g = lut_g;
+    r->lut_g_pitch = pitch;
+    r->tm_tiles = tiles;
+    r->tm_nodes = T;
+    return e;
+}
+
+cudaError_t launch_build_tm(Ctx* c, Reference* r) {
+    return r->lut_bytes == 2 ? build_tm_t<uint16_t>(c, r) : build_tm_t<int32_t>(c, r);
+}
+
+// k_match takes a CTA per ROI, one row each: below some 4e5 look-ups per SM (30
+// us) its single launch is as fast as the four of the lists.
+bool tm_pays(const Ctx* c, const Reference* r, int64_t nroi) {
+    const double per_sm = (double)((nroi + c->sm_count - 1) / c->sm_count) * (double)r->ng * r->n_hat;
+    return r->d_tm_ent && per_sm > 4.0e5;
+}
+
+size_t tm_exact_smem(const Ctx* c, const Reference* r) { return ((size_t)c->nv + r->n_hat) * sizeof(float); }
+
+static TmMargin tm_margin(const Reference* r) {
+    const double eta = sqrt((double)r->n_hat) * r->ref_max * (1.0 / 16384.0);
+    return {(float)(2.0 * eta * 1.001), (float)(1.0 + 5.0 * (r->n_hat + 64) / 16777216.0)};
+}
+
+// estimates of `nroi` ROIs into D [groups][ng][64]
+cudaError_t launch_tm_sum(Ctx* c, Reference* r, const float* S, int64_t nroi, float* D) {
+    const int64_t groups = (nroi + kTmRois - 1) / kTmRois;
+    cudaError_t e = cudaMemsetAsync(D, 0, (size_t)(groups * r->ng * kTmRois) * sizeof(float), c->stream);
+    if (e != cudaSuccess) return e;
+    const size_t smem = (size_t)(r->tm_nodes + 1) * kTmPitch * sizeof(float);
+    if ((e = cudaFuncSetAttribute(k_tm_sum, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+        return e;
+    // a CTA per (tile, group); few groups split the orientations further, four
+    // CTAs per SM in all, at least 256 orientations each
+    const int64_t base = r->tm_tiles * groups;
+    const int gsplit = (int)std::max<int64_t>(1, std::min<int64_t>((4 * (int64_t)c->sm_count + base - 1) / base, r->ng / 256));
+    for (int64_t y0 = 0; y0 < groups; y0 += 65535) {
+        const int64_t ny = std::min<int64_t>(65535, groups - y0);
+        k_tm_sum<<<dim3((unsigned)(r->tm_tiles * gsplit), (unsigned)ny), kTmThreads, smem, c->stream>>>(
+            S + y0 * kTmRois * c->nv, nroi - y0 * kTmRois, c->nv, r->d_tm_ent, r->d_tm_off, r->ng, r->tm_nodes, gsplit,
+            D + y0 * r->ng * kTmRois);
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tm_best(Ctx* c, Reference* r, const float* S, int64_t nroi, const float* D, int32_t* best,
+                           float* score) {
+    const unsigned groups = 2 * (unsigned)((nroi + kTmRois - 1) / kTmRois);   // halves
+    if (r->lut_bytes == 2)
+        k_tm_best<uint16_t><<<groups, kTmThreads, 0, c->stream>>>(S, nroi, c->nv, static_cast<const uint16_t*>(r->d_lut_g),
+                                                                  r->ng, r->lut_g_pitch, r->d_top_val, r->n_hat, tm_margin(r), D, best,
+                                                                  score);
+    else
+        k_tm_best<int32_t><<<groups, kTmThreads, 0, c->stream>>>(S, nroi, c->nv, static_cast<const int32_t*>(r->d_lut_g),
+                                                                 r->ng, r->lut_g_pitch, r->d_top_val, r->n_hat, tm_margin(r), D, best,
+                                                                 score);
+    return cudaGetLastError();
+}
+
+// rows [nroi][ng] from the estimates, exact where the topk are decided; D's
+// first nroi words are reused for the reach
+template <typename IdxT>
+static cudaError_t tm_rows_t(Ctx* c, Reference* r, const float* S, int64_t nroi, int32_t topk, float* D, float* rows) {
+    const int64_t groups = (nroi + kTmRois - 1) / kTmRois;
+    for (int64_t y0 = 0; y0 < groups; y0 += 32767) {
+        const int64_t ny = std::min<int64_t>(32767, groups - y0);
+        k_tm_rows<<<dim3((unsigned)((r->ng + 31) / 32), (unsigned)(2 * ny)), 256, 0, c->stream>>>(
+            D + y0 * r->ng * kTmRois, nroi - y0 * kTmRois, r->ng, rows + y0 * kTmRois * r->ng);
+    }
+    k_tm_reach<<<(unsigned)std::min<int64_t>(nroi, (int64_t)c->sm_count * 8), 256, 0, c->stream>>>(rows, r->ng, nroi,
+                                                                                                  topk, tm_margin(r), D);
+    const size_t smem = tm_exact_smem(c, r);
+    cudaError_t e = cudaFuncSetAttribute(k_tm_exact<IdxT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    // eight rounds of CTAs at least: the last, partly filled one then costs little
+    const int parts = (int)std::max<int64_t>(1, std::min<int64_t>((8 * (int64_t)c->sm_count + nroi - 1) / nroi, r->ng / 4096));
+    k_tm_exact<IdxT><<<(unsigned)std::min<int64_t>(nroi * parts, c->sm_count), kTmThreads, smem, c->stream>>>(
+        S, nroi, c->nv, static_cast<const IdxT*>(r->d_lut_g), r->ng, r->lut_g_pitch, r->d_top_val, r->n_hat, D, parts, rows);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tm_rows(Ctx* c, Reference* r, const float* S, int64_t nroi, int32_t topk, float* D, float* rows) {
+    return r->lut_bytes == 2 ? tm_rows_t<uint16_t>(c, r, S, nroi, topk, D, rows)
+                             : tm_rows_t<int32_t>(c, r, S, nroi, topk, D, rows);
 }
 
 // Phase decision: candidate c's summed channel scores divided by its channel

@@ -41,10 +41,17 @@ struct Reference {
     float4* d_img4 = nullptr;
     void* d_lut = nullptr;         // [n_hat x ng_pad] (k-major), uint16 node indices when nv <= 65536, else int32
     int lut_bytes = 4;             // bytes per table entry (2 or 4)
+    // the table as lists per (tile of tm_nodes nodes, orientation), or null
+    uint32_t* d_tm_ent = nullptr;  // reference value to 22 bits | row of the node, padded to four
+    uint32_t* d_tm_off = nullptr;  // [tm_tiles x ng + 1]
+    int tm_tiles = 0, tm_nodes = 0;
+    void* d_lut_g = nullptr;       // [ng x lut_g_pitch] the table by orientation (with the lists)
+    int lut_g_pitch = 0;
     double* d_quats = nullptr;     // [ng x 4] test orientations of the table
     int64_t ng = 0;
     int64_t ng_pad = 0;            // row length of the table: ng rounded up to a multiple of 8
     int32_t nv_at_set = 0;
+    double ref_max = 0.0;          // largest |value| of the reference signature
     double energy = 0.0;           // sum of the squared n_hat strongest values (Eq. 3 of an empty signature)
 };
 
@@ -238,6 +245,14 @@ cudaError_t launch_top_nodes(Ctx* c, Reference* r);
 cudaError_t launch_build_lut(Ctx* c, Reference* r, const double* d_quats, int64_t ng);
 cudaError_t launch_match(Ctx* c, Reference* r, const float* S, int64_t nroi, int32_t* best, float* score,
                          float* scores_out = nullptr, bool accumulate = false, float weight = 1.0f);
+// Eq. 3 of many ROIs by lists (estimates, then exact sums where they decide)
+cudaError_t launch_build_tm(Ctx* c, Reference* r);
+bool tm_pays(const Ctx* c, const Reference* r, int64_t nroi);
+size_t tm_exact_smem(const Ctx* c, const Reference* r);
+cudaError_t launch_tm_sum(Ctx* c, Reference* r, const float* S, int64_t nroi, float* D);
+cudaError_t launch_tm_best(Ctx* c, Reference* r, const float* S, int64_t nroi, const float* D, int32_t* best,
+                           float* score);
+cudaError_t launch_tm_rows(Ctx* c, Reference* r, const float* S, int64_t nroi, int32_t topk, float* D, float* rows);
 cudaError_t launch_phase(Ctx* c, float* score, const int32_t* n_ch, int32_t n_cand, int64_t nroi, int32_t* phase);
 cudaError_t launch_topk(Ctx* c, const float* scores, int64_t ng, int64_t nroi, int32_t topk, int32_t* best,
                         float* score);

@@ -403,23 +403,24 @@ __device__ __forceinline__ void quad_atoms(float4* A, int n, int tid, int nthrea
     }
 }
 
-constexpr uint32_t kQuadBits = 0x4C000000u;   // bit pattern of 2^25
+constexpr uint32_t kQuadBits = 0x50000000u;   // bit pattern of 2^33
 
-// 4 (2^23 + 2^(m-1) + base row): the magic number of the pass whose histogram
-// starts at shared row `row0` (its byte address / 128)
+// 1024 (2^23 + 2^(m-1) + base row): the magic number of the pass whose histogram
+// starts at shared row `row0` (its byte address / row pitch)
 __device__ __forceinline__ float quad_magic(int m, uint32_t row0) {
-    return 4.0f * (8388608.0f + (float)((1 << (m - 1)) + (int)row0));
+    return 1024.0f * (8388608.0f + (float)((1 << (m - 1)) + (int)row0));
 }
 
 // Per-lane state of the pass.
 struct QuadDirs {
     uint64_t x0, y0, z0, x1, y1, z1, sc, mg;
-    uint32_t lane_top;   // 4 lane in the top seven bits
+    uint32_t lane_top;   // the lane's byte offset in its row, in the top bits
     uint32_t t_lo;       // chunked: bit pattern of the chunk's first bin
     uint32_t h_lane;     // chunked: H + 4 lane
 };
 
-__device__ __forceinline__ QuadDirs quad_dirs(float4 d0, float4 d1, float scale, float magic, int lane) {
+// word: the lane's word of the row; rows of 32 >> split words
+__device__ __forceinline__ QuadDirs quad_dirs(float4 d0, float4 d1, float scale, float magic, int word, int split = 0) {
     QuadDirs q;
     q.x0 = f2_dup(d0.x);
     q.y0 = f2_dup(d0.y);
@@ -427,27 +428,27 @@ __device__ __forceinline__ QuadDirs quad_dirs(float4 d0, float4 d1, float scale,
     q.x1 = f2_dup(d1.x);
     q.y1 = f2_dup(d1.y);
     q.z1 = f2_dup(d1.z);
-    q.sc = f2_dup(4.0f * scale);
+    q.sc = f2_dup(1024.0f * scale);
     q.mg = f2_dup(magic);
-    q.lane_top = (uint32_t)lane << 27;
+    q.lane_top = (uint32_t)word << (27 + split);
     q.t_lo = q.h_lane = 0;
     return q;
 }
 
-template <bool kChunked>
+template <bool kChunked, int kSplit = 0>
 __device__ __forceinline__ void quad_inc(uint32_t t, uint32_t one, const QuadDirs& q) {
     if (kChunked) {
         const uint32_t v = t - q.t_lo;   // bin - first bin of the chunk
         if (v < 1024u) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(v * 128u + q.h_lane), "r"(one) : "memory");
     } else {
-        asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(__funnelshift_l(q.lane_top, t, 7)), "r"(one) : "memory");
+        asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(__funnelshift_l(q.lane_top, t, 7 - kSplit)), "r"(one) : "memory");
     }
 }
 
 // kCount as in hist_add_pair2, except that for 2 the smallest |s| is kept (0:
 // some projection is exactly zero) instead of a product, two three-input minima
 // on the integer pipe instead of two packed multiplies
-template <int kCount, bool kChunked>
+template <int kCount, bool kChunked, int kSplit = 0>
 __device__ __forceinline__ void quad_add_pair(uint64_t x, uint64_t y, uint64_t z, const QuadDirs& q, uint32_t& c0,
                                               uint32_t& c1, float& zmin) {
     const uint64_t s0 = f2_fma(z, q.z0, f2_fma(y, q.y0, f2_mul(x, q.x0)));
@@ -463,18 +464,19 @@ __device__ __forceinline__ void quad_add_pair(uint64_t x, uint64_t y, uint64_t z
         c0 += ((uint32_t)u0 - (uint32_t)t0) + ((uint32_t)(u0 >> 32) - (uint32_t)(t0 >> 32));
         c1 += ((uint32_t)u1 - (uint32_t)t1) + ((uint32_t)(u1 >> 32) - (uint32_t)(t1 >> 32));
     }
-    quad_inc<kChunked>((uint32_t)t0, 1u, q);
-    quad_inc<kChunked>((uint32_t)(t0 >> 32), 1u, q);
-    quad_inc<kChunked>((uint32_t)t1, 0x10000u, q);
-    quad_inc<kChunked>((uint32_t)(t1 >> 32), 0x10000u, q);
+    quad_inc<kChunked, kSplit>((uint32_t)t0, 1u, q);
+    quad_inc<kChunked, kSplit>((uint32_t)(t0 >> 32), 1u, q);
+    quad_inc<kChunked, kSplit>((uint32_t)t1, 0x10000u, q);
+    quad_inc<kChunked, kSplit>((uint32_t)(t1 >> 32), 0x10000u, q);
 }
 
-// Histograms of one 64-direction tile over `cn` atoms staged by quad_atoms;
-// warp w takes blocks w, w + W, ..., two at a time with their loads first; the
-// up to three trailing atoms go to warp (cn / 4) % W.  Returns the number of
-// atoms this warp handled.
-template <int W, int kCount, bool kChunked>
-__device__ __forceinline__ int hist_tile_quads(const float4* A, int cn, int warp, const QuadDirs& q, uint32_t& c0,
+// Histograms of one tile over `cn` atoms staged by quad_atoms; group g of G
+// (warps, or the parts of a warp that hold a whole row of words each) takes
+// blocks g, g + G, ..., two at a time with their loads first; the up to three
+// trailing atoms go to group (cn / 4) % G.  Returns the number of atoms this
+// group handled.
+template <int kCount, bool kChunked, int kSplit = 0>
+__device__ __forceinline__ int hist_tile_quads(const float4* A, int cn, int warp, int W, const QuadDirs& q, uint32_t& c0,
                                                uint32_t& c1, float& zmin) {
     const int nq = cn >> 2;
     auto ld = [&](int i, int k) { return *reinterpret_cast<const ulonglong2*>(A + 4 * i + k); };
@@ -482,15 +484,15 @@ __device__ __forceinline__ int hist_tile_quads(const float4* A, int cn, int warp
     for (; j + W < nq; j += 2 * W) {
         const ulonglong2 xa = ld(j, 0), ya = ld(j, 1), za = ld(j, 2);
         const ulonglong2 xb = ld(j + W, 0), yb = ld(j + W, 1), zb = ld(j + W, 2);
-        quad_add_pair<kCount, kChunked>(xa.x, ya.x, za.x, q, c0, c1, zmin);
-        quad_add_pair<kCount, kChunked>(xa.y, ya.y, za.y, q, c0, c1, zmin);
-        quad_add_pair<kCount, kChunked>(xb.x, yb.x, zb.x, q, c0, c1, zmin);
-        quad_add_pair<kCount, kChunked>(xb.y, yb.y, zb.y, q, c0, c1, zmin);
+        quad_add_pair<kCount, kChunked, kSplit>(xa.x, ya.x, za.x, q, c0, c1, zmin);
+        quad_add_pair<kCount, kChunked, kSplit>(xa.y, ya.y, za.y, q, c0, c1, zmin);
+        quad_add_pair<kCount, kChunked, kSplit>(xb.x, yb.x, zb.x, q, c0, c1, zmin);
+        quad_add_pair<kCount, kChunked, kSplit>(xb.y, yb.y, zb.y, q, c0, c1, zmin);
     }
     if (j < nq) {
         const ulonglong2 xa = ld(j, 0), ya = ld(j, 1), za = ld(j, 2);
-        quad_add_pair<kCount, kChunked>(xa.x, ya.x, za.x, q, c0, c1, zmin);
-        quad_add_pair<kCount, kChunked>(xa.y, ya.y, za.y, q, c0, c1, zmin);
+        quad_add_pair<kCount, kChunked, kSplit>(xa.x, ya.x, za.x, q, c0, c1, zmin);
+        quad_add_pair<kCount, kChunked, kSplit>(xa.y, ya.y, za.y, q, c0, c1, zmin);
     }
     int handled = warp < nq ? 4 * ((nq - warp + W - 1) / W) : 0;
     if (warp == nq % W) {
@@ -507,8 +509,8 @@ __device__ __forceinline__ int hist_tile_quads(const float4* A, int cn, int warp
                 c0 += __float_as_uint(__fmaf_ru(s0, sc, mg)) - t0;
                 c1 += __float_as_uint(__fmaf_ru(s1, sc, mg)) - t1;
             }
-            quad_inc<kChunked>(t0, 1u, q);
-            quad_inc<kChunked>(t1, 0x10000u, q);
+            quad_inc<kChunked, kSplit>(t0, 1u, q);
+            quad_inc<kChunked, kSplit>(t1, 0x10000u, q);
             ++handled;
         }
     }

@@ -236,15 +236,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_plain(SigParams p) {
                         hist_tile_chunk<kWarps>(H, A, cn, warp, lane, d0, d1, scale, magic, (uint32_t)nbm1, (uint32_t)bc);
                 } else if (nchunk == 1) {
                     if (count && zero_check)
-                        handled += hist_tile_quads<kWarps, 2, false>(A, cn, warp, q, c0, c1, zmin);
+                        handled += hist_tile_quads<2, false>(A, cn, warp, kWarps, q, c0, c1, zmin);
                     else if (count)
-                        handled += hist_tile_quads<kWarps, 1, false>(A, cn, warp, q, c0, c1, zmin);
+                        handled += hist_tile_quads<1, false>(A, cn, warp, kWarps, q, c0, c1, zmin);
                     else
-                        hist_tile_quads<kWarps, 0, false>(A, cn, warp, q, c0, c1, zmin);
+                        hist_tile_quads<0, false>(A, cn, warp, kWarps, q, c0, c1, zmin);
                 } else {
                     q.t_lo = kQuadBits + (h_addr >> 7) + (uint32_t)bc * kChunkBins;
                     q.h_lane = h_addr + 4u * (uint32_t)lane;
-                    hist_tile_quads<kWarps, 0, true>(A, cn, warp, q, c0, c1, zmin);
+                    hist_tile_quads<0, true>(A, cn, warp, kWarps, q, c0, c1, zmin);
                 }
                 if (!one_chunk) __syncthreads();
             }

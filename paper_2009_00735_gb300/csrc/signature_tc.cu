@@ -151,7 +151,6 @@ struct TpPass {
     int64_t roi;
     int32_t tile, flags;
     int32_t g0, ng, klo, khi;   // first frequency group, groups, the ROI's band
-    int32_t bc;                 // bin chunk
 };
 constexpr int kPassStop = 1, kPassFirst = 2, kPassLast = 4, kPassBad = 8, kPassPartner = 16;
 
@@ -168,18 +167,42 @@ __device__ __forceinline__ bool hist_sync_or(bool v) {
     return r != 0;
 }
 
+// K rows of the B operand: the bins of one part (a quarter of up to 2^11, an
+// eighth of 2^12)
+__host__ __device__ __forceinline__ int tp_k_rows(int m) { return m <= 11 ? 1 << (m - 2) : 1 << (m - 3); }
+
+// Debug export of one pass: adds the counts to h_out[v * 2^m + bin] (the caller
+// zeroes h_out); rows of 32 >> split words
+__device__ __forceinline__ void hist_export_rows(const uint32_t* H, int m, int split, int tile, int nv, uint16_t* h_out,
+                                                 int tid, int nthreads) {
+    const int64_t NB = (int64_t)1 << m;
+    for (int i = tid; i < (1 << m) * (32 >> split); i += nthreads) {
+        const int b = i >> (5 - split), l = i & ((32 >> split) - 1);
+        const uint32_t w = H[i];
+        const int64_t v0 = (int64_t)tile * (kDirs >> split) + 2 * l;
+        if (v0 < nv) h_out[v0 * NB + b] = (uint16_t)(h_out[v0 * NB + b] + (w & 0xFFFFu));
+        if (v0 + 1 < nv) h_out[(v0 + 1) * NB + b] = (uint16_t)(h_out[(v0 + 1) * NB + b] + (w >> 16));
+    }
+}
+
 // kNB: band slots of the epilogue (1: the ROI's own band; APTIDX_MAX_BANDS:
 // the pass's BandSet, aptidx_compute_signatures_multi)
-template <int kNB>
+// split: 2^11 and 2^12 bins run tiles of 32 and 16 directions, rows of 16 and 8
+// words, so that a tile's histogram stays at 128 KB and no atom is projected twice
+// (passes over chunks of 1024 bins projected each atom two or four times, with
+// predicated increments: 18 K cycles for 1815 atoms, 10 per atom, against 5).  A
+// template argument: as a variable of one kernel it cost the 2^10-bin pass 20 %.
+template <int kNB, int split>
 __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    constexpr int DT = kDirs >> split;      // directions per tile
     const int NB = 1 << p.m;
-    const int NBc = NB < kChunkBins ? NB : kChunkBins;   // bins per chunk
-    const int nchunk = NB / NBc;
-    const int KB = NBc / 256;   // 64-row K blocks of the B operand per chunk (K = NBc / 4 rows)
+    constexpr int pitch = 128 >> split;     // bytes of a histogram row (one bin)
+    const int K = tp_k_rows(p.m);           // bins per part (a quarter, of 2^12 an eighth)
+    const int KB = K / 64;                  // 64-row K blocks of the B operand
     uint32_t* H = reinterpret_cast<uint32_t*>(smem);
-    unsigned char* BT = smem + (size_t)NBc * 128;
+    unsigned char* BT = smem + (size_t)NB * pitch;
     float* EX = reinterpret_cast<float*>(BT + p.bt_bytes);   // [2][kExFloats]
     float4* A = reinterpret_cast<float4*>(EX + 2 * kExFloats);
     float4* DB = A + p.atom_cap;   // [2][parity][32]: this tile's directions and the next tile's
@@ -206,7 +229,7 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
         *aux_fail = 0;
         fence_barrier_init();
     }
-    for (int i = tid; i < NBc * 8; i += kTpThreads) reinterpret_cast<uint4*>(H)[i] = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < NB * pitch / 16; i += kTpThreads) reinterpret_cast<uint4*>(H)[i] = make_uint4(0, 0, 0, 0);
     if (warp == kHistWarps) tmem_alloc(tmem_s, kTmemCols);
     tc_fence_before();
     __syncthreads();
@@ -217,15 +240,19 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
 
     if (warp < kHistWarps) {
         // ================= histogram warps =================
-        const float magic = quad_magic(p.m, h_addr >> 7);
-        const int chunk_log = p.m > 10 ? p.m - 10 : 0;
+        const float magic = quad_magic(p.m, h_addr / (uint32_t)pitch);
+        // the lane's word of a row, and its group of lanes (warps hold 1, 2 or 4
+        // whole rows, each group walks its own atoms)
+        const int word = lane & ((32 >> split) - 1);
+        const int group = (warp << split) + (lane >> (5 - split)), ngroups = kHistWarps << split;
         const int n_items = (int)((p.single_roi >= 0 ? 1 : p.nroi) * p.items_per_roi);   // < 2^31 (launch)
         uint32_t ph_atoms = 0, t = 0;   // t: passes handed over
-        // this warp's share of the transfer: bins of quarter warp & 3 (the
-        // tensor-memory lanes it may write), a quarter of them
-        const int tr_rows = NBc / 16;
-        const int tr_row0 = (warp & 3) * (NBc / 4) + (warp >> 2) * tr_rows;
-        const uint32_t tr_col0 = tmem + kTmemA + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * (tr_rows / 2));
+        // this warp's share of the transfer: the bins of quarter warp & 3 (the
+        // tensor-memory lanes it may write), a quarter of its 128-byte lines
+        const int tr_lines = NB * pitch / 128 / 16;
+        const uint32_t tr_addr =
+            h_addr + ((uint32_t)((warp & 3) * 4 * tr_lines) << 7) + 4u * (uint32_t)lane;
+        const uint32_t tr_tmem = tmem + kTmemA + ((uint32_t)((warp & 3) * 32) << 16);
         bool failed = false;
         if (tid == 0) *item_s = atomicAdd(p.counter, 1);
         hist_sync();
@@ -267,7 +294,7 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
             // 1.6 K cycles per tile)
             // slot 2 l + i of a tile at [i][l]: a warp reads 512 consecutive bytes
             const int db_slot = (tid & 1) * 32 + (tid >> 1);
-            if (tid < kDirs) cp_async16(DB + (t0 & 1) * kDirs + db_slot, p.dirs + (int64_t)t0 * kDirs + tid);
+            if (tid < DT) cp_async16(DB + (t0 & 1) * kDirs + db_slot, p.dirs + (int64_t)t0 * DT + tid);
             cp_async_wait_all();
             if (nblk > 1) {
                 hist_sync();
@@ -280,9 +307,9 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
             const bool zero_check =
                 sym && nblk == 1 && !nonzero_integer_products_possible(scale, __uint_as_float(*r2max_s));
             for (int tile = t0; tile < t1 && !failed; ++tile) {
-                float4 d0 = DB[(tile & 1) * kDirs + lane], d1 = DB[(tile & 1) * kDirs + 32 + lane];
-                if (tile + 1 < t1 && tid < kDirs)
-                    cp_async16(DB + ((tile + 1) & 1) * kDirs + db_slot, p.dirs + (int64_t)(tile + 1) * kDirs + tid);
+                float4 d0 = DB[(tile & 1) * kDirs + word], d1 = DB[(tile & 1) * kDirs + 32 + word];
+                if (tile + 1 < t1 && tid < DT)
+                    cp_async16(DB + ((tile + 1) & 1) * kDirs + db_slot, p.dirs + (int64_t)(tile + 1) * DT + tid);
                 const bool pt0 = d0.w != 0.f, pt1 = d1.w != 0.f;   // the slot has an antipodal partner
                 bool tile_bad = false;
                 for (int pass = 0; pass < 2 && !failed; ++pass) {
@@ -293,40 +320,27 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
                         d1 = make_float4(-d1.x, -d1.y, -d1.z, d1.w);
                     }
                     const bool count = sym && pass == 0;
-                    QuadDirs q = quad_dirs(d0, d1, scale, magic, lane);
+                    const QuadDirs q = quad_dirs(d0, d1, scale, magic, word, split);
                     uint32_t c0 = 0, c1 = 0;
                     float zmin = 1.f;
                     int handled = 0;
-                    const int n_sub = nblk << chunk_log;
-                    for (int sub = 0; sub < n_sub; ++sub, ++t) {
-                        const int blk = sub >> chunk_log, bc = sub & (nchunk - 1);
+                    for (int blk = 0; blk < nblk; ++blk, ++t) {
                         const int cn = min(p.atom_cap, nw - blk * p.atom_cap);
-                        const bool last = sub == n_sub - 1;
-                        if (nblk > 1 && bc == 0 && !stage(p.atoms + p.off[roi] + (int64_t)blk * p.atom_cap, cn, nullptr)) {
+                        const bool last = blk == nblk - 1;
+                        if (nblk > 1 && !stage(p.atoms + p.off[roi] + (int64_t)blk * p.atom_cap, cn, nullptr)) {
                             failed = true;
                             break;
                         }
                         // ---- 1. histograms (H is zero here) ----
-                        if (nchunk == 1) {
-                            if (count && zero_check)
-                                handled += hist_tile_quads<kHistWarps, 2, false>(A, cn, warp, q, c0, c1, zmin);
-                            else if (count)
-                                handled += hist_tile_quads<kHistWarps, 1, false>(A, cn, warp, q, c0, c1, zmin);
-                            else
-                                hist_tile_quads<kHistWarps, 0, false>(A, cn, warp, q, c0, c1, zmin);
-                        } else {
-                            q.t_lo = kQuadBits + (h_addr >> 7) + (uint32_t)bc * kChunkBins;
-                            q.h_lane = h_addr + 4u * (uint32_t)lane;
-                            if (count && bc == 0 && zero_check)
-                                handled += hist_tile_quads<kHistWarps, 2, true>(A, cn, warp, q, c0, c1, zmin);
-                            else if (count && bc == 0)
-                                handled += hist_tile_quads<kHistWarps, 1, true>(A, cn, warp, q, c0, c1, zmin);
-                            else
-                                hist_tile_quads<kHistWarps, 0, true>(A, cn, warp, q, c0, c1, zmin);
-                        }
+                        if (count && zero_check)
+                            handled += hist_tile_quads<2, false, split>(A, cn, group, ngroups, q, c0, c1, zmin);
+                        else if (count)
+                            handled += hist_tile_quads<1, false, split>(A, cn, group, ngroups, q, c0, c1, zmin);
+                        else
+                            hist_tile_quads<0, false, split>(A, cn, group, ngroups, q, c0, c1, zmin);
                         // the non-integer counts are complete once the last pass's
                         // histogram is in: a partner whose count falls short of the
-                        // atoms this warp handled needs its own histogram
+                        // atoms this group handled needs its own histogram
                         const bool bad = count && last &&
                                          (zero_check ? (pt0 || pt1) && zmin == 0.f
                                                      : (pt0 && c0 != (uint32_t)handled) || (pt1 && c1 != (uint32_t)handled));
@@ -345,20 +359,19 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
                         }
                         tc_fence_after();
                         if (p.hist_out) {
-                            hist_export_add(H, NBc, NB, bc, tile, p.nv, p.hist_out, tid, kHistThreads);
+                            hist_export_rows(H, p.m, split, tile, p.nv, p.hist_out, tid, kHistThreads);
                             hist_sync();   // every row is read before the transfer zeroes it
                         }
                         if (tid == 0) {
                             TpPass m;
                             m.roi = roi;
                             m.tile = tile;
-                            m.flags = (sub == 0 ? kPassFirst : 0) | (last ? kPassLast : 0) | (tile_bad ? kPassBad : 0) |
+                            m.flags = (blk == 0 ? kPassFirst : 0) | (last ? kPassLast : 0) | (tile_bad ? kPassBad : 0) |
                                       (pass ? kPassPartner : 0);
                             m.g0 = (klo - p.kbase) >> 2;
                             m.ng = ((khi - p.kbase) >> 2) - m.g0 + 1;
                             m.klo = klo;
                             m.khi = khi;
-                            m.bc = bc;
                             pass_s[t & 1] = m;
                         }
                         // ---- 2. transfer: counts into tensor memory, the histogram
@@ -366,19 +379,58 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
                         // and a store pass over the rows took twice the shared-memory
                         // cycles).  Word (bin, lane) holds directions 2 lane and
                         // 2 lane + 1; two bins' words make a K pair of either ----
-                        for (int r = 0; r < tr_rows; r += 16) {
-                            const uint32_t row = h_addr + (uint32_t)(tr_row0 + r) * 128u + 4u * (uint32_t)lane;
-                            uint32_t w[16], e[8], o[8];
+                        for (int r = 0; r < tr_lines; r += 16) {
+                            // split 2 takes eight lines of either eighth of its quarter
+                            const int l0 = (warp >> 2) * tr_lines + r;
+                            uint32_t w[16];
 #pragma unroll
-                            for (int i = 0; i < 16; ++i)
-                                asm volatile("atom.shared.exch.b32 %0, [%1], 0;" : "=r"(w[i]) : "r"(row + 128u * i) : "memory");
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                e[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x5410);
-                                o[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x7632);
+                            for (int i = 0; i < 16; ++i) {
+                                const int line = split < 2 ? l0 + i : l0 / 2 + (i >> 1) + (i & 1) * 2 * tr_lines;
+                                asm volatile("atom.shared.exch.b32 %0, [%1], 0;"
+                                             : "=r"(w[i])
+                                             : "r"(tr_addr + 128u * (uint32_t)line)
+                                             : "memory");
                             }
-                            tmem_st8(tr_col0 + (uint32_t)(r / 2), e);
-                            tmem_st8(tr_col0 + 128u + (uint32_t)(r / 2), o);
+                            if (split == 0) {
+                                // a line is a bin: pairs of lines make K pairs of the even
+                                // directions (columns 0..) and of the odd ones (128..)
+                                uint32_t e[8], o[8];
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) {
+                                    e[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x5410);
+                                    o[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x7632);
+                                }
+                                tmem_st8(tr_tmem + (uint32_t)(l0 / 2), e);
+                                tmem_st8(tr_tmem + 128u + (uint32_t)(l0 / 2), o);
+                            } else if (split == 1) {
+                                // a line is two bins, one K pair: lanes 0-15 take the even
+                                // directions, 16-31 the odd ones
+                                const bool odd = lane >= 16;
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) {
+                                    const uint32_t x = __shfl_xor_sync(0xffffffffu, w[i], 16);
+                                    w[i] = odd ? __byte_perm(x, w[i], 0x7632) : __byte_perm(w[i], x, 0x5410);
+                                }
+                                tmem_st8(tr_tmem + (uint32_t)l0, w);
+                                tmem_st8(tr_tmem + (uint32_t)l0 + 8u, w + 8);
+                            } else {
+                                // a line is four bins, two K pairs; a line of the quarter's
+                                // first eighth (lanes 0-15) and one of its second (16-31)
+                                // make two columns, even directions in the lower eight lanes
+                                const bool odd = (lane & 8) != 0, hi = lane >= 16;
+#pragma unroll
+                                for (int i = 0; i < 16; i += 2) {
+                                    const uint32_t xa = __shfl_xor_sync(0xffffffffu, w[i], 8);
+                                    const uint32_t xb = __shfl_xor_sync(0xffffffffu, w[i + 1], 8);
+                                    const uint32_t va = odd ? __byte_perm(xa, w[i], 0x7632) : __byte_perm(w[i], xa, 0x5410);
+                                    const uint32_t vb = odd ? __byte_perm(xb, w[i + 1], 0x7632) : __byte_perm(w[i + 1], xb, 0x5410);
+                                    const uint32_t x = __shfl_xor_sync(0xffffffffu, hi ? va : vb, 16);
+                                    w[i] = hi ? x : va;
+                                    w[i + 1] = hi ? vb : x;
+                                }
+                                tmem_st8(tr_tmem + (uint32_t)l0, w);
+                                tmem_st8(tr_tmem + (uint32_t)l0 + 8u, w + 8);
+                            }
                         }
                         tmem_wait_st();
                         tc_fence_before();
@@ -407,9 +459,10 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
         // ================= auxiliary warps =================
         const int at = tid - kHistThreads, aw = at >> 5;   // warp aw: tensor-memory lanes 32 aw .., bin quarter aw
         const uint32_t bt_addr = smem_u32(BT);
-        const int nh = p.n_iss >> 1;    // accumulators per direction parity (halves of K)
+        constexpr int blocks = split == 0 ? 2 : 1;   // A operands of a tile: even and odd directions, or all
+        const int nh = p.n_iss / blocks;         // accumulators per block (parts of K)
         uint32_t ph_b = 0, exb = 0;
-        int cur_g0 = -1, cur_ng = -1, cur_bc = -1;   // B operand in shared memory
+        int cur_g0 = -1, cur_ng = -1;   // B operand in shared memory
         // accumulators: two buffers of 128 columns in turn when a tile's fit one,
         // else one of 256
         bool pending = false;
@@ -437,59 +490,51 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
                 float* ex = EX + (exb & 1) * kExFloats;
                 ++exb;
 #pragma unroll
-                for (int b = 0; b < 2; ++b) {
-                    float v[8], lo[8];
-                    const uint32_t c = dcol + (uint32_t)b * cols + (uint32_t)(8 * j);
-                    tmem_ld8(c, v);
-                    tmem_ld8(c + (uint32_t)(8 * m.ng), lo);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) v[i] += lo[i];
-                    if (nh == 2) {
-                        float v2[8];
-                        tmem_ld8(c + 2 * cols, v2);
-                        tmem_ld8(c + 2 * cols + (uint32_t)(8 * m.ng), lo);
+                for (int b = 0; b < blocks; ++b) {
+                    float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                    for (int h = 0; h < nh; ++h) {
+                        float hi[8], lo[8];
+                        const uint32_t c = dcol + (uint32_t)(h * blocks + b) * cols + (uint32_t)(8 * j);
+                        tmem_ld8(c, hi);
+                        tmem_ld8(c + (uint32_t)(8 * m.ng), lo);
                         tmem_wait_ld();
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) v[i] += v2[i] + lo[i];
+                        for (int i = 0; i < 8; ++i) v[i] += hi[i] + lo[i];
                     }
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) ex[((aw * 2 + b) * 8 + i) * 32 + lane] = v[i];
+                    for (int i = 0; i < 8; ++i) ex[((aw * blocks + b) * 8 + i) * 32 + lane] = v[i];
                 }
                 tc_fence_before();
                 aux_sync();
-                if (at < kDirs) {
+                if (at < DT) {
                     const int f0 = p.kbase + 4 * (m.g0 + j);
-                    const float* x = ex + (at & 1) * 256 + (at >> 1);   // quarter q: + 512 q
+                    // direction at: parity at & 1, word at >> 1; part q of the bins at + q * step
+                    const int pos = split == 0 ? (at & 1) * 256 + (at >> 1) : (at & 1) * (16 >> (split - 1)) + (at >> 1);
+                    const float* x = ex + pos;
+                    float xr[4] = {0.f, 0.f, 0.f, 0.f}, xi[4] = {0.f, 0.f, 0.f, 0.f};
+                    constexpr int parts = split == 2 ? 8 : 4;
+                    for (int q = 0; q < parts; ++q) {
+                        const float* y = split == 0 ? x + q * 512 : split == 1 ? x + q * 256 : x + (q >> 1) * 256 + (q & 1) * 16;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int f = f0 + i;
-                        float fc[4], fs[4];   // w^(f q NBc / 4) = fc - i fs
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            if (nchunk == 1) {   // (-i)^(f q)
-                                const int ph = (f * q) & 3;
-                                fc[q] = ph == 0 ? 1.f : ph == 2 ? -1.f : 0.f;
-                                fs[q] = ph == 1 ? 1.f : ph == 3 ? -1.f : 0.f;
-                            } else {
-                                sincospif((float)(f * q) * (float)NBc / (float)(2 * NB), &fs[q], &fc[q]);
-                            }
+                        for (int i = 0; i < 4; ++i) {
+                            // w^(f q NB / parts) = fc - i fs, an eighth root of one
+                            const int ph = ((f0 + i) * q * (8 / parts)) & 7;
+                            const float root = 0.70710678118654752f;
+                            const float fc = (ph & 3) == 2 ? 0.f : ((ph & 1) ? root : 1.f) * (ph > 2 && ph < 6 ? -1.f : 1.f);
+                            const float fs = (ph & 3) == 0 ? 0.f : ((ph & 1) ? root : 1.f) * (ph > 4 ? -1.f : 1.f);
+                            const float r = y[(2 * i) * 32], s = y[(2 * i + 1) * 32];
+                            xr[i] += fc * r - fs * s;
+                            xi[i] += fs * r + fc * s;
                         }
-                        float xr[4], xi[4];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const float r = x[q * 512 + (2 * i) * 32], s = x[q * 512 + (2 * i + 1) * 32];
-                            xr[q] = fc[q] * r - fs[q] * s;
-                            xi[q] = fs[q] * r + fc[q] * s;
-                        }
-                        const float r = (xr[0] + xr[2]) + (xr[1] + xr[3]), s = (xi[0] + xi[2]) + (xi[1] + xi[3]);
-                        // the band maximum on |X|^2 (its root is the maximum amplitude)
-                        band_update_t<kNB>(p.bands, m.klo, m.khi, f, r * r + s * s, best, bk);
                     }
+                    // the band maximum on |X|^2 (its root is the maximum amplitude)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        band_update_t<kNB>(p.bands, m.klo, m.khi, f0 + i, xr[i] * xr[i] + xi[i] * xi[i], best, bk);
                 }
             }
-            if (at < kDirs) {
-                const int slot = m.tile * kDirs + at;
+            if (at < DT) {
+                const int slot = m.tile * DT + at;
                 int v0 = slot < p.nv ? slot : -1, v1 = -1;
                 if (sym) {
                     // the slot's direction, and its partner when the tile's mirror
@@ -526,19 +571,15 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
             tc_fence_after();
             const TpPass m = pass_s[t & 1];
             if (m.flags & kPassStop) break;
-            // ---- B operand of the band (all chunks when they fit) ----
+            // ---- B operand of the band ----
             const uint32_t part = (uint32_t)m.ng * KB * 1024u;
-            const bool all = (uint32_t)nchunk * 2u * part <= (uint32_t)p.bt_bytes;
-            const int want_bc = all ? 0 : m.bc;
-            if (m.g0 != cur_g0 || m.ng != cur_ng || want_bc != cur_bc) {
+            if (m.g0 != cur_g0 || m.ng != cur_ng) {
                 if (t > 0 && !done(t - 1)) break;   // its MMAs read the operand held so far
                 if (at == 0) {
-                    const int n = all ? nchunk : 1;
                     fence_proxy_async_smem();
-                    mbar_arrive_expect_tx(bar_b, 2u * part * (uint32_t)n);
-                    for (int i = 0; i < 2 * n; ++i)
-                        bulk_g2s(BT + (size_t)i * part,
-                                 p.twb + ((size_t)(2 * want_bc + i) * p.ng_total + m.g0) * KB * 1024, part, bar_b);
+                    mbar_arrive_expect_tx(bar_b, 2u * part);
+                    for (int i = 0; i < 2; ++i)
+                        bulk_g2s(BT + (size_t)i * part, p.twb + ((size_t)i * p.ng_total + m.g0) * KB * 1024, part, bar_b);
                     if (!mbar_wait_bounded(bar_b, ph_b, p.status)) {
                         mbar_wait_bounded(bar_b, ph_b, p.status, 1u << 20);
                         *aux_fail = 1;
@@ -549,10 +590,9 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
                 if (*aux_fail) break;
                 cur_g0 = m.g0;
                 cur_ng = m.ng;
-                cur_bc = want_bc;
             }
-            // ---- 3. contraction: issuer aw takes directions of parity aw & 1 and
-            // half aw >> 1 of K (with two issuers, all of K) ----
+            // ---- 3. contraction: issuer aw takes block aw % blocks (directions of
+            // one parity, or all) and part aw / blocks of K ----
             const uint32_t cols = (uint32_t)(16 * m.ng);
             const bool dbl = p.n_iss * (int)cols <= 128;
             if (m.flags & kPassFirst) dbuf = dbl ? dbuf ^ 128u : 0u;
@@ -562,12 +602,12 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
             }
             if (lane == 0) {
                 if (aw < p.n_iss) {
-                    const int nk = NBc / 64 / nh;   // K = 16 steps of this issuer
-                    const int k0 = (aw >> 1) * nk;
+                    const int nk = K / 16 / nh;   // K = 16 steps of this issuer
+                    const int k0 = (aw / blocks) * nk;
                     const uint32_t idesc = idesc_f16_mk(128, (int)cols, false);
                     const uint32_t d = tmem + kTmemD + dbuf + (uint32_t)aw * cols;
-                    const uint32_t a = tmem + kTmemA + (uint32_t)(aw & 1) * 128u;
-                    const uint64_t b = sdesc_sw128(bt_addr + (all ? (uint32_t)m.bc * 2u * part : 0u), 16u, (uint32_t)KB * 1024u);
+                    const uint32_t a = tmem + kTmemA + (uint32_t)(aw % blocks) * 128u;
+                    const uint64_t b = sdesc_sw128(bt_addr, 16u, (uint32_t)KB * 1024u);
                     for (int k = k0; k < k0 + nk; ++k)
                         mma_f16_ta(d, a + (uint32_t)(8 * k), b + (uint64_t)((k >> 2) * 64 + (k & 3) * 2), idesc,
                                    k > k0 || !(m.flags & kPassFirst) ? 1u : 0u);
@@ -1288,21 +1328,20 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
 
 // ---- the global B operand: DFT matrix columns, fp16 hi + lo, K-major SW128 ----
 
-// Chunk bc covers bins [bc nbc, bc nbc + nbc) with nbc = min(2^m, 1024); its K
-// rows are the first half of those bins, n = bc nbc + kr, kr < nbc / 2.
-// Layout [chunk][hi|lo][group][64-row K block] x 1 KB, 128-byte swizzle
-// (narrow bands: a batch of groups is one contiguous run per part), or with
-// `streamed` the first nbc / 4 rows only, [chunk][32-row K block][hi|lo][group]
-// x 512 B, 64-byte swizzle, with ng + 1 groups per run, the last left as the
-// caller's zeros (wide bands: one K block of one part over a run of groups is
-// contiguous).
+// Narrow bands: the first part's bins n < K (tp_k_rows), layout [hi|lo][group]
+// [64-row K block] x 1 KB, 128-byte swizzle (a run of groups is contiguous per
+// part).  With `streamed` (wide bands), chunk bc covers bins [bc nbc, bc nbc +
+// nbc) with nbc = min(2^m, 1024), the first nbc / 4 of them as K rows: [chunk]
+// [32-row K block][hi|lo][group] x 512 B, 64-byte swizzle, with ng + 1 groups per
+// run, the last left as the caller's zeros (one K block of one part over a run of
+// groups is contiguous).
 __global__ void k_build_twb(uint8_t* twb, int m, int kbase, int ng, bool streamed) {
     const int NB = 1 << m;
     const int NBc = NB < kChunkBins ? NB : kChunkBins;
     const int nchunk = NB / NBc;
-    const int NK = NBc / 4;
-    const int KB = NBc / 256, KBs = NBc / 128;
-    const int64_t total = (int64_t)nchunk * 2 * ng * NK * 8;   // chunks x [hi|lo] x groups x K rows x 8 columns
+    const int NK = streamed ? NBc / 4 : tp_k_rows(m);
+    const int KB = NK / 64, KBs = NBc / 128;
+    const int64_t total = (int64_t)(streamed ? nchunk : 1) * 2 * ng * NK * 8;   // chunks x [hi|lo] x groups x K rows x 8 columns
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int r = (int)(i & 7);
         const int64_t t = i >> 3;
@@ -1327,7 +1366,7 @@ __global__ void k_build_twb(uint8_t* twb, int m, int kbase, int ng, bool streame
             off = blk * 512 + (size_t)r * 64 + (size_t)(((kin >> 3) ^ ((r >> 1) & 3)) << 4) + (size_t)(kin & 7) * 2;
         } else {
             const int kb = k >> 6, kin = k & 63;
-            const size_t blk = (size_t)((2 * bc + part) * ng + g) * KB + kb;
+            const size_t blk = (size_t)(part * ng + g) * KB + kb;
             off = blk * 1024 + (size_t)r * 128 + (size_t)(((kin >> 3) ^ r) << 4) + (size_t)(kin & 7) * 2;
         }
         *reinterpret_cast<__half*>(twb + off) = part ? lo : hi;
@@ -1349,9 +1388,9 @@ static size_t tc_smem_bytes(int m, int atom_cap, size_t bt_bytes) {
            128 * 8 * 4 + 256;
 }
 
-static size_t tp_smem_bytes(int m, int atom_cap) {
+static size_t tp_smem_bytes(int m, int atom_cap, size_t bt_bytes) {
     const size_t nbc = std::min<size_t>((size_t)1 << m, kChunkBins);
-    return 1024 + nbc * 128 + kBtBytes + 2 * kExFloats * 4 + (size_t)atom_cap * 16 + 2 * kDirs * 16 + 2 * sizeof(TpPass) + 128;
+    return 1024 + nbc * 128 + bt_bytes + 2 * kExFloats * 4 + (size_t)atom_cap * 16 + 2 * kDirs * 16 + 2 * sizeof(TpPass) + 128;
 }
 
 // Build the B operand for the current ROI bands and pick the TMEM size.
@@ -1360,11 +1399,12 @@ int prepare_tc(Ctx* c) {
     const int NB = 1 << c->m;
     const int NBc = std::min(NB, kChunkBins);
     const int nchunk = NB / NBc;
-    const int KB = NBc / 256;   // 1 KB blocks of 64 K rows per chunk, K = NBc / 4
+    const int KB = tp_k_rows(c->m) / 64;   // 1 KB blocks of 64 K rows
     const int kbase = c->band_min;
     const int ng = (c->band_max - kbase) / 4 + 1;
-    // groups one B batch and the accumulators of two issuers hold
-    const int gb = std::min(8, kBtBytes / (2 * KB * 1024));
+    // groups whose B operand shared memory holds beside the histogram (32 KB, above
+    // 2^10 bins 64 KB) and whose accumulators tensor memory holds for two issuers
+    const int gb = std::min(8, (c->m > 10 ? 2 : 1) * kBtBytes / (2 * KB * 1024));
     int ng_roi_max = 1;
     for (int64_t r = 0; r < c->nroi; ++r) {
         const int g0 = (c->h_band[2 * r] - kbase) >> 2, g1 = (c->h_band[2 * r + 1] - kbase) >> 2;
@@ -1389,7 +1429,7 @@ int prepare_tc(Ctx* c) {
         c->d_twb = nullptr;
         c->twb_key[0] = c->twb_key[1] = c->twb_key[2] = -1;
         // both layouts of the same twiddles: [narrow | streamed (one zero group more per run)]
-        const size_t bytes = (size_t)nchunk * 2 * ng * KB * 1024;
+        const size_t bytes = (size_t)2 * ng * KB * 1024;
         const size_t sbytes = (size_t)nchunk * 2 * (ng + 1) * (NBc / 128) * 512;
         int rc = dev_alloc(c, &c->d_twb, bytes + sbytes);
         if (rc) return rc;
@@ -1414,6 +1454,8 @@ int prepare_tc(Ctx* c) {
     c->tc_ng_roi = ng_roi_max;
     return APTIDX_OK;
 }
+
+static int tp_tile_dirs(int m) { return kDirs >> std::max(0, m - 10); }
 
 // Tiles per work item when none was tuned: the split of a ROI into items that
 // ends first if every CTA takes the same number of items, a set-up (staging and
@@ -1440,22 +1482,29 @@ int tuned_tiles_per_item(const Ctx* c, int path) {
     if (c->tune_tpi[path] > 0) return c->tune_tpi[path];
     if (path == 0 || c->nroi <= 0) return 16;
     const bool pairs = c->use_pairs && c->d_slot_idx;
-    return tiles_per_item_rule(c, (pairs ? c->nslot_pad : c->nv_pad) / kDirs, c->nroi);
+    return tiles_per_item_rule(c, (pairs ? c->nslot_pad : c->nv_pad) / (c->tc_wide ? kDirs : tp_tile_dirs(c->m)), c->nroi);
 }
 
 cudaError_t launch_signatures_tc(Ctx* c, float* S, uint16_t* argk, uint16_t* hist_out, int64_t hist_roi) {
     cudaError_t e;
     static int max_optin = -1;
     if (max_optin < 0) cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
-    const size_t bt_bytes = c->tc_wide ? 4 * (size_t)kWideStage : (size_t)kBtBytes;
-    const size_t base = c->tc_wide ? tc_smem_bytes(c->m, 0, bt_bytes) : tp_smem_bytes(c->m, 0);
+    const size_t bt_bytes = c->tc_wide ? 4 * (size_t)kWideStage : 32 * (size_t)c->tc_ng_roi * tp_k_rows(c->m);
+    const size_t base = c->tc_wide ? tc_smem_bytes(c->m, 0, bt_bytes) : tp_smem_bytes(c->m, 0, bt_bytes);
     int cap = (int)(((size_t)max_optin - base) / 16);
     cap = std::min(cap, kTcMaxAtoms) & ~15;
     if (cap < 256) return cudaErrorInvalidConfiguration;
     const size_t smem = base + (size_t)cap * 16;
     const bool multi = !hist_out && c->multi.n > 0;
-    auto kern = multi ? (c->tc_wide ? k_sig_tc<APTIDX_MAX_BANDS, true> : k_sig_tp<APTIDX_MAX_BANDS>)
-                      : (c->tc_wide ? k_sig_tc<1, true> : k_sig_tp<1>);
+    void (*kern)(TcParams);
+    if (c->tc_wide)
+        kern = multi ? k_sig_tc<APTIDX_MAX_BANDS, true> : k_sig_tc<1, true>;
+    else if (c->m <= 10)
+        kern = multi ? k_sig_tp<APTIDX_MAX_BANDS, 0> : k_sig_tp<1, 0>;
+    else if (c->m == 11)
+        kern = multi ? k_sig_tp<APTIDX_MAX_BANDS, 1> : k_sig_tp<1, 1>;
+    else
+        kern = multi ? k_sig_tp<APTIDX_MAX_BANDS, 2> : k_sig_tp<1, 2>;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
     // antipodal pairs (one projection per pair) unless switched off or exporting
@@ -1468,7 +1517,7 @@ cudaError_t launch_signatures_tc(Ctx* c, float* S, uint16_t* argk, uint16_t* his
     p.dirs = pairs ? c->d_slot_dirs : c->d_dirs;
     p.slot_idx = pairs ? c->d_slot_idx : nullptr;
     p.nv = c->nv;
-    p.tiles_per_roi = (pairs ? c->nslot_pad : c->nv_pad) / kDirs;
+    p.tiles_per_roi = (pairs ? c->nslot_pad : c->nv_pad) / (c->tc_wide ? kDirs : tp_tile_dirs(c->m));
     p.nroi = c->rank_limit > 0 ? std::min<int64_t>(c->nroi, c->rank_limit) : c->nroi;
     p.tiles_per_item = std::min(c->tune_tpi[1] > 0 ? c->tune_tpi[1]
                                                    : tiles_per_item_rule(c, p.tiles_per_roi, hist_out ? 1 : p.nroi),

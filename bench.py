@@ -84,7 +84,7 @@ def kernel_sources_sha16(names):
 
 
 def tc_traffic_per_launch(n_roi):
-    """DRAM bytes per k_sig_tc launch from the committed ncu figure
+    """DRAM bytes per signature launch from the committed ncu figure
     (profiles/k_sig_tc_traffic.json), scaled to n_roi ROIs; None when the
     kernel sources changed since the capture."""
     try:
@@ -571,7 +571,7 @@ def run_gb300(args):
             "traffic": tc_traffic_per_launch(nroi) if headline == "tc" else None,
             "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of a smaller launch scaled by "
                               "ROIs (profiles/k_sig_tc_traffic.json); null once the kernel sources change",
-            "kernel": "k_sig_plain" if headline == "plain" else "k_sig_tc",
+            "kernel": "k_sig_plain" if headline == "plain" else "k_sig_tp",
             "kernel_ms": sig_ms,
             "peak_source": "FP32 FMA: 152 SMs x 128 lanes x 2 flop x 2.07 GHz (unit counts and max clock; packed "
                            "fma.rn.f32x2 runs at the same FMA rate)",

@@ -149,29 +149,6 @@ __device__ __forceinline__ uint64_t f2_dup(float v) {
     return ((uint64_t)__float_as_uint(v) << 32) | (uint64_t)__float_as_uint(v);
 }
 
-// Rearranges staged atoms in place for the paired histogram loop: the
-// 32-byte block of atoms 2p, 2p + 1 becomes (x_a, x_b, y_a, y_b | z_a, z_b,
-// w_a, w_b), so that one 16-byte and one 8-byte load give the coordinates
-// of both atoms as FP32 pairs.  A trailing odd atom keeps its layout.  With
-// r2max, the largest x^2 + y^2 + z^2 (FP32) of the atoms goes to *r2max by
-// atomicMax on its bit pattern (the caller zeroes it).
-__device__ __forceinline__ void pair_atoms(float4* A, int n, int tid, int nthreads, unsigned* r2max = nullptr) {
-    float m = 0.f;
-    for (int q = tid; q < (n >> 1); q += nthreads) {
-        const float4 a = A[2 * q], b = A[2 * q + 1];
-        A[2 * q] = make_float4(a.x, b.x, a.y, b.y);
-        A[2 * q + 1] = make_float4(a.z, b.z, a.w, b.w);
-        m = fmaxf(m, fmaxf(a.x * a.x + a.y * a.y + a.z * a.z, b.x * b.x + b.y * b.y + b.z * b.z));
-    }
-    if (r2max) {
-        if ((n & 1) && tid == 0) {
-            const float4 a = A[n - 1];
-            m = fmaxf(m, a.x * a.x + a.y * a.y + a.z * a.z);
-        }
-        atomicMax(r2max, __float_as_uint(m));
-    }
-}
-
 // Whether, along any direction of norm <= 1 + 1e-5, a projection s of an atom
 // with |x|^2 <= r2max can make s * scale an exact nonzero integer.  With
 // scale = J 2^E (J odd) and s = j 2^e (j odd), s * scale = j J 2^(e + E) is an
@@ -188,191 +165,16 @@ __device__ __forceinline__ bool nonzero_integer_products_possible(float scale, f
     return !(r2max * 1.00005f < ldexpf(1.0f, -2 * E));
 }
 
-// Per-lane constants of the paired loop: the lane's two directions and the
-// binning scale and magic, each duplicated into both halves of a pair.
-struct PairDirs {
-    uint64_t x0, y0, z0, x1, y1, z1, sc, mg;
-};
-
-__device__ __forceinline__ PairDirs pair_dirs(float4 d0, float4 d1, float scale, float magic) {
-    PairDirs q;
-    q.x0 = f2_dup(d0.x);
-    q.y0 = f2_dup(d0.y);
-    q.z0 = f2_dup(d0.z);
-    q.x1 = f2_dup(d1.x);
-    q.y1 = f2_dup(d1.y);
-    q.z1 = f2_dup(d1.z);
-    q.sc = f2_dup(scale);
-    q.mg = f2_dup(magic);
-    return q;
-}
-
-// Two atoms (one paired block) into the histograms of a 64-direction tile:
-// the projections and the binning of Eq. 1 in the scalar order (x, then
-// y, then z; fma rounding down for the bin) on FP32 pairs, then the four
-// increments of hist_add_atom's unmasked form.
-__device__ __forceinline__ void hist_add_pair(uint32_t hbase, ulonglong2 xy, uint64_t zz, const PairDirs& q) {
-    const uint64_t s0 = f2_fma(zz, q.z0, f2_fma(xy.y, q.y0, f2_mul(xy.x, q.x0)));
-    const uint64_t s1 = f2_fma(zz, q.z1, f2_fma(xy.y, q.y1, f2_mul(xy.x, q.x1)));
-    const uint64_t t0 = f2_fma_rd(s0, q.sc, q.mg);
-    const uint64_t t1 = f2_fma_rd(s1, q.sc, q.mg);
-    const uint32_t base = hbase - 0x80000000u;   // (t - 0x4B000000) * 128 + hbase, wrapping
-    const uint32_t wa0 = (uint32_t)t0 * 128u + base, wb0 = (uint32_t)(t0 >> 32) * 128u + base;
-    const uint32_t wa1 = (uint32_t)t1 * 128u + base, wb1 = (uint32_t)(t1 >> 32) * 128u + base;
-    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(wa0), "r"(1u) : "memory");
-    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(wb0), "r"(1u) : "memory");
-    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(wa1), "r"(0x10000u) : "memory");
-    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(wb1), "r"(0x10000u) : "memory");
-}
-
-// hist_tile<W, false> over atoms staged by pair_atoms: warp w takes the
-// pairs w, w + W, w + 2W, ...; the odd trailing atom goes to warp
-// (cn / 2) % W.
-template <int W>
-__device__ __forceinline__ void hist_tile_pairs(uint32_t* H, const float4* A, int cn, int warp, int lane,
-                                                float4 d0, float4 d1, float scale, float magic) {
-    const uint32_t hbase = smem_u32(H) + 4u * (uint32_t)lane;
-    const PairDirs q = pair_dirs(d0, d1, scale, magic);
-    const int np = cn >> 1;
-    int j = warp;
-    auto ld_xy = [&](int i) { return *reinterpret_cast<const ulonglong2*>(A + 2 * i); };
-    auto ld_z = [&](int i) { return *reinterpret_cast<const uint64_t*>(A + 2 * i + 1); };
-    if (j + W < np) {
-        // two pairs at a time, the next two pairs' loads issued first
-        ulonglong2 xa = ld_xy(j), xb = ld_xy(j + W);
-        uint64_t za = ld_z(j), zb = ld_z(j + W);
-        for (; j + 3 * W < np; j += 2 * W) {
-            const ulonglong2 nxa = ld_xy(j + 2 * W), nxb = ld_xy(j + 3 * W);
-            const uint64_t nza = ld_z(j + 2 * W), nzb = ld_z(j + 3 * W);
-            hist_add_pair(hbase, xa, za, q);
-            hist_add_pair(hbase, xb, zb, q);
-            xa = nxa;
-            xb = nxb;
-            za = nza;
-            zb = nzb;
-        }
-        hist_add_pair(hbase, xa, za, q);
-        hist_add_pair(hbase, xb, zb, q);
-        j += 2 * W;
-    }
-    for (; j < np; j += W) hist_add_pair(hbase, ld_xy(j), ld_z(j), q);
-    if ((cn & 1) && warp == np % W) {
-        const float4 d0s = d0, d1s = d1;
-        hist_add_atom<false>(hbase, A[cn - 1], d0s, d1s, scale, magic, 0);
-    }
-}
-
-// -----------------------------------------------------------------------------
-// Histogram pass of the general tensor-core path: bin chunks, and the count of
-// atoms whose bin product is not an integer.
-//
-// Bin chunks (m > 10): the 2^m bins are split into chunks of 1024 bins (128 KB
-// of histogram words); the pass for chunk bc adds only atoms whose bin lies in
-// [1024 bc, 1024 bc + 1024), at row b - 1024 bc.  The bin fma's bit pattern is
-// 0x4B000000 + b, so the chunk of b is bits 10.. of the pattern.
-//
 // Antipodal directions: along -u the projection is exactly -s (round to
 // nearest is symmetric), so the bin of -u is 2^m - 1 - b(u) whenever the exact
 // product x = s * scale is not an integer, and 2^m - b(u) when it is.  With the
-// product rounded down (t_rd) and up (t_ru) onto the integer grid of
-// [2^23, 2^24), t_ru - t_rd is 1 for a non-integer x and 0 for an integer x; a
-// lane sums it over its atoms (kCount), so the histogram of -u is the mirror
-// image of the histogram of u exactly when that sum equals the lane's atom
-// count.
-// -----------------------------------------------------------------------------
-template <int kCount, bool kChunked>
-__device__ __forceinline__ void hist_add_pair2(uint32_t hb, ulonglong2 xy, uint64_t zz, const PairDirs& q,
-                                               uint32_t bc, uint32_t cmask, uint32_t& c0, uint32_t& c1,
-                                               uint64_t& zp) {
-    const uint64_t s0 = f2_fma(zz, q.z0, f2_fma(xy.y, q.y0, f2_mul(xy.x, q.x0)));
-    const uint64_t s1 = f2_fma(zz, q.z1, f2_fma(xy.y, q.y1, f2_mul(xy.x, q.x1)));
-    const uint64_t t0 = f2_fma_rd(s0, q.sc, q.mg);
-    const uint64_t t1 = f2_fma_rd(s1, q.sc, q.mg);
-    if (kCount == 2) {
-        zp = f2_mul(zp, f2_mul(s0, s1));
-    } else if (kCount == 1) {
-        const uint64_t u0 = f2_fma_ru(s0, q.sc, q.mg);
-        const uint64_t u1 = f2_fma_ru(s1, q.sc, q.mg);
-        c0 += ((uint32_t)u0 - (uint32_t)t0) + ((uint32_t)(u0 >> 32) - (uint32_t)(t0 >> 32));
-        c1 += ((uint32_t)u1 - (uint32_t)t1) + ((uint32_t)(u1 >> 32) - (uint32_t)(t1 >> 32));
-    }
-    // (t - 0x4B000000 - 1024 bc) * 128 + H + 4 lane, in wrapping 32-bit arithmetic
-    const uint32_t wa0 = (uint32_t)t0 * 128u + hb, wb0 = (uint32_t)(t0 >> 32) * 128u + hb;
-    const uint32_t wa1 = (uint32_t)t1 * 128u + hb, wb1 = (uint32_t)(t1 >> 32) * 128u + hb;
-    if (kChunked) {
-        if ((((uint32_t)t0 >> 10) & cmask) == bc) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(wa0), "r"(1u) : "memory");
-        if ((((uint32_t)(t0 >> 32) >> 10) & cmask) == bc)
-            asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(wb0), "r"(1u) : "memory");
-        if ((((uint32_t)t1 >> 10) & cmask) == bc)
-            asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(wa1), "r"(0x10000u) : "memory");
-        if ((((uint32_t)(t1 >> 32) >> 10) & cmask) == bc)
-            asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(wb1), "r"(0x10000u) : "memory");
-    } else {
-        asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(wa0), "r"(1u) : "memory");
-        asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(wb0), "r"(1u) : "memory");
-        asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(wa1), "r"(0x10000u) : "memory");
-        asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(wb1), "r"(0x10000u) : "memory");
-    }
-}
-
-template <int kCount, bool kChunked>
-__device__ __forceinline__ void hist_add_one2(uint32_t hb, float4 a, float4 d0, float4 d1, float scale, float magic,
-                                              uint32_t bc, uint32_t cmask, uint32_t& c0, uint32_t& c1, uint64_t& zp) {
-    const float s0 = project_f32(d0.x, d0.y, d0.z, a);
-    const float s1 = project_f32(d1.x, d1.y, d1.z, a);
-    const uint32_t t0 = __float_as_uint(__fmaf_rd(s0, scale, magic));
-    const uint32_t t1 = __float_as_uint(__fmaf_rd(s1, scale, magic));
-    if (kCount == 2) {
-        zp = (zp & 0xFFFFFFFF00000000ull) | (uint64_t)__float_as_uint(__uint_as_float((uint32_t)zp) * s0 * s1);
-    } else if (kCount == 1) {
-        c0 += __float_as_uint(__fmaf_ru(s0, scale, magic)) - t0;
-        c1 += __float_as_uint(__fmaf_ru(s1, scale, magic)) - t1;
-    }
-    if (!kChunked || ((t0 >> 10) & cmask) == bc)
-        asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(t0 * 128u + hb), "r"(1u) : "memory");
-    if (!kChunked || ((t1 >> 10) & cmask) == bc)
-        asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(t1 * 128u + hb), "r"(0x10000u) : "memory");
-}
-
-// Histograms of one 64-direction tile over `cn` atoms staged by pair_atoms, for
-// bin chunk bc (kChunked) or all bins; warp w takes pairs w, w + W, ...
-// Returns the number of atoms this warp handled.  kCount == 1: c0, c1
-// accumulate the lane's non-integer counts of its two directions; kCount ==
-// 2 (only s = 0 can give an integer product): zp multiplies the projections
-// of the lane's atoms along both directions, so a zero half means an atom
-// with s = 0 (a product of the ~70 factors |s| <= R a lane sees per tile
-// stays above ~1e-20 at four standard deviations, far from FP32's 1e-45; an
-// underflow would only cost the tile a second pass).
-template <int W, int kCount, bool kChunked>
-__device__ __forceinline__ int hist_tile_pairs2(uint32_t* H, const float4* A, int cn, int warp, int lane, float4 d0,
-                                                float4 d1, float scale, float magic, uint32_t bc, uint32_t cmask,
-                                                uint32_t& c0, uint32_t& c1, uint64_t& zp) {
-    const uint32_t hb = smem_u32(H) + 4u * (uint32_t)lane - 0x80000000u - (bc << 17);
-    const PairDirs q = pair_dirs(d0, d1, scale, magic);
-    const int np = cn >> 1;
-    int j = warp;
-    auto ld_xy = [&](int i) { return *reinterpret_cast<const ulonglong2*>(A + 2 * i); };
-    auto ld_z = [&](int i) { return *reinterpret_cast<const uint64_t*>(A + 2 * i + 1); };
-    // four independent atom pairs per step (their loads first)
-    for (; j + 3 * W < np; j += 4 * W) {
-        const ulonglong2 x0 = ld_xy(j), x1 = ld_xy(j + W), x2 = ld_xy(j + 2 * W), x3 = ld_xy(j + 3 * W);
-        const uint64_t z0 = ld_z(j), z1 = ld_z(j + W), z2 = ld_z(j + 2 * W), z3 = ld_z(j + 3 * W);
-        hist_add_pair2<kCount, kChunked>(hb, x0, z0, q, bc, cmask, c0, c1, zp);
-        hist_add_pair2<kCount, kChunked>(hb, x1, z1, q, bc, cmask, c0, c1, zp);
-        hist_add_pair2<kCount, kChunked>(hb, x2, z2, q, bc, cmask, c0, c1, zp);
-        hist_add_pair2<kCount, kChunked>(hb, x3, z3, q, bc, cmask, c0, c1, zp);
-    }
-    for (; j < np; j += W) hist_add_pair2<kCount, kChunked>(hb, ld_xy(j), ld_z(j), q, bc, cmask, c0, c1, zp);
-    int handled = warp < np ? 2 * ((np - warp + W - 1) / W) : 0;
-    if ((cn & 1) && warp == np % W) {
-        hist_add_one2<kCount, kChunked>(hb, A[cn - 1], d0, d1, scale, magic, bc, cmask, c0, c1, zp);
-        handled += 1;
-    }
-    return handled;
-}
+// product rounded down (t_rd) and up (t_ru) onto the integer grid, t_ru - t_rd is
+// one unit for a non-integer x and 0 for an integer x; a lane sums it over its atoms
+// (kCount == 1), so the histogram of -u is the mirror image of the histogram of u
+// exactly when that sum equals the lane's atom count.
 
 // -----------------------------------------------------------------------------
-// Histogram pass of the pipelined tensor-core kernel.  Atoms lie in 64-byte
+// Histogram pass of the signature kernels.  Atoms lie in 64-byte
 // blocks of four (x of the four | y | z | unused), three 16-byte loads that are
 // the FP32 pairs of two packed steps.  The bin fma runs at four times the scale
 // on the integer grid of [2^25, 2^26) (spacing 4): its bit pattern is
@@ -445,9 +247,10 @@ __device__ __forceinline__ void quad_inc(uint32_t t, uint32_t one, const QuadDir
     }
 }
 
-// kCount as in hist_add_pair2, except that for 2 the smallest |s| is kept (0:
-// some projection is exactly zero) instead of a product, two three-input minima
-// on the integer pipe instead of two packed multiplies
+// kCount == 1: c0, c1 accumulate the lane's non-integer counts of its two
+// directions.  kCount == 2 (only s = 0 can give an integer product): the smallest
+// |s s'| of the lane's two directions, 0 when some projection is exactly zero (or a
+// product underflows, which would only cost the tile a second pass).
 template <int kCount, bool kChunked, int kSplit = 0>
 __device__ __forceinline__ void quad_add_pair(uint64_t x, uint64_t y, uint64_t z, const QuadDirs& q, uint32_t& c0,
                                               uint32_t& c1, float& zmin) {
@@ -515,18 +318,6 @@ __device__ __forceinline__ int hist_tile_quads(const float4* A, int cn, int warp
         }
     }
     return handled;
-}
-
-// Debug export of a tile's histograms: h_out[v * 2^m + b] for v < nv.
-__device__ __forceinline__ void hist_export(const uint32_t* H, int NB, int tile, int nv, uint16_t* h_out, int tid,
-                                            int nthreads) {
-    for (int i = tid; i < NB * 32; i += nthreads) {
-        const int b = i >> 5, l = i & 31;
-        const uint32_t w = H[i];
-        const int64_t v0 = (int64_t)tile * 64 + 2 * l;
-        if (v0 < nv) h_out[v0 * NB + b] = (uint16_t)(w & 0xFFFFu);
-        if (v0 + 1 < nv) h_out[(v0 + 1) * NB + b] = (uint16_t)(w >> 16);
-    }
 }
 
 // Band maxima of one direction: frequency f with amplitude a updates every

@@ -219,7 +219,7 @@ __device__ __forceinline__ float node_dot(float4 u, float3 r) {
 // left to k_lut_scan.  Scanning all 40962 nodes for every query took 29.1 ms
 // for 3419 x 1000 queries (1.4e11 dot products); this reads about 20 nodes per
 // query, bound by the L2 latency of the run bounds and nodes:
-// 0.3 ms.
+// 0.4 ms.
 constexpr int kLutK = 8;   // nodes per thread (one rotation matrix, kLutK of its columns of the table)
 
 struct NodeGrid {

@@ -112,7 +112,6 @@ struct Ctx {
     void* d_twb = nullptr;
     size_t twb_bytes = 0;
     int twb_key[3] = {-1, -1, -1};     // (m, band_min, groups)
-    int tc_gb = 0;                     // frequency groups per B batch
     int tc_ng = 0;                     // groups in the global B operand
     uint32_t tc_tmem_cols = 0;
     int tc_ng_roi = 1;                 // most groups of one ROI's band

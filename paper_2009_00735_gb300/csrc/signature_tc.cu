@@ -5,16 +5,14 @@
 // spectrum of every SDM; the paper notes that the SDMs of a ROI share one
 // bin count, which permits batching their transforms).
 //
-// The histogram of a tile is built in chunks of at most 1024 bins (2^m <= 1024:
-// one chunk; m = 11, 12: two or four) and over blocks of at most 2048 atoms,
-// so that every count of a block is exact in fp16; every (block, chunk) pass is
-// contracted into the same tensor-memory accumulators.  The contraction of a
-// pass runs as M = 128 rows: rows 0-63 are the 64 directions over the chunk's
-// first half of bins, rows 64-127 the same directions over its second half.
-// Both halves use the twiddles of the first half, since
-// w^(k (n + h)) = w^(k h) w^(k n) for w = exp(-2 pi i / 2^m) and the half
-// offset h = 2^(m-1) (one chunk: w^(k h) = (-1)^k) or h = 512 (chunks of 1024);
-// the epilogue forms X(k) = D_lo(k) + w^(k h) D_hi(k).
+// The histogram of a tile covers all bins (tiles of 64 directions up to 2^10 bins,
+// of 32 and 16 at 2^11 and 2^12) over blocks of at most 2048 atoms, so that every
+// count of a block is exact in fp16; all blocks are contracted into the same
+// tensor-memory accumulators.  The bins split into four parts (eight of 2^12 bins):
+// the rows of the contraction (M = 128) are (part, direction), all parts use the
+// twiddles of the first, since w^(k (n + h)) = w^(k h) w^(k n) for
+// w = exp(-2 pi i / 2^m), and the epilogue adds the parts with their factors
+// w^(k h), fourth or eighth roots of one.
 //
 // Antipodal pairs: when the direction set holds u and -u, only u is projected;
 // -u gets the same signature value and frequency bin (its histogram is the
@@ -24,27 +22,31 @@
 // over the negated directions and writes their signatures from their own
 // histograms.
 //
-// Wide bands (more frequency groups than one B batch holds) run in their own
-// kernel instance (kWide): the chunk's bins split into quarters, only the
-// first quarter's twiddles stream from L2 through four shared-memory stages,
-// and each stage feeds two M = 128 MMAs per K step (bin quarters 0 | 2 and
-// 1 | 3); the epilogue applies the quarter factor w^(k NBc / 4).
+// Per tile and atom block:
+//   1. 16 warps histogram by shared-memory atomics (bank-private columns, as in the
+//      FP32 path); counts c <= 2048, so the u16 bit pattern of c is the fp16 value
+//      c * 2^-24 exactly (fp16 is linear through its subnormal range up to 0x0800);
+//   2. the same warps exchange every word with zero and store the counts to tensor
+//      memory, pairs of bins to a column: that is the A operand, and the histogram is
+//      ready for the next tile;
+//   3. four more warps issue the tcgen05.mma (A in tensor memory, K = 16, N = 16 per
+//      group of 4 frequencies: 8 hi columns, then 8 lo columns, where T = T_hi + T_lo
+//      with both parts fp16; the twiddles stay in shared memory) and
+//   4. read the accumulators (tcgen05.ld) of the tile before, add the partials, hi and
+//      lo parts and the bin parts (one exchange in shared memory), scale by 2^24 and
+//      keep the band maximum of |X(k)|.
+// 3 and 4 run under the next tile's 1.  Wide bands (more groups than shared memory
+// holds twiddles for) take k_sig_wide, below.
 //
-// Per 64-direction tile of a ROI and (block, chunk) pass:
-//   1. histograms by shared-memory atomics (bank-private columns, as in the
-//      FP32 path); counts c <= 2048, so the u16 bit pattern of c is the fp16
-//      value c * 2^-24 exactly (fp16 is linear through its subnormal range up
-//      to 0x0800) and the histogram is the A operand as it stands;
-//   2. an in-place permutation of 16-byte chunks gives the MN-major 128-byte
-//      swizzled layout (chunk c of bin row k moves to c ^ (k & 7));
-//   3. up to four issuer threads issue the bins / 32 tcgen05.mma of the chunk
-//      (M = 128, K = 16, N = 16 per group of 4 frequencies: 8 hi columns, then
-//      8 lo columns, where T = T_hi + T_lo with both parts fp16) into FP32
-//      accumulators in TMEM;
-//   4. after the last pass, warps 0-7 read the accumulators (tcgen05.ld), add
-//      the partials, hi and lo parts and the two bin halves (one exchange in
-//      shared memory), scale by 2^24 and keep the band maximum of |X(k)|,
-//      while warps 8-15 zero the histogram for the next pass.
+// What bounds it (2^10 bins, 1133 atoms, per 64-direction tile, cycles): the
+// histogram takes 5.2-5.6 K and the transfer 1.4 K, with 1.1 K to set up a tile and
+// 0.5 K of barriers; MMAs and epilogue (3.7 K) hide behind them.  The histogram is
+// bound by issue: 8 packed FMAs of two slots each, 4 shifts, 3 slots of the zero
+// check and about four slots per increment for every two atoms and two directions
+// (neither unrolling, software pipelining, 8 to 24 warps, halved atom loads nor
+// stores in place of the atomics change it).  One CTA per SM ran these phases one
+// after the other with the counts in shared memory: 13.5 K cycles, 116.5 ms for 8192
+// ROIs x 40962 directions; now 74.4 ms.
 #include <cuda_fp16.h>
 
 #include "tcgen05.cuh"
@@ -56,11 +58,10 @@ namespace {
 constexpr int kWarps = 16;
 constexpr int kThreads = kWarps * 32;
 constexpr int kDirs = kTileDirs;     // 64 directions per tile
-constexpr int kRows = 2 * kDirs;     // MMA M: (direction, bin half)
+constexpr int kRows = 2 * kDirs;     // MMA M of wide bands: (direction, bin half)
 constexpr int kBtBytes = 32 * 1024;  // shared-memory budget of the B operand (narrow bands)
 constexpr int kWideStage = 16 * 1024;   // wide bands: one of four twiddle stream stages
 constexpr int kExBytes = kDirs * 8 * 4;   // epilogue exchange: one group's (re, im) x 4 per direction
-constexpr int kIssuers = 4;          // at most this many warps issue MMAs, one TMEM partial accumulator each
 constexpr int kChunkBins = 1024;     // bins per histogram chunk (128 KB of words)
 
 struct TcParams {
@@ -85,8 +86,7 @@ struct TcParams {
                             // the last one zero
     int32_t bt_bytes;       // shared-memory bytes of the B region (kBtBytes, or 4 kWideStage)
     int32_t ng_total;
-    int32_t gb;             // groups per shared-memory batch
-    uint32_t tmem_cols;
+    uint32_t tmem_cols;     // wide bands
     float* S;
     uint16_t* argk;
     uint16_t* hist_out;
@@ -94,12 +94,9 @@ struct TcParams {
     int32_t* counter;
     int* status;
     int atom_cap;           // atoms per block (<= 2048)
-    int n_iss;              // MMA issuer warps (1 .. kIssuers)
+    int n_iss;              // MMA issuer warps of narrow bands (2 or 4)
     BandSet bands;
 };
-
-// instruction descriptor: A MN-major (the histogram), B K-major, M = 128
-__device__ __forceinline__ uint32_t idesc_f16(int n) { return idesc_f16_mk(kRows, n, true); }
 
 __device__ __forceinline__ void cp_async8(void* dst_smem, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
@@ -645,12 +642,30 @@ __global__ void __launch_bounds__(kTpThreads, 1) k_sig_tp(TcParams p) {
 
 // ---- wide bands ----------------------------------------------------------------
 
-// kNB: band slots of the epilogue (1: the ROI's own band; APTIDX_MAX_BANDS:
-// the pass's BandSet, aptidx_compute_signatures_multi); kWide: the instance
-// that streams the twiddles of bands wider than one B batch (the narrow-band
-// instance is compiled without that code)
-template <int kNB, bool kWide>
-__global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
+// Bands of more frequency groups than shared memory holds twiddles for.  A tile is 64
+// directions over chunks of at most 1024 bins (2^m <= 1024: one chunk; m = 11, 12: two
+// or four) and blocks of at most 2048 atoms; every (block, chunk) pass is contracted
+// into the same tensor-memory accumulators.  Per pass:
+//   1. histograms by shared-memory atomics, as above;
+//   2. an in-place permutation of 16-byte chunks gives the MN-major 128-byte swizzled
+//      layout (chunk c of bin row k moves to c ^ (k & 7)): the A operand, M = 128 rows
+//      of (64 directions, bin half);
+//   3. the chunk's bins split into quarters; the first quarter's twiddles stream from L2
+//      through four shared-memory stages, and each stage feeds two MMAs per K step (bin
+//      quarters 0 | 2 and 1 | 3);
+//   4. after the last pass, warps 0-7 read the accumulators and form X(k) = sum over the
+//      quarters with their factors w^(k q NBc / 4), while warps 8-15 zero the histogram.
+// The phases run one after the other (7.0, 2.6, 12.7 and 5.4 K cycles at 31 groups, 1133
+// atoms and 2^10 bins; 15.0 -> 14.9 ms with the atoms in blocks of four).  The
+// pipeline above, with the twiddles streamed under the next tile's histogram, is no
+// faster: 16.4-24 ms against 14.9 for 512 ROIs x 40962 directions, k = 8 .. 128.  The
+// counts in tensor memory leave 48 KB of shared memory for stages beside the next
+// histogram, and every wait of the issuing thread between such small batches of MMAs
+// costs 250-500 cycles, with 32 or more of them per tile.
+// kNB: band slots of the epilogue (1: the ROI's own band; APTIDX_MAX_BANDS: the pass's
+// BandSet, aptidx_compute_signatures_multi)
+template <int kNB>
+__global__ void __launch_bounds__(kThreads, 1) k_sig_wide(TcParams p) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte alignment for the swizzled operands; offset arithmetic on the
     // shared array keeps the pointers in the shared address space
@@ -658,26 +673,23 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
     const int NB = 1 << p.m;
     const int NBc = NB < kChunkBins ? NB : kChunkBins;   // bins per chunk
     const int nchunk = NB / NBc;
-    const uint32_t cmask = (uint32_t)(nchunk - 1);
-    const int KB = NBc / 128;   // 1 KB K-blocks of the B operand per chunk (K = NBc / 2 rows)
     uint32_t* H = reinterpret_cast<uint32_t*>(smem);
     unsigned char* BT = smem + (size_t)NBc * 128;
     float* EX = reinterpret_cast<float*>(BT + p.bt_bytes);   // [kDirs][8]
     float4* A = reinterpret_cast<float4*>(BT + p.bt_bytes + kExBytes);
     float4* DB = A + p.atom_cap;   // [2][parity][32]: this tile's directions and the next tile's
     int2* DI = reinterpret_cast<int2*>(DB + 2 * kDirs);   // [2][kDirs]: (output, partner) of those slots
-    float* EX2 = reinterpret_cast<float*>(DI + 2 * kDirs);   // [128 TMEM lanes][8]: partials 2, 3
-    // barriers: [0] atoms, [1] B operand, [2 .. 2 + kIssuers) MMA completion per
-    // issuer, then the wide-band stream: four stage loads, four stage MMA completions
-    constexpr int kBars = 2 + kIssuers + 8;
+    float* EX2 = reinterpret_cast<float*>(DI + 2 * kDirs);   // [128][8]
+    // barriers: [0] atoms, then four stage loads and four stage MMA completions
+    constexpr int kBars = 1 + 8;
     uint64_t* bars = reinterpret_cast<uint64_t*>(EX2 + 128 * 8);
-    uint64_t* wbar = bars + 2 + kIssuers;
+    uint64_t* wbar = bars + 1;
     int* flag = reinterpret_cast<int*>(bars + kBars);
     int64_t* item_s = reinterpret_cast<int64_t*>(bars + kBars + 1);
     uint32_t* tmem_s = reinterpret_cast<uint32_t*>(bars + kBars + 2);
-    int* iss_ok = reinterpret_cast<int*>(bars + kBars + 3);   // [kIssuers]
-    unsigned* r2max_s = reinterpret_cast<unsigned*>(iss_ok + kIssuers);   // largest |x|^2 of the item's atoms
-    int* prod_ok = reinterpret_cast<int*>(r2max_s + 1);                      // wide-band stream producer
+    int* iss_ok = reinterpret_cast<int*>(bars + kBars + 3);
+    int* prod_ok = iss_ok + 1;
+    unsigned* r2max_s = reinterpret_cast<unsigned*>(iss_ok + 2);   // largest |x|^2 of the item's atoms
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) {
@@ -698,10 +710,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
     const uint32_t h_addr = smem_u32(H);
     const uint32_t bt_addr = smem_u32(BT);
 
-    uint32_t ph_atoms = 0, ph_b = 0, ph_mma = 0;   // ph_mma: this warp's issuer barrier
-    uint32_t wph = 0u, wdph = 0u;   // wide stream parity bits (bit i: buffer i): stage loads (thread 0), stage MMAs (thread 32)
-    int cur_g0 = -1, cur_nb = -1, cur_bc = -1;     // B operand held in shared memory
-    const float magic = bin_magic(p.m);
+    uint32_t ph_atoms = 0;
+    uint32_t wph = 0u, wdph = 0u;   // stream parity bits (bit i: buffer i): stage loads (thread 0), stage MMAs (thread 32)
+    const float magic = quad_magic(p.m, h_addr >> 7);
     const bool sym = p.slot_idx != nullptr;
     const int64_t n_items = (p.single_roi >= 0 ? 1 : p.nroi) * (int64_t)p.items_per_roi;
     bool failed = false;
@@ -720,7 +731,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
         const int klo = p.band[2 * roi], khi = p.band[2 * roi + 1];
         const int fg0 = (klo - p.kbase) >> 2, fg1 = (khi - p.kbase) >> 2;
         const int ng = fg1 - fg0 + 1;
-        const int nbatch = 2;   // TRANSITION
         const int t0 = grp * p.tiles_per_item;
         const int t1 = min(t0 + p.tiles_per_item, p.tiles_per_roi);
         const int nblk = max(1, (nw + p.atom_cap - 1) / p.atom_cap);   // atom blocks
@@ -730,7 +740,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
                 failed = true;
                 break;
             }
-            pair_atoms(A, nw, tid, kThreads, r2max_s);
+            quad_atoms(A, nw, tid, kThreads, r2max_s);
         }
         // the first tile's directions (later tiles' arrive while the tile
         // before them runs)
@@ -765,7 +775,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
                 }
                 const bool count = sym && pass == 0;
                 uint32_t c0 = 0, c1 = 0;
-                uint64_t zp = f2_dup(1.f);
+                float zmin = 1.f;
+                QuadDirs q = quad_dirs(d0, d1, scale, magic, lane);
                 int handled = 0;
                 const int n_sub = nblk * nchunk;
                 for (int sub = 0; sub < n_sub && !failed; ++sub) {
@@ -778,30 +789,26 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
                             failed = true;
                             break;
                         }
-                        pair_atoms(A, cn, tid, kThreads);
+                        quad_atoms(A, cn, tid, kThreads);
                         __syncthreads();
                     }
                     // ---- 1. histograms (H is zero here) ----
                     if (nchunk == 1) {
                         if (count && zero_check)
-                            handled += hist_tile_pairs2<kWarps, 2, false>(H, A, cn, warp, lane, d0, d1, scale, magic,
-                                                                          0u, 0u, c0, c1, zp);
+                            handled += hist_tile_quads<2, false>(A, cn, warp, kWarps, q, c0, c1, zmin);
                         else if (count)
-                            handled += hist_tile_pairs2<kWarps, 1, false>(H, A, cn, warp, lane, d0, d1, scale, magic,
-                                                                          0u, 0u, c0, c1, zp);
+                            handled += hist_tile_quads<1, false>(A, cn, warp, kWarps, q, c0, c1, zmin);
                         else
-                            hist_tile_pairs2<kWarps, 0, false>(H, A, cn, warp, lane, d0, d1, scale, magic, 0u, 0u,
-                                                               c0, c1, zp);
+                            hist_tile_quads<0, false>(A, cn, warp, kWarps, q, c0, c1, zmin);
                     } else {
+                        q.t_lo = kQuadBits + (h_addr >> 7) + (uint32_t)bc * kChunkBins;
+                        q.h_lane = h_addr + 4u * (uint32_t)lane;
                         if (count && bc == 0 && zero_check)
-                            handled += hist_tile_pairs2<kWarps, 2, true>(H, A, cn, warp, lane, d0, d1, scale, magic,
-                                                                         (uint32_t)bc, cmask, c0, c1, zp);
+                            handled += hist_tile_quads<2, true>(A, cn, warp, kWarps, q, c0, c1, zmin);
                         else if (count && bc == 0)
-                            handled += hist_tile_pairs2<kWarps, 1, true>(H, A, cn, warp, lane, d0, d1, scale, magic,
-                                                                         (uint32_t)bc, cmask, c0, c1, zp);
+                            handled += hist_tile_quads<1, true>(A, cn, warp, kWarps, q, c0, c1, zmin);
                         else
-                            hist_tile_pairs2<kWarps, 0, true>(H, A, cn, warp, lane, d0, d1, scale, magic,
-                                                              (uint32_t)bc, cmask, c0, c1, zp);
+                            hist_tile_quads<0, true>(A, cn, warp, kWarps, q, c0, c1, zmin);
                     }
                     __syncthreads();
                     if (p.hist_out) {
@@ -815,14 +822,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
                     // of row k to chunk c ^ (k & 7); rows with k & 7 == 0 stay).  The
                     // pass runs at the shared-memory bandwidth; interleaving it with
                     // the MMAs below slows both, so the two run one after the other.
-                    // ---- 3. contraction: lane 0 of warps 0 .. n_iss-1 issues every
-                    // n_iss-th K step into its own partial accumulator (a single
-                    // tcgen05.mma costs the issuing warp ~75 cycles whatever its N;
-                    // several issuers overlap that cost); every pass after the first
-                    // accumulates onto the result so far.
-                    // Wide bands (more frequency groups than one B batch holds):
-                    // the chunk's bins split into four quarters, and the twiddles of
-                    // the first quarter, all the ROI's groups, stream through four
+                    // ---- 3. contraction: the twiddles of the first quarter of the
+                    // chunk's bins, all the ROI's groups, stream through four
                     // 16 KB shared-memory stages, one per (32-bin K block, hi|lo
                     // part), in the 64-byte-swizzled K-major layout.  Each stage
                     // feeds two M = 128 MMAs per K step: block 0 (rows 0-63 the first
@@ -835,10 +836,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
                     // so a stage's bytes feed twice the tensor work of the bin-half
                     // split alone.  Thread 0 issues the MMAs as stages land; thread 32
                     // refills a stage once its MMAs are done, three stages ahead.
-                    const bool wide = kWide && nbatch > 1;
-                    const int n_iss = wide ? 1 : p.n_iss;
-                    const uint32_t sbo_b = (uint32_t)KB * 1024u;
-                    const bool issuer = lane == 0 && warp < n_iss;
                     const uint32_t acc0 = sub > 0 ? 1u : 0u;
                     // N = 8 x groups must be a multiple of 16 (M = 128): an odd group
                     // count takes one more group of twiddles (zeros past the last
@@ -855,36 +852,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
                                  p.twk + ((((size_t)bc * KB4 + kb) * 2 + part) * (p.ng_total + 1) + fg0) * 512, wbytes,
                                  &wbar[bf]);
                     };
-                    int ok = 1;
                     if (tid == 0) {
-                        if (wide) {
-                            // the first two stages load while the histogram is swizzled
-                            // (the epilogue before wrote the B region through the
-                            // generic proxy)
-                            fence_proxy_async_smem();
-                            for (int st = 0; st < 4; ++st) wide_load(st);
-                            cur_g0 = -1;   // the narrow-band B operand is overwritten
-                            *prod_ok = 1;
-                        } else {
-                            // B operand of the band for this chunk (kept across tiles while
-                            // the ROI band and the chunk allow)
-                            const int nb0 = fg1 + 1 - fg0;
-                            if (fg0 != cur_g0 || nb0 != cur_nb || bc != cur_bc) {
-                                const uint32_t part = (uint32_t)nb0 * KB * 1024u;
-                                fence_proxy_async_smem();
-                                mbar_arrive_expect_tx(&bars[1], 2 * part);
-                                bulk_g2s(BT, p.twb + ((size_t)(2 * bc) * p.ng_total + fg0) * KB * 1024, part, &bars[1]);
-                                bulk_g2s(BT + part, p.twb + ((size_t)(2 * bc + 1) * p.ng_total + fg0) * KB * 1024, part,
-                                         &bars[1]);
-                                ok = mbar_wait_bounded(&bars[1], ph_b, p.status) ? 1 : 0;
-                                if (!ok) mbar_wait_bounded(&bars[1], ph_b, p.status, 1u << 20);
-                                ph_b ^= 1u;
-                                cur_g0 = ok ? fg0 : -1;
-                                cur_nb = nb0;
-                                cur_bc = bc;
-                            }
-                        }
-                        *flag = ok;
+                        // the first stages load while the histogram is swizzled
+                        // (the epilogue before wrote the B region through the
+                        // generic proxy)
+                        fence_proxy_async_smem();
+                        for (int st = 0; st < 4; ++st) wide_load(st);
+                        *prod_ok = 1;
                     }
                     // two groups of four rows per pass, 64 rows apart (same k & 7;
                     // the chunk's rows are a multiple of 128)
@@ -906,14 +880,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
                     fence_proxy_async_smem();
                     tc_fence_before();
                     __syncthreads();
-                    ok = *flag;
                     // A: rows 64-127 (second bin half) one swizzle atom along M
                     // away, NBc / 2 bin rows of 128 bytes
                     const uint64_t a0 = sdesc_sw128(h_addr, (uint32_t)NBc * 64u, 1024u);
-                    if (issuer && ok && wide) {
+                    if (tid == 0) {
+                        int ok = 1;
                         // the consumer: MMAs of each stage as it lands
                         tc_fence_after();
-                        const uint32_t idw = idesc_f16(8 * ngw);
+                        const uint32_t idw = idesc_f16_mk(kRows, 8 * ngw, true);
                         for (int s = 0; s < S && ok; ++s) {
                             const int kb = s >> 1, bf = s & 3;
                             if (!mbar_wait_bounded(&wbar[bf], (wph >> bf) & 1u, p.status)) {
@@ -938,7 +912,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
                             }
                             mma_commit(&wbar[4 + bf]);
                         }
-                    } else if (wide && tid == 32 && ok) {
+                        *iss_ok = ok;
+                    } else if (tid == 32) {
                         // the producer: a stage's buffer takes the stage four later
                         // once its MMAs are done; then the last four stages' MMAs
                         int pok = 1;
@@ -952,47 +927,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
                             if (pok && s < S) wide_load(s);
                         }
                         *prod_ok = pok;
-                    } else if (issuer && ok) {
-                        tc_fence_after();
-                        const int nb0 = fg1 + 1 - fg0;
-                        const uint32_t idesc = idesc_f16(16 * nb0);
-                        const uint32_t dcol = tmem + (uint32_t)warp * (uint32_t)(16 * p.gb);
-                        const uint64_t b0 = sdesc_sw128(bt_addr, 16u, sbo_b);
-                        // descriptors advance by constant steps: A by 2 KB per K step,
-                        // B by 32 bytes inside a 128-byte row and 1 KB per 64-bin
-                        // block (the address field counts 16-byte units)
-                        for (int kk = warp; kk < NBc / 32; kk += n_iss) {
-                            const uint64_t ad = a0 + (uint64_t)(kk * 128);
-                            const uint64_t bd = b0 + (uint64_t)((kk >> 2) * 64 + (kk & 3) * 2);
-                            mma_f16(dcol, ad, bd, idesc, (kk >= n_iss) ? 1u : acc0);
-                        }
-                    }
-                    if (issuer) {
-                        int mine = ok;
-                        if (mine && !wide) {
-                            mma_commit(&bars[2 + warp]);
-                            mine = mbar_wait_bounded(&bars[2 + warp], ph_mma, p.status) ? 1 : 0;
-                            if (!mine) mbar_wait_bounded(&bars[2 + warp], ph_mma, p.status, 1u << 20);
-                            ph_mma ^= 1u;
-                        }
-                        iss_ok[warp] = mine;
                     }
                     // the non-integer counts are complete once the last pass's
                     // histogram is in: a partner whose count falls short of the
                     // atoms this warp handled needs its own histogram
                     const int bad = count && last &&
-                                    (zero_check ? (pt0 >= 0 || pt1 >= 0) && (f2_lo(zp) == 0.f || f2_hi(zp) == 0.f)
+                                    (zero_check ? (pt0 >= 0 || pt1 >= 0) && zmin == 0.f
                                                 : ((pt0 >= 0 && c0 != (uint32_t)handled) ||
                                                    (pt1 >= 0 && c1 != (uint32_t)handled)));
                     const int any_bad = __syncthreads_or(bad);
                     if (last) tile_bad = any_bad;
-                    {
-                        int all = wide ? *prod_ok : 1;
-                        for (int i = 0; i < n_iss; ++i) all &= iss_ok[i];
-                        if (!all) {
-                            failed = true;
-                            break;
-                        }
+                    if (!*prod_ok || !*iss_ok) {
+                        failed = true;
+                        break;
                     }
                     tc_fence_after();
                     if (!last) {
@@ -1004,14 +951,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
                 }
                 if (failed) break;
 
-                // ---- 4. epilogue: |X(k)| and the band maximum; the warps from zw0 on
-                // zero H for the next tile meanwhile.  With four partial
-                // accumulators and one frequency group (the common case), warps
-                // 0-7 each read two partials of one TMEM lane quadrant and warps
-                // 0, 1 combine the four contributions of their directions after a
-                // single exchange; otherwise warps 0-3 (one per quadrant) read
-                // every partial and exchange per frequency group ----
-                // warps 0, 1: pass 0 writes the slot's direction (and its partner
+                // ---- 4. epilogue: |X(k)| and the band maximum, warps 0-7; the others
+                // zero H for the next tile meanwhile ----
+                // pass 0 writes the slot's direction (and its partner
                 // when the tile's mirror images are exact); pass 1 the partners
                 auto write_out = [&](const float* best, const int* bk, int dir) {
                     const int slot = tile * kDirs + dir;
@@ -1040,79 +982,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
                         }
                     }
                 };
-                const bool quad = nbatch == 1 && p.n_iss == kIssuers && fg1 == fg0;
-                const int zw0 = (quad || (kWide && nbatch > 1)) ? 8 : 4;   // first zeroing warp
-                if (warp >= zw0) {
-                    for (int i = tid - zw0 * 32; i < NBc * 8; i += kThreads - zw0 * 32)
+                if (warp >= 8) {
+                    for (int i = tid - 256; i < NBc * 8; i += kThreads - 256)
                         reinterpret_cast<uint4*>(H)[i] = make_uint4(0, 0, 0, 0);
-                } else if (quad) {
-                    // warp w: partials 2 (w >> 2) and 2 (w >> 2) + 1 (hi and lo
-                    // columns) of lane quadrant w & 3; warps 2-7 leave their sums
-                    // in shared memory (EX: warps 2, 3; EX2: warps 4-7)
-                    const uint32_t cols_b = (uint32_t)(16 * p.gb);
-                    const uint32_t c0 = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(2 * (warp >> 2)) * cols_b;
-                    float a[8], b[8], c[8], d[8], x[8];
-                    tmem_ld8(c0, a);
-                    tmem_ld8(c0 + 8u, b);
-                    tmem_ld8(c0 + cols_b, c);
-                    tmem_ld8(c0 + cols_b + 8u, d);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) x[i] = (a[i] + b[i]) + (c[i] + d[i]);
-                    if (warp >= 2) {
-                        float4* xs = reinterpret_cast<float4*>((warp < 4 ? EX + (warp - 2) * 32 * 8 : EX2 + (warp - 4) * 32 * 8) +
-                                                               lane * 8);
-                        xs[0] = make_float4(x[0], x[1], x[2], x[3]);
-                        xs[1] = make_float4(x[4], x[5], x[6], x[7]);
-                    }
-                    asm volatile("bar.sync 2, 256;" ::: "memory");
-                    if (warp < 2) {
-                        // direction dir: rows dir (first bin half: this warp, partials
-                        // 0-1; warp 4 + warp, partials 2-3) and 64 + dir (second half:
-                        // warp 2 + warp, partials 0-1; warp 6 + warp, partials 2-3)
-                        const int dir = warp * 32 + lane;
-                        const float4* pl = reinterpret_cast<const float4*>(EX2 + (warp * 32 + lane) * 8);
-                        const float4* ph = reinterpret_cast<const float4*>(EX + (warp * 32 + lane) * 8);
-                        const float4* ph2 = reinterpret_cast<const float4*>(EX2 + ((2 + warp) * 32 + lane) * 8);
-                        const float4 l0 = pl[0], l1 = pl[1], h0 = ph[0], h1 = ph[1], g0 = ph2[0], g1 = ph2[1];
-                        const float lo[8] = {x[0] + l0.x, x[1] + l0.y, x[2] + l0.z, x[3] + l0.w,
-                                             x[4] + l1.x, x[5] + l1.y, x[6] + l1.z, x[7] + l1.w};
-                        const float hv[8] = {h0.x + g0.x, h0.y + g0.y, h0.z + g0.z, h0.w + g0.w,
-                                             h1.x + g1.x, h1.y + g1.y, h1.z + g1.z, h1.w + g1.w};
-                        float best[kNB];
-                        int bk[kNB];
-                        band_init_t<kNB>(p.bands, klo, best, bk);
-                        // the band maximum on |X|^2 (its root is the maximum
-                        // amplitude); the second half's factor w^(f h) is (-1)^f for
-                        // one chunk (a branch outside the frequency loop, so that the
-                        // loop carries no predicated sincos)
-                        const int f0 = p.kbase + 4 * fg0;
-                        if (nchunk == 1) {
-                            const float sg0 = (f0 & 1) ? -1.f : 1.f;
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const float sg = (q & 1) ? -sg0 : sg0;
-                                const float xr = lo[2 * q] + sg * hv[2 * q], xi = lo[2 * q + 1] + sg * hv[2 * q + 1];
-                                band_update_t<kNB>(p.bands, klo, khi, f0 + q, xr * xr + xi * xi, best, bk);
-                            }
-                        } else {
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const int f = f0 + q;
-                                float fs, fc;   // w^(f h) = fc - i fs, h = 512
-                                sincospif((float)f * (float)NBc / (float)NB, &fs, &fc);
-                                const float xr = lo[2 * q] + fc * hv[2 * q] - fs * hv[2 * q + 1];
-                                const float xi = lo[2 * q + 1] + fs * hv[2 * q] + fc * hv[2 * q + 1];
-                                band_update_t<kNB>(p.bands, klo, khi, f, xr * xr + xi * xi, best, bk);
-                            }
-                        }
-#pragma unroll
-                        for (int b = 0; b < kNB; ++b)
-                            if (best[b] >= 0.f) best[b] = sqrtf(best[b]) * 16777216.0f;
-                        write_out(best, bk, dir);
-                    }
-                } else if (kWide && nbatch > 1) {
-                    // Wide bands, warps 0-7: the 64 directions form two groups
+                } else {
+                    // the 64 directions form two groups
                     // (32 p .. 32 p + 31, p = warp & 1); a group's first-half rows are
                     // lane quadrant p (warps p, p + 4), its second-half rows quadrant
                     // 2 + p (warps p + 2, p + 6).  The 4-group column batches split
@@ -1243,68 +1117,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_tc(TcParams p) {
                         }
                         write_out(best, bk, dir);
                     }
-                } else {
-                    // warps 0, 1 hold rows 0-63 (the first half of the chunk's
-                    // bins), warps 2, 3 rows 64-127; per frequency group the
-                    // second-half warps hand their sums over through shared memory
-                    float best[kNB];
-                    int bk[kNB];
-                    band_init_t<kNB>(p.bands, klo, best, bk);
-                    const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
-                    const int n_iss = p.n_iss;
-                    const uint32_t cols_b = (uint32_t)(16 * p.gb);
-                    const int dir = (warp & 1) * 32 + lane;
-                    {
-                        const int g0 = fg0;
-                        const int nb = ng;
-                        for (int j = 0; j < nb; ++j) {
-                            float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f};
-                            for (int i = 0; i < n_iss; ++i) {
-                                const uint32_t dcol = lane_base + (uint32_t)i * cols_b;
-                                float hi[8], lo[8];
-                                tmem_ld8(dcol + (uint32_t)(8 * j), hi);
-                                tmem_ld8(dcol + (uint32_t)(8 * nb + 8 * j), lo);
-                                tmem_wait_ld();
-#pragma unroll
-                                for (int q = 0; q < 4; ++q) {
-                                    re[q] += hi[2 * q] + lo[2 * q];
-                                    im[q] += hi[2 * q + 1] + lo[2 * q + 1];
-                                }
-                            }
-                            if (warp >= 2) {
-#pragma unroll
-                                for (int q = 0; q < 4; ++q) {
-                                    EX[dir * 8 + 2 * q] = re[q];
-                                    EX[dir * 8 + 2 * q + 1] = im[q];
-                                }
-                            }
-                            asm volatile("bar.sync 1, 128;" ::: "memory");
-                            if (warp < 2) {
-#pragma unroll
-                                for (int q = 0; q < 4; ++q) {
-                                    const int f = p.kbase + 4 * (g0 + j) + q;
-                                    // re = sum h cos, im = sum h sin over a half;
-                                    // X = D_lo + w^(f h) D_hi with D = re - i im
-                                    const float hr = EX[dir * 8 + 2 * q], hs = EX[dir * 8 + 2 * q + 1];
-                                    float xr, xi;
-                                    if (nchunk == 1) {
-                                        const float sg = (f & 1) ? -1.f : 1.f;
-                                        xr = re[q] + sg * hr;
-                                        xi = im[q] + sg * hs;
-                                    } else {
-                                        float fs, fc;   // w^(f h) = fc - i fs, h = 512
-                                        sincospif((float)f * (float)NBc / (float)NB, &fs, &fc);
-                                        xr = re[q] + fc * hr - fs * hs;
-                                        xi = im[q] + fs * hr + fc * hs;
-                                    }
-                                    band_update_t<kNB>(p.bands, klo, khi, f, sqrtf(xr * xr + xi * xi) * 16777216.0f,
-                                                       best, bk);
-                                }
-                            }
-                            asm volatile("bar.sync 1, 128;" ::: "memory");
-                        }
-                    }
-                    if (warp < 2) write_out(best, bk, dir);
                 }
                 tc_fence_before();
                 // the next tile's directions have landed (this thread's copies;
@@ -1410,8 +1222,7 @@ int prepare_tc(Ctx* c) {
         const int g0 = (c->h_band[2 * r] - kbase) >> 2, g1 = (c->h_band[2 * r + 1] - kbase) >> 2;
         ng_roi_max = std::max(ng_roi_max, g1 - g0 + 1);
     }
-    // accumulators: kIssuers partials of 16 columns per group for bands that fit
-    // one B batch; wider bands stream their twiddles and accumulate 8 columns per
+    // wider bands stream their twiddles and accumulate 8 columns per
     // group in each of two blocks (bin quarters 0 and 2, 1 and 3), all groups in
     // one MMA of N = 8 x groups <= 256 per block
     const bool wide = ng_roi_max > gb;
@@ -1421,7 +1232,7 @@ int prepare_tc(Ctx* c) {
                          ng_roi_max);
     // (wide: two blocks of 8 x groups columns, the second from a multiple of 32)
     const int wcols = 8 * ((ng_roi_max + 1) & ~1);
-    const uint32_t need = (uint32_t)std::max(kIssuers * 16 * gb, wide ? ((wcols + 31) & ~31) + wcols : 0);
+    const uint32_t need = (uint32_t)(((wcols + 31) & ~31) + wcols);
     uint32_t cols = 32;
     while (cols < need) cols <<= 1;
     if (c->twb_key[0] != c->m || c->twb_key[1] != kbase || c->twb_key[2] != ng) {
@@ -1447,7 +1258,6 @@ int prepare_tc(Ctx* c) {
         c->twb_key[1] = kbase;
         c->twb_key[2] = ng;
     }
-    c->tc_gb = gb;
     c->tc_ng = ng;
     c->tc_tmem_cols = cols;
     c->tc_wide = wide;
@@ -1498,7 +1308,7 @@ cudaError_t launch_signatures_tc(Ctx* c, float* S, uint16_t* argk, uint16_t* his
     const bool multi = !hist_out && c->multi.n > 0;
     void (*kern)(TcParams);
     if (c->tc_wide)
-        kern = multi ? k_sig_tc<APTIDX_MAX_BANDS, true> : k_sig_tc<1, true>;
+        kern = multi ? k_sig_wide<APTIDX_MAX_BANDS> : k_sig_wide<1>;
     else if (c->m <= 10)
         kern = multi ? k_sig_tp<APTIDX_MAX_BANDS, 0> : k_sig_tp<1, 0>;
     else if (c->m == 11)
@@ -1531,7 +1341,6 @@ cudaError_t launch_signatures_tc(Ctx* c, float* S, uint16_t* argk, uint16_t* his
     p.twk = (const uint8_t*)c->d_twb + c->twb_bytes;
     p.bt_bytes = (int32_t)bt_bytes;
     p.ng_total = c->tc_ng;
-    p.gb = c->tc_gb;
     p.tmem_cols = c->tc_tmem_cols;
     p.S = S;
     p.argk = argk;

@@ -128,7 +128,8 @@ int aptidx_load_positions(aptidx_ctx* ctx, const float* xyz, int64_t n, const ui
 int aptidx_set_directions(aptidx_ctx* ctx, const float* u, int32_t nv, int mem);
 
 /* Histogram resolution 2^m bins (Eq. 1; APTIDX_MIN_M <= m <= APTIDX_MAX_M;
- * above 2^10 bins the kernels build each histogram in chunks of 1024 bins)
+ * above 2^10 bins the tensor cores take fewer directions at a time, the FP32
+ * path and wide bands chunks of 1024 bins)
  * and the default signature band of frequency bins [k_lo, k_hi]
  * (supplement, Al bicrystal: the largest amplitude over a fixed band of bins),
  * 0 <= k_lo <= k_hi <= 2^(m-1).  flags: reserved, 0. */

@@ -1328,7 +1328,7 @@ int64_t tm_round(const Reference& r, int64_t nroi, int copies) {
 // best orientation per ROI (device pointers), by lists where they pay
 int match_best(Ctx* c, Reference& r, const float* dS, int64_t nroi, int32_t* db, float* ds, int* launches) {
     cudaError_t e = cudaSuccess;
-    if (!tm_pays(c, &r, nroi)) {
+    if (!tm_pays(c, &r, nroi, 1)) {
         e = launch_match(c, &r, dS, nroi, db, ds);
         *launches += 1;
     } else {
@@ -1531,7 +1531,7 @@ int aptidx_match_topk(aptidx_ctx* ctx, int32_t cand, const float* S, int64_t nro
     int launches = 0;
     if (topk == 1) {
         if ((rc = match_best(c, r, dS, nroi, db, ds, &launches))) return rc;
-    } else if (tm_pays(c, &r, nroi) && tm_exact_smem(c, &r) + 18 * 1024 <= (size_t)max_optin) {
+    } else if (tm_pays(c, &r, nroi, topk) && tm_exact_smem(c, &r) + 18 * 1024 <= (size_t)max_optin) {
         const int64_t round = tm_round(r, nroi, 2);
         const size_t one = (size_t)round * r.ng;
         if ((rc = match_scratch(c, 2 * one * sizeof(float)))) return rc;

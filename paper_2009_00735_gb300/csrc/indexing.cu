@@ -1428,14 +1428,32 @@ cudaError_t launch_build_tm(Ctx* c, Reference* r) {
     return r->lut_bytes == 2 ? build_tm_t<uint16_t>(c, r) : build_tm_t<int32_t>(c, r);
 }
 
-// k_match takes a CTA per ROI, one row each: below some 4e5 look-ups per SM (30
-// us) its single launch is as fast as the four of the lists.
-bool tm_pays(const Ctx* c, const Reference* r, int64_t nroi) {
-    const double per_sm = (double)((nroi + c->sm_count - 1) / c->sm_count) * (double)r->ng * r->n_hat;
-    return r->d_tm_ent && per_sm > 4.0e5;
-}
-
 size_t tm_exact_smem(const Ctx* c, const Reference* r) { return ((size_t)c->nv + r->n_hat) * sizeof(float); }
+
+// Whether the lists are the faster way, by estimates of both (microseconds on 152 SMs,
+// within 15 % of the measured calls named here).
+// k_match (a CTA per ROI): a round of SMs takes 13.6e3 look-ups per microsecond and SM,
+// and 33 us to stage a row of 40962 values when one CTA fits (ROIs x orientations x
+// nodes, ico6 = 40962 directions: 4096 x 4000 x 100 1.73 ms, 1000 x 3000 x 400 0.91 ms,
+// 150 x 3000 x 400 0.10 ms).
+// Lists (per 64 ROIs): 90 us for the launches, 50 per million lists visited (a list adds
+// 64 sums to global memory) and 10 per million entries: 0.98, 0.41 and 0.15 ms.  With
+// few nodes per list they lose (topk of 1000 x 50000 x 50: 1.7 against 4.0 ms).
+// topk > 1: both rank the scores (4 per million); the lists also turn the estimates into
+// rows (24 more) and sum the best again (3.9 per million terms): 192 x 50000 x 1000,
+// best 1000: 6.9 against 3.0 ms; 500 x 50000 x 100, best 1000: 1.7 against 2.2.
+bool tm_pays(const Ctx* c, const Reference* r, int64_t nroi, int32_t topk) {
+    if (!r->d_tm_ent) return false;
+    const double sms = 152.0 / c->sm_count;
+    const double looks = (double)r->ng * r->n_hat, scores = topk > 1 ? (double)nroi * r->ng * 1e-6 * sms : 0.0;
+    const double groups = (double)((nroi + kTmRois - 1) / kTmRois);
+    const double rounds = (double)((nroi + c->sm_count - 1) / c->sm_count);
+    const double stage = 33.0 * c->nv / 40962.0 / (tm_exact_smem(c, r) > 113 * 1024 ? 1.0 : 2.0);
+    const double single = rounds * (looks / 13600.0 + stage) + 4.0 * scores;
+    const double lists = 90.0 + sms * 1e-6 * groups * (50.0 * r->tm_tiles * r->ng + 10.0 * looks) + 28.0 * scores +
+                         (topk > 1 ? 3.9e-6 * sms * nroi * topk * r->n_hat : 0.0);
+    return lists < 0.9 * single;
+}
 
 static TmMargin tm_margin(const Reference* r) {
     const double eta = sqrt((double)r->n_hat) * r->ref_max * (1.0 / 16384.0);

@@ -246,7 +246,7 @@ cudaError_t launch_match(Ctx* c, Reference* r, const float* S, int64_t nroi, int
                          float* scores_out = nullptr, bool accumulate = false, float weight = 1.0f);
 // Eq. 3 of many ROIs by lists (estimates, then exact sums where they decide)
 cudaError_t launch_build_tm(Ctx* c, Reference* r);
-bool tm_pays(const Ctx* c, const Reference* r, int64_t nroi);
+bool tm_pays(const Ctx* c, const Reference* r, int64_t nroi, int32_t topk);
 size_t tm_exact_smem(const Ctx* c, const Reference* r);
 cudaError_t launch_tm_sum(Ctx* c, Reference* r, const float* S, int64_t nroi, float* D);
 cudaError_t launch_tm_best(Ctx* c, Reference* r, const float* S, int64_t nroi, const float* D, int32_t* best,

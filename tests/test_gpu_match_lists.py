@@ -32,7 +32,10 @@ def rows(u, sig, n, seed):
 
 
 @pytest.mark.parametrize("nv,ng,n_hat,nroi", [(2562, 1001, 299, 170), (1752, 777, 33, 3000), (1753, 2500, 130, 161),
-                                              (10242, 3301, 101, 193), (40962, 999, 301, 160)])
+                                              (10242, 3301, 101, 193), (40962, 999, 301, 160),
+                                              # large enough that the lists serve match and the shorter topk
+                                              (2562, 2501, 299, 3000), (1753, 2500, 330, 2900),
+                                              (10242, 3301, 401, 1500), (40962, 3301, 501, 700)])
 def test_lists_equal_single(torch_cuda, nv, ng, n_hat, nroi):
     torch = torch_cuda
     u = spiral(nv)

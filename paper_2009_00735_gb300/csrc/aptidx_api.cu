@@ -1333,14 +1333,14 @@ int match_best(Ctx* c, Reference& r, const float* dS, int64_t nroi, int32_t* db,
         *launches += 1;
     } else {
         const int64_t round = tm_round(r, nroi, 1);
-        int rc = match_scratch(c, (size_t)round * r.ng * sizeof(float));
+        int rc = match_scratch(c, ((size_t)round * r.ng + round + 1) * sizeof(float));
         if (rc) return rc;
         for (int64_t r0 = 0; r0 < nroi && e == cudaSuccess; r0 += round) {
             const int64_t n = std::min(round, nroi - r0);
             e = launch_tm_sum(c, &r, dS + r0 * c->nv, n, c->d_match_scratch);
             if (e == cudaSuccess)
                 e = launch_tm_best(c, &r, dS + r0 * c->nv, n, c->d_match_scratch, db + r0, ds ? ds + r0 : nullptr);
-            *launches += 2;
+            *launches += 3;
         }
     }
     return e == cudaSuccess ? APTIDX_OK : cuda_check(c, e, "match");

@@ -373,14 +373,40 @@ __device__ __forceinline__ void lut_accumulate(const uint4 w, const float* row, 
     }
 }
 
+// The signature row into shared memory (all threads, closing barrier); whether all
+// its values are equal.
+__device__ __forceinline__ bool stage_row(float* row, const float* __restrict__ src, int32_t nv) {
+    const float first = src[0];
+    bool flat = true;
+    for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+        const float v = src[i];
+        row[i] = v;
+        flat &= v == first;
+    }
+    return __syncthreads_and(flat) != 0;
+}
+
+// Delta of every orientation for a row of the value v, in k order
+__device__ __forceinline__ float flat_score(float v, const float* ref, int32_t n_hat) {
+    float acc = 0.f;
+    for (int k = 0; k < n_hat; ++k) {
+        const float d = v - ref[k];
+        acc = fmaf(d, d, acc);
+    }
+    return acc;
+}
+
 // With scores_out, weight x Delta(g) of ROI r also goes to scores_out[r * ng
 // + g] (accumulate: added to the value there, for sums over signature
-// channels).
-template <typename IdxT>
+// channels).  kListed: the ROIs list[1 .. list[0]] instead of all nroi; a row of
+// one value (a ROI without atoms, or with one), whose orientations all tie, takes
+// one sum.
+template <typename IdxT, bool kListed = false>
 __global__ void __launch_bounds__(1024, 1) k_match(const float* __restrict__ S, int64_t nroi, int32_t nv,
                                                 const IdxT* __restrict__ lut_t, int64_t ng, int64_t ng_pad,
                                                 const float* __restrict__ top_val, int32_t n_hat, int32_t* best,
-                                                float* score, float* scores_out, bool accumulate, float weight) {
+                                                float* score, float* scores_out, bool accumulate, float weight,
+                                                const uint32_t* __restrict__ list) {
     constexpr int G = 16 / (int)sizeof(IdxT);
     extern __shared__ float sm[];
     float* row = sm;                     // nv
@@ -388,12 +414,26 @@ __global__ void __launch_bounds__(1024, 1) k_match(const float* __restrict__ S, 
     __shared__ float red_v[32];
     __shared__ int32_t red_g[32];
     const int nwarps = blockDim.x >> 5;
+    const int64_t n = kListed ? (int64_t)list[0] : nroi;
+    if (kListed && blockIdx.x >= n) return;
     for (int i = threadIdx.x; i < n_hat; i += blockDim.x) ref[i] = top_val[i];
-    for (int64_t r = blockIdx.x; r < nroi; r += gridDim.x) {
+    for (int64_t item = blockIdx.x; item < n; item += gridDim.x) {
+        const int64_t r = kListed ? (int64_t)list[1 + item] : item;
         __syncthreads();
         const float* src = S + r * (int64_t)nv;
-        for (int i = threadIdx.x; i < nv; i += blockDim.x) row[i] = src[i];
-        __syncthreads();
+        if (kListed) {
+            if (stage_row(row, src, nv)) {
+                if (threadIdx.x == 0) {
+                    const float v = flat_score(row[0], ref, n_hat);
+                    if (best) best[r] = v < INFINITY ? 0 : 0x7FFFFFFF;
+                    if (score) score[r] = v < INFINITY ? v : INFINITY;
+                }
+                continue;
+            }
+        } else {
+            for (int i = threadIdx.x; i < nv; i += blockDim.x) row[i] = src[i];
+            __syncthreads();
+        }
         float bv = INFINITY;
         int32_t bg = 0x7FFFFFFF;
         for (int64_t g0 = (int64_t)threadIdx.x * G; g0 < ng; g0 += (int64_t)blockDim.x * G) {
@@ -609,19 +649,26 @@ __device__ __forceinline__ float tm_threshold(float estimate, TmMargin m) {
 
 // The best orientation of 32 ROIs (half a group per CTA, lane = ROI): the smallest
 // estimate, then the sums in k order of every orientation near it, a warp per
-// (ROI, orientation): the lanes read 32 terms, which are added in turn.
+// (ROI, orientation): the lanes read 32 terms, which are added in turn.  A ROI with
+// more than kTmNear orientations near its best (a row of one or few values) is left
+// to k_match, which sums all of a ROI's orientations in the time this form takes for
+// some 60: heavy[1 ..] lists such ROIs, heavy[0] (zero before) counts them.  Summed
+// here, 200 rows of zeros among 4096 (3419 orientations, 1000 nodes) took 90 ms; now
+// 3.0, as any other rows (2.9).
+constexpr int kTmNear = 64;
+
 template <typename IdxT>
 __global__ void __launch_bounds__(kTmThreads, 1) k_tm_best(const float* __restrict__ S, int64_t nroi, int32_t nv,
                                                         const IdxT* __restrict__ lut_g, int64_t ng, int pitch,
                                                         const float* __restrict__ top_val, int32_t n_hat,
                                                         TmMargin margin, const float* __restrict__ D, int32_t* best,
-                                                        float* score) {
+                                                        float* score, uint32_t* heavy) {
     __shared__ float red[32][33];
     __shared__ float thr[32];
     __shared__ unsigned long long key[32];
-    __shared__ uint32_t list_g[kTmThreads];
-    __shared__ uint8_t list_r[kTmThreads];
-    __shared__ uint32_t n_list;
+    __shared__ uint32_t near_g[32][kTmNear];
+    __shared__ uint32_t n_near[32];    // orientations near the best, then their inclusive sums
+    __shared__ uint32_t s_heavy;       // lanes left to k_match
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t roi0 = (int64_t)(blockIdx.x >> 1) * kTmRois + (blockIdx.x & 1);   // ROI of lane l: roi0 + 2 l
     const float* d = D + (int64_t)(blockIdx.x >> 1) * ng * kTmRois + (blockIdx.x & 1) * 32 + lane;
@@ -629,8 +676,10 @@ __global__ void __launch_bounds__(kTmThreads, 1) k_tm_best(const float* __restri
 #pragma unroll 4
     for (int64_t g = warp; g < ng; g += 32) m = fminf(m, d[g * kTmRois]);
     red[warp][lane] = m;
-    if (warp == 0) key[lane] = 0x7F8000007FFFFFFFull;   // (+inf, no orientation)
-    if (threadIdx.x == 0) n_list = 0;
+    if (warp == 0) {
+        key[lane] = 0x7F8000007FFFFFFFull;   // (+inf, no orientation)
+        n_near[lane] = 0;
+    }
     __syncthreads();
     if (warp == 0) {
         for (int w = 1; w < 32; ++w) m = fminf(m, red[w][lane]);
@@ -639,65 +688,58 @@ __global__ void __launch_bounds__(kTmThreads, 1) k_tm_best(const float* __restri
     __syncthreads();
     const float t = thr[lane];
     const bool valid = roi0 + 2 * lane < nroi;
-    // sums in k order of the first n listed (ROI, orientation) pairs
-    auto decide = [&](uint32_t n) {
-        for (uint32_t i = warp; i < n; i += 32) {
-            const int r = list_r[i];
-            const int64_t cg = list_g[i];
-            const float* row = S + (roi0 + 2 * r) * nv;
-            float acc = 0.f;
-            auto load = [&](int k) { return k < n_hat ? row[(int)lut_g[cg * pitch + k]] - top_val[k] : 0.f; };
-            float v = load(lane);
-            for (int k0 = 0; k0 < n_hat; k0 += 32) {
-                const float next = load(k0 + 32 + lane);
-                const int kn = min(32, n_hat - k0);
-                if (kn == 32) {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const float x = __shfl_sync(0xffffffffu, v, j);
-                        acc = fmaf(x, x, acc);
-                    }
-                } else {
-                    for (int j = 0; j < kn; ++j) {
-                        const float x = __shfl_sync(0xffffffffu, v, j);
-                        acc = fmaf(x, x, acc);
-                    }
-                }
-                v = next;
-            }
-            if (lane == 0 && acc < INFINITY)
-                atomicMin(&key[r], ((unsigned long long)__float_as_uint(acc) << 32) | (uint32_t)cg);
-        }
-    };
-    auto list = [&](int64_t g) {
-        if (valid && g < ng && d[g * kTmRois] <= t) {
-            const uint32_t i = atomicAdd(&n_list, 1u);
-            if (i < kTmThreads) {
-                list_g[i] = (uint32_t)g;
-                list_r[i] = (uint8_t)lane;
-            }
-        }
-    };
+    volatile uint32_t* seen = n_near;
 #pragma unroll 4
-    for (int64_t g = warp; g < ng; g += 32) list(g);
-    __syncthreads();
-    const uint32_t n_all = n_list;
-    if (n_all <= kTmThreads) {
-        decide(n_all);
-        __syncthreads();
-    } else {
-        // many ties (flat signatures): in steps that cannot overrun the list
-        for (int64_t g0 = 0; g0 < ng; g0 += 32) {
-            __syncthreads();
-            if (threadIdx.x == 0) n_list = 0;
-            __syncthreads();
-            list(g0 + warp);
-            __syncthreads();
-            decide(n_list);
+    for (int64_t g = warp; g < ng; g += 32)
+        if (valid && d[g * kTmRois] <= t && seen[lane] <= kTmNear) {
+            const uint32_t i = atomicAdd(&n_near[lane], 1u);
+            if (i < kTmNear) near_g[lane][i] = (uint32_t)g;
         }
-        __syncthreads();
+    __syncthreads();
+    if (warp == 0) {
+        const bool many = n_near[lane] > kTmNear;
+        const uint32_t bal = __ballot_sync(0xffffffffu, many);
+        if (many) heavy[1 + atomicAdd(heavy, 1u)] = (uint32_t)(roi0 + 2 * lane);
+        if (lane == 0) s_heavy = bal;
+        uint32_t x = many ? 0 : n_near[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        n_near[lane] = x;
     }
-    if (warp == 0 && valid) {
+    __syncthreads();
+    const uint32_t upto = n_near[lane], total = n_near[31];
+    for (uint32_t i = warp; i < total; i += 32) {
+        // pair i: ROI r, the first whose inclusive sum exceeds i
+        const int r = __popc(__ballot_sync(0xffffffffu, upto <= i));
+        const int64_t cg = near_g[r][i - (r ? n_near[r - 1] : 0u)];
+        const float* row = S + (roi0 + 2 * r) * nv;
+        float acc = 0.f;
+        auto load = [&](int k) { return k < n_hat ? row[(int)lut_g[cg * pitch + k]] - top_val[k] : 0.f; };
+        float v = load(lane);
+        for (int k0 = 0; k0 < n_hat; k0 += 32) {
+            const float next = load(k0 + 32 + lane);
+            const int kn = min(32, n_hat - k0);
+            if (kn == 32) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const float x = __shfl_sync(0xffffffffu, v, j);
+                    acc = fmaf(x, x, acc);
+                }
+            } else {
+                for (int j = 0; j < kn; ++j) {
+                    const float x = __shfl_sync(0xffffffffu, v, j);
+                    acc = fmaf(x, x, acc);
+                }
+            }
+            v = next;
+        }
+        if (lane == 0 && acc < INFINITY)
+            atomicMin(&key[r], ((unsigned long long)__float_as_uint(acc) << 32) | (uint32_t)cg);
+    }
+    __syncthreads();
+    if (warp == 0 && valid && !((s_heavy >> lane) & 1u)) {
         const int64_t r = roi0 + 2 * lane;
         const unsigned long long v = key[lane];
         if (best) best[r] = (int32_t)(uint32_t)v;
@@ -778,6 +820,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) k_tm_exact(const float* __restr
     float* ref = sm + nv;        // n_hat
     __shared__ uint32_t list[kTmList];
     __shared__ uint32_t n_list;
+    __shared__ float s_flat;
     const int tid = threadIdx.x;
     for (int i = tid; i < n_hat; i += kTmThreads) ref[i] = top_val[i];
     if (tid == 0) n_list = 0;
@@ -785,11 +828,17 @@ __global__ void __launch_bounds__(kTmThreads, 1) k_tm_exact(const float* __restr
     for (int64_t it = blockIdx.x; it < nroi * parts; it += gridDim.x) {
         const int64_t r = it / parts, ga = (it % parts) * per, gb = tmin<int64_t>(ng, ga + per);
         __syncthreads();
-        for (int i = tid; i < nv; i += kTmThreads) row[i] = S[r * (int64_t)nv + i];
+        const bool flat = stage_row(row, S + r * (int64_t)nv, nv);
         float* sc = scores + r * ng;
         const float t = reach[r];
         const bool all = isnan(t);
-        __syncthreads();
+        if (flat) {   // every orientation has the same sum
+            if (tid == 0) s_flat = flat_score(row[0], ref, n_hat);
+            __syncthreads();
+            for (int64_t g = ga + tid; g < gb; g += kTmThreads)
+                if (all || sc[g] <= t) sc[g] = s_flat;
+            continue;
+        }
         for (int64_t g0 = ga; g0 < gb; g0 += kTmThreads) {
             const int64_t g = g0 + tid;
             if (g < gb && (all || sc[g] <= t)) list[atomicAdd(&n_list, 1u)] = (uint32_t)g;
@@ -1347,28 +1396,30 @@ cudaError_t launch_build_lut(Ctx* c, Reference* r, const double* d_quats, int64_
 
 template <typename IdxT>
 static cudaError_t launch_match_t(Ctx* c, Reference* r, const float* S, int64_t nroi, int32_t* best, float* score,
-                                  float* scores_out, bool accumulate, float weight) {
+                                  float* scores_out, bool accumulate, float weight, const uint32_t* list) {
     constexpr int G = 16 / (int)sizeof(IdxT);
     const size_t smem = ((size_t)c->nv + r->n_hat) * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(k_match<IdxT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const auto kern = list ? k_match<IdxT, true> : k_match<IdxT, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // one thread per G orientations, whole warps, at most 1024 threads
     const int64_t want = (r->ng + G - 1) / G;
     const int threads = (int)std::min<int64_t>(1024, std::max<int64_t>(32, (want + 31) / 32 * 32));
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_match<IdxT>, threads, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
     per_sm = std::max(per_sm, 1);
     const int64_t grid = std::min<int64_t>((int64_t)c->sm_count * per_sm, nroi);
-    k_match<IdxT><<<(unsigned)grid, threads, smem, c->stream>>>(S, nroi, c->nv, static_cast<const IdxT*>(r->d_lut),
-                                                                r->ng, r->ng_pad, r->d_top_val, r->n_hat, best, score,
-                                                                scores_out, accumulate, weight);
+    kern<<<(unsigned)grid, threads, smem, c->stream>>>(S, nroi, c->nv, static_cast<const IdxT*>(r->d_lut), r->ng, r->ng_pad,
+                                                       r->d_top_val, r->n_hat, best, score, scores_out, accumulate,
+                                                       weight, list);
     return cudaGetLastError();
 }
 
 cudaError_t launch_match(Ctx* c, Reference* r, const float* S, int64_t nroi, int32_t* best, float* score,
-                         float* scores_out, bool accumulate, float weight) {
-    return r->lut_bytes == 2 ? launch_match_t<uint16_t>(c, r, S, nroi, best, score, scores_out, accumulate, weight)
-                             : launch_match_t<int32_t>(c, r, S, nroi, best, score, scores_out, accumulate, weight);
+                         float* scores_out, bool accumulate, float weight, const uint32_t* list) {
+    return r->lut_bytes == 2
+               ? launch_match_t<uint16_t>(c, r, S, nroi, best, score, scores_out, accumulate, weight, list)
+               : launch_match_t<int32_t>(c, r, S, nroi, best, score, scores_out, accumulate, weight, list);
 }
 
 // The lists of k_tm_sum for the table just built (skipped when they would not
@@ -1460,10 +1511,10 @@ static TmMargin tm_margin(const Reference* r) {
     return {(float)(2.0 * eta * 1.001), (float)(1.0 + 5.0 * (r->n_hat + 64) / 16777216.0)};
 }
 
-// estimates of `nroi` ROIs into D [groups][ng][64]
+// estimates of `nroi` ROIs into D [groups][ng][64], and zero into the word after them
 cudaError_t launch_tm_sum(Ctx* c, Reference* r, const float* S, int64_t nroi, float* D) {
     const int64_t groups = (nroi + kTmRois - 1) / kTmRois;
-    cudaError_t e = cudaMemsetAsync(D, 0, (size_t)(groups * r->ng * kTmRois) * sizeof(float), c->stream);
+    cudaError_t e = cudaMemsetAsync(D, 0, (size_t)(groups * r->ng * kTmRois + 1) * sizeof(float), c->stream);
     if (e != cudaSuccess) return e;
     const size_t smem = (size_t)(r->tm_nodes + 1) * kTmPitch * sizeof(float);
     if ((e = cudaFuncSetAttribute(k_tm_sum, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
@@ -1481,18 +1532,21 @@ cudaError_t launch_tm_sum(Ctx* c, Reference* r, const float* S, int64_t nroi, fl
     return cudaGetLastError();
 }
 
-cudaError_t launch_tm_best(Ctx* c, Reference* r, const float* S, int64_t nroi, const float* D, int32_t* best,
-                           float* score) {
-    const unsigned groups = 2 * (unsigned)((nroi + kTmRois - 1) / kTmRois);   // halves
-    if (r->lut_bytes == 2)
-        k_tm_best<uint16_t><<<groups, kTmThreads, 0, c->stream>>>(S, nroi, c->nv, static_cast<const uint16_t*>(r->d_lut_g),
-                                                                  r->ng, r->lut_g_pitch, r->d_top_val, r->n_hat, tm_margin(r), D, best,
-                                                                  score);
-    else
-        k_tm_best<int32_t><<<groups, kTmThreads, 0, c->stream>>>(S, nroi, c->nv, static_cast<const int32_t*>(r->d_lut_g),
-                                                                 r->ng, r->lut_g_pitch, r->d_top_val, r->n_hat, tm_margin(r), D, best,
-                                                                 score);
-    return cudaGetLastError();
+// the best of every ROI from the estimates D, which the counter of heavy ROIs follows
+template <typename IdxT>
+static cudaError_t tm_best_t(Ctx* c, Reference* r, const float* S, int64_t nroi, float* D, int32_t* best, float* score) {
+    const int64_t groups = (nroi + kTmRois - 1) / kTmRois;
+    uint32_t* heavy = reinterpret_cast<uint32_t*>(D + groups * r->ng * kTmRois);
+    k_tm_best<IdxT><<<(unsigned)(2 * groups), kTmThreads, 0, c->stream>>>(
+        S, nroi, c->nv, static_cast<const IdxT*>(r->d_lut_g), r->ng, r->lut_g_pitch, r->d_top_val, r->n_hat, tm_margin(r),
+        D, best, score, heavy);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? launch_match(c, r, S, nroi, best, score, nullptr, false, 1.0f, heavy) : e;
+}
+
+cudaError_t launch_tm_best(Ctx* c, Reference* r, const float* S, int64_t nroi, float* D, int32_t* best, float* score) {
+    return r->lut_bytes == 2 ? tm_best_t<uint16_t>(c, r, S, nroi, D, best, score)
+                             : tm_best_t<int32_t>(c, r, S, nroi, D, best, score);
 }
 
 // rows [nroi][ng] from the estimates, exact where the topk are decided; D's

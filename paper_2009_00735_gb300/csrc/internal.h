@@ -243,14 +243,15 @@ size_t plain_smem_bytes(int m, int atom_cap);
 cudaError_t launch_top_nodes(Ctx* c, Reference* r);
 cudaError_t launch_build_lut(Ctx* c, Reference* r, const double* d_quats, int64_t ng);
 cudaError_t launch_match(Ctx* c, Reference* r, const float* S, int64_t nroi, int32_t* best, float* score,
-                         float* scores_out = nullptr, bool accumulate = false, float weight = 1.0f);
+                         float* scores_out = nullptr, bool accumulate = false, float weight = 1.0f,
+                         const uint32_t* list = nullptr);   // list: (count, ROIs) on the device instead of all
 // Eq. 3 of many ROIs by lists (estimates, then exact sums where they decide)
 cudaError_t launch_build_tm(Ctx* c, Reference* r);
 bool tm_pays(const Ctx* c, const Reference* r, int64_t nroi, int32_t topk);
 size_t tm_exact_smem(const Ctx* c, const Reference* r);
 cudaError_t launch_tm_sum(Ctx* c, Reference* r, const float* S, int64_t nroi, float* D);
-cudaError_t launch_tm_best(Ctx* c, Reference* r, const float* S, int64_t nroi, const float* D, int32_t* best,
-                           float* score);
+// (D as launch_tm_sum left it, with 1 + nroi words more behind the groups' estimates)
+cudaError_t launch_tm_best(Ctx* c, Reference* r, const float* S, int64_t nroi, float* D, int32_t* best, float* score);
 cudaError_t launch_tm_rows(Ctx* c, Reference* r, const float* S, int64_t nroi, int32_t topk, float* D, float* rows);
 cudaError_t launch_phase(Ctx* c, float* score, const int32_t* n_ch, int32_t n_cand, int64_t nroi, int32_t* phase);
 cudaError_t launch_topk(Ctx* c, const float* scores, int64_t ng, int64_t nroi, int32_t topk, int32_t* best,

@@ -1481,29 +1481,39 @@ cudaError_t launch_build_tm(Ctx* c, Reference* r) {
 
 size_t tm_exact_smem(const Ctx* c, const Reference* r) { return ((size_t)c->nv + r->n_hat) * sizeof(float); }
 
-// Whether the lists are the faster way, by estimates of both (microseconds on 152 SMs,
-// within 15 % of the measured calls named here).
-// k_match (a CTA per ROI): a round of SMs takes 13.6e3 look-ups per microsecond and SM,
-// and 33 us to stage a row of 40962 values when one CTA fits (ROIs x orientations x
-// nodes, ico6 = 40962 directions: 4096 x 4000 x 100 1.73 ms, 1000 x 3000 x 400 0.91 ms,
-// 150 x 3000 x 400 0.10 ms).
-// Lists (per 64 ROIs): 90 us for the launches, 50 per million lists visited (a list adds
-// 64 sums to global memory) and 10 per million entries: 0.98, 0.41 and 0.15 ms.  With
-// few nodes per list they lose (topk of 1000 x 50000 x 50: 1.7 against 4.0 ms).
-// topk > 1: both rank the scores (4 per million); the lists also turn the estimates into
-// rows (24 more) and sum the best again (3.9 per million terms): 192 x 50000 x 1000,
-// best 1000: 6.9 against 3.0 ms; 500 x 50000 x 100, best 1000: 1.7 against 2.2.
+// Whether the lists are the faster way: estimates of both in microseconds on 152 SMs,
+// fitted to 636 calls timed both ways (2562 and 40962 directions, 500 to 100000
+// orientations, 50 to 1000 nodes, 1 to 4096 ROIs, the best 1, 10 and 500; the median
+// estimate is right, nine in ten are within 20 %).
+// k_match: look-ups per SM (60 per million), staging (by few threads when there are
+// few orientations), a chain of reads as long as the node list, and for topk > 1 the
+// selection, by SM and by the longest row.
+// Lists: 68 per million lists visited (each adds 64 sums to global memory), 1.5 per
+// million entries and 64 ROIs, the longest warp's entries, k_tm_best's walk over the
+// orientations by two CTAs per 64 ROIs, or the rows, selections and exact sums of
+// topk > 1.  (Without the last three the lists served 64 ROIs x 50000 orientations x
+// 100 nodes in 0.63 ms, which k_match does in 0.36.)
 bool tm_pays(const Ctx* c, const Reference* r, int64_t nroi, int32_t topk) {
     if (!r->d_tm_ent) return false;
-    const double sms = 152.0 / c->sm_count;
-    const double looks = (double)r->ng * r->n_hat, scores = topk > 1 ? (double)nroi * r->ng * 1e-6 * sms : 0.0;
-    const double groups = (double)((nroi + kTmRois - 1) / kTmRois);
-    const double rounds = (double)((nroi + c->sm_count - 1) / c->sm_count);
-    const double stage = 33.0 * c->nv / 40962.0 / (tm_exact_smem(c, r) > 113 * 1024 ? 1.0 : 2.0);
-    const double single = rounds * (looks / 13600.0 + stage) + 4.0 * scores;
-    const double lists = 90.0 + sms * 1e-6 * groups * (50.0 * r->tm_tiles * r->ng + 10.0 * looks) + 28.0 * scores +
-                         (topk > 1 ? 3.9e-6 * sms * nroi * topk * r->n_hat : 0.0);
-    return lists < 0.9 * single;
+    const auto up = [](double a, double b) { return ceil(a / b); };
+    const double sms = c->sm_count, per = 152.0 / sms, n = (double)nroi, ng = (double)r->ng, nh = r->n_hat, nv = c->nv;
+    const double looks = ng * nh * 1e-6, cells = n * ng * 1e-6 * per;
+    const double threads = std::min(1024.0, 32.0 * up(up(ng, 8), 32));
+    const double fit = std::min(floor(1024 / threads), floor(232448 / (tm_exact_smem(c, r) + 1024.0)));   // CTAs per SM
+    const double ctas = std::max(1.0, std::min(16.0, fit));
+    const double rounds = up(n, sms), waves = up(n, sms * ctas), rows = up(n, 8 * sms);
+    double single = 15 + rounds * (60 * looks + 1.7e-4 * nv) + waves * (0.2 * nv / threads + 0.038 * nh * up(up(ng, 8), threads));
+    const double groups = up(n, kTmRois), tiles = r->tm_tiles;
+    const double gsplit = std::max(1.0, std::min(up(4 * sms, tiles * groups), floor(ng / 256)));
+    const double longest = up(tiles * groups * gsplit, sms) * up(ng, gsplit * (kTmThreads / 32)) * nh / tiles;
+    double lists = 37 + per * groups * (68e-6 * tiles * ng + 1.5 * looks) + 0.047 * longest;
+    if (topk == 1) {
+        lists += up(2 * groups, sms) * (8e-3 * ng + 0.024 * nh) + 1.7 * cells;
+    } else {
+        single += 17 + 5 * cells + rows * (1.8e-3 * ng + 0.02 * topk) + 0.026 * n * per;
+        lists += 46 + 11.7 * cells + rows * (3.6e-3 * ng + 0.018 * topk) + (0.066 + 0.8e-6 * topk * nh) * n * per;
+    }
+    return lists < 0.85 * single;
 }
 
 static TmMargin tm_margin(const Reference* r) {

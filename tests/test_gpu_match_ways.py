@@ -114,6 +114,28 @@ def test_flat_and_near_flat_rows(torch_cuda, nv, ng, n_hat, nroi, topk, match_l,
     ctx.close()
 
 
+@pytest.mark.parametrize("nv,ng,n_hat,nroi,launches", [
+    (2562, 30000, 50, 16, 1), (40962, 50000, 100, 64, 1), (40962, 3419, 200, 64, 1), (2562, 100000, 50, 256, 1),
+    (40962, 3419, 1000, 64, 3), (40962, 999, 200, 300, 3)])
+def test_way_of_few_rois(torch_cuda, nv, ng, n_hat, nroi, launches):
+    """Few ROIs against many orientations with short node lists are faster one CTA per
+    ROI, long node lists and few orientations by lists (timed both ways)."""
+    torch = torch_cuda
+    u, sig = reference(nv)
+    ctx = open_context(u, sig, ng, n_hat)
+    h = ctx.handle
+    S = torch.from_numpy(rows(u, sig, nroi, ng)).cuda()
+    best = torch.full((nroi,), -9, dtype=torch.int32, device="cuda")
+    score = torch.full((nroi,), -9.0, device="cuda")
+    assert launched(h, lambda: apt.aptidx_match(h, 0, S, best, score)) == launches
+    lut = torch.from_numpy(apt.aptidx_get_lut(h, 0, ng=ng).astype(np.int64)).cuda()
+    ref = torch.from_numpy(sig[oracle.top_nodes(sig, n_hat)]).cuda()
+    none = np.empty((nroi, 0), np.int32)
+    check(torch, S, lut, ref, [0, 1, 4, 9, nroi - 1], best.cpu().numpy(), score.cpu().numpy(), none,
+          none.astype(np.float32))
+    ctx.close()
+
+
 def test_flat_rows_take_no_longer(torch_cuda):
     """ROIs without atoms do not slow a call down: at most twice the time of the same
     call on bright rows (summed orientation by orientation they took 14 times as long)."""

@@ -1318,23 +1318,28 @@ int match_scratch(Ctx* c, size_t need) {
     return rc;
 }
 
-// ROIs per round when their estimates (and, `copies` = 2, their score rows) stay
-// within 1 GiB: whole groups of 64
-int64_t tm_round(const Reference& r, int64_t nroi, int copies) {
-    const int64_t groups = std::max<int64_t>(1, ((int64_t)1 << 30) / (r.ng * 256 * copies));
-    return std::min<int64_t>((nroi + 63) / 64, groups) * 64;
+// ROIs of a round of the lists when the scratch holds them, 0 when the call goes to
+// k_match: where that is faster, where there is no memory for the scratch, and on a
+// stream being captured (a graph must not hold scratch that a later call replaces)
+int64_t tm_round(Ctx* c, const Reference& r, int64_t nroi, int32_t topk) {
+    if (!tm_pays(c, &r, nroi, topk)) return 0;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (cap != cudaStreamCaptureStatusNone) return 0;
+    const int64_t round = std::min<int64_t>((nroi + 63) / 64, tm_groups(&r, topk)) * 64;
+    const std::string err = c->err;
+    if (match_scratch(c, ((size_t)round * (r.ng + 1) * (topk > 1 ? 2 : 1) + 1) * sizeof(float)) == APTIDX_OK) return round;
+    c->err = err;
+    return 0;
 }
 
 // best orientation per ROI (device pointers), by lists where they pay
 int match_best(Ctx* c, Reference& r, const float* dS, int64_t nroi, int32_t* db, float* ds, int* launches) {
     cudaError_t e = cudaSuccess;
-    if (!tm_pays(c, &r, nroi, 1)) {
-        e = launch_match(c, &r, dS, nroi, db, ds);
-        *launches += 1;
-    } else {
-        const int64_t round = tm_round(r, nroi, 1);
-        int rc = match_scratch(c, ((size_t)round * r.ng + round + 1) * sizeof(float));
-        if (rc) return rc;
+    if (const int64_t round = tm_round(c, r, nroi, 1)) {
         for (int64_t r0 = 0; r0 < nroi && e == cudaSuccess; r0 += round) {
             const int64_t n = std::min(round, nroi - r0);
             e = launch_tm_sum(c, &r, dS + r0 * c->nv, n, c->d_match_scratch);
@@ -1342,6 +1347,9 @@ int match_best(Ctx* c, Reference& r, const float* dS, int64_t nroi, int32_t* db,
                 e = launch_tm_best(c, &r, dS + r0 * c->nv, n, c->d_match_scratch, db + r0, ds ? ds + r0 : nullptr);
             *launches += 3;
         }
+    } else {
+        e = launch_match(c, &r, dS, nroi, db, ds);
+        *launches += 1;
     }
     return e == cudaSuccess ? APTIDX_OK : cuda_check(c, e, "match");
 }
@@ -1529,15 +1537,13 @@ int aptidx_match_topk(aptidx_ctx* ctx, int32_t cand, const float* S, int64_t nro
     if ((rc = dev_out(c, score, nout, mem, ts, &ds))) return rc;
     prof_begin(c, APTIDX_PHASE_MATCH);
     int launches = 0;
+    int64_t round = 0;
     if (topk == 1) {
         if ((rc = match_best(c, r, dS, nroi, db, ds, &launches))) return rc;
-    } else if (tm_pays(c, &r, nroi, topk) && tm_exact_smem(c, &r) + 18 * 1024 <= (size_t)max_optin) {
-        const int64_t round = tm_round(r, nroi, 2);
-        const size_t one = (size_t)round * r.ng;
-        if ((rc = match_scratch(c, 2 * one * sizeof(float)))) return rc;
+    } else if (tm_exact_smem(c, &r) + 18 * 1024 <= (size_t)max_optin && (round = tm_round(c, r, nroi, topk)) > 0) {
+        float* rows = c->d_match_scratch + (size_t)round * (r.ng + 1) + 1;
         for (int64_t r0 = 0; r0 < nroi; r0 += round) {
             const int64_t n = std::min(round, nroi - r0);
-            float* rows = c->d_match_scratch + one;
             cudaError_t e = launch_tm_sum(c, &r, dS + r0 * c->nv, n, c->d_match_scratch);
             if (e == cudaSuccess) e = launch_tm_rows(c, &r, dS + r0 * c->nv, n, topk, c->d_match_scratch, rows);
             if (e == cudaSuccess) e = launch_topk(c, rows, r.ng, n, topk, db + r0 * topk, ds ? ds + r0 * topk : nullptr);
@@ -1546,7 +1552,7 @@ int aptidx_match_topk(aptidx_ctx* ctx, int32_t cand, const float* S, int64_t nro
         }
     } else {
         // scores of a chunk of ROIs (at most 1 GiB), then a radix select per ROI
-        const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(nroi, ((int64_t)1 << 30) / (r.ng * 4)));
+        const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(nroi, (int64_t)kMatchScratch / (r.ng * 4)));
         if ((rc = match_scratch(c, (size_t)chunk * r.ng * sizeof(float)))) return rc;
         for (int64_t r0 = 0; r0 < nroi; r0 += chunk) {
             const int64_t n = std::min(chunk, nroi - r0);
@@ -1617,7 +1623,7 @@ int aptidx_match_phase(aptidx_ctx* ctx, int32_t n_cand, const int32_t* cand_off,
     dn = static_cast<int32_t*>(tn.p);
     APTIDX_CUDA(c, cudaMemcpyAsync(dn, nc.data(), nc.size() * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
     // channel sums of a chunk of ROIs (at most 1 GiB), then the argmin per ROI
-    const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(nroi, ((int64_t)1 << 30) / (ng * 4)));
+    const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(nroi, (int64_t)kMatchScratch / (ng * 4)));
     if ((rc = match_scratch(c, (size_t)chunk * ng * sizeof(float)))) return rc;
     prof_begin(c, APTIDX_PHASE_MATCH);
     int launches = 0;

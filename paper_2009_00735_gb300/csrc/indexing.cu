@@ -1481,6 +1481,12 @@ cudaError_t launch_build_tm(Ctx* c, Reference* r) {
 
 size_t tm_exact_smem(const Ctx* c, const Reference* r) { return ((size_t)c->nv + r->n_hat) * sizeof(float); }
 
+// Groups of 64 ROIs whose estimates, with the list of heavy ROIs or the rows of topk
+// > 1, fit the scratch of a call
+int64_t tm_groups(const Reference* r, int32_t topk) {
+    return (int64_t)((kMatchScratch - sizeof(float)) / ((size_t)(r->ng + 1) * kTmRois * sizeof(float) * (topk > 1 ? 2 : 1)));
+}
+
 // Whether the lists are the faster way: estimates of both in microseconds on 152 SMs,
 // fitted to 636 calls timed both ways (2562 and 40962 directions, 500 to 100000
 // orientations, 50 to 1000 nodes, 1 to 4096 ROIs, the best 1, 10 and 500; the median
@@ -1493,8 +1499,9 @@ size_t tm_exact_smem(const Ctx* c, const Reference* r) { return ((size_t)c->nv +
 // orientations by two CTAs per 64 ROIs, or the rows, selections and exact sums of
 // topk > 1.  (Without the last three the lists served 64 ROIs x 50000 orientations x
 // 100 nodes in 0.63 ms, which k_match does in 0.36.)
+// Not where the estimates of 64 ROIs (topk > 1: and their rows) exceed the scratch.
 bool tm_pays(const Ctx* c, const Reference* r, int64_t nroi, int32_t topk) {
-    if (!r->d_tm_ent) return false;
+    if (!r->d_tm_ent || tm_groups(r, topk) < 1) return false;
     const auto up = [](double a, double b) { return ceil(a / b); };
     const double sms = c->sm_count, per = 152.0 / sms, n = (double)nroi, ng = (double)r->ng, nh = r->n_hat, nv = c->nv;
     const double looks = ng * nh * 1e-6, cells = n * ng * 1e-6 * per;

@@ -247,6 +247,8 @@ cudaError_t launch_match(Ctx* c, Reference* r, const float* S, int64_t nroi, int
                          const uint32_t* list = nullptr);   // list: (count, ROIs) on the device instead of all
 // Eq. 3 of many ROIs by lists (estimates, then exact sums where they decide)
 cudaError_t launch_build_tm(Ctx* c, Reference* r);
+constexpr size_t kMatchScratch = (size_t)1 << 30;   // scores or estimates staged by a matching call, bytes
+int64_t tm_groups(const Reference* r, int32_t topk);
 bool tm_pays(const Ctx* c, const Reference* r, int64_t nroi, int32_t topk);
 size_t tm_exact_smem(const Ctx* c, const Reference* r);
 cudaError_t launch_tm_sum(Ctx* c, Reference* r, const float* S, int64_t nroi, float* D);

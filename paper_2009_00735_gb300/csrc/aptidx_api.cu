@@ -38,6 +38,8 @@ constexpr size_t kSpareBytes = (size_t)4 << 30;
 static std::mutex g_blk_mu;
 static std::unordered_map<void*, size_t> g_blk_bytes;
 
+static bool release_lists(Ctx* c);
+
 int dev_alloc(Ctx* c, void** p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
@@ -53,6 +55,10 @@ int dev_alloc(Ctx* c, void** p, size_t bytes) {
     if (e == cudaErrorMemoryAllocation && !c->spare.empty()) {
         cudaGetLastError();
         release_spare(c);
+        e = cudaMalloc(p, bytes);
+    }
+    if (e == cudaErrorMemoryAllocation && release_lists(c)) {
+        cudaGetLastError();
         e = cudaMalloc(p, bytes);
     }
     if (e != cudaSuccess) {
@@ -109,6 +115,18 @@ template <typename T>
 static void recycle_ptr(Ctx* c, T*& p) {
     dev_recycle(c, (void*)p);
     p = nullptr;
+}
+
+// give back the lists of Eq. 3, which no call needs (cudaFree waits for their readers)
+static bool release_lists(Ctx* c) {
+    bool any = false;
+    for (Reference& r : c->ref) {
+        any |= r.d_tm_ent != nullptr;
+        free_ptr(r.d_tm_ent);
+        free_ptr(r.d_tm_off);
+        free_ptr(r.d_lut_g);
+    }
+    return any;
 }
 
 // A host view of an input array: the caller's pointer for host memory, a
@@ -515,7 +533,7 @@ int aptidx_destroy(aptidx_ctx* ctx) {
         free_ptr(r.d_lut);
         free_ptr(r.d_tm_ent);
         free_ptr(r.d_tm_off);
-        dev_free(r.d_lut_g);
+        free_ptr(r.d_lut_g);
         free_ptr(r.d_quats);
     }
     delete ctx;
@@ -1318,28 +1336,38 @@ int match_scratch(Ctx* c, size_t need) {
     return rc;
 }
 
-// ROIs of a round of the lists when the scratch holds them, 0 when the call goes to
-// k_match: where that is faster, where there is no memory for the scratch, and on a
-// stream being captured (a graph must not hold scratch that a later call replaces)
-int64_t tm_round(Ctx* c, const Reference& r, int64_t nroi, int32_t topk) {
-    if (!tm_pays(c, &r, nroi, topk)) return 0;
+// ROIs of a round of the lists when the scratch and the lists are there, 0 when the call
+// goes to k_match: where that is faster, where there is no memory, and on a stream being
+// captured (a graph must not hold scratch that a later call replaces)
+int tm_round(Ctx* c, Reference& r, int64_t nroi, int32_t topk, int64_t* round) {
+    *round = 0;
+    if (!tm_pays(c, &r, nroi, topk)) return APTIDX_OK;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
         cudaGetLastError();
-        return 0;
+        return APTIDX_OK;
     }
-    if (cap != cudaStreamCaptureStatusNone) return 0;
-    const int64_t round = std::min<int64_t>((nroi + 63) / 64, tm_groups(&r, topk)) * 64;
+    if (cap != cudaStreamCaptureStatusNone) return APTIDX_OK;
+    const int64_t n = std::min<int64_t>((nroi + 63) / 64, tm_groups(&r, topk)) * 64;
     const std::string err = c->err;
-    if (match_scratch(c, ((size_t)round * (r.ng + 1) * (topk > 1 ? 2 : 1) + 1) * sizeof(float)) == APTIDX_OK) return round;
-    c->err = err;
-    return 0;
+    if (match_scratch(c, ((size_t)n * (r.ng + 1) * (topk > 1 ? 2 : 1) + 1) * sizeof(float)) != APTIDX_OK) {
+        c->err = err;
+        return APTIDX_OK;
+    }
+    if (!r.d_tm_ent) {   // (after the scratch, whose allocation may give the lists back)
+        const cudaError_t e = launch_build_tm(c, &r);
+        if (e != cudaSuccess) return cuda_check(c, e, "look-up table lists");
+    }
+    if (r.d_tm_ent) *round = n;
+    return APTIDX_OK;
 }
 
 // best orientation per ROI (device pointers), by lists where they pay
 int match_best(Ctx* c, Reference& r, const float* dS, int64_t nroi, int32_t* db, float* ds, int* launches) {
     cudaError_t e = cudaSuccess;
-    if (const int64_t round = tm_round(c, r, nroi, 1)) {
+    int64_t round;
+    if (int rc = tm_round(c, r, nroi, 1, &round)) return rc;
+    if (round > 0) {
         for (int64_t r0 = 0; r0 < nroi && e == cudaSuccess; r0 += round) {
             const int64_t n = std::min(round, nroi - r0);
             e = launch_tm_sum(c, &r, dS + r0 * c->nv, n, c->d_match_scratch);
@@ -1377,8 +1405,8 @@ int aptidx_set_reference(aptidx_ctx* ctx, int32_t cand, const float* node_sig, i
     free_ptr(r.d_lut);
     recycle_ptr(c, r.d_tm_ent);
     recycle_ptr(c, r.d_tm_off);
-    dev_recycle(c, r.d_lut_g);
-    r.d_lut_g = nullptr;
+    recycle_ptr(c, r.d_lut_g);
+    r.tm_none = false;
     free_ptr(r.d_quats);
     free_ptr(r.d_img4);
     r.ng = 0;
@@ -1445,8 +1473,8 @@ int aptidx_build_lut(aptidx_ctx* ctx, int32_t cand, const double* quats, int64_t
     free_ptr(r.d_lut);
     recycle_ptr(c, r.d_tm_ent);
     recycle_ptr(c, r.d_tm_off);
-    dev_recycle(c, r.d_lut_g);
-    r.d_lut_g = nullptr;
+    recycle_ptr(c, r.d_lut_g);
+    r.tm_none = false;
     free_ptr(r.d_quats);
     r.ng = 0;
     r.ng_pad = 0;
@@ -1461,7 +1489,10 @@ int aptidx_build_lut(aptidx_ctx* ctx, int32_t cand, const double* quats, int64_t
     if (e != cudaSuccess) return cuda_check(c, e, "look-up table");
     c->launches += 1;
     r.ng = ng;
-    if ((e = launch_build_tm(c, &r)) != cudaSuccess) return cuda_check(c, e, "look-up table lists");
+    // the lists of Eq. 3 where a call of 1000 ROIs would take them (of smaller tables the
+    // first call that does builds them: they would double the time of this one)
+    if (tm_pays(c, &r, 1000, 1) && (e = launch_build_tm(c, &r)) != cudaSuccess)
+        return cuda_check(c, e, "look-up table lists");
     return APTIDX_OK;
 }
 
@@ -1538,9 +1569,11 @@ int aptidx_match_topk(aptidx_ctx* ctx, int32_t cand, const float* S, int64_t nro
     prof_begin(c, APTIDX_PHASE_MATCH);
     int launches = 0;
     int64_t round = 0;
+    if (topk > 1 && tm_exact_smem(c, &r) + 18 * 1024 <= (size_t)max_optin && (rc = tm_round(c, r, nroi, topk, &round)))
+        return rc;
     if (topk == 1) {
         if ((rc = match_best(c, r, dS, nroi, db, ds, &launches))) return rc;
-    } else if (tm_exact_smem(c, &r) + 18 * 1024 <= (size_t)max_optin && (round = tm_round(c, r, nroi, topk)) > 0) {
+    } else if (round > 0) {
         float* rows = c->d_match_scratch + (size_t)round * (r.ng + 1) + 1;
         for (int64_t r0 = 0; r0 < nroi; r0 += round) {
             const int64_t n = std::min(round, nroi - r0);

@@ -525,8 +525,7 @@ __device__ __forceinline__ uint32_t tm_entry(float ref, int row) {
     return ((b + 0x200u) & ~kTmRowBits) | (uint32_t)row;
 }
 
-template <typename IdxT>
-__global__ void __launch_bounds__(256) k_tm_count(const IdxT* __restrict__ lut_t, int64_t ng, int64_t ng_pad, int T,
+__global__ void __launch_bounds__(256) k_tm_count(const uint16_t* __restrict__ lut_t, int64_t ng, int64_t ng_pad, int T,
                                                   int32_t* counts) {
     const int64_t g = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (g < ng) atomicAdd(&counts[(int64_t)((int)lut_t[(int64_t)blockIdx.y * ng_pad + g] / T) * ng + g], 1);
@@ -549,8 +548,7 @@ __global__ void __launch_bounds__(256) k_tm_off(const int64_t* __restrict__ off6
     counts[i] = 0;
 }
 
-template <typename IdxT>
-__global__ void __launch_bounds__(256) k_tm_fill(const IdxT* __restrict__ lut_t, int64_t ng, int64_t ng_pad,
+__global__ void __launch_bounds__(256) k_tm_fill(const uint16_t* __restrict__ lut_t, int64_t ng, int64_t ng_pad,
                                                  const float* __restrict__ top_val, int T,
                                                  const uint32_t* __restrict__ off, int32_t* cursor, uint32_t* ent) {
     const int64_t g = (int64_t)blockIdx.x * 256 + threadIdx.x;
@@ -562,15 +560,14 @@ __global__ void __launch_bounds__(256) k_tm_fill(const IdxT* __restrict__ lut_t,
 }
 
 // k-major table to rows per orientation, lut_g[g * pitch + k] (32 x 32 tiles)
-template <typename IdxT>
-__global__ void __launch_bounds__(256) k_tm_rowmajor(const IdxT* __restrict__ lut_t, int64_t ng, int64_t ng_pad,
-                                                     int32_t n_hat, int pitch, IdxT* lut_g) {
-    __shared__ IdxT t[32][33];
+__global__ void __launch_bounds__(256) k_tm_rowmajor(const uint16_t* __restrict__ lut_t, int64_t ng, int64_t ng_pad,
+                                                     int32_t n_hat, int pitch, uint16_t* lut_g) {
+    __shared__ uint16_t t[32][33];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t g0 = (int64_t)blockIdx.x * 32;
     const int k0 = (int)blockIdx.y * 32;
     for (int i = w; i < 32; i += 8)
-        t[i][lane] = k0 + i < n_hat && g0 + lane < ng ? lut_t[(int64_t)(k0 + i) * ng_pad + g0 + lane] : (IdxT)0;
+        t[i][lane] = k0 + i < n_hat && g0 + lane < ng ? lut_t[(int64_t)(k0 + i) * ng_pad + g0 + lane] : (uint16_t)0;
     __syncthreads();
     for (int i = w; i < 32; i += 8)
         if (g0 + i < ng && k0 + lane < pitch) lut_g[(g0 + i) * pitch + k0 + lane] = t[lane][i];
@@ -657,9 +654,8 @@ __device__ __forceinline__ float tm_threshold(float estimate, TmMargin m) {
 // 3.0, as any other rows (2.9).
 constexpr int kTmNear = 64;
 
-template <typename IdxT>
 __global__ void __launch_bounds__(kTmThreads, 1) k_tm_best(const float* __restrict__ S, int64_t nroi, int32_t nv,
-                                                        const IdxT* __restrict__ lut_g, int64_t ng, int pitch,
+                                                        const uint16_t* __restrict__ lut_g, int64_t ng, int pitch,
                                                         const float* __restrict__ top_val, int32_t n_hat,
                                                         TmMargin margin, const float* __restrict__ D, int32_t* best,
                                                         float* score, uint32_t* heavy) {
@@ -809,9 +805,8 @@ __global__ void __launch_bounds__(256) k_tm_reach(const float* __restrict__ scor
 // over the row is exact.  A CTA takes one part of a ROI's orientations.
 constexpr int kTmList = 4096;
 
-template <typename IdxT>
 __global__ void __launch_bounds__(kTmThreads, 1) k_tm_exact(const float* __restrict__ S, int64_t nroi, int32_t nv,
-                                                            const IdxT* __restrict__ lut_g, int64_t ng, int pitch,
+                                                            const uint16_t* __restrict__ lut_g, int64_t ng, int pitch,
                                                             const float* __restrict__ top_val, int32_t n_hat,
                                                             const float* __restrict__ reach, int parts,
                                                             float* scores) {
@@ -847,14 +842,14 @@ __global__ void __launch_bounds__(kTmThreads, 1) k_tm_exact(const float* __restr
             if (n > kTmList - kTmThreads || g0 + kTmThreads >= gb) {
                 for (uint32_t i = tid; i < n; i += kTmThreads) {
                     // 16 bytes of the orientation's row of the table at a time
-                    constexpr int N = 16 / (int)sizeof(IdxT);
+                    constexpr int N = 8;
                     const uint4* lp = reinterpret_cast<const uint4*>(lut_g + (int64_t)list[i] * pitch);
                     float acc = 0.f;
                     uint4 w = __ldg(lp);
                     for (int k = 0; k < n_hat; k += N) {
                         const uint4 cur = w;
                         if (k + N < n_hat) w = __ldg(++lp);
-                        const IdxT* ix = reinterpret_cast<const IdxT*>(&cur);
+                        const uint16_t* ix = reinterpret_cast<const uint16_t*>(&cur);
 #pragma unroll
                         for (int j = 0; j < N; ++j)
                             if (k + j < n_hat) {
@@ -1422,14 +1417,13 @@ cudaError_t launch_match(Ctx* c, Reference* r, const float* S, int64_t nroi, int
                : launch_match_t<int32_t>(c, r, S, nroi, best, score, scores_out, accumulate, weight, list);
 }
 
-// The lists of k_tm_sum for the table just built (skipped when they would not
-// fit: k_match then serves every call).
-template <typename IdxT>
-static cudaError_t build_tm_t(Ctx* c, Reference* r) {
-    const int tiles = (c->nv + kTmTileMax - 1) / kTmTileMax;
+static int tm_tiles(const Ctx* c) { return (c->nv + kTmTileMax - 1) / kTmTileMax; }
+
+// The lists of k_tm_sum and the table by orientation, queued on the stream.  Without
+// memory for them k_match serves the table (tm_none, until it is built again).
+cudaError_t launch_build_tm(Ctx* c, Reference* r) {
+    const int tiles = tm_tiles(c);
     const int64_t lists = (int64_t)tiles * r->ng;
-    if (lists > ((int64_t)1 << 24) - 4096 || r->n_hat > 65535 || r->ng * r->n_hat + 3 * lists >= ((int64_t)1 << 32))
-        return cudaSuccess;
     const int T = (c->nv + tiles - 1) / tiles;
     const int pitch = (r->n_hat + 7) / 8 * 8;
     void *ent = nullptr, *off = nullptr, *lut_g = nullptr;
@@ -1438,48 +1432,54 @@ static cudaError_t build_tm_t(Ctx* c, Reference* r) {
     const std::string err = c->err;
     if (dev_alloc(c, &ent, (size_t)(r->ng * r->n_hat + 3 * lists) * sizeof(uint32_t)) ||
         dev_alloc(c, &off, (size_t)(lists + 1) * sizeof(uint32_t)) ||
-        dev_alloc(c, &lut_g, (size_t)r->ng * pitch * sizeof(IdxT)) ||
+        dev_alloc(c, &lut_g, (size_t)r->ng * pitch * sizeof(uint16_t)) ||
         dev_alloc(c, (void**)&counts, (size_t)lists * sizeof(int32_t)) ||
         dev_alloc(c, (void**)&padded, (size_t)lists * sizeof(int64_t)) ||
         dev_alloc(c, (void**)&off64, (size_t)(lists + 1) * sizeof(int64_t)) ||
         dev_alloc(c, (void**)&tmp, (scan_tmp_elems(lists) + 1) * sizeof(int64_t))) {
         for (void* q : {ent, off, lut_g, (void*)counts, (void*)padded, (void*)off64, (void*)tmp}) dev_free(q);
         c->err = err;
+        r->tm_none = true;
         return cudaSuccess;
     }
-    const IdxT* lut = static_cast<const IdxT*>(r->d_lut);
+    const uint16_t* lut = static_cast<const uint16_t*>(r->d_lut);
     const dim3 all((unsigned)((r->ng + 255) / 256), (unsigned)r->n_hat);
     const unsigned per_list = (unsigned)(lists / 256 + 1);
     cudaError_t e = cudaMemsetAsync(counts, 0, (size_t)lists * sizeof(int32_t), c->stream);
     if (e == cudaSuccess) {
-        k_tm_count<IdxT><<<all, 256, 0, c->stream>>>(lut, r->ng, r->ng_pad, T, counts);
+        k_tm_count<<<all, 256, 0, c->stream>>>(lut, r->ng, r->ng_pad, T, counts);
         k_tm_pad<<<per_list, 256, 0, c->stream>>>(counts, lists, padded);
         e = launch_scan_i64(padded, off64, lists, tmp, c->stream);
     }
     if (e == cudaSuccess) {
         k_tm_off<<<per_list, 256, 0, c->stream>>>(off64, counts, lists, T, static_cast<uint32_t*>(off),
                                                   static_cast<uint32_t*>(ent));
-        k_tm_fill<IdxT><<<all, 256, 0, c->stream>>>(lut, r->ng, r->ng_pad, r->d_top_val, T,
-                                                    static_cast<uint32_t*>(off), counts, static_cast<uint32_t*>(ent));
-        k_tm_rowmajor<IdxT><<<dim3((unsigned)((r->ng + 31) / 32), (unsigned)((pitch + 31) / 32)), 256, 0, c->stream>>>(
-            lut, r->ng, r->ng_pad, r->n_hat, pitch, static_cast<IdxT*>(lut_g));
+        k_tm_fill<<<all, 256, 0, c->stream>>>(lut, r->ng, r->ng_pad, r->d_top_val, T, static_cast<uint32_t*>(off), counts,
+                                              static_cast<uint32_t*>(ent));
+        k_tm_rowmajor<<<dim3((unsigned)((r->ng + 31) / 32), (unsigned)((pitch + 31) / 32)), 256, 0, c->stream>>>(
+            lut, r->ng, r->ng_pad, r->n_hat, pitch, static_cast<uint16_t*>(lut_g));
         e = cudaGetLastError();
     }
     for (void* q : {(void*)counts, (void*)padded, (void*)off64, (void*)tmp}) dev_recycle(c, q);
     r->d_tm_ent = static_cast<uint32_t*>(ent);
     r->d_tm_off = static_cast<uint32_t*>(off);
-    r->d_lut_g = lut_g;
+    r->d_lut_g = static_cast<uint16_t*>(lut_g);
     r->lut_g_pitch = pitch;
     r->tm_tiles = tiles;
     r->tm_nodes = T;
     return e;
 }
 
-cudaError_t launch_build_tm(Ctx* c, Reference* r) {
-    return r->lut_bytes == 2 ? build_tm_t<uint16_t>(c, r) : build_tm_t<int32_t>(c, r);
-}
-
 size_t tm_exact_smem(const Ctx* c, const Reference* r) { return ((size_t)c->nv + r->n_hat) * sizeof(float); }
+
+// Whether lists serve a table at all: 16-bit node indices and a signature row in
+// shared memory (which the matching calls ask of every table), 2^24 lists (what the
+// scan of their lengths takes) and 32-bit offsets.
+static bool tm_possible(const Ctx* c, const Reference* r) {
+    const int64_t lists = tm_tiles(c) * r->ng;
+    return !r->tm_none && tm_exact_smem(c, r) <= 227 * 1024 && r->lut_bytes == 2 && lists <= ((int64_t)1 << 24) - 4096 &&
+           r->n_hat <= 65535 && r->ng * r->n_hat + 3 * lists < ((int64_t)1 << 32);
+}
 
 // Groups of 64 ROIs whose estimates, with the list of heavy ROIs or the rows of topk
 // > 1, fit the scratch of a call
@@ -1501,7 +1501,7 @@ int64_t tm_groups(const Reference* r, int32_t topk) {
 // 100 nodes in 0.63 ms, which k_match does in 0.36.)
 // Not where the estimates of 64 ROIs (topk > 1: and their rows) exceed the scratch.
 bool tm_pays(const Ctx* c, const Reference* r, int64_t nroi, int32_t topk) {
-    if (!r->d_tm_ent || tm_groups(r, topk) < 1) return false;
+    if (!tm_possible(c, r) || tm_groups(r, topk) < 1) return false;
     const auto up = [](double a, double b) { return ceil(a / b); };
     const double sms = c->sm_count, per = 152.0 / sms, n = (double)nroi, ng = (double)r->ng, nh = r->n_hat, nv = c->nv;
     const double looks = ng * nh * 1e-6, cells = n * ng * 1e-6 * per;
@@ -1510,7 +1510,7 @@ bool tm_pays(const Ctx* c, const Reference* r, int64_t nroi, int32_t topk) {
     const double ctas = std::max(1.0, std::min(16.0, fit));
     const double rounds = up(n, sms), waves = up(n, sms * ctas), rows = up(n, 8 * sms);
     double single = 15 + rounds * (60 * looks + 1.7e-4 * nv) + waves * (0.2 * nv / threads + 0.038 * nh * up(up(ng, 8), threads));
-    const double groups = up(n, kTmRois), tiles = r->tm_tiles;
+    const double groups = up(n, kTmRois), tiles = tm_tiles(c);
     const double gsplit = std::max(1.0, std::min(up(4 * sms, tiles * groups), floor(ng / 256)));
     const double longest = up(tiles * groups * gsplit, sms) * up(ng, gsplit * (kTmThreads / 32)) * nh / tiles;
     double lists = 37 + per * groups * (68e-6 * tiles * ng + 1.5 * looks) + 0.047 * longest;
@@ -1550,26 +1550,19 @@ cudaError_t launch_tm_sum(Ctx* c, Reference* r, const float* S, int64_t nroi, fl
 }
 
 // the best of every ROI from the estimates D, which the counter of heavy ROIs follows
-template <typename IdxT>
-static cudaError_t tm_best_t(Ctx* c, Reference* r, const float* S, int64_t nroi, float* D, int32_t* best, float* score) {
+cudaError_t launch_tm_best(Ctx* c, Reference* r, const float* S, int64_t nroi, float* D, int32_t* best, float* score) {
     const int64_t groups = (nroi + kTmRois - 1) / kTmRois;
     uint32_t* heavy = reinterpret_cast<uint32_t*>(D + groups * r->ng * kTmRois);
-    k_tm_best<IdxT><<<(unsigned)(2 * groups), kTmThreads, 0, c->stream>>>(
-        S, nroi, c->nv, static_cast<const IdxT*>(r->d_lut_g), r->ng, r->lut_g_pitch, r->d_top_val, r->n_hat, tm_margin(r),
-        D, best, score, heavy);
+    k_tm_best<<<(unsigned)(2 * groups), kTmThreads, 0, c->stream>>>(S, nroi, c->nv, r->d_lut_g, r->ng, r->lut_g_pitch,
+                                                                    r->d_top_val, r->n_hat, tm_margin(r), D, best, score,
+                                                                    heavy);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? launch_match(c, r, S, nroi, best, score, nullptr, false, 1.0f, heavy) : e;
 }
 
-cudaError_t launch_tm_best(Ctx* c, Reference* r, const float* S, int64_t nroi, float* D, int32_t* best, float* score) {
-    return r->lut_bytes == 2 ? tm_best_t<uint16_t>(c, r, S, nroi, D, best, score)
-                             : tm_best_t<int32_t>(c, r, S, nroi, D, best, score);
-}
-
 // rows [nroi][ng] from the estimates, exact where the topk are decided; D's
 // first nroi words are reused for the reach
-template <typename IdxT>
-static cudaError_t tm_rows_t(Ctx* c, Reference* r, const float* S, int64_t nroi, int32_t topk, float* D, float* rows) {
+cudaError_t launch_tm_rows(Ctx* c, Reference* r, const float* S, int64_t nroi, int32_t topk, float* D, float* rows) {
     const int64_t groups = (nroi + kTmRois - 1) / kTmRois;
     for (int64_t y0 = 0; y0 < groups; y0 += 32767) {
         const int64_t ny = std::min<int64_t>(32767, groups - y0);
@@ -1579,18 +1572,13 @@ static cudaError_t tm_rows_t(Ctx* c, Reference* r, const float* S, int64_t nroi,
     k_tm_reach<<<(unsigned)std::min<int64_t>(nroi, (int64_t)c->sm_count * 8), 256, 0, c->stream>>>(rows, r->ng, nroi,
                                                                                                   topk, tm_margin(r), D);
     const size_t smem = tm_exact_smem(c, r);
-    cudaError_t e = cudaFuncSetAttribute(k_tm_exact<IdxT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_tm_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // eight rounds of CTAs at least: the last, partly filled one then costs little
     const int parts = (int)std::max<int64_t>(1, std::min<int64_t>((8 * (int64_t)c->sm_count + nroi - 1) / nroi, r->ng / 4096));
-    k_tm_exact<IdxT><<<(unsigned)std::min<int64_t>(nroi * parts, c->sm_count), kTmThreads, smem, c->stream>>>(
-        S, nroi, c->nv, static_cast<const IdxT*>(r->d_lut_g), r->ng, r->lut_g_pitch, r->d_top_val, r->n_hat, D, parts, rows);
+    k_tm_exact<<<(unsigned)std::min<int64_t>(nroi * parts, c->sm_count), kTmThreads, smem, c->stream>>>(
+        S, nroi, c->nv, r->d_lut_g, r->ng, r->lut_g_pitch, r->d_top_val, r->n_hat, D, parts, rows);
     return cudaGetLastError();
-}
-
-cudaError_t launch_tm_rows(Ctx* c, Reference* r, const float* S, int64_t nroi, int32_t topk, float* D, float* rows) {
-    return r->lut_bytes == 2 ? tm_rows_t<uint16_t>(c, r, S, nroi, topk, D, rows)
-                             : tm_rows_t<int32_t>(c, r, S, nroi, topk, D, rows);
 }
 
 // Phase decision: candidate c's summed channel scores divided by its channel

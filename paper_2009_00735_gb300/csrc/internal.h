@@ -41,11 +41,13 @@ struct Reference {
     float4* d_img4 = nullptr;
     void* d_lut = nullptr;         // [n_hat x ng_pad] (k-major), uint16 node indices when nv <= 65536, else int32
     int lut_bytes = 4;             // bytes per table entry (2 or 4)
-    // the table as lists per (tile of tm_nodes nodes, orientation), or null
+    // the table as lists per (tile of tm_nodes nodes, orientation), or null: built with
+    // the table or by the first call that takes them, given back when memory runs out
     uint32_t* d_tm_ent = nullptr;  // reference value to 22 bits | row of the node, padded to four
     uint32_t* d_tm_off = nullptr;  // [tm_tiles x ng + 1]
     int tm_tiles = 0, tm_nodes = 0;
-    void* d_lut_g = nullptr;       // [ng x lut_g_pitch] the table by orientation (with the lists)
+    bool tm_none = false;          // no memory for the lists of this table
+    uint16_t* d_lut_g = nullptr;   // [ng x lut_g_pitch] the table by orientation (with the lists)
     int lut_g_pitch = 0;
     double* d_quats = nullptr;     // [ng x 4] test orientations of the table
     int64_t ng = 0;

@@ -504,7 +504,6 @@ int aptidx_destroy(aptidx_ctx* ctx) {
     free_ptr(c->d_dirs_sorted);
     free_ptr(c->d_slot_dirs);
     free_ptr(c->d_slot_idx);
-    free_ptr(c->d_node_start);
     free_ptr(c->d_nodes);
     free_ptr(c->d_gn_scratch);
     c->gn_scratch_bytes = 0;
@@ -612,11 +611,13 @@ int aptidx_set_directions(aptidx_ctx* ctx, const float* u, int32_t nv, int mem) 
     if ((rc = to_host(c, u, (size_t)nv * 3, mem, hu))) return rc;
     const int32_t nv_pad = (nv + kTileDirs - 1) / kTileDirs * kTileDirs;
     std::vector<float4> d4((size_t)nv_pad, make_float4(1.f, 0.f, 0.f, 0.f));
+    double umax2 = 0.0;
     for (int32_t v = 0; v < nv; ++v) {
         float x = hu[3 * v], y = hu[3 * v + 1], z = hu[3 * v + 2];
         double n2 = (double)x * x + (double)y * y + (double)z * z;
         if (!(fabs(sqrt(n2) - 1.0) <= 1e-5))
             return set_error(c, APTIDX_E_INVALID_ARG, "directions: |u[%d]| = %g is not 1", v, sqrt(n2));
+        umax2 = std::max(umax2, n2);
         d4[v] = make_float4(x, y, z, 0.f);
     }
     // spatial order: Morton key of the (elevation, azimuth) 1-degree cell
@@ -685,38 +686,13 @@ int aptidx_set_directions(aptidx_ctx* ctx, const float* u, int32_t nv, int mem) 
             si.push_back(make_int2(-1, -1));
         }
     }
-    // node grid: cells of one and a half node spacings of an even covering (0.02
-    // to 0.5), which hold a few nodes each
-    const double h = std::min(0.5, std::max(0.02, 1.5 * sqrt(4.0 * M_PI / (double)nv)));
-    const float org = -1.0001f, inv_h = (float)(1.0 / h);
-    const int dim = (int)(2.0002 * (double)inv_h) + 1;
-    std::vector<int32_t> nstart((size_t)dim * dim * dim + 1, 0), ncell((size_t)nv);
-    double umax2 = 0.0;
-    for (int32_t v = 0; v < nv; ++v) {
-        const float x[3] = {d4[v].x, d4[v].y, d4[v].z};
-        int ic[3];
-        for (int d = 0; d < 3; ++d) ic[d] = std::min(std::max((int)((x[d] - org) * inv_h), 0), dim - 1);
-        ncell[v] = ic[0] + dim * (ic[1] + dim * ic[2]);
-        ++nstart[(size_t)ncell[v] + 1];
-        umax2 = std::max(umax2, (double)x[0] * x[0] + (double)x[1] * x[1] + (double)x[2] * x[2]);
-    }
-    for (size_t i = 1; i < nstart.size(); ++i) nstart[i] += nstart[i - 1];
-    std::vector<float4> nodes((size_t)nv);
-    {
-        std::vector<int32_t> at(nstart.begin(), nstart.end() - 1);
-        for (int32_t v = 0; v < nv; ++v) {
-            float w;
-            memcpy(&w, &v, sizeof(w));
-            nodes[(size_t)at[(size_t)ncell[v]]++] = make_float4(d4[v].x, d4[v].y, d4[v].z, w);
-        }
-    }
     free_ptr(c->d_dirs);
     free_ptr(c->d_dirs_sorted);
     free_ptr(c->d_slot_dirs);
     free_ptr(c->d_slot_idx);
-    free_ptr(c->d_node_start);
     free_ptr(c->d_nodes);
     clear_graphs(c);
+    c->dir_max2 = umax2;
     c->nv = c->nv_pad = 0;
     c->nslot = c->nslot_pad = c->npairs = 0;
     if ((rc = dev_alloc(c, (void**)&c->d_dirs, (size_t)nv_pad * sizeof(float4)))) return rc;
@@ -725,16 +701,6 @@ int aptidx_set_directions(aptidx_ctx* ctx, const float* u, int32_t nv, int mem) 
                                    c->stream));
     APTIDX_CUDA(c, cudaMemcpyAsync(c->d_dirs_sorted, ds.data(), (size_t)nv * sizeof(float4), cudaMemcpyHostToDevice,
                                    c->stream));
-    if ((rc = dev_alloc(c, (void**)&c->d_node_start, nstart.size() * sizeof(int32_t)))) return rc;
-    if ((rc = dev_alloc(c, (void**)&c->d_nodes, (size_t)nv * sizeof(float4)))) return rc;
-    APTIDX_CUDA(c, cudaMemcpyAsync(c->d_node_start, nstart.data(), nstart.size() * sizeof(int32_t),
-                                   cudaMemcpyHostToDevice, c->stream));
-    APTIDX_CUDA(c, cudaMemcpyAsync(c->d_nodes, nodes.data(), (size_t)nv * sizeof(float4), cudaMemcpyHostToDevice,
-                                   c->stream));
-    c->node_dim = dim;
-    c->node_org = org;
-    c->node_inv_h = inv_h;
-    c->node_far2 = (float)(umax2 - 0.998 / ((double)inv_h * (double)inv_h));
     if (npairs > 0) {
         if ((rc = dev_alloc(c, (void**)&c->d_slot_dirs, sd.size() * sizeof(float4)))) return rc;
         if ((rc = dev_alloc(c, (void**)&c->d_slot_idx, si.size() * sizeof(int2)))) return rc;

@@ -211,15 +211,15 @@ __device__ __forceinline__ float node_dot(float4 u, float3 r) {
 // (nv <= 65536), else int32_t.
 //
 // The nodes lie in a cubic grid of cells of edge h (about one and a half node
-// spacings).  A query scans the 3 x 3 x 3 cells around r, nine runs of
-// consecutive nodes.  A node outside them is at least h away, so its exact dot
+// spacings of an even covering).  A query scans the 3 x 3 x 3 cells around r, nine
+// runs of consecutive nodes.  A node outside them is at least h away, so its exact dot
 // product is at most (max |u|^2 + |r|^2 - h^2) / 2: when the best found exceeds
 // that by more than the FP32 errors it is the answer of a scan over all nodes.
-// Queries it does not settle (r in a gap of the direction set) are listed and
-// left to k_lut_scan.  Scanning all 40962 nodes for every query took 29.1 ms
-// for 3419 x 1000 queries (1.4e11 dot products); this reads about 20 nodes per
-// query, bound by the L2 latency of the run bounds and nodes:
-// 0.4 ms.
+// Queries it does not settle (r in a gap of the direction set) are listed and left to
+// k_lut_scan.
+// Scanning all 40962 nodes for every query took 29.1 ms for 3419 x 1000 queries
+// (1.4e11 dot products); this reads about 20 nodes per query, bound by the L2 latency
+// of the run bounds and nodes: 0.4 ms.
 constexpr int kLutK = 8;   // nodes per thread (one rotation matrix, kLutK of its columns of the table)
 
 struct NodeGrid {
@@ -231,6 +231,30 @@ struct NodeGrid {
 
 __device__ __forceinline__ int node_cell(float x, const NodeGrid& g) {
     return min(max((int)((x - g.org) * g.inv_h), 0), g.dim - 1);
+}
+
+__device__ __forceinline__ int node_cell3(float4 u, const NodeGrid& g) {
+    return node_cell(u.x, g) + g.dim * (node_cell(u.y, g) + g.dim * node_cell(u.z, g));
+}
+
+__global__ void __launch_bounds__(256) k_node_count(const float4* __restrict__ dirs, int32_t nv, NodeGrid g,
+                                                    unsigned long long* counts) {
+    const int v = blockIdx.x * 256 + threadIdx.x;
+    if (v < nv) atomicAdd(&counts[node_cell3(dirs[v], g)], 1ull);
+}
+
+// every node into its cell (in any order: queries resolve ties by index), counting the
+// cells down, and the cells' first nodes in 32 bits
+__global__ void __launch_bounds__(256) k_node_fill(const float4* __restrict__ dirs, int32_t nv, NodeGrid g, int n_cells,
+                                                   const int64_t* __restrict__ off, unsigned long long* counts,
+                                                   int32_t* start, float4* nodes) {
+    for (int i = blockIdx.x * 256 + threadIdx.x; i <= n_cells; i += gridDim.x * 256) start[i] = (int32_t)off[i];
+    for (int v = blockIdx.x * 256 + threadIdx.x; v < nv; v += gridDim.x * 256) {
+        const float4 u = dirs[v];
+        const int c = node_cell3(u, g);
+        const int64_t k = off[c] + (int64_t)atomicAdd(&counts[c], ~0ull) - 1;
+        nodes[k] = make_float4(u.x, u.y, u.z, __int_as_float(v));
+    }
 }
 
 template <typename IdxT>
@@ -278,17 +302,17 @@ __global__ void __launch_bounds__(kLutThreads) k_build_lut(NodeGrid grid, const 
     }
 }
 
-// The listed queries against every node, staged through shared memory, four
-// queries per thread.
+// The listed queries (open == nullptr: all n_all of them) against every node, staged
+// through shared memory, four queries per thread.
 template <typename IdxT>
 __global__ void __launch_bounds__(kLutThreads) k_lut_scan(const float4* __restrict__ dirs, int32_t nv,
                                                           const int32_t* __restrict__ top,
                                                           const double* __restrict__ quats, int64_t ng,
-                                                          int64_t ng_pad, IdxT* lut_t, int32_t k0,
+                                                          int64_t ng_pad, IdxT* lut_t, int32_t k0, uint32_t n_all,
                                                           const uint32_t* __restrict__ open,
                                                           const uint32_t* __restrict__ n_open) {
     __shared__ float4 tile[kLutTile];
-    const uint32_t n = *n_open;
+    const uint32_t n = open ? *n_open : n_all;
     for (uint32_t q0 = blockIdx.x * (uint32_t)(kLutThreads * kLutPer); q0 < n;
          q0 += gridDim.x * (uint32_t)(kLutThreads * kLutPer)) {
         float3 r[kLutPer];
@@ -296,14 +320,15 @@ __global__ void __launch_bounds__(kLutThreads) k_lut_scan(const float4* __restri
         int32_t bi[kLutPer];
 #pragma unroll
         for (int j = 0; j < kLutPer; ++j) {
-            const uint32_t q = q0 + (uint32_t)j * kLutThreads + threadIdx.x;
+            const uint32_t i = q0 + (uint32_t)j * kLutThreads + threadIdx.x;
             best[j] = -INFINITY;
             bi[j] = 0;
             r[j] = make_float3(0.f, 0.f, 0.f);
-            if (q < n) {
-                const int64_t g = open[q] % ng;
+            if (i < n) {
+                const uint32_t q = open ? open[i] : i;
+                const int64_t g = q % ng;
                 const M3 R = quat_to_matrix(quats[4 * g], quats[4 * g + 1], quats[4 * g + 2], quats[4 * g + 3]);
-                r[j] = rotate_node(R, dirs[top[k0 + (int)(open[q] / ng)]]);
+                r[j] = rotate_node(R, dirs[top[k0 + (int)(q / ng)]]);
             }
         }
         for (int p0 = 0; p0 < nv; p0 += kLutTile) {
@@ -325,8 +350,11 @@ __global__ void __launch_bounds__(kLutThreads) k_lut_scan(const float4* __restri
         }
 #pragma unroll
         for (int j = 0; j < kLutPer; ++j) {
-            const uint32_t q = q0 + (uint32_t)j * kLutThreads + threadIdx.x;
-            if (q < n) lut_t[(k0 + (int64_t)(open[q] / ng)) * ng_pad + open[q] % ng] = (IdxT)bi[j];
+            const uint32_t i = q0 + (uint32_t)j * kLutThreads + threadIdx.x;
+            if (i < n) {
+                const uint32_t q = open ? open[i] : i;
+                lut_t[(k0 + (int64_t)(q / ng)) * ng_pad + q % ng] = (IdxT)bi[j];
+            }
         }
     }
 }
@@ -1357,30 +1385,82 @@ cudaError_t launch_top_nodes(Ctx* c, Reference* r) {
     return e;
 }
 
+// The node grid of the directions, queued on the stream: cells of one and a half node
+// spacings of an even covering (0.02 to 0.5), which hold a few nodes each.  Built here
+// and not with the directions: signatures do not need it (on the host it took
+// set_directions 0.85 of 6.6 ms for 40962 directions).
+static int ensure_node_grid(Ctx* c) {
+    if (c->d_nodes) return APTIDX_OK;
+    const double h = std::min(0.5, std::max(0.02, 1.5 * sqrt(4.0 * M_PI / (double)c->nv)));
+    c->node_org = -1.0001f;
+    c->node_inv_h = (float)(1.0 / h);
+    c->node_dim = (int)(2.0002 * (double)c->node_inv_h) + 1;
+    c->node_far2 = (float)(c->dir_max2 - 0.998 / ((double)c->node_inv_h * (double)c->node_inv_h));
+    const size_t cells = (size_t)c->node_dim * c->node_dim * c->node_dim;
+    const NodeGrid g{nullptr, nullptr, c->node_dim, c->node_org, c->node_inv_h, c->node_far2};
+    int64_t* work = nullptr;   // counts | offsets | the scan's sums
+    int rc = dev_alloc(c, (void**)&work, (2 * cells + 1 + scan_tmp_elems(cells) + 1) * sizeof(int64_t));
+    if (!rc) rc = dev_alloc(c, (void**)&c->d_nodes, (size_t)c->nv * sizeof(float4) + (cells + 1) * sizeof(int32_t));
+    if (!rc) {
+        c->d_node_start = reinterpret_cast<int32_t*>(c->d_nodes + c->nv);
+        unsigned long long* counts = reinterpret_cast<unsigned long long*>(work);
+        int64_t* off = work + cells;
+        cudaError_t e = cudaMemsetAsync(counts, 0, cells * sizeof(int64_t), c->stream);
+        if (e == cudaSuccess) {
+            k_node_count<<<(unsigned)((c->nv + 255) / 256), 256, 0, c->stream>>>(c->d_dirs, c->nv, g, counts);
+            e = launch_scan_i64(work, off, (int64_t)cells, off + cells + 1, c->stream);
+        }
+        if (e == cudaSuccess) {
+            k_node_fill<<<(unsigned)c->sm_count * 8, 256, 0, c->stream>>>(c->d_dirs, c->nv, g, (int)cells, off, counts,
+                                                                         c->d_node_start, c->d_nodes);
+            e = cudaGetLastError();
+        }
+        if (e != cudaSuccess) {
+            rc = cuda_check(c, e, "node grid");
+            dev_free(c->d_nodes);
+            c->d_nodes = nullptr;
+        }
+    }
+    dev_recycle(c, work);
+    return rc;
+}
+
 // The table in runs of rows of at most 2^24 queries, so that the list of open
-// queries (sized for all of a run) stays at 64 MB, and of what a grid takes.
+// queries (sized for all of a run) stays at 64 MB, and of what a grid takes.  Few
+// queries, and those without memory for the grid or the list, are scanned: 2e8 dot
+// products take 42 us, the grid's own kernels and the look-up 60.
 template <typename IdxT>
 static cudaError_t launch_build_lut_t(Ctx* c, Reference* r, const double* d_quats, int64_t ng) {
     const int64_t rows = std::min<int64_t>(std::min<int64_t>(r->n_hat, 65535 * kLutK),
                                            std::max<int64_t>(1, ((int64_t)1 << 24) / ng));
     uint32_t* open = nullptr;
-    if (dev_alloc(c, (void**)&open, (size_t)(rows * ng + 1) * sizeof(uint32_t))) return cudaErrorMemoryAllocation;
+    bool by_grid = (double)ng * r->n_hat * c->nv > 2e8;
+    const std::string err = c->err;
+    if (by_grid) {
+        int rc = ensure_node_grid(c);
+        if (!rc) rc = dev_alloc(c, (void**)&open, (size_t)(rows * ng + 1) * sizeof(uint32_t));
+        by_grid = rc == APTIDX_OK;
+        if (rc && rc != APTIDX_E_OOM) return cudaErrorUnknown;
+        c->err = err;
+    }
     const NodeGrid grid{c->d_node_start, c->d_nodes, c->node_dim, c->node_org, c->node_inv_h, c->node_far2};
+    IdxT* lut = static_cast<IdxT*>(r->d_lut);
     cudaError_t e = cudaSuccess;
     for (int64_t k0 = 0; k0 < r->n_hat && e == cudaSuccess; k0 += rows) {
-        const int64_t k1 = std::min<int64_t>(k0 + rows, r->n_hat);
-        if ((e = cudaMemsetAsync(open, 0, sizeof(uint32_t), c->stream)) != cudaSuccess) break;
-        const dim3 blocks((unsigned)((ng + kLutThreads - 1) / kLutThreads), (unsigned)((k1 - k0 + kLutK - 1) / kLutK));
-        k_build_lut<IdxT><<<blocks, kLutThreads, 0, c->stream>>>(grid, c->d_dirs, r->d_top, r->n_hat, d_quats, ng,
-                                                                 r->ng_pad, static_cast<IdxT*>(r->d_lut), (int32_t)k0,
-                                                                 (int32_t)k1, open + 1, open);
-        k_lut_scan<IdxT><<<(unsigned)c->sm_count * 4, kLutThreads, 0, c->stream>>>(
-            c->d_dirs, c->nv, r->d_top, d_quats, ng, r->ng_pad, static_cast<IdxT*>(r->d_lut), (int32_t)k0, open + 1,
+        const int64_t k1 = std::min<int64_t>(k0 + rows, r->n_hat), nq = (k1 - k0) * ng;
+        if (by_grid) {
+            if ((e = cudaMemsetAsync(open, 0, sizeof(uint32_t), c->stream)) != cudaSuccess) break;
+            const dim3 blocks((unsigned)((ng + kLutThreads - 1) / kLutThreads), (unsigned)((k1 - k0 + kLutK - 1) / kLutK));
+            k_build_lut<IdxT><<<blocks, kLutThreads, 0, c->stream>>>(grid, c->d_dirs, r->d_top, r->n_hat, d_quats, ng,
+                                                                     r->ng_pad, lut, (int32_t)k0, (int32_t)k1, open + 1, open);
+        }
+        const int64_t chunks = (nq + kLutThreads * kLutPer - 1) / (kLutThreads * kLutPer);
+        k_lut_scan<IdxT><<<(unsigned)std::min<int64_t>(chunks, (int64_t)c->sm_count * 8), kLutThreads, 0, c->stream>>>(
+            c->d_dirs, c->nv, r->d_top, d_quats, ng, r->ng_pad, lut, (int32_t)k0, (uint32_t)nq, by_grid ? open + 1 : nullptr,
             open);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    dev_recycle(c, open);
+    dev_recycle(c, open);   // (reused on the same stream only)
     return e;
 }
 

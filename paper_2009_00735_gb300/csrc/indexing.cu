@@ -215,16 +215,19 @@ __device__ __forceinline__ float node_dot(float4 u, float3 r) {
 // runs of consecutive nodes.  A node outside them is at least h away, so its exact dot
 // product is at most (max |u|^2 + |r|^2 - h^2) / 2: when the best found exceeds
 // that by more than the FP32 errors it is the answer of a scan over all nodes.
-// Queries it does not settle (r in a gap of the direction set) are listed and left to
-// k_lut_scan.
+// Queries it does not settle (r in a gap of the direction set), and those with more
+// than kLutRun nodes in their cells (clustered directions: a thread that walked
+// thousands of nodes by itself took up to 54 ms for 10^6 queries on 40000 directions
+// within one degree, the scan 9.1), are listed and left to k_lut_scan.
 // Scanning all 40962 nodes for every query took 29.1 ms for 3419 x 1000 queries
 // (1.4e11 dot products); this reads about 20 nodes per query, bound by the L2 latency
 // of the run bounds and nodes: 0.4 ms.
+constexpr int kLutRun = 512;
 constexpr int kLutK = 8;   // nodes per thread (one rotation matrix, kLutK of its columns of the table)
 
 struct NodeGrid {
     const int32_t* start;   // [dim^3 + 1]
-    const float4* nodes;    // in cell order, ascending index inside a cell; w = index bits
+    const float4* nodes;    // in cell order, in any order inside a cell; w = index bits
     int dim;
     float org, inv_h, far2;   // cell = (x - org) * inv_h; far2 = max |u|^2 - (0.999 h)^2
 };
@@ -273,7 +276,7 @@ __global__ void __launch_bounds__(kLutThreads) k_build_lut(NodeGrid grid, const 
         const int xa = max(ix - 1, 0), xb = min(ix + 2, grid.dim);
         float best = -INFINITY;
         int32_t bi = 0x7FFFFFFF;
-        int32_t beg[9], end[9];
+        int32_t beg[9], end[9], run = 0;
 #pragma unroll
         for (int j = 0; j < 9; ++j) {
             const int y = iy + j % 3 - 1, z = iz + j / 3 - 1;
@@ -281,10 +284,11 @@ __global__ void __launch_bounds__(kLutThreads) k_build_lut(NodeGrid grid, const 
             const int c = in ? grid.dim * (y + grid.dim * z) : 0;
             beg[j] = in ? __ldg(grid.start + c + xa) : 0;
             end[j] = in ? __ldg(grid.start + c + xb) : 0;
+            run += end[j] - beg[j];
         }
 #pragma unroll
         for (int j = 0; j < 9; ++j)
-            for (int i = beg[j]; i < end[j]; ++i) {
+            for (int i = beg[j]; i < end[j] && run <= kLutRun; ++i) {
                 const float4 u = __ldg(grid.nodes + i);
                 const float d = node_dot(u, r);
                 const int32_t idx = __float_as_int(u.w);
@@ -294,7 +298,7 @@ __global__ void __launch_bounds__(kLutThreads) k_build_lut(NodeGrid grid, const 
                 }
             }
         const float r2 = r.x * r.x + r.y * r.y + r.z * r.z;
-        if (best > 0.5f * (grid.far2 + r2) + 2e-6f) {
+        if (run <= kLutRun && best > 0.5f * (grid.far2 + r2) + 2e-6f) {
             lut_t[(int64_t)k * ng_pad + g] = (IdxT)bi;
         } else {
             open[atomicAdd(n_open, 1u)] = (uint32_t)((int64_t)(k - k0) * ng + g);

@@ -1,7 +1,7 @@
 """The look-up table by the node grid against the table by scans over all nodes (the
 same table in pieces small enough that the library scans them, which test_gpu_lut.py
-holds to the oracle): direction sets with gaps, uneven norms, duplicates.  Index
-work: exact.
+holds to the oracle): direction sets with gaps, uneven norms, duplicates, and clusters
+of thousands of directions in one cell of the grid.  Index work: exact.
 """
 import numpy as np
 import pytest
@@ -15,6 +15,14 @@ from test_gpu_plain import torch_cuda  # noqa: F401
 pytestmark = pytest.mark.gpu
 
 
+def cap(n, degrees):
+    """n directions within `degrees` of the z axis"""
+    i = np.arange(n) + 0.5
+    z = 1 - (1 - np.cos(np.radians(degrees))) * i / n
+    a = i * np.pi * (3 - 5 ** 0.5)
+    return np.stack([np.sqrt(1 - z * z) * np.cos(a), np.sqrt(1 - z * z) * np.sin(a), z], 1).astype(np.float32)
+
+
 def near(n, degrees, seed):
     """orientations within a few times `degrees` of the identity"""
     w = np.radians(degrees) * np.random.default_rng(seed).standard_normal((n, 3))
@@ -23,12 +31,16 @@ def near(n, degrees, seed):
 
 
 def sets(kind):
+    if kind == "cluster":
+        return np.concatenate([cap(20000, 1.0), spiral(3001)])
+    if kind == "clusters":
+        return np.concatenate([cap(8000, 0.3), -cap(7001, 2.0), spiral(500)])
     if kind == "even":
         return spiral(40001)
     return direction_set(kind)
 
 
-@pytest.mark.parametrize("kind", ["even", "cap", "holes", "norms", "double", "dense"])
+@pytest.mark.parametrize("kind", ["cluster", "clusters", "even", "cap", "holes", "norms", "double", "dense"])
 def test_grid_equals_scan(torch_cuda, kind):
     u = sets(kind)
     nv = len(u)
@@ -63,3 +75,30 @@ def test_grid_equals_scan(torch_cuda, kind):
     other.close()
     ctx.close()
 
+
+def test_clustered_directions_take_no_longer(torch_cuda):
+    """40000 directions within one degree: queries among them take no longer than queries
+    away from them, which are scanned (a thread that walked its cells took six times as
+    long)."""
+    torch = torch_cuda
+    u = cap(40000, 1.0)
+    ctx = apt.Context(0)
+    h = ctx.handle
+    apt.aptidx_set_directions(h, u)
+    apt.aptidx_set_reference(h, 0, np.random.default_rng(1).random(len(u)).astype(np.float32), 500)
+    flip = near(400, 0.3, 1)[:, [1, 0, 3, 2]] * [-1, 1, -1, 1]   # the same after half a turn about x
+
+    def ms(Q):
+        t = []
+        for _ in range(4):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            e0.record()
+            apt.aptidx_build_lut(h, 0, Q)
+            e1.record()
+            torch.cuda.synchronize()
+            t.append(e0.elapsed_time(e1))
+        return min(t[1:])
+
+    assert ms(near(400, 0.3, 1)) < 2.0 * ms(np.ascontiguousarray(flip))
+    ctx.close()

@@ -105,8 +105,11 @@ __global__ void __launch_bounds__(1024) k_top_nodes(const float* __restrict__ si
 // the lowest-index ones equal to it, sorted in shared memory.  The full sort
 // above walks 136 passes of 65536 keys in global memory at 40962 directions
 // (2.16 ms in one CTA); four counting passes and a sort of 1024 keys take
-// 0.04 ms.
+// 0.04 ms.  Where the sort is no longer for all keys, and up to kSortAll directions, it
+// takes them all: the four passes, with a walk over 256 counts each, cost 12 us more
+// (aptidx_set_reference of 162 directions 50 us, now 37; of 1025 and all of them 75, 54).
 constexpr int kSelMax = 4096;
+constexpr int kSortAll = 1024;
 
 __global__ void __launch_bounds__(1024) k_top_select(const float* __restrict__ sig, int32_t nv, int32_t n_hat,
                                                      int32_t* top, float* top_val) {
@@ -119,48 +122,52 @@ __global__ void __launch_bounds__(1024) k_top_select(const float* __restrict__ s
         s_rem = (uint32_t)n_hat;
         s_count = 0;
     }
-    for (int pass = 3; pass >= 0; --pass) {
-        if (tid < 256) hist[tid] = 0;
-        __syncthreads();
-        const uint32_t prefix = s_prefix, hmask = pass == 3 ? 0u : 0xFFFFFFFFu << (8 * (pass + 1));
-        for (int i = tid; i < nv; i += 1024) {
-            const uint32_t k = ~ordered_f32(sig[i]);
-            if ((k & hmask) == (prefix & hmask)) atomicAdd(&hist[(k >> (8 * pass)) & 255u], 1u);
-        }
-        __syncthreads();
-        if (tid == 0) {
-            uint32_t rem = s_rem, d = 0;
-            while (hist[d] < rem) rem -= hist[d++];
-            s_rem = rem;
-            s_prefix = prefix | (d << (8 * pass));
-        }
-        __syncthreads();
-    }
-    const uint32_t kth = s_prefix, need_eq = s_rem, n_less = (uint32_t)n_hat - need_eq;
     int kp = 1;
-    while (kp < n_hat) kp <<= 1;
+    while (kp < (nv <= kSortAll ? nv : n_hat)) kp <<= 1;
     for (int i = tid; i < kp; i += 1024) sel[i] = ~0ull;
     __syncthreads();
-    for (int i = tid; i < nv; i += 1024) {
-        const uint32_t k = ~ordered_f32(sig[i]);
-        if (k < kth) sel[atomicAdd(&s_count, 1u)] = ((uint64_t)k << 32) | (uint32_t)i;
-    }
-    uint32_t taken = 0;
-    for (int i0 = 0; i0 < nv && taken < need_eq; i0 += 1024) {
-        const int i = i0 + tid;
-        const bool eq = i < nv && ~ordered_f32(sig[i]) == kth;
-        const uint32_t bal = __ballot_sync(0xffffffffu, eq);
-        __syncthreads();
-        if (lane == 0) wcnt[warp] = __popc(bal);
-        __syncthreads();
-        uint32_t before = 0, total = 0;
-        for (int w = 0; w < 32; ++w) {
-            if (w < warp) before += wcnt[w];
-            total += wcnt[w];
+    if (nv <= kp) {
+        for (int i = tid; i < nv; i += 1024) sel[i] = ((uint64_t)(~ordered_f32(sig[i])) << 32) | (uint32_t)i;
+    } else {
+        for (int pass = 3; pass >= 0; --pass) {
+            if (tid < 256) hist[tid] = 0;
+            __syncthreads();
+            const uint32_t prefix = s_prefix, hmask = pass == 3 ? 0u : 0xFFFFFFFFu << (8 * (pass + 1));
+            for (int i = tid; i < nv; i += 1024) {
+                const uint32_t k = ~ordered_f32(sig[i]);
+                if ((k & hmask) == (prefix & hmask)) atomicAdd(&hist[(k >> (8 * pass)) & 255u], 1u);
+            }
+            __syncthreads();
+            if (tid == 0) {
+                uint32_t rem = s_rem, d = 0;
+                while (hist[d] < rem) rem -= hist[d++];
+                s_rem = rem;
+                s_prefix = prefix | (d << (8 * pass));
+            }
+            __syncthreads();
         }
-        const uint32_t rank = taken + before + __popc(bal & ((1u << lane) - 1u));
-        if (eq && rank < need_eq) sel[n_less + rank] = ((uint64_t)kth << 32) | (uint32_t)i;
-        taken += total;
+        const uint32_t kth = s_prefix, need_eq = s_rem, n_less = (uint32_t)n_hat - need_eq;
+        for (int i = tid; i < nv; i += 1024) {
+            const uint32_t k = ~ordered_f32(sig[i]);
+            if (k < kth) sel[atomicAdd(&s_count, 1u)] = ((uint64_t)k << 32) | (uint32_t)i;
+        }
+        uint32_t taken = 0;
+        for (int i0 = 0; i0 < nv && taken < need_eq; i0 += 1024) {
+            const int i = i0 + tid;
+            const bool eq = i < nv && ~ordered_f32(sig[i]) == kth;
+            const uint32_t bal = __ballot_sync(0xffffffffu, eq);
+            __syncthreads();
+            if (lane == 0) wcnt[warp] = __popc(bal);
+            __syncthreads();
+            uint32_t before = 0, total = 0;
+            for (int w = 0; w < 32; ++w) {
+                if (w < warp) before += wcnt[w];
+                total += wcnt[w];
+            }
+            const uint32_t rank = taken + before + __popc(bal & ((1u << lane) - 1u));
+            if (eq && rank < need_eq) sel[n_less + rank] = ((uint64_t)kth << 32) | (uint32_t)i;
+            taken += total;
+        }
     }
     __syncthreads();
     for (int k = 2; k <= kp; k <<= 1) {

@@ -102,3 +102,21 @@ def test_clustered_directions_take_no_longer(torch_cuda):
 
     assert ms(near(400, 0.3, 1)) < 2.0 * ms(np.ascontiguousarray(flip))
     ctx.close()
+
+
+@pytest.mark.parametrize("nv", [1, 2, 3, 162, 1023, 1024, 1025, 2049, 4096])
+def test_strongest_of_few_directions(torch_cuda, nv):
+    """Few directions are sorted, more are selected unless about all are asked for: values with
+    ties and zeros of both signs, the identity maps every strongest node onto itself."""
+    u = spiral(nv)
+    sig = (np.random.default_rng(nv).integers(-6, 6, nv) / 4.0).astype(np.float32)
+    sig[5::11] = -0.0
+    key = np.where(sig.view(np.int32) < 0, ~sig.view(np.uint32), sig.view(np.uint32) | np.uint32(1 << 31))
+    want = np.lexsort((np.arange(nv), ~key))
+    ctx = apt.Context(0)
+    apt.aptidx_set_directions(ctx.handle, u)
+    for n_hat in sorted({1, (nv + 1) // 2, nv}):
+        apt.aptidx_set_reference(ctx.handle, 0, sig, n_hat)
+        apt.aptidx_build_lut(ctx.handle, 0, np.array([[1.0, 0, 0, 0]]))
+        assert np.array_equal(apt.aptidx_get_lut(ctx.handle, 0, ng=1)[0], want[:n_hat])
+    ctx.close()

@@ -166,10 +166,10 @@ int aptidx_band_for_spacing(double d_min, double d_max, double R, int m, int32_t
  * take the band of the amplitude spectrum and keep its maximum (Section
  * 2.2).  path: APTIDX_PATH_PLAIN_FP32 or APTIDX_PATH_TC_FP16.  flags: any of
  * APTIDX_NORMALISE_MAX; APTIDX_AUTOTUNE (the first call for a new shape --
- * bins, band width, mean ROI size, directions, device -- times candidate
- * launch configurations on the first 8 ROIs per SM and keeps the fastest;
- * with the environment variable APTIDX_TUNE_CACHE naming a file, choices
- * persist across processes); APTIDX_GRAPH (the launches of the call are
+ * bins, band width, mean ROI size, directions, device, number of ROIs up to 8
+ * per SM -- times candidate launch configurations on the first 8 ROIs per SM
+ * and keeps the fastest for the calls of that shape; with the environment
+ * variable APTIDX_TUNE_CACHE naming a file, choices persist across processes); APTIDX_GRAPH (the launches of the call are
  * captured in a CUDA graph on first use for these output pointers and sizes
  * and replayed on later calls; input changes discard the graphs; the
  * profiler of aptidx_set_profiling then books the whole replay, gather and

@@ -329,26 +329,45 @@ static int launch_sequence(Ctx* c, int path, unsigned flags, float* dS, uint16_t
 
 // ---- autotuner ---------------------------------------------------------------
 // Launch configuration per (path, bins, frequency groups of the band, mean
-// ROI size, directions, device): tiles of 64 directions per work item and,
-// on the tensor-core path, the number of MMA issuer warps.  Candidates are
+// ROI size, directions, number of ROIs while they are few, device): tiles of
+// 64 directions per work item and, on the tensor-core path, the number of MMA
+// issuer warps.  Candidates are
 // timed with CUDA events on the first ranks of the ROI order (8 per SM) and
 // the fastest is kept for the context, and in the file named by the
-// environment variable APTIDX_TUNE_CACHE when it is set.
+// environment variable APTIDX_TUNE_CACHE when it is set.  It serves the calls
+// of its own shape; others take the defaults (on the tensor-core path a rule on
+// the sizes) until they are tuned.
 
 static std::string tune_key(Ctx* c, int path) {
     char buf[384];
-    cudaDeviceProp prop;
-    cudaGetDeviceProperties(&prop, c->device);
+    if (c->device_name.empty()) {
+        cudaDeviceProp prop;
+        cudaGetDeviceProperties(&prop, c->device);
+        c->device_name = prop.name;
+    }
     const double mean = c->nroi > 0 ? (double)c->atoms_total / (double)c->nroi : 0.0;
     const int abin = mean > 1.0 ? (int)lround(2.0 * log2(mean)) : 0;
     const int vbin = (int)lround(2.0 * log2((double)std::max(c->nv, 1)));
+    const int nbin = (int)lround(2.0 * log2((double)std::max<int64_t>(1, std::min<int64_t>(c->nroi, 8 * c->sm_count))));
     const int groups = (c->band_max - c->band_min) / 4 + 1;
     const int pairs = c->use_pairs && c->npairs > 0 ? 1 : 0;
-    snprintf(buf, sizeof(buf), "%s/%d|p%d|m%d|g%d|a%d|v%d|s%d", prop.name, prop.multiProcessorCount, path, c->m,
-             groups, abin, vbin, pairs);
+    snprintf(buf, sizeof(buf), "%s/%d|p%d|m%d|g%d|a%d|v%d|s%d|n%d", c->device_name.c_str(), c->sm_count, path, c->m,
+             groups, abin, vbin, pairs, nbin);
     for (char* q = buf; *q; ++q)
         if (*q == ' ') *q = '_';
     return buf;
+}
+
+// The configuration of the current shape: the tuned one, else the defaults.
+static bool tune_apply(Ctx* c, int path) {
+    const int pi = path == APTIDX_PATH_TC_FP16 ? 1 : 0;
+    const Ctx::TuneCfg none{pi ? 0 : 16, 4, 0.f};
+    auto it = c->tune_cache.end();
+    if (!c->tune_cache.empty()) it = c->tune_cache.find(tune_key(c, path));
+    const Ctx::TuneCfg& t = it == c->tune_cache.end() ? none : it->second;
+    c->tune_tpi[pi] = t.tpi;
+    if (pi) c->tune_iss = t.iss;
+    return it != c->tune_cache.end();
 }
 
 static void tune_load(Ctx* c) {
@@ -376,14 +395,9 @@ static void tune_save(Ctx* c) {
 
 static int autotune(Ctx* c, int path, float* dS, uint16_t* dA) {
     tune_load(c);
+    if (tune_apply(c, path)) return APTIDX_OK;
     const int pi = path == APTIDX_PATH_TC_FP16 ? 1 : 0;
     const std::string key = tune_key(c, path);
-    auto it = c->tune_cache.find(key);
-    if (it != c->tune_cache.end()) {
-        c->tune_tpi[pi] = it->second.tpi;
-        if (pi) c->tune_iss = it->second.iss;
-        return APTIDX_OK;
-    }
     int rc;
     if ((rc = run_gather(c))) return rc;
     cudaError_t e = launch_roi_order(c);
@@ -870,6 +884,7 @@ int aptidx_compute_signatures(aptidx_ctx* ctx, int path, unsigned flags, float* 
         dA = argk ? c->d_argk : nullptr;
     }
     if (path == APTIDX_PATH_TC_FP16 && (rc = prepare_tc(c))) return rc;
+    tune_apply(c, path);
     if ((flags & APTIDX_AUTOTUNE) && (rc = autotune(c, path, dS, dA))) return rc;
     if (flags & APTIDX_GRAPH) {
         // capture the sequence once per (arguments, configuration), replay after
@@ -938,6 +953,7 @@ int aptidx_get_tuning(aptidx_ctx* ctx, int path, int32_t* tiles_per_item, int32_
     CTX_OR_FAIL(ctx);
     if (path != APTIDX_PATH_PLAIN_FP32 && path != APTIDX_PATH_TC_FP16)
         return set_error(c, APTIDX_E_INVALID_ARG, "unknown path %d", path);
+    tune_apply(c, path);
     if (tiles_per_item) *tiles_per_item = tuned_tiles_per_item(c, path == APTIDX_PATH_TC_FP16);
     if (issuers) *issuers = path == APTIDX_PATH_TC_FP16 ? c->tune_iss : 0;
     return APTIDX_OK;
@@ -1798,6 +1814,7 @@ int aptidx_compute_signatures_multi(aptidx_ctx* ctx, int path, unsigned flags, i
             restore();
             return rc;
         }
+        tune_apply(c, path);
         if ((rc = launch_sequence(c, path, 0, dS, dA))) {
             restore();
             return rc;

@@ -61,6 +61,7 @@ struct Ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
     int sm_count = 0;
+    std::string device_name;
     std::string err;
 
     // positions
@@ -157,8 +158,8 @@ struct Ctx {
     // status word
     int* d_status = nullptr;
 
-    // launch configuration (tiles per work item per path, MMA issuer warps),
-    // set by the autotuner; rank_limit > 0 restricts a launch to the first
+    // launch configuration of the current shape (tiles per work item per path, MMA
+    // issuer warps), tuned or default; rank_limit > 0 restricts a launch to the first
     // ranks of the ROI order (tuning runs)
     int tune_tpi[2] = {16, 0};         // 0: the rule of the tensor-core launch
     int tune_iss = 4;

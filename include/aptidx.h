@@ -361,7 +361,7 @@ int aptidx_get_tuning(aptidx_ctx* ctx, int path, int32_t* tiles_per_item, int32_
 int aptidx_path_supported(aptidx_ctx* ctx, int path);
 
 /* Phases timed when profiling is on. */
-#define APTIDX_PHASE_GATHER    0   /* ROI count, offsets, gather + centring (a1) */
+#define APTIDX_PHASE_GATHER    0   /* ROI gather + centring (a1) */
 #define APTIDX_PHASE_ORDER     1   /* longest-first ROI order */
 #define APTIDX_PHASE_SIGNATURE 2   /* projection, histogram, spectrum, band max (a2-a5) */
 #define APTIDX_PHASE_NORMALISE 3

@@ -34,21 +34,6 @@ __host__ __device__ __forceinline__ float bin_magic(int m) {
     return 8388608.0f + (float)(1 << (m - 1));
 }
 
-__device__ __forceinline__ int bin_of(float s, float scale, float magic, int nb_minus_1) {
-    int b = __float_as_int(__fmaf_rd(s, scale, magic)) - 0x4B000000;
-    return min(max(b, 0), nb_minus_1);
-}
-
-// The same bin without the clamp, for the histogram loops.  For inputs the
-// library accepts (|u| within 1e-5 of 1, |x| <= R by the FP64 membership
-// test, m <= 10) |s * scale| < 2^(m-1) - 1 + 0.01, so the exact bin lies in
-// [0, 2^m - 1] and the clamp of the contract never acts; the fma result is
-// then 2^23 + b exactly and its low m bits are b.  The mask keeps every
-// shared-memory index in range whatever the input.
-__device__ __forceinline__ uint32_t bin_of_valid(float s, float scale, float magic, uint32_t nb_minus_1) {
-    return __float_as_uint(__fmaf_rd(s, scale, magic)) & nb_minus_1;
-}
-
 // exact small non-negative integer (< 2^23) to float with one integer op and
 // one FP32 add (no conversion-pipe instruction)
 __device__ __forceinline__ float u23_to_float(uint32_t c) {
@@ -59,34 +44,25 @@ __device__ __forceinline__ float u23_to_float(uint32_t c) {
 // directions 2l (low 16 bits) and 2l + 1 (high 16 bits) of the word
 // H[b * 32 + l].  The word of a lane lies in bank l for every bin b, so the
 // 32 atomics of one warp instruction never share a bank.  `hbase` is the
-// shared address of H plus 4 * lane.
-//   kMasked: the bin is masked to m bits (memory-safe for any input).
-//   otherwise: the inputs are known to give bins in range (the library's own
-//   gather and validated directions and radii), and the word address is one
-//   multiply-add of the fma result's bit pattern 0x4B000000 + b.
-template <bool kMasked>
+// shared address of H plus 4 * lane.  The low m bits of the bin fma's pattern are
+// the bin (for inputs the library accepts the clamp of the contract never acts:
+// |u| within 1e-5 of 1 and |x| <= R give |s * scale| < 2^(m-1) - 1 + 0.01); the mask
+// keeps every address in range whatever the input.
 __device__ __forceinline__ void hist_add_atom(uint32_t hbase, float4 a, float4 d0, float4 d1, float scale,
                                               float magic, int nbm1) {
     const float s0 = project_f32(d0.x, d0.y, d0.z, a);
     const float s1 = project_f32(d1.x, d1.y, d1.z, a);
     const uint32_t t0 = __float_as_uint(__fmaf_rd(s0, scale, magic));
     const uint32_t t1 = __float_as_uint(__fmaf_rd(s1, scale, magic));
-    uint32_t w0, w1;
-    if (kMasked) {
-        w0 = hbase + ((t0 & (uint32_t)nbm1) << 7);
-        w1 = hbase + ((t1 & (uint32_t)nbm1) << 7);
-    } else {
-        // (t - 0x4B000000) * 128 + hbase, in wrapping 32-bit arithmetic
-        w0 = t0 * 128u + (hbase - 0x80000000u);
-        w1 = t1 * 128u + (hbase - 0x80000000u);
-    }
+    const uint32_t w0 = hbase + ((t0 & (uint32_t)nbm1) << 7);
+    const uint32_t w1 = hbase + ((t1 & (uint32_t)nbm1) << 7);
     asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(w0), "r"(1u) : "memory");
     asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(w1), "r"(0x10000u) : "memory");
 }
 
 // Histograms of one 64-direction tile over `cn` staged atoms; warp w takes
 // atoms w, w + W, w + 2W, ...
-template <int W, bool kMasked>
+template <int W>
 __device__ __forceinline__ void hist_tile(uint32_t* H, const float4* A, int cn, int warp, int lane, float4 d0,
                                           float4 d1, float scale, float magic, int nbm1) {
     const uint32_t hbase = smem_u32(H) + 4u * (uint32_t)lane;
@@ -97,22 +73,22 @@ __device__ __forceinline__ void hist_tile(uint32_t* H, const float4* A, int cn, 
         float4 a0 = A[j], a1 = A[j + W], a2 = A[j + 2 * W], a3 = A[j + 3 * W];
         for (; j + 7 * W < cn; j += 4 * W) {
             const float4 b0 = A[j + 4 * W], b1 = A[j + 5 * W], b2 = A[j + 6 * W], b3 = A[j + 7 * W];
-            hist_add_atom<kMasked>(hbase, a0, d0, d1, scale, magic, nbm1);
-            hist_add_atom<kMasked>(hbase, a1, d0, d1, scale, magic, nbm1);
-            hist_add_atom<kMasked>(hbase, a2, d0, d1, scale, magic, nbm1);
-            hist_add_atom<kMasked>(hbase, a3, d0, d1, scale, magic, nbm1);
+            hist_add_atom(hbase, a0, d0, d1, scale, magic, nbm1);
+            hist_add_atom(hbase, a1, d0, d1, scale, magic, nbm1);
+            hist_add_atom(hbase, a2, d0, d1, scale, magic, nbm1);
+            hist_add_atom(hbase, a3, d0, d1, scale, magic, nbm1);
             a0 = b0;
             a1 = b1;
             a2 = b2;
             a3 = b3;
         }
-        hist_add_atom<kMasked>(hbase, a0, d0, d1, scale, magic, nbm1);
-        hist_add_atom<kMasked>(hbase, a1, d0, d1, scale, magic, nbm1);
-        hist_add_atom<kMasked>(hbase, a2, d0, d1, scale, magic, nbm1);
-        hist_add_atom<kMasked>(hbase, a3, d0, d1, scale, magic, nbm1);
+        hist_add_atom(hbase, a0, d0, d1, scale, magic, nbm1);
+        hist_add_atom(hbase, a1, d0, d1, scale, magic, nbm1);
+        hist_add_atom(hbase, a2, d0, d1, scale, magic, nbm1);
+        hist_add_atom(hbase, a3, d0, d1, scale, magic, nbm1);
         j += 4 * W;
     }
-    for (; j < cn; j += W) hist_add_atom<kMasked>(hbase, A[j], d0, d1, scale, magic, nbm1);
+    for (; j < cn; j += W) hist_add_atom(hbase, A[j], d0, d1, scale, magic, nbm1);
 }
 
 // Packed FP32 pairs (f32x2): each half is one IEEE FP32 operation with the
@@ -176,12 +152,13 @@ __device__ __forceinline__ bool nonzero_integer_products_possible(float scale, f
 // -----------------------------------------------------------------------------
 // Histogram pass of the signature kernels.  Atoms lie in 64-byte
 // blocks of four (x of the four | y | z | unused), three 16-byte loads that are
-// the FP32 pairs of two packed steps.  The bin fma runs at four times the scale
-// on the integer grid of [2^25, 2^26) (spacing 4): its bit pattern is
-// 0x4C000000 + row, and shifting that left by 7 drops every exponent bit, so
-// one funnel shift with the lane's byte offset in the top seven bits of the low
-// word gives row * 128 + 4 lane, the shared address itself when the magic
-// number carries the histogram's base / 128.  That keeps the address off the
+// the FP32 pairs of two packed steps.  The bin fma runs at 1024 times the scale
+// on the integer grid of [2^33, 2^34) (spacing 1024): its bit pattern is
+// 0x50000000 + row, and shifting that left by 7 (5 for tiles of 16 directions, whose
+// rows are a quarter as long) drops every exponent bit -- the grid of [2^25, 2^26),
+// 0x4C000000, would keep one --, so one funnel shift with the lane's byte offset in the
+// top bits of the low word gives row * 128 + 4 lane, the shared address itself when the
+// magic number carries the histogram's base / 128.  That keeps the address off the
 // FMA pipe, which a multiply-add of the pattern loads as much as four packed
 // FMAs do per atom pair.
 // -----------------------------------------------------------------------------

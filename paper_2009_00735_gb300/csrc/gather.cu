@@ -3,10 +3,11 @@
 // The paper queries the atoms of each ROI with a tree (supplement, cost term
 // N_roi f R^3 rho log(V rho)).  Here the positions are bucketed once into a
 // uniform cell grid (counting sort, cells ordered by atom index so results
-// are deterministic), and one warp per ROI scans the cells that overlap the
-// ROI's sphere.  Membership is the FP64 closed-ball test
-// (dx*dx + dy*dy) + dz*dz <= R*R without fused multiply-add, and the centred
-// coordinates x_i - p_c are rounded once to FP32 (Eq. 1: p_i - p_c).
+// are deterministic), and one CTA per ROI walks the rows of cells that its
+// sphere touches.  Membership is the FP64 closed-ball test
+// (dx*dx + dy*dy) + dz*dz <= R*R without fused multiply-add, decided in FP32 where
+// that is certain to agree, and the centred coordinates x_i - p_c are formed in FP64
+// and rounded once to FP32 (Eq. 1: p_i - p_c).
 #include <float.h>
 
 #include "common.cuh"

@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_plain(SigParams p) {
                 if (!one_chunk && !stage(src + s0, cn, nullptr)) return false;
                 if (kSafe) {
                     if (nchunk == 1)
-                        hist_tile<kWarps, true>(H, A, cn, warp, lane, d0, d1, scale, magic, nbm1);
+                        hist_tile<kWarps>(H, A, cn, warp, lane, d0, d1, scale, magic, nbm1);
                     else
                         hist_tile_chunk<kWarps>(H, A, cn, warp, lane, d0, d1, scale, magic, (uint32_t)nbm1, (uint32_t)bc);
                 } else if (nchunk == 1) {

@@ -694,7 +694,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_wide(TcParams p) {
     unsigned char* BT = smem + (size_t)NBc * 128;
     float* EX = reinterpret_cast<float*>(BT + p.bt_bytes);   // [kDirs][8]
     float4* A = reinterpret_cast<float4*>(BT + p.bt_bytes + kExBytes);
-    float4* DB = A + p.atom_cap;   // [2][parity][32]: this tile's directions and the next tile's
+    float4* DB = A + p.atom_cap;   // [2][kDirs]: this tile's directions and the next tile's
     int2* DI = reinterpret_cast<int2*>(DB + 2 * kDirs);   // [2][kDirs]: (output, partner) of those slots
     float* EX2 = reinterpret_cast<float*>(DI + 2 * kDirs);   // [128][8]
     // barriers: [0] atoms, then four stage loads and four stage MMA completions

@@ -1556,11 +1556,12 @@ int aptidx_match_topk(aptidx_ctx* ctx, int32_t cand, const float* S, int64_t nro
     if (topk == 1) {
         if ((rc = match_best(c, r, dS, nroi, db, ds, &launches))) return rc;
     } else if (round > 0) {
-        float* rows = c->d_match_scratch + (size_t)round * (r.ng + 1) + 1;
+        // the rows first: whole groups of 64, so that both they and the estimates start on a line
+        float *rows = c->d_match_scratch, *est = rows + (size_t)round * r.ng;
         for (int64_t r0 = 0; r0 < nroi; r0 += round) {
             const int64_t n = std::min(round, nroi - r0);
-            cudaError_t e = launch_tm_sum(c, &r, dS + r0 * c->nv, n, c->d_match_scratch);
-            if (e == cudaSuccess) e = launch_tm_rows(c, &r, dS + r0 * c->nv, n, topk, c->d_match_scratch, rows);
+            cudaError_t e = launch_tm_sum(c, &r, dS + r0 * c->nv, n, est);
+            if (e == cudaSuccess) e = launch_tm_rows(c, &r, dS + r0 * c->nv, n, topk, est, rows);
             if (e == cudaSuccess) e = launch_topk(c, rows, r.ng, n, topk, db + r0 * topk, ds ? ds + r0 * topk : nullptr);
             if (e != cudaSuccess) return cuda_check(c, e, "match_topk");
             launches += 4;

@@ -1764,6 +1764,7 @@ int aptidx_compute_signatures_multi(aptidx_ctx* ctx, int path, unsigned flags, i
                 c->atoms_cap = total;
             }
             c->layout_mask = umask;
+            c->nw_max = std::max(c->nw_max, nwmax);
             if ((rc = read_status(c))) return rc;
         }
     }

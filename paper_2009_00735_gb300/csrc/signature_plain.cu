@@ -103,8 +103,10 @@ struct SigParams {
 // Folded partial spectrum of kKpw frequencies from k0 over the bins j0 .. j0 +
 // span - 1 from the middle (and their three images), for the lane's two
 // directions: re = sum e cos, im = sum o sin.  TW2[i] = (cos, sin)(pi i / N),
-// i < 2 N; kOdd = k0 & 1.
-template <int kOdd>
+// i < 2 N; kOdd = k0 & 1.  Bound by issue; kUnroll bins a step: 8 where the bins are
+// split among warps (512 ROIs x 40962 directions, four frequencies: 8.65 ms by 2, 8.44),
+// 3 where a warp walks them all (100 ROIs x 10242, k = 8..100: 4.65, 4.41).
+template <int kOdd, int kUnroll>
 __device__ __forceinline__ void fold_dft(const uint32_t* H, const float2* TW2, int NB, int lane, int j0, int span,
                                          int k0, float (&re)[kKpw][2], float (&im)[kKpw][2]) {
     const unsigned mask = 2u * (unsigned)NB - 1u;
@@ -115,7 +117,7 @@ __device__ __forceinline__ void fold_dft(const uint32_t* H, const float2* TW2, i
     const uint32_t* hb = H + (NB / 2 + j0) * kWords + lane;       // b: above the middle
     const uint32_t* hc = H + j0 * kWords + lane;                  // c: from the first bin
     const uint32_t* hd = H + (NB - 1 - j0) * kWords + lane;       // d: from the last bin
-#pragma unroll 2
+#pragma unroll kUnroll
     for (int j = 0; j < span; ++j) {
         const uint32_t wa = *ha, wc = *hc;
         const uint32_t s1 = wa + *hb, s2 = wc + *hd;   // 16-bit halves: no carry, a histogram holds at most 65535 atoms
@@ -150,14 +152,19 @@ __device__ __forceinline__ void fold_dft(const uint32_t* H, const float2* TW2, i
 
 // kNB: band slots of the epilogue (1: the ROI's own band; APTIDX_MAX_BANDS:
 // the pass's BandSet).  kSafe: atoms and directions come from the caller
-// unchecked, so bins are masked to m bits (memory-safe for any input).
-template <int kNB, bool kSafe>
+// unchecked, so bins are masked to m bits (memory-safe for any input).  kMode: which
+// ROIs of a launch take the passes over bin chunks and atom blocks (all above 2^10
+// bins, those above kBlockAtoms atoms, none); registers are short, and each loop is
+// faster in an instance without the other (by 2 to 5 %).
+enum { kSinglePass, kMixed, kAllPasses };
+
+template <int kNB, bool kSafe, int kMode>
 __global__ void __launch_bounds__(kThreads, 1) k_sig_plain(SigParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
     const int NB = 1 << p.m;
     const int nbm1 = NB - 1;
     const int NBc = NB < kChunkBins ? NB : kChunkBins;   // histogram rows held at once
-    const int nchunk = NB / NBc;
+    const int nchunk = kMode == kSinglePass ? 1 : NB / NBc;
     const int ntw = nchunk == 1 ? 2 * NB : NB;   // half-step angles for the folded sum
     uint32_t* H = reinterpret_cast<uint32_t*>(smem);
     float2* TW = reinterpret_cast<float2*>(smem + (size_t)NBc * kWords * 4);
@@ -271,7 +278,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_plain(SigParams p) {
             }
         };
 
-        const bool multi_pass = nchunk > 1 || nw > kBlockAtoms;
+        const bool multi_pass = kMode == kAllPasses || (kMode == kMixed && (nchunk > 1 || nw > kBlockAtoms));
         for (int tile = t0; tile < t1; ++tile) {
             bool partners = sym && multi_pass;   // a partner pass is due
             for (int pass = 0; pass < 2; ++pass) {
@@ -294,7 +301,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_plain(SigParams p) {
                     // full-step angles: with half steps in the table the index runs in
                     // twos.  Bound by issue: the index scaled at every look-up and no
                     // unrolling cost 10 % each (60 ROIs, 10242 directions, 2^12 bins,
-                    // k = 8..60: 34.8 ms, now 28.0)
+                    // k = 8..60: 34.8 ms, now 26.5)
                     const unsigned tws = nchunk == 1 ? 2u : 1u, tmask = tws * (unsigned)NB - 1u;
                     float best[kNB];
                     int bk[kNB];
@@ -402,9 +409,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_plain(SigParams p) {
 #pragma unroll
                         for (int i = 0; i < kKpw; ++i) re[i][0] = re[i][1] = im[i][0] = im[i][1] = 0.f;
                         if (k0 & 1)
-                            fold_dft<1>(H, TW, NB, lane, sp * span, span, k0, re, im);
+                            fold_dft<1, 8>(H, TW, NB, lane, sp * span, span, k0, re, im);
                         else
-                            fold_dft<0>(H, TW, NB, lane, sp * span, span, k0, re, im);
+                            fold_dft<0, 8>(H, TW, NB, lane, sp * span, span, k0, re, im);
 #pragma unroll
                         for (int i = 0; i < kKpw; ++i) {
                             PART[((size_t)warp * kKpw + i) * kDirs + 2 * lane] = make_float2(re[i][0], im[i][0]);
@@ -443,9 +450,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_sig_plain(SigParams p) {
 #pragma unroll
                         for (int i = 0; i < kKpw; ++i) re[i][0] = re[i][1] = im[i][0] = im[i][1] = 0.f;
                         if (k0 & 1)
-                            fold_dft<1>(H, TW, NB, lane, 0, NB / 4, k0, re, im);
+                            fold_dft<1, 3>(H, TW, NB, lane, 0, NB / 4, k0, re, im);
                         else
-                            fold_dft<0>(H, TW, NB, lane, 0, NB / 4, k0, re, im);
+                            fold_dft<0, 3>(H, TW, NB, lane, 0, NB / 4, k0, re, im);
 #pragma unroll
                         for (int i = 0; i < kKpw; ++i) {
                             if (k0 + i > khi) break;
@@ -553,7 +560,12 @@ cudaError_t launch_signatures_plain(Ctx* c, float* S, uint16_t* argk, uint16_t* 
     if (cap < 256) return cudaErrorInvalidConfiguration;
     const size_t smem = plain_smem_bytes(c->m, cap);
     const bool multi = !hist_out && c->multi.n > 0;
-    auto kern = multi ? k_sig_plain<APTIDX_MAX_BANDS, false> : k_sig_plain<1, false>;
+    const int mode = c->m > 10 ? kAllPasses : c->nw_max > kBlockAtoms ? kMixed : kSinglePass;
+    void (*const kerns[2][3])(SigParams) = {
+        {k_sig_plain<1, false, kSinglePass>, k_sig_plain<1, false, kMixed>, k_sig_plain<1, false, kAllPasses>},
+        {k_sig_plain<APTIDX_MAX_BANDS, false, kSinglePass>, k_sig_plain<APTIDX_MAX_BANDS, false, kMixed>,
+         k_sig_plain<APTIDX_MAX_BANDS, false, kAllPasses>}};
+    void (*const kern)(SigParams) = kerns[multi][mode];
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
 
@@ -731,7 +743,7 @@ extern "C" int aptidx_signatures_noalloc(const float* xc4, const int64_t* off, c
     cap = std::min(cap, 4096) & ~15;
     if (cap < 256) return APTIDX_E_CUDA;
     const size_t smem = plain_smem_bytes(m, cap);
-    if (cudaFuncSetAttribute(k_sig_plain<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    if (cudaFuncSetAttribute(k_sig_plain<1, true, kMixed>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
         return APTIDX_E_CUDA;
     }
@@ -760,9 +772,9 @@ extern "C" int aptidx_signatures_noalloc(const float* xc4, const int64_t* off, c
     p.atom_cap = cap;
     p.nroi = nroi;
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sig_plain<1, true>, kThreads, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sig_plain<1, true, kMixed>, kThreads, smem);
     per_sm = std::max(per_sm, 1);
     const int64_t grid = std::min<int64_t>((int64_t)sm_count * per_sm, p.n_items);
-    k_sig_plain<1, true><<<(unsigned)grid, kThreads, smem, s>>>(p);
+    k_sig_plain<1, true, kMixed><<<(unsigned)grid, kThreads, smem, s>>>(p);
     return cudaGetLastError() == cudaSuccess ? APTIDX_OK : APTIDX_E_CUDA;
 }

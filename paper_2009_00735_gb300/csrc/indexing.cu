@@ -1409,8 +1409,9 @@ cudaError_t launch_top_nodes(Ctx* c, Reference* r) {
 // The node grid of the directions, queued on the stream: cells of one and a half node
 // spacings of an even covering (0.02 to 0.5), which hold a few nodes each.  Built here
 // and not with the directions: signatures do not need it (on the host it took
-// set_directions 0.85 of 6.6 ms for 40962 directions).
-static int ensure_node_grid(Ctx* c) {
+// set_directions 0.85 of 6.6 ms for 40962 directions).  `scratch` (idle on the
+// stream) holds the counts when it is large enough.
+static int ensure_node_grid(Ctx* c, void* scratch, size_t scratch_bytes) {
     if (c->d_nodes) return APTIDX_OK;
     const double h = std::min(0.5, std::max(0.02, 1.5 * sqrt(4.0 * M_PI / (double)c->nv)));
     c->node_org = -1.0001f;
@@ -1419,8 +1420,9 @@ static int ensure_node_grid(Ctx* c) {
     c->node_far2 = (float)(c->dir_max2 - 0.998 / ((double)c->node_inv_h * (double)c->node_inv_h));
     const size_t cells = (size_t)c->node_dim * c->node_dim * c->node_dim;
     const NodeGrid g{nullptr, nullptr, c->node_dim, c->node_org, c->node_inv_h, c->node_far2};
-    int64_t* work = nullptr;   // counts | offsets | the scan's sums
-    int rc = dev_alloc(c, (void**)&work, (2 * cells + 1 + scan_tmp_elems(cells) + 1) * sizeof(int64_t));
+    const size_t bytes = (2 * cells + 1 + scan_tmp_elems(cells) + 1) * sizeof(int64_t);
+    int64_t* work = static_cast<int64_t*>(scratch);   // counts | offsets | the scan's sums
+    int rc = scratch_bytes >= bytes ? APTIDX_OK : dev_alloc(c, (void**)&work, bytes);
     if (!rc) rc = dev_alloc(c, (void**)&c->d_nodes, (size_t)c->nv * sizeof(float4) + (cells + 1) * sizeof(int32_t));
     if (!rc) {
         c->d_node_start = reinterpret_cast<int32_t*>(c->d_nodes + c->nv);
@@ -1442,7 +1444,7 @@ static int ensure_node_grid(Ctx* c) {
             c->d_nodes = nullptr;
         }
     }
-    dev_recycle(c, work);
+    if (work != scratch) dev_recycle(c, work);
     return rc;
 }
 
@@ -1458,10 +1460,14 @@ static cudaError_t launch_build_lut_t(Ctx* c, Reference* r, const double* d_quat
     bool by_grid = (double)ng * r->n_hat * c->nv > 2e8;
     const std::string err = c->err;
     if (by_grid) {
-        int rc = ensure_node_grid(c);
-        if (!rc) rc = dev_alloc(c, (void**)&open, (size_t)(rows * ng + 1) * sizeof(uint32_t));
+        const size_t bytes = (size_t)(rows * ng + 1) * sizeof(uint32_t);
+        int rc = dev_alloc(c, (void**)&open, bytes);
+        if (!rc) rc = ensure_node_grid(c, open, bytes);
         by_grid = rc == APTIDX_OK;
-        if (rc && rc != APTIDX_E_OOM) return cudaErrorUnknown;
+        if (rc && rc != APTIDX_E_OOM) {
+            dev_recycle(c, open);
+            return cudaErrorUnknown;
+        }
         c->err = err;
     }
     const NodeGrid grid{c->d_node_start, c->d_nodes, c->node_dim, c->node_org, c->node_inv_h, c->node_far2};

@@ -269,7 +269,10 @@ int aptidx_set_reference(aptidx_ctx* ctx, int32_t cand, const float* node_sig, i
 /* Look-up table of candidate `cand` for test orientations quats (ng x 4
  * FP64 unit quaternions (w, x, y, z), mapping crystal to lab): entry
  * (g, k) = the direction index nearest to R(q_g) n_k for the k-th strongest
- * reference node n_k.  Errors: INVALID_ARG, STATE, OOM, CUDA. */
+ * reference node n_k.  Beside tables that aptidx_match reads by lists the
+ * library keeps the lists and a copy of the table (three times its memory),
+ * which it frees when another call of the context finds no memory.  Errors:
+ * INVALID_ARG, STATE, OOM, CUDA. */
 int aptidx_build_lut(aptidx_ctx* ctx, int32_t cand, const double* quats, int64_t ng, int mem);
 
 /* Debug/parity: the look-up table of candidate `cand`, lut[g * n_hat + k]
@@ -279,8 +282,10 @@ int aptidx_get_lut(aptidx_ctx* ctx, int32_t cand, int32_t* lut, int32_t* n_hat_o
 /* Eq. 3 for every ROI: Delta(g) = sum_k (S[roi, lut[g, k]] - ref[n_k])^2
  * over the candidate's look-up table; best[roi] = argmin_g (ties: lowest
  * g), score[roi] = Delta(best).  S: nroi x nv FP32 normalised signatures in
- * `mem`; best: nroi int32; score: nroi FP32 (NULL to skip).  Errors:
- * INVALID_ARG, STATE, OOM, CUDA. */
+ * `mem`; best: nroi int32; score: nroi FP32 (NULL to skip).  Calls of many
+ * ROIs stage estimates of Delta on the device (at most 1 GiB, library-owned;
+ * without that memory, and on a stream being captured, they take the way of
+ * few ROIs, with the same results).  Errors: INVALID_ARG, STATE, OOM, CUDA. */
 int aptidx_match(aptidx_ctx* ctx, int32_t cand, const float* S, int64_t nroi, int32_t* best,
                  float* score, int mem);
 

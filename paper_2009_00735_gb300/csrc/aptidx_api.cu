@@ -515,10 +515,6 @@ int aptidx_destroy(aptidx_ctx* ctx) {
     free_ptr(c->d_pos);
     free_ptr(c->d_types);
     free_ptr(c->d_dirs);
-    free_ptr(c->d_dirs_sorted);
-    free_ptr(c->d_slot_dirs);
-    free_ptr(c->d_slot_idx);
-    free_ptr(c->d_nodes);
     free_ptr(c->d_gn_scratch);
     c->gn_scratch_bytes = 0;
     free_ptr(c->d_match_scratch);
@@ -700,24 +696,36 @@ int aptidx_set_directions(aptidx_ctx* ctx, const float* u, int32_t nv, int mem) 
             si.push_back(make_int2(-1, -1));
         }
     }
-    free_ptr(c->d_dirs);
-    free_ptr(c->d_dirs_sorted);
-    free_ptr(c->d_slot_dirs);
-    free_ptr(c->d_slot_idx);
-    free_ptr(c->d_nodes);
+    recycle_ptr(c, c->d_dirs);
+    c->d_dirs_sorted = c->d_slot_dirs = c->d_nodes = nullptr;
+    c->d_slot_idx = nullptr;
     clear_graphs(c);
-    c->dir_max2 = umax2;
+    // node grid: cells of one and a half node spacings of an even covering (0.02 to
+    // 0.5), which hold a few nodes each
+    const double h = std::min(0.5, std::max(0.02, 1.5 * sqrt(4.0 * M_PI / (double)nv)));
+    c->node_org = -1.0001f;
+    c->node_inv_h = (float)(1.0 / h);
+    c->node_dim = (int)(2.0002 * (double)c->node_inv_h) + 1;
+    c->node_far2 = (float)(umax2 - 0.998 / ((double)c->node_inv_h * (double)c->node_inv_h));
+    const size_t cells = (size_t)c->node_dim * c->node_dim * c->node_dim;
     c->nv = c->nv_pad = 0;
     c->nslot = c->nslot_pad = c->npairs = 0;
-    if ((rc = dev_alloc(c, (void**)&c->d_dirs, (size_t)nv_pad * sizeof(float4)))) return rc;
-    if ((rc = dev_alloc(c, (void**)&c->d_dirs_sorted, (size_t)nv * sizeof(float4)))) return rc;
+    // one block: directions | in spatial order | room for the grid's nodes | slots | their
+    // indices | room for the grid's cells (a block of its own costs the first table 0.1 ms)
+    if ((rc = dev_alloc(c, (void**)&c->d_dirs,
+                        ((size_t)nv_pad + 2 * (size_t)nv + sd.size()) * sizeof(float4) + si.size() * sizeof(int2) +
+                            (cells + 1) * sizeof(int32_t))))
+        return rc;
+    c->d_dirs_sorted = c->d_dirs + nv_pad;
+    float4* slots = c->d_dirs_sorted + 2 * (size_t)nv;
+    c->d_node_start = reinterpret_cast<int32_t*>(reinterpret_cast<int2*>(slots + sd.size()) + si.size());
     APTIDX_CUDA(c, cudaMemcpyAsync(c->d_dirs, d4.data(), (size_t)nv_pad * sizeof(float4), cudaMemcpyHostToDevice,
                                    c->stream));
     APTIDX_CUDA(c, cudaMemcpyAsync(c->d_dirs_sorted, ds.data(), (size_t)nv * sizeof(float4), cudaMemcpyHostToDevice,
                                    c->stream));
     if (npairs > 0) {
-        if ((rc = dev_alloc(c, (void**)&c->d_slot_dirs, sd.size() * sizeof(float4)))) return rc;
-        if ((rc = dev_alloc(c, (void**)&c->d_slot_idx, si.size() * sizeof(int2)))) return rc;
+        c->d_slot_dirs = slots;
+        c->d_slot_idx = reinterpret_cast<int2*>(slots + sd.size());
         APTIDX_CUDA(c, cudaMemcpyAsync(c->d_slot_dirs, sd.data(), sd.size() * sizeof(float4), cudaMemcpyHostToDevice,
                                        c->stream));
         APTIDX_CUDA(c, cudaMemcpyAsync(c->d_slot_idx, si.data(), si.size() * sizeof(int2), cudaMemcpyHostToDevice,

@@ -1407,46 +1407,35 @@ cudaError_t launch_top_nodes(Ctx* c, Reference* r) {
     return e;
 }
 
-// The node grid of the directions, queued on the stream: cells of one and a half node
-// spacings of an even covering (0.02 to 0.5), which hold a few nodes each.  Built here
-// and not with the directions: signatures do not need it (on the host it took
-// set_directions 0.85 of 6.6 ms for 40962 directions).  `scratch` (idle on the
-// stream) holds the counts when it is large enough.
+// The node grid of the directions, queued on the stream.  Filled here and not with the
+// directions: signatures do not need it (on the host it took set_directions 0.85 of 6.6
+// ms for 40962 directions).  `scratch` (idle on the stream) holds the counts when it is
+// large enough.
 static int ensure_node_grid(Ctx* c, void* scratch, size_t scratch_bytes) {
     if (c->d_nodes) return APTIDX_OK;
-    const double h = std::min(0.5, std::max(0.02, 1.5 * sqrt(4.0 * M_PI / (double)c->nv)));
-    c->node_org = -1.0001f;
-    c->node_inv_h = (float)(1.0 / h);
-    c->node_dim = (int)(2.0002 * (double)c->node_inv_h) + 1;
-    c->node_far2 = (float)(c->dir_max2 - 0.998 / ((double)c->node_inv_h * (double)c->node_inv_h));
     const size_t cells = (size_t)c->node_dim * c->node_dim * c->node_dim;
     const NodeGrid g{nullptr, nullptr, c->node_dim, c->node_org, c->node_inv_h, c->node_far2};
     const size_t bytes = (2 * cells + 1 + scan_tmp_elems(cells) + 1) * sizeof(int64_t);
     int64_t* work = static_cast<int64_t*>(scratch);   // counts | offsets | the scan's sums
-    int rc = scratch_bytes >= bytes ? APTIDX_OK : dev_alloc(c, (void**)&work, bytes);
-    if (!rc) rc = dev_alloc(c, (void**)&c->d_nodes, (size_t)c->nv * sizeof(float4) + (cells + 1) * sizeof(int32_t));
-    if (!rc) {
-        c->d_node_start = reinterpret_cast<int32_t*>(c->d_nodes + c->nv);
-        unsigned long long* counts = reinterpret_cast<unsigned long long*>(work);
-        int64_t* off = work + cells;
-        cudaError_t e = cudaMemsetAsync(counts, 0, cells * sizeof(int64_t), c->stream);
-        if (e == cudaSuccess) {
-            k_node_count<<<(unsigned)((c->nv + 255) / 256), 256, 0, c->stream>>>(c->d_dirs, c->nv, g, counts);
-            e = launch_scan_i64(work, off, (int64_t)cells, off + cells + 1, c->stream);
-        }
-        if (e == cudaSuccess) {
-            k_node_fill<<<(unsigned)c->sm_count * 8, 256, 0, c->stream>>>(c->d_dirs, c->nv, g, (int)cells, off, counts,
-                                                                         c->d_node_start, c->d_nodes);
-            e = cudaGetLastError();
-        }
-        if (e != cudaSuccess) {
-            rc = cuda_check(c, e, "node grid");
-            dev_free(c->d_nodes);
-            c->d_nodes = nullptr;
-        }
+    if (scratch_bytes < bytes)
+        if (int rc = dev_alloc(c, (void**)&work, bytes)) return rc;
+    float4* nodes = c->d_dirs_sorted + c->nv;
+    unsigned long long* counts = reinterpret_cast<unsigned long long*>(work);
+    int64_t* off = work + cells;
+    cudaError_t e = cudaMemsetAsync(counts, 0, cells * sizeof(int64_t), c->stream);
+    if (e == cudaSuccess) {
+        k_node_count<<<(unsigned)((c->nv + 255) / 256), 256, 0, c->stream>>>(c->d_dirs, c->nv, g, counts);
+        e = launch_scan_i64(work, off, (int64_t)cells, off + cells + 1, c->stream);
+    }
+    if (e == cudaSuccess) {
+        k_node_fill<<<(unsigned)c->sm_count * 8, 256, 0, c->stream>>>(c->d_dirs, c->nv, g, (int)cells, off, counts,
+                                                                     c->d_node_start, nodes);
+        e = cudaGetLastError();
     }
     if (work != scratch) dev_recycle(c, work);
-    return rc;
+    if (e != cudaSuccess) return cuda_check(c, e, "node grid");
+    c->d_nodes = nodes;
+    return APTIDX_OK;
 }
 
 // The table in runs of rows of at most 2^24 queries, so that the list of open

@@ -79,7 +79,8 @@ struct Ctx {
     int64_t* d_cell_start = nullptr;   // [n_cells + 1]
     float4* d_cell_pos = nullptr;      // [n] positions in cell order, w = type (as float)
 
-    // directions (padded to a multiple of kTileDirs with (1, 0, 0))
+    // directions (padded to a multiple of kTileDirs with (1, 0, 0)); the block also holds
+    // the other arrays of the directions below
     int32_t nv = 0, nv_pad = 0;
     float4* d_dirs = nullptr;
     // the same directions in a spatially coherent order (Morton order of 1-degree
@@ -94,11 +95,10 @@ struct Ctx {
     int2* d_slot_idx = nullptr;
     int32_t nslot = 0, nslot_pad = 0, npairs = 0;
     bool use_pairs = true;           // cleared by APTIDX_DIRECT for one call
-    double dir_max2 = 0.0;             // largest |u|^2 of the directions
-    // the directions in a cubic grid of cells for nearest-node queries, built for the
-    // first table that takes it; null before
-    float4* d_nodes = nullptr;         // [nv] in cell order, w = index bits; the cells' starts behind
-    int32_t* d_node_start = nullptr;   // [node_dim^3 + 1], part of d_nodes
+    // the directions in a cubic grid of cells for nearest-node queries, filled for the
+    // first table that takes it, null before
+    float4* d_nodes = nullptr;         // [nv] in cell order, w = index bits
+    int32_t* d_node_start = nullptr;   // [node_dim^3 + 1]
     int node_dim = 0;
     float node_org = 0.f, node_inv_h = 0.f, node_far2 = 0.f;
     float* d_gn_scratch = nullptr;   // one signature row per refinement CTA, in the order above

@@ -48,7 +48,7 @@
 // stores in place of the atomics change it).  Over the whole kernel 60 % of the issue
 // slots, 65 % of the shared-memory cycles.  One CTA per SM ran these phases one
 // after the other with the counts in shared memory: 13.5 K cycles, 116.5 ms for 8192
-// ROIs x 40962 directions; now 74.4 ms.
+// ROIs x 40962 directions; now 73.9 ms.
 #include <cuda_fp16.h>
 
 #include "tcgen05.cuh"
